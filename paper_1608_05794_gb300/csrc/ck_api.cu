@@ -224,6 +224,7 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     r.lA2 = (double)(std::log2((long double)a[0]));
     r.beta = a[1];
     r.EoR2 = (double)((long double)a[2] / (Rg * ln2));
+    r.EoR = r.EoR2 * LN2;
     r.type = (int8_t)d->rtype[i];
     r.rev = (int8_t)d->reversible[i];
     if (r.rev == 2) {
@@ -238,11 +239,14 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
       r.lA02 = (double)(std::log2((long double)a0[0]));
       r.beta0 = a0[1];
       r.E0oR2 = (double)((long double)a0[2] / (Rg * ln2));
+      r.E0oR = r.E0oR2 * LN2;
     }
     int nr = 0, np = 0;
     for (int s = 0; s < 3; ++s) {
-      r.sp[s] = (int16_t)d->reac[i * 3 + s];
-      r.sp[3 + s] = (int16_t)d->prod[i * 3 + s];
+      // empty slots hold species S, whose entries the team kernels set to the
+      // neutral element of the product or sum they enter
+      r.sp[s] = (int16_t)(d->reac[i * 3 + s] >= 0 ? d->reac[i * 3 + s] : S);
+      r.sp[3 + s] = (int16_t)(d->prod[i * 3 + s] >= 0 ? d->prod[i * 3 + s] : S);
       nr += d->reac[i * 3 + s] >= 0;
       np += d->prod[i * 3 + s] >= 0;
     }
@@ -352,7 +356,7 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
         ent[sb + 0 * S + k].push_back({nu, li});
         ent[sb + 1 * S + k].push_back({nu, chunk + li});
         ent[sb + 2 * S + k].push_back({nu, 2 * chunk + li});
-        ent[sb + 3 * S + k].push_back({nu, pbase + 6});
+        if (r.type) ent[sb + 3 * S + k].push_back({nu, pbase + 6});
       }
     }
     std::vector<int> order_e;

@@ -20,29 +20,34 @@ constexpr double INV_LN2 = 1.4426950408889634074;
 constexpr double R_OVER_P0 = R_GAS / P_STD;               // R T / p0 is the molar volume at p0, m^3/mol
 constexpr double P0_OVER_R = P_STD / R_GAS;
 
-// One reaction, 96 bytes, read uniformly by all lanes (thread-per-reactor
-// kernels) or by one lane per reaction (team kernels).  The loader sorts the
-// reactions by (type, reversible, reactant count, product count) so that
-// neighbouring lanes of a team kernel take the same branches.
+// One reaction, 112 bytes, read uniformly by all lanes (thread-per-reactor
+// kernels) or by one lane per reaction (team kernels, in 16-byte loads; the
+// last two hold the fall-off limit and are loaded for fall-off reactions
+// only).  The loader sorts the reactions by (type, reversible, reactant
+// count, product count) so that neighbouring lanes of a team kernel take the
+// same branches.
 struct __align__(16) RxnRec {
   double lA2;    // log2 A (SI)
   double beta;   // temperature exponent
   double EoR2;   // Ea / (R ln 2), K
-  double lA02;   // Lindemann low-pressure limit: log2 A0
-  double beta0;
-  double E0oR2;
-  double dnu_d;    // sum of product minus reactant coefficients, as FP64
-  double nreac_d;  // reactant count, as FP64
-  double nprod_d;  // product count, as FP64
-  int16_t sp[6];    // reactant slots 0..2, product slots 3..5, -1 padded
+  double EoR;    // EoR2 * LN2 (as rounded by that product): d ln k_f/dT
+  int16_t sp[6];    // reactant slots 0..2, product slots 3..5, padded with S
   int8_t type;      // 0 elementary, 1 third-body, 2 Lindemann
   int8_t rev;       // 1 reversible through K_c, 2 explicit reverse Arrhenius
   int8_t dnu;
-  int8_t nreac, nprod, pad0;
+  int8_t nreac;
+  int8_t nprod, pad0;
   int16_t eff_beg, eff_cnt;  // slice of the efficiency table (eff - 1 != 0)
   int16_t rev_ix;            // rev == 2: row of the explicit reverse table
+  double dnu_d;    // sum of product minus reactant coefficients, as FP64
+  double nreac_d;  // reactant count, as FP64
+  double nprod_d;  // product count, as FP64
+  double lA02;   // Lindemann low-pressure limit: log2 A0
+  double beta0;
+  double E0oR2;
+  double E0oR;   // E0oR2 * LN2
 };
-static_assert(sizeof(RxnRec) == 96, "RxnRec layout");
+static_assert(sizeof(RxnRec) == 112, "RxnRec layout");
 
 // Jacobian partials stored per reaction: reactant slots 0..2, product slots
 // 3..5, and slot 6 = dc/d[M] * (k_f prod' - k_r prod'').

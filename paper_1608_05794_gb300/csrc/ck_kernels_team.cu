@@ -20,7 +20,7 @@ __global__ void k_jacobian(const __grid_constant__ DevMech d, int64_t N, const d
   double* J = sm;
   double* ys = J + (size_t)n * n;
   double* fs = ys + n;
-  TeamBufs b = carve_bufs(fs + n, d.S, d.chunk);
+  TeamBufs b = carve_bufs(fs + n, d.S, d.chunk, d.chunk);
   Mix x;
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
@@ -43,7 +43,7 @@ __global__ void k_jacobian_fd(const __grid_constant__ DevMech d, int64_t N, cons
   double* fs = ys + n;
   double* yt = fs + n;
   double* ft = yt + n;
-  TeamBufs b = carve_bufs(ft + n, d.S, d.chunk);
+  TeamBufs b = carve_bufs(ft + n, d.S, d.chunk, d.chunk);
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
     __syncthreads();
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
   double* yv = sm;
   double* yt = yv + n;
   double* kk = yt + n;  // six stages, n each
-  TeamBufs b = carve_bufs(kk + 6 * n, d.S, d.chunk);
+  TeamBufs b = carve_bufs(kk + 6 * n, d.S, d.chunk, 64);
   Mix x;
   const bool fixed = sp.fixed_h > 0.0;
   const int tid = threadIdx.x, P = blockDim.x;

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(G * G, G == 8 ? 6 : 1) k_ros4(const __grid_con
   int* piv = reinterpret_cast<int*>(invd + n);
   // the LU's scratch (lu_scratch_words: at most 578 doubles) reuses the
   // team buffers, free while factoring (9 S + 10 chunk + 48 >= 688 doubles)
-  TeamBufs b = carve_bufs(invd + n + (n + 1) / 2, d.S, d.chunk);
+  TeamBufs b = carve_bufs(invd + n + (n + 1) / 2, d.S, d.chunk, d.chunk);
   float* M32 = reinterpret_cast<float*>(M);  // PREC >= 1: FP32 factors over the FP64 matrix
   double* Mg = m64g ? m64g + (size_t)blockIdx.x * ros4_scratch_doubles(n) : nullptr;
   const bool keep_j = Mg != nullptr && sp.jac == 0;

@@ -29,26 +29,54 @@ __device__ __forceinline__ double team_sum(double v, double* red) {
   return s;
 }
 
-// K block-wide sums at once (each in the order of team_sum, so the values
-// are those of K calls), with one pair of barriers.  K <= 4, blockDim <= 256.
-template <int K>
-__device__ __forceinline__ void team_sum_n(double (&v)[K], double* red) {
+// Butterfly sums of 2, 4 or 8 values over the 32 lanes of a warp, packed:
+// after the first exchange each half of the warp carries half of the values,
+// and so on, so that 4 sums cost 6 adds instead of 20 (an FP64 add costs the
+// warp 64 cycles of its pipe however few lanes carry something useful).
+// Every value is summed by the same tree as warp_allsum (strides 16, 8, 4,
+// 2, 1; only the order of the two operands of an add may differ), so the sums
+// are bitwise those of warp_allsum.  The sum of value q ends in every lane
+// whose leading lane bits (16 first) spell q: lane q * (32 / N) holds it.
+__device__ __forceinline__ double pack_step(double keep_lo, double keep_hi, int o) {
+  const bool hi = (threadIdx.x & o) != 0;
+  return (hi ? keep_hi : keep_lo) + __shfl_xor_sync(0xffffffffu, hi ? keep_lo : keep_hi, o);
+}
+__device__ __forceinline__ double warp_sum_pack2(double a, double b) {
+  double v = pack_step(a, b, 16);
 #pragma unroll
-  for (int q = 0; q < K; ++q) v[q] = warp_allsum(v[q]);
-  const int nw = blockDim.x >> 5;
-  if (nw == 1) return;
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_sum_pack4(double a, double b, double c, double d) {
+  double v = pack_step(pack_step(a, c, 16), pack_step(b, d, 16), 8);
 #pragma unroll
-    for (int q = 0; q < K; ++q) red[8 * q + (threadIdx.x >> 5)] = v[q];
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ double warp_sum_pack8(const double (&a)[8]) {
+  const double p0 = pack_step(a[0], a[4], 16), p1 = pack_step(a[1], a[5], 16);
+  const double p2 = pack_step(a[2], a[6], 16), p3 = pack_step(a[3], a[7], 16);
+  double v = pack_step(pack_step(p0, p2, 8), pack_step(p1, p3, 8), 4);
+#pragma unroll
+  for (int o = 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// A sum over the species taken by one warp: g[q] holds the part of lanes 32 q
+// to 32 q + 31 of a team of b.vp threads; the parts are summed each by the
+// warp tree and then in order, as team_sum does.  ng parts (1..4), the rest
+// must be zero.  The total reaches every lane.
+__device__ __forceinline__ double warp_sum_groups(const double (&g)[4], int ng) {
+  if (ng == 1) return warp_allsum(g[0]);
+  if (ng == 2) {
+    const double v = warp_sum_pack2(g[0], g[1]);
+    return __shfl_sync(0xffffffffu, v, 0) + __shfl_sync(0xffffffffu, v, 16);
   }
-  __syncthreads();
-#pragma unroll
-  for (int q = 0; q < K; ++q) {
-    double s = 0.0;
-    for (int i = 0; i < nw; ++i) s += red[8 * q + i];
-    v[q] = s;
-  }
+  const double v = warp_sum_pack4(g[0], g[1], g[2], g[3]);
+  double s = __shfl_sync(0xffffffffu, v, 0) + __shfl_sync(0xffffffffu, v, 8);
+  s += __shfl_sync(0xffffffffu, v, 16);
+  if (ng > 3) s += __shfl_sync(0xffffffffu, v, 24);
+  return s;
 }
 
 __device__ __forceinline__ void team_sync() {
@@ -60,230 +88,254 @@ __device__ __forceinline__ void team_sync() {
 // The Jacobian processes reactions in chunks of m.chunk (64 if n <= 56, else
 // 256), so the per-reaction arrays hold one chunk; the right-hand side, which
 // keeps one value per reaction, uses them as one array of 10 m.chunk values
-// when all reactions fit.  cs aliases Gp (free once the reaction passes are
-// done).  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k = (S/R -
-// H/RT)_k / ln 2, so that 1/K_c of Eq. kc is a product of species factors.
+// when all reactions fit.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
+// (S/R - H/RT)_k / ln 2, so that 1/K_c of Eq. kc is a product of species
+// factors.  Entry S of X, Gp, Gm (1) and hRT (0) stands for an empty reaction
+// slot.  After the reaction passes of the Jacobian, X, Gp and Gm are reused
+// (dense, cs, eW).
 struct TeamBufs {
-  double *X, *Gp, *hRT, *cpR, *Gm, *wd, *aT, *E, *u, *cs;  // [S]
-  double *q, *dqT, *D;                                        // [chunk]
-  double* P;                                                  // [chunk * JP] Jacobian partials
-  double* red;                                                // [48]
+  double *X, *Gp, *Gm, *hRT;              // [S + 1]
+  double *cpR, *wd, *aT, *E, *u;          // [S]; wd, aT, E, u contiguous
+  double *q, *dqT, *D;                    // [chunk]
+  double* P;                              // [chunk * JP] Jacobian partials
+  double* red;                            // [TEAM_RED] reductions and scalars (SC_*)
+  int vp;                                 // lanes that the species sums are grouped by (64 or 256)
+};
+
+// Scalars of one evaluation, formed once by one warp (an FP64 instruction
+// costs every warp that issues it a full slot) and read by all from red[].
+constexpr int TEAM_RED = 64;
+enum : int {
+  SC_INVT = 32, SC_LNT, SC_LOG2T, SC_T2, SC_T3, SC_T4,  // functions of T
+  SC_PW,                                                // (R T / p0)^dnu, dnu = -2..2
+  SC_WBAR = SC_PW + 5, SC_RHO, SC_INVRHO, SC_CTOT,      // mixture
+  SC_TDOT, SC_ICPM, SC_POW,
+  SC_SUM = 52                                           // the Jacobian's seven species sums
 };
 
 // Mixture quantities shared by the RHS and the Jacobian.
 struct Mix {
-  double T, invT, lnT, log2T, T2, T3, T4, rho, invrho, Wbar, Ctot;
-  double dcpm;  // this thread's part of sum_k Y_k/W_k d(cp_k/R)/dT (Jacobian only)
+  double T, invT, log2T, rho, invrho, Wbar, Ctot;
 };
 
+// Groups of 32 species (at most 4).
+__device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
+
 // Species pass: rho, [X_k], Gibbs / enthalpy / heat-capacity polynomials.
+// The mixture (a chain of sums and divisions) and the functions of T (a chain
+// through log T) are formed side by side by two warps, everything else of
+// the species by all of them: a polynomial pass of 32 species is one work
+// item, dealt to the warps in turn.
 __device__ __forceinline__ void team_species(const DevMech& m, double p, const double* y,
-                                             TeamBufs& b, Mix& x, bool want_dcp, const double* tab) {
-  const int S = m.S;
-  x.T = y[0];
-  // the temperature functions are formed by the first warp alone (an FP64
-  // instruction costs every warp that issues it a full slot) and handed to
-  // the others through red[40..45] across the barriers of the sum below
-  double* tf = b.red + 40;
-  if (threadIdx.x < 32) {
-    x.invT = rcp_rn(x.T);
-    x.lnT = log(x.T);
-    x.log2T = x.lnT * INV_LN2;
-    x.T2 = x.T * x.T;
-    x.T3 = x.T2 * x.T;
-    x.T4 = x.T3 * x.T;
-    if (threadIdx.x == 0) {
-      tf[0] = x.invT;
-      tf[1] = x.lnT;
-      tf[2] = x.log2T;
-      tf[3] = x.T2;
-      tf[4] = x.T3;
-      tf[5] = x.T4;
+                                             TeamBufs& b, Mix& x, const double* tab) {
+  const int S = m.S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int SG = species_groups(S);
+  double* red = b.red;
+  const double T = y[0];
+  x.T = T;
+  if (warp == nw - 1) {
+    const double invT = rcp_rn(T), lnT = log(T);
+    const double T2 = T * T, T3 = T2 * T;
+    const double up = T * R_OVER_P0, dn = invT * P0_OVER_R;
+    if (lane == 0) {
+      red[SC_INVT] = invT;
+      red[SC_LNT] = lnT;
+      red[SC_LOG2T] = lnT * INV_LN2;
+      red[SC_T2] = T2;
+      red[SC_T3] = T3;
+      red[SC_T4] = T3 * T;
+      red[SC_PW] = dn * dn;
+      red[SC_PW + 1] = dn;
+      red[SC_PW + 2] = 1.0;
+      red[SC_PW + 3] = up;
+      red[SC_PW + 4] = up * up;
     }
   }
-  double s = 0.0;
-  for (int k = threadIdx.x; k < S; k += blockDim.x) s = fma(y[1 + k], m.invW[k], s);
-  const double sumYW = team_sum(s, b.red);
-  if (threadIdx.x >= 32) {
-    x.invT = tf[0];
-    x.lnT = tf[1];
-    x.log2T = tf[2];
-    x.T2 = tf[3];
-    x.T3 = tf[4];
-    x.T4 = tf[5];
-  }
-  // the mean molar mass, rho and 1 / rho likewise by the first warp,
-  // through red[32..34]
-  double* sc = b.red + 32;
-  if (threadIdx.x < 32) {
-    x.Wbar = rcp_rn(sumYW);
-    x.rho = m.cv ? p : p / (R_GAS * x.T * sumYW);  // constant volume: p is the density
-    x.invrho = rcp_rn(x.rho);
-    if (threadIdx.x == 0) {
-      sc[0] = x.Wbar;
-      sc[1] = x.rho;
-      sc[2] = x.invrho;
+  if (warp == 0) {
+    double yw[4], part[4] = {0.0, 0.0, 0.0, 0.0};
+    const bool fold = b.vp == 64;  // species 64 + t joins species t in its lane's part
+    const int ng = fold && SG > 2 ? 2 : SG;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      yw[q] = 0.0;
+      if (q < SG) {
+        const int k = 32 * q + lane;
+        const double yk = k < S ? y[1 + k] : 0.0, iw = k < S ? m.invW[k] : 0.0;
+        yw[q] = yk * iw;
+        if (q >= 2 && fold) part[q - 2] = fma(yk, iw, part[q - 2]);
+        else part[q] = yw[q];
+      }
+    }
+    const double sumYW = warp_sum_groups(part, ng);
+    const double Wbar = rcp_rn(sumYW);
+    const double rho = m.cv ? p : p / (R_GAS * T * sumYW);  // constant volume: p is the density
+    const double invrho = rcp_rn(rho);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) part[q] = 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < SG) {
+        const int k = 32 * q + lane;
+        const double xk = k < S ? rho * yw[q] : 0.0;
+        if (k < S) b.X[k] = xk;
+        if (q >= 2 && fold) part[q - 2] += xk;
+        else part[q] = xk;
+      }
+    const double Ctot = warp_sum_groups(part, ng);
+    if (lane == 0) {
+      red[SC_WBAR] = Wbar;
+      red[SC_RHO] = rho;
+      red[SC_INVRHO] = invrho;
+      red[SC_CTOT] = Ctot;
+      b.X[S] = b.Gp[S] = b.Gm[S] = 1.0;
+      b.hRT[S] = 0.0;
     }
   }
-  if (blockDim.x > 32) {
-    __syncthreads();
-    if (threadIdx.x >= 32) {
-      x.Wbar = sc[0];
-      x.rho = sc[1];
-      x.invrho = sc[2];
+  for (int k = threadIdx.x; k < 4 * S; k += blockDim.x) b.wd[k] = 0.0;  // wd, aT, E, u
+  team_sync();
+  x.invT = red[SC_INVT];
+  x.log2T = red[SC_LOG2T];
+  x.Wbar = red[SC_WBAR];
+  x.rho = red[SC_RHO];
+  x.invrho = red[SC_INVRHO];
+  x.Ctot = red[SC_CTOT];
+  const double lnT = red[SC_LNT], T2 = red[SC_T2], T3 = red[SC_T3], T4 = red[SC_T4];
+  for (int it = warp; it < 2 * SG; it += nw) {
+    const bool gibbs = it < SG;
+    const int k = 32 * (gibbs ? it : it - SG) + lane;
+    if (k < S) {
+      const double* a = m.thermo + k * TH_PER_SPECIES + (T < m.tmid[k] ? 0 : TH_STRIDE);
+      if (gibbs) {
+        double g = fma(a[11], lnT, a[12]);
+        g = fma(a[13], T, g);
+        g = fma(a[14], T2, g);
+        g = fma(a[15], T3, g);
+        g = fma(a[16], T4, g);
+        g = fma(a[17], x.invT, g);
+        ck_exp2_pm(g, tab, b.Gp[k], b.Gm[k]);
+      } else {
+        b.cpR[k] = fma(a[4], T4, fma(a[3], T3, fma(a[2], T2, fma(a[1], T, a[0]))));
+        b.hRT[k] = fma(a[10], x.invT, fma(a[9], T4, fma(a[8], T3, fma(a[7], T2, fma(a[6], T, a[5])))));
+      }
     }
   }
-  double c = 0.0, dcpm = 0.0;
-  for (int k = threadIdx.x; k < S; k += blockDim.x) {
-    const double xk = x.rho * (y[1 + k] * m.invW[k]);
-    b.X[k] = xk;
-    c += xk;
-    const double* a = m.thermo + k * TH_PER_SPECIES + (x.T < m.tmid[k] ? 0 : TH_STRIDE);
-    double g = fma(a[11], x.lnT, a[12]);
-    g = fma(a[13], x.T, g);
-    g = fma(a[14], x.T2, g);
-    g = fma(a[15], x.T3, g);
-    g = fma(a[16], x.T4, g);
-    g = fma(a[17], x.invT, g);
-    ck_exp2_pm(g, tab, b.Gp[k], b.Gm[k]);
-    b.cpR[k] = fma(a[4], x.T4, fma(a[3], x.T3, fma(a[2], x.T2, fma(a[1], x.T, a[0]))));
-    b.hRT[k] = fma(a[10], x.invT, fma(a[9], x.T4, fma(a[8], x.T3, fma(a[7], x.T2, fma(a[6], x.T, a[5])))));
-    if (want_dcp)
-      dcpm = fma(y[1 + k] * m.invW[k], fma(4.0 * a[4], x.T3, fma(3.0 * a[3], x.T2, fma(2.0 * a[2], x.T, a[1]))), dcpm);
-    b.wd[k] = 0.0;
-    b.aT[k] = 0.0;
-    b.E[k] = 0.0;
-    b.u[k] = 0.0;
-  }
-  x.dcpm = dcpm;
-  x.Ctot = team_sum(c, b.red);
 }
 
-// A 96-byte reaction record in six 16-byte loads (the fields are then read
-// from registers).
+// A reaction record without its fall-off limit (the last two vectors) in
+// 16-byte loads; the fields are then read from registers.
 __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
   RxnRec r;
   const int4* s = reinterpret_cast<const int4*>(src);
   int4* t = reinterpret_cast<int4*>(&r);
 #pragma unroll
-  for (int q = 0; q < 6; ++q) t[q] = __ldg(s + q);
+  for (int q = 0; q < 5; ++q) t[q] = __ldg(s + q);
   return r;
 }
 
-// Rates of one reaction at the mixture state.  With want_jac also the
-// partial-derivative pieces used by the Jacobian (see team_jacobian).
-__device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec& r, const Mix& x,
-                                              const TeamBufs& b, const double* tab, int i,
-                                              bool want_jac) {
-  // i: index of the reaction inside the current chunk
+// Rates of one reaction at the mixture state.  JAC: also the partial-
+// derivative pieces used by the Jacobian (see team_jacobian).  i: index of
+// the reaction inside the current chunk.  Empty slots read the neutral
+// entries of the species arrays (a product with 1, a sum with 0, exact), so
+// that reactions of every molecularity take the same instructions.
+template <bool JAC>
+__device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
+                                              const TeamBufs& b, const double* tab, int i) {
+  const RxnRec r = load_rxn(src);
   const double* X = b.X;
   const double l2kf = fma(-r.EoR2, x.invT, fma(r.beta, x.log2T, r.lA2));
   const double kf = ck_exp2(l2kf, tab);
-  double fwd = X[r.sp[0]];
-  if (r.nreac > 1) fwd *= X[r.sp[1]];
-  if (r.nreac > 2) fwd *= X[r.sp[2]];
+  const int s0 = r.sp[0], s1 = r.sp[1], s2 = r.sp[2], s3 = r.sp[3], s4 = r.sp[4], s5 = r.sp[5];
+  const double x0 = X[s0], x1 = X[s1], x2 = X[s2], y0 = X[s3], y1 = X[s4], y2 = X[s5];
+  const double fwd = x0 * x1 * x2;
   double kr = 0.0, rv = 0.0, dlnkc = 0.0;
   if (r.rev == 2) {
     // explicit reverse Arrhenius; for the Jacobian, d ln k_r/dT enters as
     // d ln k_f/dT - d ln K_c/dT, so dlnkc carries their difference
     const double* ra = m.revp + 3 * r.rev_ix;
     kr = ck_exp2(fma(-ra[2], x.invT, fma(ra[1], x.log2T, ra[0])), tab);
-    rv = X[r.sp[3]];
-    if (r.nprod > 1) rv *= X[r.sp[4]];
-    if (r.nprod > 2) rv *= X[r.sp[5]];
-    if (want_jac) {
-      const double dlnkf = fma(r.EoR2 * LN2, x.invT, r.beta) * x.invT;
+    rv = y0 * y1 * y2;
+    if (JAC) {
+      const double dlnkf = fma(r.EoR, x.invT, r.beta) * x.invT;
       dlnkc = dlnkf - fma(ra[2] * LN2, x.invT, ra[1]) * x.invT;
     }
   } else if (r.rev) {
     // 1/K_c = (R T/p0)^dnu prod_reactants Gp prod_products Gm (Eq. kc)
-    double kci = rt_over_p0_pow(r.dnu, x.T, x.invT) * b.Gp[r.sp[0]];
-    kci *= b.Gm[r.sp[3]];
-    if (r.nreac > 1) kci *= b.Gp[r.sp[1]];
-    if (r.nprod > 1) kci *= b.Gm[r.sp[4]];
-    if (r.nreac > 2) kci *= b.Gp[r.sp[2]];
-    if (r.nprod > 2) kci *= b.Gm[r.sp[5]];
+    double kci = b.red[SC_PW + 2 + r.dnu] * b.Gp[s0];
+    kci *= b.Gm[s3];
+    kci *= b.Gp[s1];
+    kci *= b.Gm[s4];
+    kci *= b.Gp[s2];
+    kci *= b.Gm[s5];
     kr = kf * kci;
-    rv = X[r.sp[3]];
-    if (r.nprod > 1) rv *= X[r.sp[4]];
-    if (r.nprod > 2) rv *= X[r.sp[5]];
-    if (want_jac) {
+    rv = y0 * y1 * y2;
+    if (JAC) {
       // d ln K_c / dT = (sum_j nu_j H_j/(R T) - dnu) / T
-      double hs = b.hRT[r.sp[3]];
-      if (r.nprod > 1) hs += b.hRT[r.sp[4]];
-      if (r.nprod > 2) hs += b.hRT[r.sp[5]];
-      hs -= b.hRT[r.sp[0]];
-      if (r.nreac > 1) hs -= b.hRT[r.sp[1]];
-      if (r.nreac > 2) hs -= b.hRT[r.sp[2]];
+      double hs = b.hRT[s3];
+      hs += b.hRT[s4];
+      hs += b.hRT[s5];
+      hs -= b.hRT[s0];
+      hs -= b.hRT[s1];
+      hs -= b.hRT[s2];
       dlnkc = (hs - r.dnu_d) * x.invT;
     }
   }
   const double net = fma(-kr, rv, kf * fwd);
-  double c = 1.0, dcdM = 0.0, dcdT = 0.0, M = 0.0;
-  const double dlnkf = fma(r.EoR2 * LN2, x.invT, r.beta) * x.invT;
+  double q = net, ckf = kf, ckr = kr, w = 0.0, M = 0.0, dcdT = 0.0;
+  const double dlnkf = fma(r.EoR, x.invT, r.beta) * x.invT;
   if (r.type) {
+    double c, dcdM;
     M = x.Ctot;
     for (int e = r.eff_beg; e < r.eff_beg + r.eff_cnt; ++e) M = fma(m.eff_m1[e], X[m.eff_sp[e]], M);
     if (r.type == 1) {
       c = M;
       dcdM = 1.0;
     } else {
-      const double l2k0 = fma(-r.E0oR2, x.invT, fma(r.beta0, x.log2T, r.lA02));
+      const double2 f0 = __ldg(reinterpret_cast<const double2*>(src) + 5);  // lA02, beta0
+      const double2 f1 = __ldg(reinterpret_cast<const double2*>(src) + 6);  // E0oR2, E0oR
+      const double l2k0 = fma(-f1.x, x.invT, fma(f0.y, x.log2T, f0.x));
       const double k0_kf = ck_exp2(l2k0 - l2kf, tab);
       const double Pr = k0_kf * M;
       const double inv1p = rcp_rn(1.0 + Pr);
       c = Pr * inv1p;
       dcdM = k0_kf * inv1p * inv1p;
-      if (want_jac) {
-        const double dlnk0 = fma(r.E0oR2 * LN2, x.invT, r.beta0) * x.invT;
-        dcdT = Pr * (dlnk0 - dlnkf) * inv1p * inv1p;
+      if (JAC) {
+        const double ds = fma(fma(f1.y, x.invT, f0.y), x.invT, -dlnkf);
+        dcdT = Pr * ds * inv1p * inv1p;
       }
     }
+    q = c * net;
+    if (JAC) {
+      ckf = c * kf;
+      ckr = c * kr;
+      w = dcdM * net;
+      b.P[(size_t)i * JP + 6] = w;
+    }
   }
-  const double q = c * net;
   b.q[i] = q;
-  if (want_jac) {
-    const double ckf = c * kf, ckr = c * kr;
-    const double w = dcdM * net;
+  if (JAC) {
     // d q / d[X] slot by slot: c k_f prod of the other reactant slots, and
     // -c k_r prod of the other product slots
     double* P = b.P + (size_t)i * JP;
-    const double x0 = X[r.sp[0]];
-    if (r.nreac == 1) {
-      P[0] = ckf;
-    } else if (r.nreac == 2) {
-      const double x1 = X[r.sp[1]];
-      P[0] = ckf * x1;
-      P[1] = ckf * x0;
-    } else {
-      const double x1 = X[r.sp[1]], x2 = X[r.sp[2]];
-      P[0] = ckf * (x1 * x2);
-      P[1] = ckf * (x0 * x2);
-      P[2] = ckf * (x0 * x1);
-    }
+    P[0] = ckf * (x1 * x2);
+    P[1] = ckf * (x0 * x2);
+    P[2] = ckf * (x0 * x1);
     if (r.rev) {
-      const double y0 = X[r.sp[3]];
-      if (r.nprod == 1) {
-        P[3] = -ckr;
-      } else if (r.nprod == 2) {
-        const double y1 = X[r.sp[4]];
-        P[3] = -ckr * y1;
-        P[4] = -ckr * y0;
-      } else {
-        const double y1 = X[r.sp[4]], y2 = X[r.sp[5]];
-        P[3] = -ckr * (y1 * y2);
-        P[4] = -ckr * (y0 * y2);
-        P[5] = -ckr * (y0 * y1);
-      }
+      P[3] = -ckr * (y1 * y2);
+      P[4] = -ckr * (y0 * y2);
+      P[5] = -ckr * (y0 * y1);
     }
-    P[6] = w;
     // D = sum_j dq/d[X_j] [X_j]: Euler's theorem for the mass-action
     // products (homogeneous of degree nreac / nprod) plus the [M] part.
-    const double D = fma(ckf * fwd, r.nreac_d, -(ckr * rv) * r.nprod_d) + M * w;
-    b.D[i] = D;
+    double D = fma(ckf * fwd, r.nreac_d, -(ckr * rv) * r.nprod_d);
     // dq/dT at fixed [X], then the total derivative at fixed Y (d[X]/dT =
     // -[X]/T at constant pressure, 0 at constant volume)
-    const double dqTX = fma(dcdT, net, ckf * fwd * dlnkf - ckr * rv * (dlnkf - dlnkc));
+    const double tA = __dmul_rn(ckf, fwd), tB = __dmul_rn(ckr, rv);
+    double dqTX = fma(tA, dlnkf, -__dmul_rn(tB, __dadd_rn(dlnkf, -dlnkc)));
+    if (r.type) {
+      D = fma(M, w, D);
+      dqTX = fma(dcdT, net, dqTX);
+    }
+    b.D[i] = D;
     b.dqT[i] = m.cv ? dqTX : fma(-D, x.invT, dqTX);
   }
 }
@@ -292,39 +344,37 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec& r,
 static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p,
                                              const double* y, double* f, TeamBufs b) {
   Mix x;
-  team_species(m, p, y, b, x, false, tab);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int S = m.S, SG = species_groups(S);
+  team_species(m, p, y, b, x, tab);
   team_sync();
+  const double invrho = x.invrho;
   const int NC = m.n_chunks, CH = m.chunk;
   if (m.R <= (3 + JP) * CH) {
     // the right-hand side needs one value per reaction, so the whole chunk
     // scratch (q, dqT, D, P are contiguous) holds every rate of progress at
     // once: one reaction pass and one gather, two barriers in all.  The
     // gather sums in the same order as the chunked form below.
-    for (int i = threadIdx.x; i < m.R; i += blockDim.x) {
-      const RxnRec r = load_rxn(m.rxn + i);
-      team_reaction(m, r, x, b, tab, i, false);
-    }
+    for (int i = threadIdx.x; i < m.R; i += blockDim.x) team_reaction<false>(m, m.rxn + i, x, b, tab, i);
     team_sync();
-    for (int kk = threadIdx.x; kk < m.S; kk += blockDim.x) {
+    for (int kk = threadIdx.x; kk < S; kk += blockDim.x) {
       const int k = m.rsp[kk];
-      double w = b.wd[k];
+      double w = 0.0;
       for (int e = m.csr_ptr[k]; e < m.csr_ptr[k + 1]; ++e) {
         const CsrTerm t = m.csr[e];
         w = fma(t.nu, b.q[t.rx], w);
       }
       b.wd[k] = w;
+      f[1 + k] = w * (m.W[k] * invrho);
     }
     team_sync();
   } else {
     for (int c = 0; c < NC; ++c) {
       const int base = c * CH;
       for (int li = threadIdx.x; li < CH; li += blockDim.x)
-        if (base + li < m.R) {
-          const RxnRec r = load_rxn(m.rxn + base + li);
-          team_reaction(m, r, x, b, tab, li, false);
-        }
+        if (base + li < m.R) team_reaction<false>(m, m.rxn + base + li, x, b, tab, li);
       team_sync();
-      for (int k = threadIdx.x; k < m.S; k += blockDim.x) {
+      for (int k = threadIdx.x; k < S; k += blockDim.x) {
         const int* cp = m.csr_cptr + k * (NC + 1) + c;
         double w = b.wd[k];
         for (int e = cp[0]; e < cp[1]; ++e) {
@@ -332,24 +382,50 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
           w = fma(t.nu, b.q[t.rx - base], w);
         }
         b.wd[k] = w;
+        if (c == NC - 1) f[1 + k] = w * (m.W[k] * invrho);
       }
       team_sync();
     }
   }
-  const double invrho = x.invrho;
-  const double cvf = m.cv ? 1.0 : 0.0;  // constant volume: U/RT = H/RT - 1, cv/R = cp/R - 1
-  double cpm = 0.0, hw = 0.0;
-  for (int k = threadIdx.x; k < m.S; k += blockDim.x) {
-    const double w = b.wd[k];
-    cpm = fma(y[1 + k] * m.invW[k], b.cpR[k] - cvf, cpm);
-    hw = fma(b.hRT[k] - cvf, w, hw);
-    f[1 + k] = w * (m.W[k] * invrho);
+  // dT/dt by the last warp: its two species sums and the division.  Constant
+  // volume: U/RT = H/RT - 1, cv/R = cp/R - 1.
+  if (warp == nw - 1) {
+    double cpm[4] = {0.0, 0.0, 0.0, 0.0}, hw[4] = {0.0, 0.0, 0.0, 0.0};
+    const bool fold = b.vp == 64;
+    const int ng = fold && SG > 2 ? 2 : SG;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q < SG) {
+        const int k = 32 * q + lane;
+        if (k < S) {
+          double c = b.cpR[k], h = b.hRT[k];
+          if (m.cv) {
+            c -= 1.0;
+            h -= 1.0;
+          }
+          const double yk = y[1 + k] * m.invW[k], w = b.wd[k];
+          if (q >= 2 && fold) {
+            cpm[q - 2] = fma(yk, c, cpm[q - 2]);
+            hw[q - 2] = fma(h, w, hw[q - 2]);
+          } else {
+            cpm[q] = fma(yk, c, 0.0);
+            hw[q] = fma(h, w, 0.0);
+          }
+        }
+      }
+    double sc, sh;
+    if (ng <= 2) {
+      const double v = warp_sum_pack4(cpm[0], cpm[1], hw[0], hw[1]);
+      // lanes 0-15: cpm, 16-31: hw, both from one add
+      const double s = v + __shfl_xor_sync(0xffffffffu, v, 8);
+      sc = __shfl_sync(0xffffffffu, s, 0);
+      sh = __shfl_sync(0xffffffffu, s, 16);
+    } else {
+      sc = warp_sum_groups(cpm, ng);
+      sh = warp_sum_groups(hw, ng);
+    }
+    if (lane == 0) f[0] = -x.T * sh / (x.rho * sc);
   }
-  double sums[2] = {cpm, hw};
-  team_sum_n(sums, b.red);
-  cpm = sums[0];
-  hw = sums[1];
-  if (threadIdx.x == 0) f[0] = -x.T * hw / (x.rho * cpm);
   team_sync();
 }
 
@@ -370,10 +446,12 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 //   J[1+k][1+j] = W_k (A_kj + u_k) / W_j,   J[1+k][0] = W_k a_k / rho,
 //   J[0][1+j]   = -(T cs_j / cvm + Tdot cv_j / cvm) / W_j,
 //   J[0][0]     = -(sum cv_k wdot_k + T sum U_k/RT a_k)/(rho cvm) - Tdot dcpm/cvm.
+// Needs b.vp >= S (one species a lane in the sums).
 static __device__ void team_jacobian(const DevMech& m, const double* tab, double p, const double* y,
                               double* f, double* J, TeamBufs& b, Mix& x) {
-  const int S = m.S, n = m.n;
-  team_species(m, p, y, b, x, true, tab);
+  const int S = m.S, n = m.n, SG = species_groups(S);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  team_species(m, p, y, b, x, tab);
   // species block A starts at zero (the whole matrix is cleared: the
   // temperature row and column are written whole further down); chunk by
   // chunk, every entry touched by the chunk and every species sum (wdot,
@@ -386,10 +464,7 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
   for (int c = 0; c < NC; ++c) {
     const int base = c * CH;
     for (int li = threadIdx.x; li < CH; li += blockDim.x)
-      if (base + li < m.R) {
-        const RxnRec r = load_rxn(m.rxn + base + li);
-        team_reaction(m, r, x, b, tab, li, true);
-      }
+      if (base + li < m.R) team_reaction<true>(m, m.rxn + base + li, x, b, tab, li);
     team_sync();
     // every target of the chunk (species-block entries and the per-species
     // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
@@ -406,62 +481,68 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
     }
     team_sync();
   }
-  // column sums for the temperature row, and the RHS itself.  Constant
-  // volume: rho is fixed, so every term that comes from d rho/dT or
+  // Constant volume: rho is fixed, so every term that comes from d rho/dT or
   // d rho/dY (cpf) drops out, and U/RT = H/RT - 1, cv/R = cp/R - 1 take the
   // places of H/RT and cp/R (cvf).  The contributions were pre-scaled by
   // W_k/W_j, so J holds A'_kj = W_k A_kj / W_j here.
   const double invrho = x.invrho;
   const double cvf = m.cv ? 1.0 : 0.0, cpf = 1.0 - cvf;
-  double cpm = 0.0, hw = 0.0, he = 0.0, dcpm = x.dcpm, cw = 0.0, ha = 0.0, eu = 0.0;
+  double* eW = b.Gm;     // e_k / W_k, for the column sums
+  double* dense = b.X;   // dense part of the species block, W_k u_k + W_k Wbar (wdot_k - E_k) / rho
+  double* cs = b.Gp;
   for (int k = threadIdx.x; k < S; k += blockDim.x) {
-    const double yk = y[1 + k] * m.invW[k];
-    const double e = b.hRT[k] - cvf, c = b.cpR[k] - cvf;
-    cpm = fma(yk, c, cpm);
-    hw = fma(e, b.wd[k], hw);
-    he = fma(b.hRT[k], b.E[k], he);
-    cw = fma(c, b.wd[k], cw);
-    ha = fma(e, b.aT[k], ha);
-    eu = fma(e, b.u[k], eu);
     f[1 + k] = b.wd[k] * (m.W[k] * invrho);
-    // per row: e_k / W_k for the column sums, and the dense part of the
-    // species block, W_k u_k + W_k Wbar (wdot_k - E_k) / rho (constant p)
-    b.hRT[k] = e * m.invW[k];
-    b.u[k] = m.W[k] * fma(cpf * x.Wbar * invrho, b.wd[k] - b.E[k], b.u[k]);
-  }
-  double s4[4] = {cpm, dcpm, hw, he}, s3[3] = {cw, ha, eu};
-  team_sum_n(s4, b.red);
-  team_sum_n(s3, b.red);
-  cpm = s4[0];
-  dcpm = s4[1];
-  hw = s4[2];
-  he = s4[3];
-  cw = s3[0];
-  ha = s3[1];
-  eu = s3[2];
-  // Tdot and 1 / cpm by the first warp, handed over through red[35..36]
-  // across the barrier below
-  double Tdot = 0.0, inv_cpm = 0.0;
-  double* sc = b.red + 32;
-  if (threadIdx.x < 32) {
-    Tdot = -x.T * hw / (x.rho * cpm);
-    inv_cpm = rcp_rn(cpm);
-    if (threadIdx.x == 0) {
-      sc[3] = Tdot;
-      sc[4] = inv_cpm;
-    }
-  }
-  // cs_j = sum_k e_k (A_kj + u_k) = W_j sum_k (e_k / W_k) A'_kj + sum_k e_k u_k
-  for (int j = threadIdx.x; j < S; j += blockDim.x) {
-    double s = 0.0;
-    for (int k = 0; k < S; ++k) s = fma(b.hRT[k], J[(size_t)(1 + k) * n + 1 + j], s);
-    b.cs[j] = fma(m.W[j], s, eu);
+    eW[k] = (b.hRT[k] - cvf) * m.invW[k];
+    dense[k] = m.W[k] * fma(cpf * x.Wbar * invrho, b.wd[k] - b.E[k], b.u[k]);
   }
   team_sync();
-  if (threadIdx.x >= 32) {
-    Tdot = sc[3];
-    inv_cpm = sc[4];
+  // the last warp: the seven species sums (cpm, dcpm, hw, he, cw, ha, eu),
+  // Tdot and 1 / cpm; the others: cs'_j = sum_k (e_k / W_k) A'_kj
+  double* sums = b.red + SC_SUM;
+  if (warp == nw - 1) {
+    const double T2 = b.red[SC_T2], T3 = b.red[SC_T3];
+    double sv = 0.0;  // lane q: sum q over the groups so far
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      if (g < SG) {
+        const int k = 32 * g + lane;
+        double v[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        if (k < S) {
+          const double* a = m.thermo + k * TH_PER_SPECIES + (x.T < m.tmid[k] ? 0 : TH_STRIDE);
+          const double yk = y[1 + k] * m.invW[k];
+          const double e = b.hRT[k] - cvf, c = b.cpR[k] - cvf;
+          v[0] = fma(yk, c, 0.0);
+          v[1] = fma(yk, fma(4.0 * a[4], T3, fma(3.0 * a[3], T2, fma(2.0 * a[2], x.T, a[1]))), 0.0);
+          v[2] = fma(e, b.wd[k], 0.0);
+          v[3] = fma(b.hRT[k], b.E[k], 0.0);
+          v[4] = fma(c, b.wd[k], 0.0);
+          v[5] = fma(e, b.aT[k], 0.0);
+          v[6] = fma(e, b.u[k], 0.0);
+        }
+        const double s = warp_sum_pack8(v);  // lane 4 q holds sum q
+        sv = g == 0 ? s : sv + s;
+      }
+    const double cpm = __shfl_sync(0xffffffffu, sv, 0), hw = __shfl_sync(0xffffffffu, sv, 8);
+    const double Tdot = -x.T * hw / (x.rho * cpm);
+    const double inv_cpm = rcp_rn(cpm);
+    if ((lane & 3) == 0 && lane < 28) sums[lane >> 2] = sv;
+    if (lane == 0) {
+      b.red[SC_TDOT] = Tdot;
+      b.red[SC_ICPM] = inv_cpm;
+    }
   }
+  // (a team of one warp does both; otherwise the column sums start at warp 0)
+  for (int g = warp; g < SG; g += nw) {
+    const int j = 32 * g + lane;
+    if (j < S) {
+      double s = 0.0;
+      for (int k = 0; k < S; ++k) s = fma(eW[k], J[(size_t)(1 + k) * n + 1 + j], s);
+      cs[j] = s;
+    }
+  }
+  team_sync();
+  const double dcpm = sums[1], he = sums[3], cw = sums[4], ha = sums[5], eu = sums[6];
+  const double Tdot = b.red[SC_TDOT], inv_cpm = b.red[SC_ICPM];
   // species block (J_kj = A'_kj + dense_k / W_j) and temperature column
   // entries e = k S + j of the species block, (k, j) advanced without
   // dividing by the runtime S
@@ -470,7 +551,7 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
     int k = threadIdx.x / S, j = threadIdx.x - k * S;
     for (; k < S;) {
       double* a = J + (size_t)(1 + k) * n + 1 + j;
-      *a = fma(b.u[k], m.invW[j], *a);
+      *a = fma(dense[k], m.invW[j], *a);
       k += dk;
       j += dj;
       if (j >= S) {
@@ -483,12 +564,15 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
     J[(size_t)(1 + k) * n] = m.W[k] * invrho * fma(cpf * b.wd[k], x.invT, b.aT[k]);
   const double inv_rc = invrho * inv_cpm;
   for (int j = threadIdx.x; j < S; j += blockDim.x) {
-    const double t1 = x.T * (x.rho * b.cs[j] - cpf * x.Wbar * he) * inv_rc;
-    const double t2 = Tdot * fma(b.cpR[j] - cvf, inv_cpm, -cpf * x.Wbar);
-    J[1 + j] = -(t1 + t2) * m.invW[j];
+    // cs_j = sum_k e_k (A_kj + u_k) = W_j sum_k (e_k / W_k) A'_kj + sum_k e_k u_k
+    const double csj = fma(m.W[j], cs[j], eu);
+    const double cW = __dmul_rn(cpf, x.Wbar);
+    const double in = fma(x.rho, csj, -__dmul_rn(cW, he));
+    const double tt = fma(__dmul_rn(x.T, in), inv_rc, __dmul_rn(Tdot, fma(b.cpR[j] - cvf, inv_cpm, -cW)));
+    J[1 + j] = -tt * m.invW[j];
   }
   if (threadIdx.x == 0) {
-    J[0] = -fma(x.T, ha, cw) * inv_rc - Tdot * fma(dcpm, inv_cpm, -cpf * x.invT);
+    J[0] = fma(-fma(x.T, ha, cw), inv_rc, -__dmul_rn(Tdot, fma(dcpm, inv_cpm, -cpf * x.invT)));
     f[0] = Tdot;
   }
   team_sync();

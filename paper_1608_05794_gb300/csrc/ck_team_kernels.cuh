@@ -10,25 +10,27 @@
 
 namespace ck {
 
-static __host__ __device__ __forceinline__ int team_bufs_doubles(int S, int chunk) { return 9 * S + (3 + JP) * chunk + 48; }
+static __host__ __device__ __forceinline__ int team_bufs_doubles(int S, int chunk) {
+  return 4 * (S + 1) + 5 * S + (3 + JP) * chunk + TEAM_RED;
+}
 
-static __device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH) {
+static __device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH, int vp) {
   TeamBufs b;
   b.X = base;
-  b.Gp = b.X + S;
-  b.hRT = b.Gp + S;
-  b.cpR = b.hRT + S;
-  b.Gm = b.cpR + S;
-  b.wd = b.Gm + S;
+  b.Gp = b.X + S + 1;
+  b.Gm = b.Gp + S + 1;
+  b.hRT = b.Gm + S + 1;
+  b.cpR = b.hRT + S + 1;
+  b.wd = b.cpR + S;
   b.aT = b.wd + S;
   b.E = b.aT + S;
   b.u = b.E + S;
-  b.cs = b.Gp;  // column sums reuse Gp (free after the reaction passes)
   b.q = b.u + S;
   b.dqT = b.q + CH;
   b.D = b.dqT + CH;
   b.P = b.D + CH;
   b.red = b.P + (size_t)JP * CH;
+  b.vp = vp;
   return b;
 }
 
@@ -77,14 +79,14 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
 }
 
 // x^q, the step-size controller's power, by the first warp alone and handed
-// to the others through red[37]: pow is long, and every warp that runs it
+// to the others through red[SC_POW]: pow is long, and every warp that runs it
 // pays all of its FP64 instructions.  x is the same in every thread; every
 // thread must call it.
 static __device__ __forceinline__ double team_pow(double x, double q, double* red) {
   if (blockDim.x == 32) return pow(x, q);
-  if (threadIdx.x == 0) red[37] = pow(x, q);
+  if (threadIdx.x == 0) red[SC_POW] = pow(x, q);
   __syncthreads();
-  return red[37];
+  return red[SC_POW];
 }
 
 // ------------------------------------------------------------------ ROS4
