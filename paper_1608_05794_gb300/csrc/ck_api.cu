@@ -305,17 +305,26 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     }
   }
   csr_ptr[S] = (int32_t)csr_rx.size();
-  // team kernels walk the reactions in chunks of the CTA size
-  const int chunk = (S + 1 <= 56) ? 64 : 256;
+  // team kernels walk the reactions in chunks: equal shares of at most what
+  // the team's shared memory has room for
+  const int n1 = S + 1;
+  auto shares = [&](int most) { return R ? (R + (R + most - 1) / most - 1) / ((R + most - 1) / most) : 1; };
+  const int chunk = shares(n1 <= 24 ? 64 : (n1 <= 64 ? 112 : 60));
   const int n_chunks = (R + chunk - 1) / chunk;
-  std::vector<int32_t> csr_cptr((size_t)S * (n_chunks + 1));
-  for (int k = 0; k < S; ++k) {
-    int e = csr_ptr[k];
-    for (int c = 0; c <= n_chunks; ++c) {
-      while (e < csr_ptr[k + 1] && csr_rx[e] < c * chunk) ++e;
-      csr_cptr[(size_t)k * (n_chunks + 1) + c] = (c == n_chunks) ? csr_ptr[k + 1] : e;
+  const int rhs_chunk = shares(n1 <= 64 ? 512 : 392);
+  const int n_rhs_chunks = (R + rhs_chunk - 1) / rhs_chunk;
+  auto cut = [&](int size, int count) {  // first CSR entry of every species and chunk
+    std::vector<int32_t> c((size_t)S * (count + 1));
+    for (int k = 0; k < S; ++k) {
+      int e = csr_ptr[k];
+      for (int i = 0; i <= count; ++i) {
+        while (e < csr_ptr[k + 1] && csr_rx[e] < i * size) ++e;
+        c[(size_t)k * (count + 1) + i] = (i == count) ? csr_ptr[k + 1] : e;
+      }
     }
-  }
+    return c;
+  };
+  const std::vector<int32_t> jac_cptr = cut(chunk, n_chunks), csr_cptr = cut(rhs_chunk, n_rhs_chunks);
   // Jacobian assembly, chunk by chunk, as one list of targets, each adding a
   // fixed-order sum of coef * src[pidx] (src: the chunk's per-reaction
   // arrays q, dq/dT, D and the partials P, contiguous in shared memory):
@@ -335,7 +344,7 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   for (int c = 0; c < n_chunks; ++c) {
     std::vector<std::vector<std::pair<double, int32_t>>> ent((size_t)S * S + 4 * (size_t)S);
     for (int k = 0; k < S; ++k) {
-      for (int e = csr_cptr[(size_t)k * (n_chunks + 1) + c]; e < csr_cptr[(size_t)k * (n_chunks + 1) + c + 1];
+      for (int e = jac_cptr[(size_t)k * (n_chunks + 1) + c]; e < jac_cptr[(size_t)k * (n_chunks + 1) + c + 1];
            ++e) {
         const int i = csr_rx[e];
         const int li = i - c * chunk;
@@ -386,7 +395,7 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     jc_ptr.push_back((int32_t)jc.size());
   }
   // species ordered by the length of their CSR rows (longest first), so
-  // that the lanes of one warp gather similar counts in the one-pass RHS
+  // that the lanes of one warp gather similar counts in the RHS
   std::vector<int16_t> rsp(S);
   {
     std::vector<int> ks(S);
@@ -494,6 +503,8 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   dm.csr = reinterpret_cast<const CsrTerm*>(b + off_csr);
   dm.chunk = chunk;
   dm.n_chunks = n_chunks;
+  dm.rhs_chunk = rhs_chunk;
+  dm.n_rhs_chunks = n_rhs_chunks;
   dm.csr_cptr = reinterpret_cast<const int32_t*>(b + off_csr_cptr);
   dm.jc_ptr = reinterpret_cast<const int32_t*>(b + off_jc_ptr);
   dm.jc = reinterpret_cast<const JcEntry*>(b + off_jc);

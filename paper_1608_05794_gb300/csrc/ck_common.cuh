@@ -96,20 +96,22 @@ struct DevMech {
   const CsrTerm* csr;     // [csr_nnz]
   const double* tab;      // [256] 2^(j/256)
   const double* revp;     // [n_rev][3] explicit reverse: log2 A_r, beta_r, Ea_r / (R ln 2)
-  // Team kernels walk the reactions in chunks of `chunk` (= CTA size).
-  // csr_cptr[k (n_chunks + 1) + c] = first CSR entry of species k whose
-  // reaction lies in chunk c or later.  Jacobian assembly, chunk c: the
+  // Team kernels walk the reactions in chunks: of `chunk` for the Jacobian,
+  // of `rhs_chunk` for a right-hand side whose team has no room for all R
+  // rates.  csr_cptr[k (n_rhs_chunks + 1) + c] = first CSR entry of species k
+  // whose reaction lies in right-hand-side chunk c or later.  Jacobian
+  // assembly, chunk c: the
   // targets jc[e], e in [jc_ptr[c], jc_ptr[c+1]) (flat index idx: the
   // species-block entry J[idx] below n^2, else the per-species sums wd, aT,
   // E, u at idx - n^2), each add the sum over t in [jc[e].beg, jc[e].end)
   // of jt[t].coef * src[jt[t].pidx] (src: the chunk's q, dq/dT, D and
   // partials P, JP per reaction, contiguous).
-  int chunk, n_chunks;
+  int chunk, n_chunks, rhs_chunk, n_rhs_chunks;
   const int32_t* csr_cptr;
   const int32_t* jc_ptr;
   const JcEntry* jc;
   const JcTerm* jt;
-  const int16_t* rsp;     // [S] species order of the one-pass RHS gather, longest row first
+  const int16_t* rsp;     // [S] species order of the RHS gather, longest row first
 };
 
 // ---------------------------------------------------------------- 2^x

@@ -35,10 +35,9 @@ enum : int32_t { DEVERR_STAGE_TIMEOUT = 1 };
 
 // Launch configuration knobs chosen by the host (variant / autotuner).
 struct LaunchCfg {
-  int team_warps = 0;   // warps per reactor for team kernels (0: heuristic)
   int ctas_per_sm = 0;  // 0: as many as fit
   int precision = 0;    // ROS4 linear algebra: 0 FP64, 1 FP32 + FP64 refinement
-  int grid_side = 0;    // ROS4 team: 0 automatic, 8 or 16 threads per side
+  int grid_side = 0;    // ROS4 team: 16 takes the largest team whatever the size
 };
 
 cudaError_t launch_rhs(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
@@ -62,15 +61,15 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, double* scratch,
                         size_t scratch_bytes, bool may_alloc);
 size_t ros4_scratch_bytes_max();
-// launch_ros4 for one team grid (G x G threads, T x T tiles, n <= G T), each
-// in its own translation unit (ck_ros4_GxT.cu).
+// launch_ros4 for one team size (warps), each in its own translation unit
+// (ck_ros4_wN.cu).
 #define CK_ROS4_TILE_LAUNCHER(NAME)                                                                          \
   cudaError_t NAME(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt, double* h_io, \
                    const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue, cudaStream_t st,   \
                    const LaunchCfg& cfg, double* scratch, size_t scratch_bytes, bool may_alloc);
-CK_ROS4_TILE_LAUNCHER(launch_ros4_8x7)
-CK_ROS4_TILE_LAUNCHER(launch_ros4_16x7)
-CK_ROS4_TILE_LAUNCHER(launch_ros4_16x9)
+CK_ROS4_TILE_LAUNCHER(launch_ros4_w2)
+CK_ROS4_TILE_LAUNCHER(launch_ros4_w4)
+CK_ROS4_TILE_LAUNCHER(launch_ros4_w8)
 #undef CK_ROS4_TILE_LAUNCHER
 cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                          double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,

@@ -6,71 +6,82 @@
 #include <cuda_runtime.h>
 
 #include <mutex>
-#include <type_traits>
 
 #include "ck_team_kernels.cuh"
 
 namespace ck {
 
+// Threads of a team for a mechanism or matrix of dimension n: one warp for
+// the smallest (no barriers), otherwise three warps (an odd number spreads
+// the single-warp phases of neighbouring CTAs over the SM's four schedulers)
+// or eight.
+static int team_size(int n) { return n <= 24 ? 32 : (n <= 64 ? 96 : 256); }
+
 // ------------------------------------------------------------------ Jacobian
-__global__ void k_jacobian(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
-                           const double* __restrict__ y, double* __restrict__ jac) {
+__global__ void __launch_bounds__(256) k_jacobian(const __grid_constant__ DevMech d, int64_t N,
+                                                  const double* __restrict__ p, const double* __restrict__ y,
+                                                  double* __restrict__ jac) {
   extern __shared__ __align__(16) double sm[];
   const int n = d.n;
   double* J = sm;
   double* ys = J + (size_t)n * n;
   double* fs = ys + n;
-  TeamBufs b = carve_bufs(fs + n, d.S, d.chunk, d.chunk);
-  Mix x;
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
-    __syncthreads();
-    team_jacobian(d, d.tab, p[r], ys, fs, J, b, x);
+    team_sync();
+    team_jacobian(d, d.tab, p[r], ys, fs, J, carve_bufs(fs + n, d.S, d.chunk, 256));
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = J[e];
-    __syncthreads();
+    team_sync();
   }
 }
 
 // Forward-difference Jacobians (one CTA per reactor), as ROS4 builds them
 // with the forward-difference option at step size h[r].
-__global__ void k_jacobian_fd(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
-                              const double* __restrict__ y, const double* __restrict__ h, double rtol,
-                              double atol, double* __restrict__ jac) {
+__global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ DevMech d, int64_t N,
+                                                     const double* __restrict__ p, const double* __restrict__ y,
+                                                     const double* __restrict__ h, double rtol, double atol,
+                                                     double* __restrict__ jac) {
   extern __shared__ __align__(16) double sm[];
-  const int n = d.n;
-  double* J = sm;
-  double* ys = J + (size_t)n * n;
-  double* fs = ys + n;
-  double* yt = fs + n;
-  double* ft = yt + n;
-  TeamBufs b = carve_bufs(ft + n, d.S, d.chunk, d.chunk);
+  const int n = d.n, ys = n * n;
+  const RhsQ qq{ys + 4 * n + species_doubles(d.S), d.rhs_chunk};
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
-    __syncthreads();
-    team_jacobian_fd(d, d.tab, p[r], ys, h[r], rtol, atol, fs, J, yt, ft, b);
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = J[e];
-    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x) sm[ys + i] = y[r * n + i];
+    team_sync();
+    team_jacobian_fd(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, ys + 2 * n, ys + 3 * n, ys + 4 * n,
+                     n > 64 ? 256 : 64, qq);
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = sm[e];
+    team_sync();
   }
 }
 
 // ------------------------------------------------------------------ batched LU
-template <int G, int T>
-__global__ void __launch_bounds__(G * G, 1) k_lu_factor(int64_t batch, int dim, double* __restrict__ a,
-                                                      int32_t* __restrict__ piv, int32_t* __restrict__ info) {
+// Shared memory, in doubles: the matrix, 1 / U_kk, the row tables and pivots.
+static __host__ __device__ __forceinline__ size_t lu_doubles(int dim) {
+  return (((size_t)dim * dim + 1) & ~(size_t)1) + 4 * (size_t)dim + 2 * (size_t)dim;
+}
+__global__ void __launch_bounds__(256) k_lu_factor(int64_t batch, int dim, double* __restrict__ a,
+                                                   int32_t* __restrict__ piv, int32_t* __restrict__ info) {
   extern __shared__ __align__(16) double sm[];
+  __shared__ int flag;
+  const int nn = dim * dim;
   double* A = sm;
-  double* invd = A + (size_t)dim * dim;
-  int* pv = reinterpret_cast<int*>(invd + dim);
-  double* scratch = invd + 2 * dim;  // lu_scratch_words<G, T>() doubles
-  const int64_t nn = (int64_t)dim * dim;
+  LuRow<double>* lr = reinterpret_cast<LuRow<double>*>(A + ((nn + 1) & ~1));
+  double* invd = reinterpret_cast<double*>(lr + 2 * dim);
+  int* rof = reinterpret_cast<int*>(invd + dim);
+  int* pv = rof + dim;
+  const float rc = 1.0f / (float)dim;
   for (int64_t m = blockIdx.x; m < batch; m += gridDim.x) {
-    for (int64_t e = threadIdx.x; e < nn; e += blockDim.x) A[e] = a[m * nn + e];
-    __syncthreads();
-    const int inf = lu_reg<G, T>(A, dim, pv, invd, scratch);
-    for (int64_t e = threadIdx.x; e < nn; e += blockDim.x) a[m * nn + e] = A[e];
+    double* am = a + m * nn;
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) A[e] = am[e];
+    team_sync();
+    const int inf = lu_flat<false>(A, dim, rof, pv, invd, lr, &flag);
+    for (int e = threadIdx.x; e < nn; e += blockDim.x) {
+      const int i = flat_row(e, rc);
+      am[e] = A[(rof[i] >> 8) + (e - i * dim)];
+    }
     for (int i = threadIdx.x; i < dim; i += blockDim.x) piv[m * dim + i] = pv[i];
     if (threadIdx.x == 0) info[m] = inf;
-    __syncthreads();
+    team_sync();
   }
 }
 
@@ -103,7 +114,7 @@ __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu
 // right-hand sides are evaluated by the team, so a reactor's working set
 // (8 n-vectors and one chunk of reaction scratch) stays in shared memory and
 // the number of steps of one reactor never holds back another.
-__global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
+__global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
                                                    double* __restrict__ y, const double* __restrict__ dt,
                                                    double* h_io, SolverParams sp, int32_t* steps,
                                                    int32_t* status, int32_t* queue) {
@@ -113,8 +124,10 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
   double* yv = sm;
   double* yt = yv + n;
   double* kk = yt + n;  // six stages, n each
-  TeamBufs b = carve_bufs(kk + 6 * n, d.S, d.chunk, 64);
-  Mix x;
+  constexpr int vp = 64;
+  const int o_y = 0, o_t = n, o_k = 2 * n, bufs = 8 * n;
+  double* red = sm + bufs;
+  const RhsQ qq{bufs + species_doubles(d.S), d.rhs_chunk};
   const bool fixed = sp.fixed_h > 0.0;
   const int tid = threadIdx.x, P = blockDim.x;
   double* k0 = kk;
@@ -142,7 +155,7 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
       if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0(d, d.tab, pr, yv, tf, sp.rtol, sp.atol, k0, yt, k1, b, x);
+      else h = team_h0(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
       const double hmin = 1e-15 * tf;
       double t = 0.0;
       bool last_rej = false, last_nf = false;
@@ -152,38 +165,38 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
         const double hh = clamped ? tf - t : h;
         if (hh < hmin) { st = last_nf ? ST_NONFINITE : ST_HMIN; break; }
         // k_s = hh f(y + sum_j a_sj k_j)
-        team_rhs(d, d.tab, pr, yv, k0, b);
+        team_rhs(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k0[i] *= hh;
           yt[i] = fma(RK_A21, k0[i], yv[i]);
         }
         team_sync();
-        team_rhs(d, d.tab, pr, yt, k1, b);
+        team_rhs(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k1[i] *= hh;
           yt[i] = fma(RK_A32, k1[i], fma(RK_A31, k0[i], yv[i]));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, yt, k2, b);
+        team_rhs(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k2[i] *= hh;
           yt[i] = fma(RK_A43, k2[i], fma(RK_A42, k1[i], fma(RK_A41, k0[i], yv[i])));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, yt, k3, b);
+        team_rhs(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k3[i] *= hh;
           yt[i] = fma(RK_A54, k3[i], fma(RK_A53, k2[i], fma(RK_A52, k1[i], fma(RK_A51, k0[i], yv[i]))));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, yt, k4, b);
+        team_rhs(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k4[i] *= hh;
           yt[i] = fma(RK_A65, k4[i],
                       fma(RK_A64, k3[i], fma(RK_A63, k2[i], fma(RK_A62, k1[i], fma(RK_A61, k0[i], yv[i])))));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, yt, k5, b);
+        team_rhs(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k1, whose weights are 0)
         int nf = 0;
         for (int i = tid; i < n; i += P) {
@@ -202,7 +215,7 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
           ++acc;
           continue;
         }
-        const double e = team_wrms(n, k1, yv, yt, sp.rtol, sp.atol, b.red);
+        const double e = team_wrms(n, k1, yv, yt, sp.rtol, sp.atol, red, vp);
         if (nf || !isfinite(e)) {
           ++rej;
           h = FAC_MIN * hh;
@@ -211,7 +224,7 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
           continue;
         }
         last_nf = false;
-        const double pe = (e == 0.0) ? 0.0 : team_pow(e, -0.2, b.red);
+        const double pe = (e == 0.0) ? 0.0 : team_pow(e, -0.2, red);
         if (e < 1.0) {
           for (int i = tid; i < n; i += P) yv[i] = yt[i];
           team_sync();
@@ -243,30 +256,13 @@ __global__ void __launch_bounds__(64) k_rkf45_team(const __grid_constant__ DevMe
 }
 
 // ------------------------------------------------------------------ launchers
-static int team_threads(int n, const LaunchCfg& cfg) {
-  int w = cfg.team_warps;
-  if (w <= 0) w = (n <= 24) ? 1 : (n <= 64 ? 2 : 4);
-  if (w > 8) w = 8;
-  return 32 * w;
-}
-
-
-// Thread grid of the register-tiled LU for dimension n: G x G threads with
-// T x T tiles (n <= G T).
-template <class F>
-static cudaError_t with_grid(int n, F f, int side = 0) {
-  if (side == 16 && n <= 112) return f(std::integral_constant<int, 16>{}, std::integral_constant<int, 7>{});
-  if (n <= 56) return f(std::integral_constant<int, 8>{}, std::integral_constant<int, 7>{});
-  if (n <= 112) return f(std::integral_constant<int, 16>{}, std::integral_constant<int, 7>{});
-  if (n <= 144) return f(std::integral_constant<int, 16>{}, std::integral_constant<int, 9>{});
-  return cudaErrorInvalidValue;
-}
 cudaError_t launch_jacobian(const HostMech& hm, int64_t n, const double* p, const double* y,
                             double* jac, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * ((size_t)nn * nn + 2 * nn + team_bufs_doubles(hm.S, hm.d.chunk));
-  const int threads = hm.d.chunk;
+  const size_t smem =
+      sizeof(double) * ((size_t)nn * nn + 2 * nn + species_doubles(hm.S) + jac_doubles(hm.S, hm.d.chunk));
+  const int threads = team_size(nn);
   const int grid = team_grid(k_jacobian, threads, smem, n, cfg);
   k_jacobian<<<grid, threads, smem, st>>>(hm.d, n, p, y, jac);
   return cudaGetLastError();
@@ -276,8 +272,8 @@ cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, c
                                double rtol, double atol, double* jac, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + team_bufs_doubles(hm.S, hm.d.chunk));
-  const int threads = hm.d.chunk;
+  const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const int threads = team_size(nn);
   const int grid = team_grid(k_jacobian_fd, threads, smem, n, cfg);
   k_jacobian_fd<<<grid, threads, smem, st>>>(hm.d, n, p, y, h, rtol, atol, jac);
   return cudaGetLastError();
@@ -287,14 +283,11 @@ cudaError_t launch_lu_factor(int64_t batch, int dim, double* a, int32_t* piv, in
                              cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
   LaunchCfg cfg;
-  return with_grid(dim, [&](auto Gc, auto Tc) {
-    constexpr int G = decltype(Gc)::value, T = decltype(Tc)::value;
-    const size_t smem = sizeof(double) * ((size_t)dim * dim + 2 * dim + lu_scratch_words<G, T>());
-    auto kern = k_lu_factor<G, T>;
-    const int grid = team_grid(kern, G * G, smem, batch, cfg);
-    kern<<<grid, G * G, smem, st>>>(batch, dim, a, piv, info);
-    return cudaGetLastError();
-  });
+  const size_t smem = sizeof(double) * lu_doubles(dim);
+  const int threads = team_size(dim);
+  const int grid = team_grid(k_lu_factor, threads, smem, batch, cfg);
+  k_lu_factor<<<grid, threads, smem, st>>>(batch, dim, a, piv, info);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_lu_solve(int64_t batch, int dim, const double* lu, const int32_t* piv,
@@ -302,7 +295,7 @@ cudaError_t launch_lu_solve(int64_t batch, int dim, const double* lu, const int3
   if (batch <= 0) return cudaSuccess;
   const size_t smem = sizeof(double) * ((size_t)dim * dim + 3 * dim);
   LaunchCfg cfg;
-  const int threads = team_threads(dim, cfg);
+  const int threads = dim <= 24 ? 32 : (dim <= 64 ? 64 : 128);
   const int grid = team_grid(k_lu_solve, threads, smem, batch, cfg);
   k_lu_solve<<<grid, threads, smem, st>>>(batch, dim, lu, piv, b);
   return cudaGetLastError();
@@ -330,12 +323,7 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
   const int nn = hm.d.n;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  auto* fn = (cfg.grid_side == 16 && nn <= 112) ? launch_ros4_16x7
-             : nn <= 56                         ? launch_ros4_8x7
-             : nn <= 112                        ? launch_ros4_16x7
-             : nn <= 144                        ? launch_ros4_16x9
-                                                : nullptr;
-  if (!fn) return cudaErrorInvalidValue;
+  auto* fn = cfg.grid_side == 16 ? launch_ros4_w8 : (nn <= 24 ? launch_ros4_w2 : (nn <= 64 ? launch_ros4_w4 : launch_ros4_w8));
   return fn(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg, scratch, scratch_bytes, may_alloc);
 }
 
@@ -344,11 +332,12 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
                               int32_t* status, int32_t* queue, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * (8 * (size_t)nn + team_bufs_doubles(hm.S, hm.d.chunk));
-  const int grid = team_grid(k_rkf45_team, 64, smem, n, cfg);
+  const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 128);
+  const int grid = team_grid(k_rkf45_team, threads, smem, n, cfg);
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  k_rkf45_team<<<grid, 64, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
+  k_rkf45_team<<<grid, threads, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
   return cudaGetLastError();
 }
 

@@ -1,28 +1,29 @@
 // The ROS4 integrator kernel (Sec. 2 transformed form, App. C, driven by
-// Algorithm 1): one CTA per reactor, iteration matrix in shared memory,
-// register-tiled LU, warp solves; and its launcher for one thread grid.
-// Included by one translation unit per thread grid (ck_ros4_*.cu).
+// Algorithm 1): one CTA per reactor, iteration matrix in shared memory, and
+// its launcher for one team size.  Included by one translation unit per team
+// size (ck_ros4_*.cu).
 #pragma once
+#include <type_traits>
+
 #include "ck_team_kernels.cuh"
 
 namespace ck {
 
 // Stage solve of the precision form: the iteration matrix is factored in
-// FP32 (M32, piv, invd32) and each solve is refined against the FP64 matrix
+// FP32 (M32, rof, invd32) and each solve is refined against the FP64 matrix
 // M64 (the CTA's copy in global memory, L2-resident): x = LU32^-1 b, then
 // REFINE times r = b - M64 x (FP64), x += LU32^-1 r.
 // b (in u) is overwritten with x; xf (n floats) and x (n doubles) are scratch
-// that must not hold anything the caller still needs (stage 4 reuses the
-// third stage's f, so the first three solves take u4's buffer as xf).
-static __device__ void refined_solve(const double* M64, const float* M32, int n, const int* piv,
+// that must not hold anything the caller still needs.
+static __device__ void refined_solve(const double* M64, const float* M32, int n, const int* rof,
                               const float* invd32, double* u, float* xf, double* x, int refine) {
   const int tid = threadIdx.x, P = blockDim.x;
   for (int i = tid; i < n; i += P) xf[i] = (float)u[i];
-  __syncthreads();
-  if (tid < 32) warp_lu_solve<true>(M32, n, piv, invd32, xf);
-  __syncthreads();
+  team_sync();
+  if (tid < 32) warp_lu_solve<true>(M32, n, rof, invd32, xf);
+  team_sync();
   for (int i = tid; i < n; i += P) x[i] = (double)xf[i];
-  __syncthreads();
+  team_sync();
   for (int it = 0; it < refine; ++it) {
     for (int i = tid; i < n; i += P) {
       const double* row = M64 + (size_t)i * n;
@@ -37,19 +38,30 @@ static __device__ void refined_solve(const double* M64, const float* M32, int n,
       for (; j < n; ++j) s0 = fma(-row[j], x[j], s0);
       xf[i] = (float)((s0 + s1) + (s2 + s3));
     }
-    __syncthreads();
-    if (tid < 32) warp_lu_solve<true>(M32, n, piv, invd32, xf);
-    __syncthreads();
+    team_sync();
+    if (tid < 32) warp_lu_solve<true>(M32, n, rof, invd32, xf);
+    team_sync();
     for (int i = tid; i < n; i += P) x[i] += (double)xf[i];
-    __syncthreads();
+    team_sync();
   }
   for (int i = tid; i < n; i += P) u[i] = x[i];
-  __syncthreads();
+  team_sync();
 }
+
+// Step control, worked out by the first warp and read by all.
+struct Ros4Ctl {
+  double hh, dg;                          // step size, 1 / (hh gamma)
+  double c21, c31, c32, c41, c42, c43;    // -c_ij / hh
+  int go, accept;
+};
 
 // PREC 0: FP64 LU and solves.  PREC 1 / 2: FP32 LU and solves with one /
 // two steps of FP64 iterative refinement (the rates, K_c, the temperature
 // equation, the error norm and the step control stay FP64).
+//
+// P: threads of a team, at least n; the stage vectors are kept one component
+// a thread, in registers.  MINB: resident teams an SM that the register
+// allocation allows for.
 //
 // m64g (may be NULL for PREC 0) holds ros4_scratch_doubles(n) doubles per
 // CTA, m64g[blockIdx.x][.]: global memory, 23 KB a CTA at n = 54 (21 MB for
@@ -74,78 +86,98 @@ static __device__ void refined_solve(const double* M64, const float* M32, int n,
 //     the last n for each h) and its FP32 factors in the first half of the
 //     shared FP64 matrix, so both forms need the same shared memory and
 //     residency.
-template <int G, int T, int PREC>
-__global__ void __launch_bounds__(G * G, G == 8 ? 6 : 1) k_ros4(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
+template <int P, int MINB, int PREC>
+__global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
                                                  double* __restrict__ y, const double* __restrict__ dt,
                                                  double* h_io, SolverParams sp, int32_t* steps,
                                                  int32_t* status, int32_t* queue, double* __restrict__ m64g) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ int slot;
-  const int n = d.n;
+  __shared__ int slot, flag;
+  __shared__ Ros4Ctl ctl;
+  using F = typename std::conditional<PREC == 0, double, float>::type;  // type of the factors
+  const int n = d.n, nn = n * n;
   const double* tab = d.tab;  // 2 KB, stays in L1
+  const Ros4Layout L(n, d.S, d.chunk, d.rhs_chunk);
   double* M = sm;
-  double* yv = M + (size_t)n * n;
-  double* F0 = yv + n;
-  double* F = F0 + n;
-  double* Yt = F + n;
-  double* u1 = Yt + n;
-  double* u2 = u1 + n;
-  double* u3 = u2 + n;
-  double* u4 = u3 + n;
-  double* invd = u4 + n;
-  int* piv = reinterpret_cast<int*>(invd + n);
-  // the LU's scratch (lu_scratch_words: at most 578 doubles) reuses the
-  // team buffers, free while factoring (9 S + 10 chunk + 48 >= 688 doubles)
-  TeamBufs b = carve_bufs(invd + n + (n + 1) / 2, d.S, d.chunk, d.chunk);
-  float* M32 = reinterpret_cast<float*>(M);  // PREC >= 1: FP32 factors over the FP64 matrix
+  double* yv = sm + L.yv;
+  double* F0 = sm + L.f0;
+  double* Yt = sm + L.yt;
+  double* ub = sm + L.ub;
+  double* invd = sm + L.invd;
+  int* rof = reinterpret_cast<int*>(sm + L.rof);
+  double* red = sm + L.bufs;
+  LuRow<F>* lr = reinterpret_cast<LuRow<F>*>(sm + L.lr);
+  F* MF = reinterpret_cast<F*>(M);         // PREC >= 1: FP32 factors over the FP64 matrix
+  F* invF = reinterpret_cast<F*>(invd);
+  float* xf = reinterpret_cast<float*>(invd) + n;  // PREC >= 1: the other half of invd
   double* Mg = m64g ? m64g + (size_t)blockIdx.x * ros4_scratch_doubles(n) : nullptr;
   const bool keep_j = Mg != nullptr && sp.jac == 0;
-  Mix x;
   const bool fixed = sp.fixed_h > 0.0;
-  const int tid = threadIdx.x, P = blockDim.x;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const bool own = tid < n;
   for (;;) {
     const int r = team_next(queue, &slot);
     if (r >= N) break;
-    for (int i = tid; i < n; i += P) yv[i] = y[(int64_t)r * n + i];
+    if (own) yv[tid] = y[(int64_t)r * n + tid];
     const double pr = p[r];
     const double tf = dt[r];
-    __syncthreads();
-    int bad = 0;
-    for (int i = tid; i < n; i += P) bad |= !isfinite(yv[i]);
+    team_sync();
+    int bad = own && !isfinite(yv[tid]);
     bad = __syncthreads_or(bad);
     bad |= !(pr > 0.0) || !isfinite(pr) || !(yv[0] > 0.0) || !isfinite(tf) || !(tf >= 0.0);
-    int st = ST_OK, acc = 0, rej = 0;
-    double h = 0.0;
+    // the first warp's view of the step control
+    int st = ST_OK, acc = 0, rej = 0, sing_run = 0;
+    double h = 0.0, t = 0.0, hh = 0.0;
+    bool last_rej = false, last_nf = false, clamped = false;
     if (bad) {
       st = ST_BADINPUT;
     } else if (tf > 0.0) {
       if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0(d, tab, pr, yv, tf, sp.rtol, sp.atol, F0, Yt, F, b, x);
+      else h = team_h0(d, tab, pr, L.yv, tf, sp.rtol, sp.atol, L.f0, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
       const double hmin = 1e-15 * tf;
-      double t = 0.0;
-      bool last_rej = false, last_nf = false;
-      int sing_run = 0;
+      // the next attempt: its step size, or the end of the integration
+      auto next = [&](int accept) {
+        int go = 0;
+        if (t < tf) {
+          if (acc + rej >= sp.max_steps) {
+            st = ST_MAXSTEPS;
+          } else {
+            clamped = h >= tf - t;
+            hh = clamped ? tf - t : h;
+            if (hh < hmin) st = last_nf ? ST_NONFINITE : ST_HMIN;
+            else go = 1;
+          }
+        }
+        const double ih = rcp_rn(hh), dg = rcp_rn(hh * ROS_GAMMA);
+        if (tid == 0) {
+          ctl.hh = hh;
+          ctl.dg = dg;
+          ctl.c21 = -ROS_C21 * ih;
+          ctl.c31 = -ROS_C31 * ih;
+          ctl.c32 = -ROS_C32 * ih;
+          ctl.c41 = -ROS_C41 * ih;
+          ctl.c42 = -ROS_C42 * ih;
+          ctl.c43 = -ROS_C43 * ih;
+          ctl.go = go;
+          ctl.accept = accept;
+        }
+      };
+      if (warp == 0) next(0);
       bool have_j = false;   // J of yv in Mg (analytic form with a copy only)
       bool have_f = false;   // F0 = f(yv)
-      while (t < tf) {
-        if (acc + rej >= sp.max_steps) { st = ST_MAXSTEPS; break; }
-        const bool clamped = h >= tf - t;
-        const double hh = clamped ? tf - t : h;
-        if (hh < hmin) { st = last_nf ? ST_NONFINITE : ST_HMIN; break; }
+      team_sync();
+      while (ctl.go) {
         // J and f at y (or the copy kept since a rejected attempt at the
         // same y); A = J - I/(hh gamma) = -M; LU of A
-        const int nn = n * n;
         if (!have_j) {
-          if (sp.jac == 1) team_jacobian_fd(d, tab, pr, yv, hh, sp.rtol, sp.atol, F0, M, Yt, F, b, have_f);
-          else team_jacobian(d, tab, pr, yv, F0, M, b, x);
-          team_sync();
+          if (sp.jac == 1) team_jacobian_fd(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, M, L.yt, L.ub, L.bufs, L.vp, L.rhs_q, have_f);
+          else team_jacobian(d, tab, pr, yv, F0, M, carve_bufs(sm + L.bufs, d.S, d.chunk, L.vp));
           if (Mg && (keep_j || PREC)) {
             for (int e = tid; e < nn; e += P) Mg[e] = M[e];
-            if (PREC)
-              for (int i = tid; i < n; i += P) Mg[nn + i] = M[(size_t)i * n + i];
-            __syncthreads();
+            if (PREC && own) Mg[nn + tid] = M[(size_t)tid * n + tid];
+            team_sync();
           }
           have_j = keep_j;
           have_f = true;
@@ -153,119 +185,134 @@ __global__ void __launch_bounds__(G * G, G == 8 ? 6 : 1) k_ros4(const __grid_con
           for (int e = tid; e < nn; e += P) M[e] = Mg[e];
           team_sync();
         }
-        const double dg = rcp_rn(hh * ROS_GAMMA);
-        int info;
         if (PREC == 0) {
-          for (int i = tid; i < n; i += P) M[(size_t)i * n + i] -= dg;
-          team_sync();
-          info = lu_reg<G, T, true>(M, n, piv, invd, b.X);
+          if (own) M[(size_t)tid * n + tid] -= ctl.dg;
         } else {
-          for (int i = tid; i < n; i += P) Mg[(size_t)i * n + i] = Mg[nn + i] - dg;
+          if (own) Mg[(size_t)tid * n + tid] = Mg[nn + tid] - ctl.dg;
           __syncthreads();
-          for (int e = tid; e < nn; e += P) M32[e] = (float)Mg[e];
-          __syncthreads();
-          info = lu_reg<G, T, true>(M32, n, piv, reinterpret_cast<float*>(invd), reinterpret_cast<float*>(b.X));
+          for (int e = tid; e < nn; e += P) MF[e] = (F)Mg[e];
         }
+        team_sync();
+        const int info = lu_flat<true>(MF, n, rof, nullptr, invF, lr, &flag);
         if (info) {
-          ++rej;
-          if (++sing_run >= SINGULAR_LIMIT) { st = ST_SINGULAR; break; }
-          h = 0.5 * hh;
-          last_rej = true;
+          if (warp == 0) {
+            ++rej;
+            if (++sing_run >= SINGULAR_LIMIT) {
+              st = ST_SINGULAR;
+              if (tid == 0) ctl.go = 0;
+            } else {
+              h = 0.5 * hh;
+              last_rej = true;
+              next(0);
+            }
+          }
+          team_sync();
           continue;
         }
-        sing_run = 0;
-        const double ih = rcp_rn(hh);
+        auto solve = [&]() {  // ub <- A^-1 ub
+          team_sync();
+          if constexpr (PREC == 0) {
+            if (warp == 0) warp_lu_solve<true>(M, n, rof, invd, ub);
+            team_sync();
+          } else {
+            refined_solve(Mg, MF, n, rof, invF, ub, xf, Yt, PREC);
+          }
+        };
+        double u1 = 0.0, u2 = 0.0, u3 = 0.0, u4 = 0.0, f3 = 0.0;
+        const double yi = own ? yv[tid] : 0.0;
         // stage 1: M u1 = f(y), solved as A v1 = f(y) with v = -u (A = -M)
-        for (int i = tid; i < n; i += P) u1[i] = F0[i];
-        team_sync();
-        if (PREC == 0) {
-          if (tid < 32) warp_lu_solve<true>(M, n, piv, invd, u1);
-          __syncthreads();
-        } else {
-          refined_solve(Mg, M32, n, piv, reinterpret_cast<const float*>(invd), u1, reinterpret_cast<float*>(u4), Yt, PREC);
-        }
+        if (own) ub[tid] = F0[tid];
+        solve();
         // stage 2: M u2 = f(y + a21 u1) + (c21/h) u1
-        for (int i = tid; i < n; i += P) Yt[i] = fma(-ROS_A21, u1[i], yv[i]);
-        team_sync();
-        team_rhs(d, tab, pr, Yt, F, b);
-        for (int i = tid; i < n; i += P) u2[i] = fma(-ROS_C21 * ih, u1[i], F[i]);
-        team_sync();
-        if (PREC == 0) {
-          if (tid < 32) warp_lu_solve<true>(M, n, piv, invd, u2);
-          __syncthreads();
-        } else {
-          refined_solve(Mg, M32, n, piv, reinterpret_cast<const float*>(invd), u2, reinterpret_cast<float*>(u4), Yt, PREC);
+        if (own) {
+          u1 = ub[tid];
+          Yt[tid] = fma(-ROS_A21, u1, yi);
         }
+        team_sync();
+        team_rhs(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        if (own) ub[tid] = fma(ctl.c21, u1, ub[tid]);
+        solve();
         // stage 3: M u3 = f(y + a31 u1 + a32 u2) + (c31 u1 + c32 u2)/h
-        for (int i = tid; i < n; i += P) Yt[i] = fma(-ROS_A32, u2[i], fma(-ROS_A31, u1[i], yv[i]));
-        team_sync();
-        team_rhs(d, tab, pr, Yt, F, b);
-        for (int i = tid; i < n; i += P)
-          u3[i] = fma(-ROS_C32 * ih, u2[i], fma(-ROS_C31 * ih, u1[i], F[i]));
-        team_sync();
-        if (PREC == 0) {
-          if (tid < 32) warp_lu_solve<true>(M, n, piv, invd, u3);
-          __syncthreads();
-        } else {
-          refined_solve(Mg, M32, n, piv, reinterpret_cast<const float*>(invd), u3, reinterpret_cast<float*>(u4), Yt, PREC);
+        if (own) {
+          u2 = ub[tid];
+          Yt[tid] = fma(-ROS_A32, u2, fma(-ROS_A31, u1, yi));
         }
+        team_sync();
+        team_rhs(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        if (own) {
+          f3 = ub[tid];
+          ub[tid] = fma(ctl.c32, u2, fma(ctl.c31, u1, f3));
+        }
+        solve();
         // stage 4: same argument as stage 3 (a4j = a3j, a43 = 0), so f is reused
-        for (int i = tid; i < n; i += P)
-          u4[i] = fma(-ROS_C43 * ih, u3[i], fma(-ROS_C42 * ih, u2[i], fma(-ROS_C41 * ih, u1[i], F[i])));
+        if (own) {
+          u3 = ub[tid];
+          ub[tid] = fma(ctl.c43, u3, fma(ctl.c42, u2, fma(ctl.c41, u1, f3)));
+        }
+        solve();
+        // y* = y + sum m_i u_i, e = sum E_i u_i; u_i = -v_i; the norm
+        // sqrt(mean (e_i / (atol + rtol max(|y_i|, |y*_i|)))^2)
+        double yn = 0.0, s = 0.0;
+        if (own) {
+          u4 = ub[tid];
+          yn = fma(-ROS_M4, u4, fma(-ROS_M3, u3, fma(-ROS_M2, u2, fma(-ROS_M1, u1, yi))));
+          const double e = fma(-ROS_E4, u4, fma(-ROS_E3, u3, fma(-ROS_E2, u2, -ROS_E1 * u1)));
+          if (!fixed) {
+            const double v = e / (sp.atol + sp.rtol * fmax(fabs(yi), fabs(yn)));
+            s = v * v;
+          }
+        }
+        if (32 * warp < n) {
+          s = warp_allsum(s);
+          if ((tid & 31) == 0) red[warp] = s;
+        }
+        const int nf = __syncthreads_or(own && !isfinite(yn));
+        if (warp == 0) {
+          int accept = 1;
+          if (fixed) {
+            t = clamped ? tf : t + hh;
+            ++acc;
+          } else {
+            double q = 0.0;
+            for (int g = 0; 32 * g < n; ++g) q += red[g];
+            const double e = sqrt(q / n);
+            if (nf || !isfinite(e)) {
+              ++rej;
+              h = FAC_MIN * hh;
+              last_rej = true;
+              last_nf = true;
+              accept = 0;
+            } else {
+              last_nf = false;
+              const double pe = (e == 0.0) ? 0.0 : pow(e, -0.25);
+              if (e < 1.0) {
+                t = clamped ? tf : t + hh;
+                ++acc;
+                double fac = (e == 0.0) ? FAC_MAX : fmin(FAC_MAX, fmax(FAC_MIN, SAFETY * pe));
+                if (last_rej) fac = fmin(1.0, fac);
+                h = hh * fac;
+                last_rej = false;
+              } else {
+                ++rej;
+                h = hh * fmax(FAC_MIN, SAFETY * pe);
+                last_rej = true;
+                accept = 0;
+              }
+            }
+          }
+          sing_run = 0;
+          next(accept);
+        }
         team_sync();
-        if (PREC == 0) {
-          if (tid < 32) warp_lu_solve<true>(M, n, piv, invd, u4);
-          __syncthreads();
-        } else {
-          refined_solve(Mg, M32, n, piv, reinterpret_cast<const float*>(invd), u4, reinterpret_cast<float*>(F), Yt, PREC);
-        }
-        // y* = y + sum m_i u_i (into Yt), e = sum E_i u_i (into F); u_i = -v_i
-        int nf = 0;
-        for (int i = tid; i < n; i += P) {
-          const double yn =
-              fma(-ROS_M4, u4[i], fma(-ROS_M3, u3[i], fma(-ROS_M2, u2[i], fma(-ROS_M1, u1[i], yv[i]))));
-          Yt[i] = yn;
-          F[i] = fma(-ROS_E4, u4[i], fma(-ROS_E3, u3[i], fma(-ROS_E2, u2[i], -ROS_E1 * u1[i])));
-          nf |= !isfinite(yn);
-        }
-        nf = __syncthreads_or(nf);
-        if (fixed) {
-          for (int i = tid; i < n; i += P) yv[i] = Yt[i];
-          team_sync();
-          t = clamped ? tf : t + hh;
-          ++acc;
+        if (ctl.accept) {
+          if (own) yv[tid] = yn;
           have_j = have_f = false;
-          continue;
         }
-        const double e = team_wrms(n, F, yv, Yt, sp.rtol, sp.atol, b.red);
-        if (nf || !isfinite(e)) {
-          ++rej;
-          h = FAC_MIN * hh;
-          last_rej = true;
-          last_nf = true;
-          continue;
-        }
-        last_nf = false;
-        const double pe = (e == 0.0) ? 0.0 : team_pow(e, -0.25, b.red);
-        if (e < 1.0) {
-          for (int i = tid; i < n; i += P) yv[i] = Yt[i];
-          team_sync();
-          t = clamped ? tf : t + hh;
-          ++acc;
-          have_j = have_f = false;
-          double fac = (e == 0.0) ? FAC_MAX : fmin(FAC_MAX, fmax(FAC_MIN, SAFETY * pe));
-          if (last_rej) fac = fmin(1.0, fac);
-          h = hh * fac;
-          last_rej = false;
-        } else {
-          ++rej;
-          h = hh * fmax(FAC_MIN, SAFETY * pe);
-          last_rej = true;
-        }
+        team_sync();
       }
     }
-    __syncthreads();
-    for (int i = tid; i < n; i += P) y[(int64_t)r * n + i] = yv[i];
+    team_sync();
+    if (own) y[(int64_t)r * n + tid] = yv[tid];
     if (tid == 0) {
       if (h_io && st != ST_BADINPUT && tf > 0.0) h_io[r] = h;
       if (steps) {
@@ -274,21 +321,22 @@ __global__ void __launch_bounds__(G * G, G == 8 ? 6 : 1) k_ros4(const __grid_con
       }
       status[r] = st;
     }
-    __syncthreads();
+    team_sync();
   }
 }
 
-// Launch k_ros4<G, T, precision> (the body of launch_ros4 for one thread
-// grid; each grid is compiled in its own translation unit).
-template <int G, int T>
-cudaError_t launch_ros4_tile(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
+// Launch k_ros4<P, MINB, precision> (the body of launch_ros4 for one team
+// size; each is compiled in its own translation unit).
+template <int P, int MINB>
+cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                              double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,
                              int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, double* scratch,
                              size_t scratch_bytes, bool may_alloc) {
   const int nn = hm.d.n;
-  const size_t smem = ros4_smem_bytes(nn, hm.S, hm.d.chunk);
-  auto kern = cfg.precision == 2 ? k_ros4<G, T, 2> : (cfg.precision == 1 ? k_ros4<G, T, 1> : k_ros4<G, T, 0>);
-  const int grid = team_grid(kern, G * G, smem, n, cfg);
+  const size_t smem = sizeof(double) * Ros4Layout(nn, hm.S, hm.d.chunk, hm.d.rhs_chunk).doubles;
+  auto kern = cfg.precision == 2 ? k_ros4<P, MINB, 2>
+                                 : (cfg.precision == 1 ? k_ros4<P, MINB, 1> : k_ros4<P, MINB, 0>);
+  const int grid = team_grid(kern, P, smem, n, cfg);
   // per-CTA copies of J (every form) and the FP64 iteration matrices of
   // the precision form: the caller's scratch when it is large enough, else
   // a stream-ordered allocation around the launch, else (allocation-free
@@ -305,7 +353,7 @@ cudaError_t launch_ros4_tile(const HostMech& hm, int64_t n, const double* p, dou
   } else if (cfg.precision) {
     return cudaErrorNotSupported;
   }
-  kern<<<grid, G * G, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);
+  kern<<<grid, P, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);
   cudaError_t k = cudaGetLastError();
   if (owned) {
     cudaError_t f = cudaFreeAsync(m64g, st);

@@ -85,10 +85,10 @@ __device__ __forceinline__ void team_sync() {
 }
 
 // Shared-memory work arrays of one team.
-// The Jacobian processes reactions in chunks of m.chunk (64 if n <= 56, else
-// 256), so the per-reaction arrays hold one chunk; the right-hand side, which
-// keeps one value per reaction, uses them as one array of 10 m.chunk values
-// when all reactions fit.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
+// The Jacobian processes reactions in chunks of m.chunk, so the per-reaction
+// arrays hold one chunk; the right-hand side, which keeps one value per
+// reaction, takes all reactions at once when the caller's q holds them, else
+// chunks of m.rhs_chunk.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
 // (S/R - H/RT)_k / ln 2, so that 1/K_c of Eq. kc is a product of species
 // factors.  Entry S of X, Gp, Gm (1) and hRT (0) stands for an empty reaction
 // slot.  After the reaction passes of the Jacobian, X, Gp and Gm are reused
@@ -98,13 +98,38 @@ struct TeamBufs {
   double *cpR, *wd, *aT, *E, *u;          // [S]; wd, aT, E, u contiguous
   double *q, *dqT, *D;                    // [chunk]
   double* P;                              // [chunk * JP] Jacobian partials
-  double* red;                            // [TEAM_RED] reductions and scalars (SC_*)
+  double* red;                            // [TEAM_RED_DOUBLES] reductions and scalars (SC_*)
   int vp;                                 // lanes that the species sums are grouped by (64 or 256)
 };
 
+// [red | X Gp Gm hRT | cpR | wd ... : a right-hand side needs species_doubles(S)
+// doubles up to and with wd; a Jacobian continues with aT E u and the chunk.
+constexpr int TEAM_RED_DOUBLES = 64;
+__host__ __device__ __forceinline__ constexpr int species_doubles(int S) { return TEAM_RED_DOUBLES + 4 * (S + 1) + 2 * S; }
+__host__ __device__ __forceinline__ constexpr int jac_doubles(int S, int chunk) { return 3 * S + (3 + JP) * chunk; }
+
+__device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH, int vp) {
+  TeamBufs b;
+  b.red = base;
+  b.X = b.red + TEAM_RED_DOUBLES;
+  b.Gp = b.X + S + 1;
+  b.Gm = b.Gp + S + 1;
+  b.hRT = b.Gm + S + 1;
+  b.cpR = b.hRT + S + 1;
+  b.wd = b.cpR + S;
+  b.aT = b.wd + S;
+  b.E = b.aT + S;
+  b.u = b.E + S;
+  b.q = b.u + S;
+  b.dqT = b.q + CH;
+  b.D = b.dqT + CH;
+  b.P = b.D + CH;
+  b.vp = vp;
+  return b;
+}
+
 // Scalars of one evaluation, formed once by one warp (an FP64 instruction
 // costs every warp that issues it a full slot) and read by all from red[].
-constexpr int TEAM_RED = 64;
 enum : int {
   SC_INVT = 32, SC_LNT, SC_LOG2T, SC_T2, SC_T3, SC_T4,  // functions of T
   SC_PW,                                                // (R T / p0)^dnu, dnu = -2..2
@@ -118,6 +143,12 @@ struct Mix {
   double T, invT, log2T, rho, invrho, Wbar, Ctot;
 };
 
+// Where a right-hand side keeps its rates of progress: offset in shared
+// memory and how many (all m.R, or m.rhs_chunk).
+struct RhsQ {
+  int off, chunk;
+};
+
 // Groups of 32 species (at most 4).
 __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 
@@ -126,6 +157,7 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // through log T) are formed side by side by two warps, everything else of
 // the species by all of them: a polynomial pass of 32 species is one work
 // item, dealt to the warps in turn.
+template <bool JAC>
 __device__ __forceinline__ void team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
   const int S = m.S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -191,7 +223,8 @@ __device__ __forceinline__ void team_species(const DevMech& m, double p, const d
       b.hRT[S] = 0.0;
     }
   }
-  for (int k = threadIdx.x; k < 4 * S; k += blockDim.x) b.wd[k] = 0.0;  // wd, aT, E, u
+  if (JAC)
+    for (int k = threadIdx.x; k < 4 * S; k += blockDim.x) b.wd[k] = 0.0;  // wd, aT, E, u
   team_sync();
   x.invT = red[SC_INVT];
   x.log2T = red[SC_LOG2T];
@@ -299,6 +332,7 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
       c = Pr * inv1p;
       dcdM = k0_kf * inv1p * inv1p;
       if (JAC) {
+        const double dlnk0 = fma(f1.y, x.invT, f0.y) * x.invT;
         const double ds = fma(fma(f1.y, x.invT, f0.y), x.invT, -dlnkf);
         dcdT = Pr * ds * inv1p * inv1p;
       }
@@ -340,52 +374,54 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
   }
 }
 
-// f(y) for one reactor.  y, f: shared memory, n = S + 1.
-static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p,
-                                             const double* y, double* f, TeamBufs b) {
+// f(y) for one reactor.  Arrays by their offsets (doubles) in the CTA's
+// dynamic shared memory, so that this out-of-line function still addresses
+// shared memory directly: y_o, f_o the vectors (n = S + 1; f may not be y),
+// bufs_o the work arrays (species_doubles), q_o the rates of progress (m.R
+// doubles if they fit the caller's layout, else m.rhs_chunk; q_all tells).
+static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p, int y_o, int f_o,
+                                             int bufs_o, int vp, RhsQ qq) {
+  extern __shared__ __align__(16) double sm[];
+  const double* y = sm + y_o;
+  double* f = sm + f_o;
+  TeamBufs b = carve_bufs(sm + bufs_o, m.S, 0, vp);
+  b.q = sm + qq.off;
   Mix x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int S = m.S, SG = species_groups(S);
-  team_species(m, p, y, b, x, tab);
+  team_species<false>(m, p, y, b, x, tab);
   team_sync();
   const double invrho = x.invrho;
-  const int NC = m.n_chunks, CH = m.chunk;
-  if (m.R <= (3 + JP) * CH) {
-    // the right-hand side needs one value per reaction, so the whole chunk
-    // scratch (q, dqT, D, P are contiguous) holds every rate of progress at
-    // once: one reaction pass and one gather, two barriers in all.  The
-    // gather sums in the same order as the chunked form below.
-    for (int i = threadIdx.x; i < m.R; i += blockDim.x) team_reaction<false>(m, m.rxn + i, x, b, tab, i);
+  // every chunk: its rates of progress, then one fixed-order gather per
+  // species, longest rows first so that the lanes of a warp do similar work
+  // (one chunk when q holds all reactions)
+  const int CH = qq.chunk;
+  for (int base = 0;;) {
+    const int cnt = m.R - base < CH ? m.R - base : CH;
+    for (int li = threadIdx.x; li < cnt; li += blockDim.x) team_reaction<false>(m, m.rxn + base + li, x, b, tab, li);
     team_sync();
+    const bool last = base + cnt >= m.R;
     for (int kk = threadIdx.x; kk < S; kk += blockDim.x) {
       const int k = m.rsp[kk];
+      int e = m.csr_ptr[k], e1 = m.csr_ptr[k + 1];
       double w = 0.0;
-      for (int e = m.csr_ptr[k]; e < m.csr_ptr[k + 1]; ++e) {
+      if (CH < m.R) {
+        const int c = base / CH;
+        const int* cp = m.csr_cptr + k * (m.n_rhs_chunks + 1) + c;
+        e = cp[0];
+        e1 = cp[1];
+        if (c) w = b.wd[k];
+      }
+      for (; e < e1; ++e) {
         const CsrTerm t = m.csr[e];
-        w = fma(t.nu, b.q[t.rx], w);
+        w = fma(t.nu, b.q[t.rx - base], w);
       }
       b.wd[k] = w;
-      f[1 + k] = w * (m.W[k] * invrho);
+      if (last) f[1 + k] = w * (m.W[k] * invrho);
     }
     team_sync();
-  } else {
-    for (int c = 0; c < NC; ++c) {
-      const int base = c * CH;
-      for (int li = threadIdx.x; li < CH; li += blockDim.x)
-        if (base + li < m.R) team_reaction<false>(m, m.rxn + base + li, x, b, tab, li);
-      team_sync();
-      for (int k = threadIdx.x; k < S; k += blockDim.x) {
-        const int* cp = m.csr_cptr + k * (NC + 1) + c;
-        double w = b.wd[k];
-        for (int e = cp[0]; e < cp[1]; ++e) {
-          const CsrTerm t = m.csr[e];
-          w = fma(t.nu, b.q[t.rx - base], w);
-        }
-        b.wd[k] = w;
-        if (c == NC - 1) f[1 + k] = w * (m.W[k] * invrho);
-      }
-      team_sync();
-    }
+    if (last) break;
+    base += CH;
   }
   // dT/dt by the last warp: its two species sums and the division.  Constant
   // volume: U/RT = H/RT - 1, cv/R = cp/R - 1.
@@ -448,10 +484,11 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 //   J[0][0]     = -(sum cv_k wdot_k + T sum U_k/RT a_k)/(rho cvm) - Tdot dcpm/cvm.
 // Needs b.vp >= S (one species a lane in the sums).
 static __device__ void team_jacobian(const DevMech& m, const double* tab, double p, const double* y,
-                              double* f, double* J, TeamBufs& b, Mix& x) {
+                              double* f, double* J, TeamBufs b) {
+  Mix x;
   const int S = m.S, n = m.n, SG = species_groups(S);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  team_species(m, p, y, b, x, tab);
+  team_species<true>(m, p, y, b, x, tab);
   // species block A starts at zero (the whole matrix is cleared: the
   // temperature row and column are written whole further down); chunk by
   // chunk, every entry touched by the chunk and every species sum (wdot,
@@ -543,7 +580,8 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
   team_sync();
   const double dcpm = sums[1], he = sums[3], cw = sums[4], ha = sums[5], eu = sums[6];
   const double Tdot = b.red[SC_TDOT], inv_cpm = b.red[SC_ICPM];
-  // species block (J_kj = A'_kj + dense_k / W_j) and temperature column
+  // species block (J_kj = A'_kj + dense_k / W_j) and temperature column and
+  // row, each product rounded as written
   // entries e = k S + j of the species block, (k, j) advanced without
   // dividing by the runtime S
   {
@@ -578,344 +616,221 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
   team_sync();
 }
 
-// LU with partial pivoting, register-tiled.  The CTA is a G x G grid of
-// threads laid out column-major: thread t = tc G + tr holds the elements
-// (tr + G r, tc + G c), r, c < T, of the n x n row-major matrix A (shared
-// memory, n <= G T) in registers, so the G owners of a matrix column are G
-// consecutive lanes of one warp.  An FP64 instruction costs a full warp slot
-// of the FP64 pipe however few lanes are active, and the non-FP64 work
-// around it sets how densely those slots fill, so step k (slot row and
-// column kq = k / G, position kt = k % G):
-//   1. the owners of column k pick the pivot among rows i >= k (magnitudes
-//      compared as integers: the bit pattern of |v| orders like |v|, NaN
-//      above +inf; ties take the smallest row) with shuffles of (magnitude,
-//      row) inside their group, fetch the pivot's value from the lane that
-//      holds its row, form 1 / pivot, and write the column below the
-//      diagonal, as it stands after the exchange of rows k and p (row p
-//      takes row k's entry), to lb; their whole warp scales it into the
-//      multipliers;
-//   2. barrier; the owners of rows k and p exchange the two rows through
-//      shared memory, which also publishes the new row k (the pivot row) in
-//      ub; barrier;
-//   3. every thread applies A_ij -= l_i u_j to its tile; column k below the
-//      diagonal becomes the multipliers.
-// Two barriers a step.  The slot bounds of a step are compile-time
-// constants (the step is instantiated for every kq), so the update carries
-// no per-element predicates: rows and columns beyond n are zero and lb / ub
-// are zero-padded there, and only slot row and column kq need per-thread
-// tests.  lb is double-buffered because the next pivot's owners write it
-// while other warps may still read the current one.
-// PRE = false: piv[k] receives the row swapped with row k (LAPACK order) and
-// A the factors.  PRE = true (the form the stage solves of ROS4 take): piv
-// receives the composite row permutation (row i of PA is row piv[i] of A),
-// and the strict upper triangle of U is stored pre-divided by its diagonal,
-// so that a solve gathers b once and needs no division in back
-// substitution.  On return A holds the unit lower factor below the diagonal
-// and the upper factor on and above it; invd[k] = 1 / U_kk.  Returns 0, or
-// k+1 when pivot k is zero or not finite (the same in every thread).
-// scratch: lu_scratch_words<G, T>() doubles of shared memory.
+// LU with partial pivoting of the n x n row-major matrix A (shared memory,
+// n <= 144) by the whole team, in place.  An FP64 instruction costs a full
+// warp slot of a pipe that takes 64 cycles a slot, while shared memory has
+// bandwidth to spare beside it (an update moves 3 loads and a store per
+// slot), so the trailing matrix stays in shared memory and its elements are
+// dealt to the lanes one by one, as a flat list: a pivot with m rows below it
+// costs ceil(m^2 / 32) slots, with no lanes lost to the edges of a tile, and
+// the team keeps no tile in registers (which lets more warps reside).
+// Rows are never moved: rows k.. of the permuted matrix are listed, with
+// their multipliers, in a row table (LuRow), rebuilt for every pivot.
+// One barrier a pivot: while the other warps update columns k + 2.. with
+// pivot k, one warp (a different one each time) updates column k + 1, picks
+// pivot k + 1 in it and forms its multipliers and row table (two tables, used
+// in turn).  Every element receives its updates in pivot order, so the
+// factors do not depend on how the elements are dealt.
+// Pivot: the largest magnitude of rows i >= k, ties to the smallest row
+// (magnitudes compared as integers: the bit pattern of |v| orders like |v|,
+// NaN above +inf).
+// On return rof[i] holds row i of PA as (its offset in A << 8) | row, A the
+// unit lower factor below the diagonal and the upper factor on and above it
+// (row i of them at offset rof[i] >> 8), invd[k] = 1 / U_kk.  PRE: the strict
+// upper triangle is stored divided by its diagonal, so that back
+// substitution needs no division.  lpiv (may be NULL) receives the row that
+// pivot k was swapped with (LAPACK order).  Returns 0, or k + 1 when pivot k
+// is zero or not finite (the same in every thread; A then holds the matrix as
+// updated by the pivots before k).
+// lr: 2 n entries of scratch, flag: one int of shared memory.
+template <class F>
+struct __align__(2 * sizeof(F)) LuRow {
+  F l;      // multiplier
+  int pk;   // (offset << 8) | row of A
+};
+
 // Bits of |v| as an unsigned integer (orders like |v|; NaN above +inf).
 __device__ __forceinline__ unsigned long long abs_key(double v) {
   return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
 }
 __device__ __forceinline__ unsigned long long abs_key(float v) {
-  return (unsigned long long)((unsigned)__float_as_int(v) & 0x7fffffffu);
+  return (unsigned long long)((unsigned)__float_as_int(v) & 0x7fffffffu) << 32;
 }
 __device__ __forceinline__ unsigned long long inf_key(double) { return 0x7ff0000000000000ULL; }
-__device__ __forceinline__ unsigned long long inf_key(float) { return 0x7f800000ULL; }
+__device__ __forceinline__ unsigned long long inf_key(float) { return 0x7f80000000000000ULL; }
 
-template <int G, int T>
-__host__ __device__ constexpr int lu_scratch_words() { return 4 * G * T + 2; }
+constexpr int LU_MAX_N = 144;
 
-
-// Slot row ps (>= KQ; the same in every thread) of a tile out to / in from
-// a shared row buffer.  The switch is on a CTA-uniform value, so only the
-// taken case executes, instead of a predicated copy of every slot row.
-template <int G, int T, int KQ, class F>
-__device__ __forceinline__ void lu_slot_row_out(const F (&a)[T][T], int ps, int tn, F* row) {
-  const int tc = threadIdx.x / G;
-  if constexpr (KQ < T) {
-    if (ps == KQ) {
-#pragma unroll
-      for (int c = 0; c < T; ++c)
-        if (c < tn) row[tc + G * c] = a[KQ][c];
-    } else {
-      lu_slot_row_out<G, T, KQ + 1>(a, ps, tn, row);
-    }
-  }
-}
-template <int G, int T, int KQ, class F>
-__device__ __forceinline__ void lu_slot_row_in(F (&a)[T][T], int ps, int tn, const F* row) {
-  const int tc = threadIdx.x / G;
-  if constexpr (KQ < T) {
-    if (ps == KQ) {
-#pragma unroll
-      for (int c = 0; c < T; ++c)
-        if (c < tn) a[KQ][c] = row[tc + G * c];
-    } else {
-      lu_slot_row_in<G, T, KQ + 1>(a, ps, tn, row);
-    }
-  }
-}
-
-// Pivot search of step k = KQ G + kt in its branch-free form, run by every
-// lane of the warp that holds column k: each group of G lanes searches its
-// own column, so the warp stays converged, and the group of column k alone
-// stores the multipliers (column k below the diagonal, as it stands after
-// the exchange of rows k and p, times 1 / pivot, each lane scaling its own
-// rows) in lb.  Returns the pivot row, or -1 when the pivot is zero or not
-// finite; ip receives 1 / pivot.  The results are bitwise those of the
-// owner-group form in lu_step.
-template <int G, int T, int KQ, bool FULL, class F>
-__device__ __forceinline__ int lu_pivot(const F (&a)[T][T], int n, int kt, F* scratch, F& ip) {
-  constexpr int GT = G * T;
-  const int tid = threadIdx.x, tr = tid % G, tc = tid / G;
-  const int k = KQ * G + kt;
-  const int tn = FULL ? T : (n + G - 1) / G;
-  F* lb = scratch + (k & 1) * GT;
-  const unsigned long long INFB = inf_key(F(0));
+// Pivot k, by one warp: column k updated with pivot k - 1, the pivot of rows
+// k.., and the multipliers and row order of the rows below it.
+template <class F>
+__device__ __forceinline__ void lu_panel(F* A, int n, int k, int* rof, int* lpiv, F* invd, LuRow<F>* lr, int* flag) {
+  constexpr int Q = (LU_MAX_N + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  const LuRow<F>* prev = lr + ((k + 1) & 1) * n;
+  LuRow<F>* next = lr + (k & 1) * n;
+  const F u = k > 0 ? A[(rof[k > 0 ? k - 1 : 0] >> 8) + k] : F(0);
+  F v[Q];
+  int pk[Q];
   unsigned long long best = 0;
   F bv = F(0);
-  int bi = n;
+  int bi = n, bpk = 0;
 #pragma unroll
-  for (int r = KQ; r < T; ++r) {
-    if (r >= tn) break;
-    const int i = tr + G * r;
-    const bool ok = (r > KQ || tr >= kt) && i < n;
-    const unsigned long long key = abs_key(a[r][KQ]);
-    const bool take = ok && key > best;
-    best = take ? key : best;
-    bv = take ? a[r][KQ] : bv;
-    bi = take ? i : bi;
-  }
-#pragma unroll
-  for (int off = 1; off < G; off <<= 1) {
-    const unsigned long long ok_ = __shfl_xor_sync(0xffffffffu, best, off, G);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, off, G);
-    const bool take = ok_ > best || (ok_ == best && oi < bi);
-    best = take ? ok_ : best;
-    bi = take ? oi : bi;
-  }
-  const int p = bi;
-  const bool sing = p >= n || best == 0 || best >= INFB;
-  bv = __shfl_sync(0xffffffffu, bv, p % G, G);  // the value from the lane that holds row p
-  const F akk = __shfl_sync(0xffffffffu, a[KQ][KQ], kt, G);
-  ip = rcp_rn(sing ? F(1) : bv);
-  if (tc == kt && !sing) {
-#pragma unroll
-    for (int r = KQ; r < T; ++r) {
-      if (r >= tn) break;
-      const int i = tr + G * r;
-      if (i > k && i < n) lb[i] = ((i == p) ? akk : a[r][KQ]) * ip;
-    }
-  }
-  return sing ? -1 : p;
-}
-
-// The pivot of step k, published by lane tr = 0 of column k's group.
-template <int G, bool PRE, class F>
-__device__ __forceinline__ void lu_publish(int k, int p, F ip, int* piv, F* invd, int* sp) {
-  const int tid = threadIdx.x;
-  if (tid / G == k % G && tid % G == 0) {
-    *sp = p;
-    if (p >= 0) {
-      invd[k] = ip;
-      if (PRE) {
-        const int t = piv[k];
-        piv[k] = piv[p];
-        piv[p] = t;
-      } else {
-        piv[k] = p;
-      }
-    }
-  }
-}
-
-// One pivot step at compile-time slot kq (see lu_reg).  Returns false when
-// the pivot is zero or not finite.
-template <int G, int T, int KQ, bool PRE, bool FULL, class F>
-__device__ __forceinline__ bool lu_step(F (&a)[T][T], int n, int kt, int* piv, F* invd, F* scratch) {
-  constexpr int GT = G * T;
-  const int tid = threadIdx.x, tr = tid % G, tc = tid / G, lane = tid & 31;
-  const int k = KQ * G + kt;
-  // slots that hold rows / columns below n (warp-uniform); FULL: all T
-  const int tn = FULL ? T : (n + G - 1) / G;
-  F* lb = scratch + (k & 1) * GT;
-  F* ub = scratch + 2 * GT;
-  F* xb = scratch + 3 * GT;
-  int* sp = reinterpret_cast<int*>(scratch + 4 * GT);
-  const unsigned long long INFB = inf_key(F(0));
-  // 1. pivot search, reciprocal and multipliers: the warp holding column k.
-  // The branch-free form measured faster everywhere but in the full-tile
-  // FP64 factorization of the 8 x 8 team, which keeps the owner-group form.
-  constexpr bool BF = !(G == 8 && FULL && sizeof(F) == 8);
-  const int owner_warp = (kt * G) >> 5;
-  if constexpr (BF) {
-    if ((tid >> 5) == owner_warp) {
-      F ip;
-      const int p0 = lu_pivot<G, T, KQ, FULL>(a, n, kt, scratch, ip);
-      lu_publish<G, PRE>(k, p0, ip, piv, invd, sp);
-    }
-  } else if ((tid >> 5) == owner_warp) {
-    const int base = (kt * G) & 31;  // first lane of the owner group
-    bool sing = false;
-    F ip = F(0);
-    if (tc == kt) {
-      const unsigned gmask = (G >= 32 ? 0xffffffffu : ((1u << G) - 1u)) << base;
-      unsigned long long best = 0;
-      F bv = F(0);
-      int bi = n;
-#pragma unroll
-      for (int r = KQ; r < T; ++r) {
-        if (r >= tn) break;
-        const int i = tr + G * r;
-        const bool ok = (r > KQ || tr >= kt) && i < n;
-        const unsigned long long key = abs_key(a[r][KQ]);
-        if (ok && key > best) {
+  for (int q = 0; q < Q; ++q) {
+    const int i = k + lane + 32 * q;
+    v[q] = F(0);
+    pk[q] = 0;
+    if (k + 32 * q < n) {  // warp-uniform
+      if (i < n) {
+        const LuRow<F> r = prev[i];
+        pk[q] = r.pk;
+        v[q] = A[(r.pk >> 8) + k];
+        if (k > 0) v[q] = fma(-r.l, u, v[q]);
+        const unsigned long long key = abs_key(v[q]);
+        if (key > best) {
           best = key;
-          bv = a[r][KQ];
+          bv = v[q];
           bi = i;
-        }
-      }
-#pragma unroll
-      for (int off = 1; off < G; off <<= 1) {
-        const unsigned long long ok_ = __shfl_xor_sync(gmask, best, off, G);
-        const int oi = __shfl_xor_sync(gmask, bi, off, G);
-        if (ok_ > best || (ok_ == best && oi < bi)) {
-          best = ok_;
-          bi = oi;
-        }
-      }
-      const int p = bi;
-      sing = p >= n || best == 0 || best >= INFB;
-      bv = __shfl_sync(gmask, bv, p % G, G);  // the value from the lane that holds row p
-      // column k as it stands after the exchange: row p takes row k's entry
-      const F akk = __shfl_sync(gmask, a[KQ][KQ], kt, G);
-      if (!sing) {
-        ip = rcp_rn(bv);
-#pragma unroll
-        for (int r = KQ; r < T; ++r) {
-          if (r >= tn) break;
-          const int i = tr + G * r;
-          if (i > k && i < n) lb[i] = (i == p) ? akk : a[r][KQ];
-        }
-      }
-      if (tr == 0) {
-        *sp = sing ? -1 : p;
-        if (!sing) {
-          invd[k] = ip;
-          if (PRE) {
-            const int t = piv[k];
-            piv[k] = piv[p];
-            piv[p] = t;
-          } else {
-            piv[k] = p;
-          }
+          bpk = r.pk;
         }
       }
     }
-    __syncwarp();
-    sing = __shfl_sync(0xffffffffu, (int)sing, base) != 0;
-    ip = __shfl_sync(0xffffffffu, ip, base);
-    if (!sing)
-      for (int i = k + 1 + lane; i < n; i += 32) lb[i] *= ip;
   }
-  __syncthreads();
-  const int p = *sp;
-  if (p < 0) return false;
-  // 2. exchange rows k and p; the new row k (the pivot row) lands in ub
-  const int pt = p % G, ps = p / G;
-  if (tr == kt) {
+  const unsigned hi = (unsigned)(best >> 32);
+  const unsigned H = __reduce_max_sync(0xffffffffu, hi);
+  unsigned L = 0;
+  if (sizeof(F) == 8) L = __reduce_max_sync(0xffffffffu, hi == H ? (unsigned)best : 0u);
+  const bool mine = hi == H && (sizeof(F) < 8 || (unsigned)best == L);
+  const int p = (int)__reduce_min_sync(0xffffffffu, mine ? (unsigned)bi : (unsigned)n);
+  const unsigned long long top = ((unsigned long long)H << 32) | L;
+  if (p >= n || top == 0 || top >= inf_key(F(0))) {
 #pragma unroll
-    for (int c = 0; c < T; ++c)
-      if (c < tn) (p != k ? xb : ub)[tc + G * c] = a[KQ][c];
+    for (int q = 0; q < Q; ++q) {
+      const int i = k + lane + 32 * q;
+      if (i < n) {
+        A[(pk[q] >> 8) + k] = v[q];
+        rof[i] = pk[q];  // the row order as it stands
+      }
+    }
+    if (lane == 0) *flag = k + 1;
+    return;
   }
-  if (p != k && tr == pt) lu_slot_row_out<G, T, KQ>(a, ps, tn, ub);
-  __syncthreads();
-  if (p != k) {
-    if (tr == kt) {
-#pragma unroll
-      for (int c = 0; c < T; ++c)
-        if (c < tn) a[KQ][c] = ub[tc + G * c];
-    }
-    if (tr == pt) lu_slot_row_in<G, T, KQ>(a, ps, tn, xb);
+  const int from = (p - k) & 31;
+  bv = __shfl_sync(0xffffffffu, bv, from);
+  bpk = __shfl_sync(0xffffffffu, bpk, from);
+  const F vk = __shfl_sync(0xffffffffu, v[0], 0);
+  const int pkk = __shfl_sync(0xffffffffu, pk[0], 0);
+  const F ip = rcp_rn(bv);
+  if (lane == 0) {
+    rof[k] = bpk;
+    A[(bpk >> 8) + k] = bv;
+    invd[k] = ip;
+    if (lpiv) lpiv[k] = p;
   }
-  // 3. rank-one update of the trailing tile; column k takes the multipliers.
-  // Slots at or beyond tn hold only padding and are left alone.
-  F u[T];
 #pragma unroll
-  for (int c = KQ; c < T; ++c) u[c] = c < tn ? ub[tc + G * c] : F(0);
-  // slot column KQ needs work only in warps holding a column >= k (the G
-  // lanes of a column are consecutive, so the warp's largest tc is its last
-  // lane's): a warp-uniform test that lets the other warps skip it.  The
-  // FP32 factorization of the precision form measured faster without it.
-  const bool wcol = sizeof(F) < 8 || ((tid | 31) / G) >= kt;
-#pragma unroll
-  for (int r = KQ; r < T; ++r) {
-    if (r >= tn) break;
-    const bool live = r > KQ || tr > kt;  // row tr + G r lies below row k
-    const F li = live ? lb[tr + G * r] : F(0);
-#pragma unroll
-    for (int c = KQ + 1; c < T; ++c) {
-      if (c >= tn) break;
-      a[r][c] = fma(-li, u[c], a[r][c]);
+  for (int q = 0; q < Q; ++q) {
+    const int i = k + lane + 32 * q;
+    if (k + 32 * q < n) {
+      // row p takes row k's entry
+      LuRow<F> r;
+      r.l = (i == p ? vk : v[q]) * ip;
+      r.pk = i == p ? pkk : pk[q];
+      if (i > k && i < n) {
+        next[i] = r;
+        A[(r.pk >> 8) + k] = r.l;
+      }
     }
-    if (wcol) {
-      if (tc > kt) a[r][KQ] = fma(-li, u[KQ], a[r][KQ]);
-      else if (tc == kt && live) a[r][KQ] = li;
-    }
-  }
-  return true;
-}
-
-template <int G, int T, bool PRE, bool FULL, int KQ, class F>
-__device__ __forceinline__ int lu_slots(F (&a)[T][T], int n, int* piv, F* invd, F* scratch) {
-  if constexpr (KQ < T) {
-    for (int kt = 0; kt < G; ++kt) {
-      if (KQ * G + kt >= n) return 0;
-      if (!lu_step<G, T, KQ, PRE, FULL>(a, n, kt, piv, invd, scratch)) return KQ * G + kt + 1;
-    }
-    return lu_slots<G, T, PRE, FULL, KQ + 1>(a, n, piv, invd, scratch);
-  } else {
-    return 0;
   }
 }
 
-template <int G, int T, bool PRE = false, class F>
-__device__ int lu_reg(F* A, int n, int* piv, F* invd, F* scratch) {
-  const int tid = threadIdx.x, tr = tid % G, tc = tid / G;
-  for (int e = tid; e < lu_scratch_words<G, T>(); e += blockDim.x) scratch[e] = F(0);
-  for (int i = tid; i < n; i += blockDim.x) piv[i] = i;
-  F a[T][T];
-#pragma unroll
-  for (int r = 0; r < T; ++r)
-#pragma unroll
-    for (int c = 0; c < T; ++c) {
-      const int i = tr + G * r, j = tc + G * c;
-      a[r][c] = (i < n && j < n) ? A[i * n + j] : F(0);
-    }
-  __syncthreads();
-  // every slot holds real rows and columns (n > G (T - 1)): the steps need no
-  // run-time slot bound
-  const int info = (n > G * (T - 1)) ? lu_slots<G, T, PRE, true, 0>(a, n, piv, invd, scratch)
-                                     : lu_slots<G, T, PRE, false, 0>(a, n, piv, invd, scratch);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < T; ++r) {
-    const int i = tr + G * r;
-    const F di = (PRE && i < n) ? invd[i] : F(1);
-#pragma unroll
-    for (int c = 0; c < T; ++c) {
-      const int j = tc + G * c;
-      // slot (r, c) lies wholly above the diagonal when c > r and wholly
-      // below it when c < r (tr, tc < G), so only c == r needs the test
-      F v = a[r][c];
-      if (PRE && (c > r || (c == r && tc > tr))) v = a[r][c] * di;
-      if (i < n && j < n) A[i * n + j] = v;
-    }
+// Element e of a list of rows of c elements: its row, for e < 2^14, c <= 144
+// (rc = 1 / c in FP32: (e + 1/2) / c is at least 1 / (2 c) away from an
+// integer, far more than its rounding error of 2^-22 e / c).
+__device__ __forceinline__ int flat_row(int e, float rc) { return (int)(((float)e + 0.5f) * rc); }
+
+template <bool PRE, class F>
+__device__ __noinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd, LuRow<F>* lr, int* flag) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int i = tid; i < n; i += blockDim.x) {
+    lr[n + i].pk = (i * n) << 8 | i;
+    if (lpiv) lpiv[i] = i;
   }
-  __syncthreads();
-  return info;
+  if (tid == 0) *flag = 0;
+  team_sync();
+  if (warp == 0) lu_panel(A, n, 0, rof, lpiv, invd, lr, flag);
+  team_sync();
+  if (*flag) return *flag;
+  constexpr int C0 = 10;  // a panel costs its warp about as much as this many updates of 32 elements
+  int pw = 1 % nw;        // the warp of the next panel
+  for (int k = 0; k + 1 < n; ++k) {
+    const int m = n - 1 - k, mc = m - 1, E = m * mc, NG = (E + 31) >> 5;
+    // groups of 32 elements: the panel's warp takes the last gp, the others
+    // share the rest
+    int gp = NG, g0 = 0, gs = 1, g1 = NG;
+    if (nw > 1) {
+      const int per = (NG + C0 + nw - 1) / nw;
+      gp = per > C0 ? per - C0 : 0;
+      if (warp == pw) {
+        g0 = NG - gp;
+      } else {
+        g0 = warp - pw - 1;
+        if (g0 < 0) g0 += nw;
+        gs = nw - 1;
+        g1 = NG - gp;
+      }
+    }
+    if (warp == pw) lu_panel(A, n, k + 1, rof, lpiv, invd, lr, flag);
+    const LuRow<F>* R = lr + (k & 1) * n + k + 1;
+    const F* U = A + (rof[k] >> 8) + k + 2;
+    F* A2 = A + k + 2;
+    const float rc = 1.0f / (float)(mc > 0 ? mc : 1);
+    int g = g0;
+    for (; g + 3 * gs < g1; g += 4 * gs) {
+      F l[4], u[4], a[4];
+      int o[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int e0 = 32 * (g + t * gs) + lane, e = e0 < E ? e0 : E - 1;
+        const int i = flat_row(e, rc), j = e - i * mc;
+        const LuRow<F> r = R[i];
+        l[t] = r.l;
+        u[t] = U[j];
+        o[t] = (r.pk >> 8) + j;
+        a[t] = A2[o[t]];
+        if (e0 >= E) o[t] = -1;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const F w = fma(-l[t], u[t], a[t]);
+        if (o[t] >= 0) A2[o[t]] = w;
+      }
+    }
+    for (; g < g1; g += gs) {
+      const int e = 32 * g + lane;
+      if (e < E) {
+        const int i = flat_row(e, rc), j = e - i * mc;
+        const LuRow<F> r = R[i];
+        F* a = A2 + (r.pk >> 8) + j;
+        *a = fma(-r.l, U[j], *a);
+      }
+    }
+    if (++pw == nw) pw = 0;
+    team_sync();
+    if (*flag) return *flag;
+  }
+  if (PRE) {
+    // rows r and n - 2 - r of the strict upper triangle have n elements together
+    const int E = n * (n - 1) / 2;
+    const float rc = 1.0f / (float)n;
+    for (int e = tid; e < E; e += blockDim.x) {
+      const int r = flat_row(e, rc), c = e - r * n, m = n - 1 - r;
+      const int i = c < m ? r : n - 2 - r, j = c < m ? r + 1 + c : n - 1 - r + (c - m);
+      F* a = A + (rof[i] >> 8) + j;
+      *a = *a * invd[i];
+    }
+    team_sync();
+  }
+  return 0;
 }
 
 // Solve (LU) x = b in place with one warp (b in shared memory).  Must be
@@ -924,8 +839,9 @@ __device__ int lu_reg(F* A, int n, int* piv, F* invd, F* scratch) {
 // earlier blocks is a matrix-vector product (one row per lane, four partial
 // sums in a fixed order), the diagonal block a substitution whose solved
 // value is broadcast by a shuffle.
-// PRE: the factors and permutation come from lu_reg<G, T, true> (gather by
-// the composite permutation, U pre-divided by its diagonal).
+// PRE: the factors come from lu_flat<true> (rows listed in its row table rof,
+// passed as piv: gather by it, U pre-divided by its diagonal); else rows in
+// order and piv[k] the row swapped with row k.
 template <bool PRE = false, class F>
 __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv, const F* invd, F* b) {
   const int lane = threadIdx.x & 31;
@@ -935,7 +851,7 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
 #pragma unroll
     for (int q = 0; q < MAXR; ++q) {
       const int i = lane + 32 * q;
-      g[q] = i < n ? b[piv[i]] : F(0);
+      g[q] = i < n ? b[piv[i] & 255] : F(0);
     }
     __syncwarp();
 #pragma unroll
@@ -959,8 +875,8 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     const int i = B0 + lane;
     const bool act = i < n;
     F s0 = act ? b[i] : F(0), s1 = F(0), s2 = F(0), s3 = F(0);
+    const F* Li = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * n);
     if (act) {
-      const F* Li = A + (size_t)i * n;
       int j = 0;
       for (; j + 4 <= B0; j += 4) {
         s0 = fma(-Li[j], b[j], s0);
@@ -974,7 +890,7 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     const int m = min(32, n - B0);
     for (int jj = 0; jj < m; ++jj) {
       const F yj = __shfl_sync(0xffffffffu, s, jj);
-      if (act && lane > jj) s = fma(-A[(size_t)i * n + B0 + jj], yj, s);
+      if (act && lane > jj) s = fma(-Li[B0 + jj], yj, s);
     }
     if (act) b[i] = s;
     __syncwarp();
@@ -985,8 +901,8 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     const bool act = i < n;
     const int m = min(32, n - B1);
     F s0 = act ? (PRE ? b[i] * invd[i] : b[i]) : F(0), s1 = F(0), s2 = F(0), s3 = F(0);
+    const F* Ui = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * n);
     if (act) {
-      const F* Ui = A + (size_t)i * n;
       int j = B1 + 32;
       for (; j + 4 <= n; j += 4) {
         s0 = fma(-Ui[j], b[j], s0);
@@ -1000,7 +916,7 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     for (int jj = m - 1; jj >= 0; --jj) {
       if (!PRE && lane == jj) s *= invd[i];
       const F xj = __shfl_sync(0xffffffffu, s, jj);
-      if (act && lane < jj) s = fma(-A[(size_t)i * n + B1 + jj], xj, s);
+      if (act && lane < jj) s = fma(-Ui[B1 + jj], xj, s);
     }
     if (act) b[i] = s;
     __syncwarp();

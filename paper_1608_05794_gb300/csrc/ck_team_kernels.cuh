@@ -10,36 +10,12 @@
 
 namespace ck {
 
-static __host__ __device__ __forceinline__ int team_bufs_doubles(int S, int chunk) {
-  return 4 * (S + 1) + 5 * S + (3 + JP) * chunk + TEAM_RED;
-}
-
-static __device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH, int vp) {
-  TeamBufs b;
-  b.X = base;
-  b.Gp = b.X + S + 1;
-  b.Gm = b.Gp + S + 1;
-  b.hRT = b.Gm + S + 1;
-  b.cpR = b.hRT + S + 1;
-  b.wd = b.cpR + S;
-  b.aT = b.wd + S;
-  b.E = b.aT + S;
-  b.u = b.E + S;
-  b.q = b.u + S;
-  b.dqT = b.q + CH;
-  b.D = b.dqT + CH;
-  b.P = b.D + CH;
-  b.red = b.P + (size_t)JP * CH;
-  b.vp = vp;
-  return b;
-}
-
 // Next reactor index for this CTA from the global queue (same in every thread).
 static __device__ __forceinline__ int team_next(int32_t* queue, int* slot) {
   if (threadIdx.x == 0) *slot = atomicAdd(queue, 1);
-  __syncthreads();
+  team_sync();
   const int r = *slot;
-  __syncthreads();
+  team_sync();
   return r;
 }
 
@@ -50,20 +26,26 @@ static __device__ __forceinline__ int team_next(int32_t* queue, int* slot) {
 // (f(y + s_j e_j) - f(y)) / s_j with s_j = max(sqrt(U) |y_j|, s0 / w_j).
 // f0 = f(y) is computed here (unless have_f0: the caller already holds it
 // for this y) and reused as the first stage's f; the n columns cost n team
-// RHS evaluations.  Yt, F: n-vector scratch.
-static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const double* tab, double p,
-                                                     const double* y, double h, double rtol, double atol,
-                                                     double* f0, double* J, double* Yt, double* F, TeamBufs b,
-                                                     bool have_f0 = false) {
+// RHS evaluations.  y_o, f0_o, yt_o, f_o: offsets of n-vectors in shared
+// memory (the last two scratch); bufs_o, vp, qq as in team_rhs.
+static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const double* tab, double p, int y_o, double h,
+                                                     double rtol, double atol, int f0_o, double* J, int yt_o,
+                                                     int f_o, int bufs_o, int vp, RhsQ qq, bool have_f0 = false) {
+  extern __shared__ __align__(16) double sm[];
+  const double* y = sm + y_o;
+  const double* f0 = sm + f0_o;
+  const double* F = sm + f_o;
+  double* Yt = sm + yt_o;
   const int n = d.n;
-  if (!have_f0) team_rhs(d, tab, p, y, f0, b);
+  if (!have_f0) team_rhs(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double v = f0[i] / (atol + rtol * fabs(y[i]));
-    s = fma(v, v, s);
-    Yt[i] = y[i];
-  }
-  const double fn = sqrt(team_sum(s, b.red) / n);
+  if ((int)threadIdx.x < vp)
+    for (int i = threadIdx.x; i < n; i += vp) {
+      const double v = f0[i] / (atol + rtol * fabs(y[i]));
+      s = fma(v, v, s);
+      Yt[i] = y[i];
+    }
+  const double fn = sqrt(team_sum(s, sm + bufs_o) / n);
   const double U = 2.220446049250313080847e-16;  // 2^-52
   const double srur = 1.490116119384765625e-8;   // 2^-26 = sqrt(U)
   const double s0 = (fn != 0.0) ? 1000.0 * fabs(h) * U * n * fn : 1.0;
@@ -71,7 +53,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
     const double sj = fmax(srur * fabs(y[j]), s0 * (atol + rtol * fabs(y[j])));
     if (threadIdx.x == 0) Yt[j] = y[j] + sj;
     team_sync();
-    team_rhs(d, tab, p, Yt, F, b);
+    team_rhs(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
     for (int i = threadIdx.x; i < n; i += blockDim.x) J[(size_t)i * n + j] = (F[i] - f0[i]) / sj;
     if (threadIdx.x == 0) Yt[j] = y[j];
     team_sync();
@@ -89,50 +71,87 @@ static __device__ __forceinline__ double team_pow(double x, double q, double* re
   return red[SC_POW];
 }
 
-// ------------------------------------------------------------------ ROS4
 // Weighted RMS norm over the team (reading shared with the oracle:
-// sqrt(mean (e_i / (atol + rtol max(|y_i|, |ynew_i|)))^2)).
-static __device__ __forceinline__ double team_wrms(int n, const double* e, const double* y0,
-                                            const double* y1, double rtol, double atol, double* red) {
+// sqrt(mean (e_i / (atol + rtol max(|y_i|, |ynew_i|)))^2)).  vp: the lanes
+// that the components are dealt to (as the species sums).
+static __device__ __forceinline__ double team_wrms(int n, const double* e, const double* y0, const double* y1,
+                                                   double rtol, double atol, double* red, int vp) {
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double sc = atol + rtol * fmax(fabs(y0[i]), fabs(y1[i]));
-    const double v = e[i] / sc;
-    s = fma(v, v, s);
-  }
+  if ((int)threadIdx.x < vp)
+    for (int i = threadIdx.x; i < n; i += vp) {
+      const double sc = atol + rtol * fmax(fabs(y0[i]), fabs(y1[i]));
+      const double v = e[i] / sc;
+      s = fma(v, v, s);
+    }
   s = team_sum(s, red);
   return sqrt(s / n);
 }
 
 // Initial step, Hairer-Norsett-Wanner starting-step algorithm (order 4).
-static __device__ double team_h0(const DevMech& d, const double* tab, double p, const double* y0, double tspan,
-                          double rtol, double atol, double* f0, double* y1, double* f1, TeamBufs& b,
-                          Mix& x) {
+// Offsets, vp and qq as in team_rhs; f0, y1, f1 are scratch vectors.
+static __device__ __noinline__ double team_h0(const DevMech& d, const double* tab, double p, int y0_o, double tspan,
+                                              double rtol, double atol, int f0_o, int y1_o, int f1_o, int bufs_o,
+                                              int vp, RhsQ qq) {
+  extern __shared__ __align__(16) double sm[];
+  const double *y0 = sm + y0_o, *f0 = sm + f0_o, *f1 = sm + f1_o;
+  double *y1 = sm + y1_o, *red = sm + bufs_o;
   const int n = d.n;
-  team_rhs(d, tab, p, y0, f0, b);
+  const bool lane_in = (int)threadIdx.x < vp;
+  team_rhs(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
   double s0 = 0.0, s1 = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double sc = atol + rtol * fabs(y0[i]);
-    s0 = fma(y0[i] / sc, y0[i] / sc, s0);
-    s1 = fma(f0[i] / sc, f0[i] / sc, s1);
-  }
-  const double d0 = sqrt(team_sum(s0, b.red) / n);
-  const double d1 = sqrt(team_sum(s1, b.red) / n);
+  if (lane_in)
+    for (int i = threadIdx.x; i < n; i += vp) {
+      const double sc = atol + rtol * fabs(y0[i]);
+      s0 = fma(y0[i] / sc, y0[i] / sc, s0);
+      s1 = fma(f0[i] / sc, f0[i] / sc, s1);
+    }
+  const double d0 = sqrt(team_sum(s0, red) / n);
+  const double d1 = sqrt(team_sum(s1, red) / n);
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   for (int i = threadIdx.x; i < n; i += blockDim.x) y1[i] = fma(ha, f0[i], y0[i]);
   team_sync();
-  team_rhs(d, tab, p, y1, f1, b);
+  team_rhs(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
   double s2 = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double sc = atol + rtol * fabs(y0[i]);
-    const double v = (f1[i] - f0[i]) / sc;
-    s2 = fma(v, v, s2);
-  }
-  const double d2 = sqrt(team_sum(s2, b.red) / n) / ha;
+  if (lane_in)
+    for (int i = threadIdx.x; i < n; i += vp) {
+      const double sc = atol + rtol * fabs(y0[i]);
+      const double v = (f1[i] - f0[i]) / sc;
+      s2 = fma(v, v, s2);
+    }
+  const double d2 = sqrt(team_sum(s2, red) / n) / ha;
   const double dm = fmax(d1, d2);
   const double hb = (dm <= 1e-15) ? fmax(1e-6, ha * 1e-3) : pow(0.01 / dm, 0.2);
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
+
+// Shared memory of one k_ros4 CTA, in doubles: the matrix, y and f(y), the
+// team's work arrays, and behind them the Jacobian's chunk or, at other times,
+// the stage vectors, the factors' row table and the rates of progress (or the
+// LU's scratch).
+struct Ros4Layout {
+  int vp, yv, f0, bufs, yt, ub, invd, rof, lr;
+  RhsQ rhs_q;
+  size_t doubles;
+  __host__ __device__ Ros4Layout(int n, int S, int chunk, int rhs_chunk) {
+    vp = n > 64 ? 256 : 64;
+    yv = n * n;
+    f0 = yv + n;
+    bufs = f0 + n;
+    const int t = bufs + species_doubles(S);
+    yt = t;
+    ub = yt + n;
+    invd = ub + n;
+    rof = invd + n;
+    const int after = (rof + (n + 1) / 2 + 1) & ~1;  // 16-byte aligned
+    lr = after;
+    rhs_q.off = after;
+    rhs_q.chunk = rhs_chunk;
+    int most = t + jac_doubles(S, chunk);
+    if (after + 4 * n > most) most = after + 4 * n;
+    if (after + rhs_chunk > most) most = after + rhs_chunk;
+    doubles = (size_t)most;
+  }
+};
 
 // ------------------------------------------------------------------ launch helpers
 // Persistent grid: as many CTAs of `kernel` as fit on every SM (or the
@@ -147,11 +166,6 @@ static inline int team_grid(K kernel, int threads, size_t smem, int64_t work, co
   int64_t g = (int64_t)per_sm * sm_count();
   if (work < g) g = work;
   return (int)(g < 1 ? 1 : g);
-}
-
-// Shared memory of one k_ros4 CTA for a mechanism of n = S + 1.
-inline size_t ros4_smem_bytes(int n, int S, int chunk) {
-  return sizeof(double) * ((size_t)n * n + 9 * (size_t)n + (n + 1) / 2 + team_bufs_doubles(S, chunk));
 }
 
 }  // namespace ck
