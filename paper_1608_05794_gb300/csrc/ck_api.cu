@@ -307,93 +307,111 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   csr_ptr[S] = (int32_t)csr_rx.size();
   // team kernels walk the reactions in chunks: equal shares of at most what
   // the team's shared memory has room for
-  const int n1 = S + 1;
+  const int n1 = S + 1, NN = n1 * n1;
   auto shares = [&](int most) { return R ? (R + (R + most - 1) / most - 1) / ((R + most - 1) / most) : 1; };
-  const int chunk = shares(n1 <= 24 ? 64 : (n1 <= 64 ? 112 : 60));
-  const int n_chunks = (R + chunk - 1) / chunk;
+  int first_typed = 0;
+  while (first_typed < R && rx[first_typed].type == 0) ++first_typed;
   const int rhs_chunk = shares(n1 <= 64 ? 512 : 392);
   const int n_rhs_chunks = (R + rhs_chunk - 1) / rhs_chunk;
-  auto cut = [&](int size, int count) {  // first CSR entry of every species and chunk
-    std::vector<int32_t> c((size_t)S * (count + 1));
-    for (int k = 0; k < S; ++k) {
-      int e = csr_ptr[k];
-      for (int i = 0; i <= count; ++i) {
-        while (e < csr_ptr[k + 1] && csr_rx[e] < i * size) ++e;
-        c[(size_t)k * (count + 1) + i] = (i == count) ? csr_ptr[k + 1] : e;
-      }
+  std::vector<int32_t> csr_cptr((size_t)S * (n_rhs_chunks + 1));  // first CSR entry of every species and chunk
+  for (int k = 0; k < S; ++k) {
+    int e = csr_ptr[k];
+    for (int i = 0; i <= n_rhs_chunks; ++i) {
+      while (e < csr_ptr[k + 1] && csr_rx[e] < i * rhs_chunk) ++e;
+      csr_cptr[(size_t)k * (n_rhs_chunks + 1) + i] = (i == n_rhs_chunks) ? csr_ptr[k + 1] : e;
     }
-    return c;
-  };
-  const std::vector<int32_t> jac_cptr = cut(chunk, n_chunks), csr_cptr = cut(rhs_chunk, n_rhs_chunks);
+  }
   // Jacobian assembly, chunk by chunk, as one list of targets, each adding a
-  // fixed-order sum of coef * src[pidx] (src: the chunk's per-reaction
-  // arrays q, dq/dT, D and the partials P, contiguous in shared memory):
+  // fixed-order sum of coef * src[pidx] (src: the chunk's per-reaction values
+  // q, dq/dT, D, the partials and the typed reactions' w, contiguous in shared
+  // memory):
   // - species-block entries A[k][j] += nu_ki * P[i][slot] for every slot of
-  //   reaction i holding species j (and nu_ki (eff_ij - 1) * P[i][6] for the
+  //   reaction i holding species j (and nu_ki (eff_ij - 1) * w[i] for the
   //   third-body corrections), target index (1 + k) n + 1 + j;
   // - per species k the four sums over its reactions in the chunk, wdot_k
-  //   (nu q), a_k (nu dq/dT), E_k (nu D) and u_k (nu P[i][6]), target index
+  //   (nu q), a_k (nu dq/dT), E_k (nu D) and u_k (nu w), target index
   //   n^2 + a S + k for a = 0..3, terms in the CSR order.
   // Longest lists first, so that lanes running the same iteration do similar
-  // amounts of work.
-  std::vector<int32_t> jc_ptr(1, 0);
-  std::vector<JcEntry> jc;
-  std::vector<JcTerm> jt;
+  // amounts of work.  The terms of a target come in reaction order whatever
+  // the chunks, so its sum does not depend on them.
+  struct JacHost {
+    int chunk = 1, n_chunks = 1, scratch = 0;
+    std::vector<int32_t> jc_ptr;
+    std::vector<JcEntry> jc;
+    std::vector<JcTerm> jt;
+  };
   int n_jterms = 0;
-  const int NN = (S + 1) * (S + 1);
-  for (int c = 0; c < n_chunks; ++c) {
-    std::vector<std::vector<std::pair<double, int32_t>>> ent((size_t)S * S + 4 * (size_t)S);
-    for (int k = 0; k < S; ++k) {
-      for (int e = jac_cptr[(size_t)k * (n_chunks + 1) + c]; e < jac_cptr[(size_t)k * (n_chunks + 1) + c + 1];
-           ++e) {
-        const int i = csr_rx[e];
-        const int li = i - c * chunk;
-        const double nu = csr_nu[e];
-        const RxnRec& r = rx[i];
-        const int32_t pbase = 3 * chunk + li * JP;
-        // coefficients carry W_k / W_j, the factor of the species block
-        // dY_k/dY_j (so the assembly needs no per-entry rescaling)
-        auto wr = [&](int j) { return (double)((long double)W[k] / (long double)W[j]); };
-        for (int s2 = 0; s2 < r.nreac; ++s2)
-          ent[(size_t)k * S + r.sp[s2]].push_back({nu * wr(r.sp[s2]), pbase + s2});
-        if (r.rev)
-          for (int s2 = 0; s2 < r.nprod; ++s2)
-            ent[(size_t)k * S + r.sp[3 + s2]].push_back({nu * wr(r.sp[3 + s2]), pbase + 3 + s2});
-        for (int q = r.eff_beg; q < r.eff_beg + r.eff_cnt; ++q)
-          ent[(size_t)k * S + eff_sp[q]].push_back({nu * eff_m1[q] * wr(eff_sp[q]), pbase + 6});
-        const size_t sb = (size_t)S * S;
-        ent[sb + 0 * S + k].push_back({nu, li});
-        ent[sb + 1 * S + k].push_back({nu, chunk + li});
-        ent[sb + 2 * S + k].push_back({nu, 2 * chunk + li});
-        if (r.type) ent[sb + 3 * S + k].push_back({nu, pbase + 6});
+  auto jac_table = [&](int chunk) {
+    JacHost t;
+    t.chunk = chunk;
+    t.n_chunks = R ? (R + chunk - 1) / chunk : 1;
+    t.jc_ptr.push_back(0);
+    n_jterms = 0;
+    int typed_most = 0;
+    for (int c = 0; c < t.n_chunks; ++c) {
+      const int base = c * chunk, end = std::min(R, base + chunk), ft = std::max(first_typed - base, 0);
+      typed_most = std::max(typed_most, end - std::max(base, first_typed));
+      std::vector<std::vector<std::pair<double, int32_t>>> ent((size_t)S * S + 4 * (size_t)S);
+      for (int k = 0; k < S; ++k) {
+        for (int e = csr_ptr[k]; e < csr_ptr[k + 1]; ++e) {
+          const int i = csr_rx[e];
+          if (i < base || i >= end) continue;
+          const int li = i - base;
+          const double nu = csr_nu[e];
+          const RxnRec& r = rx[i];
+          const int32_t pbase = 3 * chunk + li * 6, pw = JAC_PER_RXN * chunk + li - ft;
+          // coefficients carry W_k / W_j, the factor of the species block
+          // dY_k/dY_j (so the assembly needs no per-entry rescaling)
+          auto wr = [&](int j) { return (double)((long double)W[k] / (long double)W[j]); };
+          for (int s2 = 0; s2 < r.nreac; ++s2)
+            ent[(size_t)k * S + r.sp[s2]].push_back({nu * wr(r.sp[s2]), pbase + s2});
+          if (r.rev)
+            for (int s2 = 0; s2 < r.nprod; ++s2)
+              ent[(size_t)k * S + r.sp[3 + s2]].push_back({nu * wr(r.sp[3 + s2]), pbase + 3 + s2});
+          for (int q = r.eff_beg; q < r.eff_beg + r.eff_cnt; ++q)
+            ent[(size_t)k * S + eff_sp[q]].push_back({nu * eff_m1[q] * wr(eff_sp[q]), pw});
+          const size_t sb = (size_t)S * S;
+          ent[sb + 0 * S + k].push_back({nu, li});
+          ent[sb + 1 * S + k].push_back({nu, chunk + li});
+          ent[sb + 2 * S + k].push_back({nu, 2 * chunk + li});
+          if (r.type) ent[sb + 3 * S + k].push_back({nu, pw});
+        }
       }
+      std::vector<int> order_e;
+      for (size_t e = 0; e < ent.size(); ++e)
+        if (c == 0 || !ent[e].empty()) order_e.push_back((int)e);
+      std::stable_sort(order_e.begin(), order_e.end(),
+                       [&](int a, int b) { return ent[a].size() > ent[b].size(); });
+      for (int e : order_e) {
+        JcEntry h{};
+        if (e < S * S) {
+          const int k = e / S, j = e % S;
+          h.idx = (1 + k) * n1 + 1 + j;
+          n_jterms += (int)ent[e].size();
+        } else {
+          h.idx = NN + (e - S * S);
+        }
+        h.beg = (int32_t)t.jt.size();
+        for (auto& cc : ent[e]) {
+          JcTerm u{};
+          u.coef = cc.first;
+          u.pidx = cc.second;
+          t.jt.push_back(u);
+        }
+        h.end = (int32_t)t.jt.size();
+        t.jc.push_back(h);
+      }
+      t.jc_ptr.push_back((int32_t)t.jc.size());
     }
-    std::vector<int> order_e;
-    for (size_t e = 0; e < ent.size(); ++e)
-      if (!ent[e].empty()) order_e.push_back((int)e);
-    std::stable_sort(order_e.begin(), order_e.end(),
-                     [&](int a, int b) { return ent[a].size() > ent[b].size(); });
-    for (int e : order_e) {
-      JcEntry h{};
-      if (e < S * S) {
-        const int k = e / S, j = e % S;
-        h.idx = (1 + k) * (S + 1) + 1 + j;
-        n_jterms += (int)ent[e].size();
-      } else {
-        h.idx = NN + (e - S * S);
-      }
-      h.beg = (int32_t)jt.size();
-      for (auto& cc : ent[e]) {
-        JcTerm t{};
-        t.coef = cc.first;
-        t.pidx = cc.second;
-        jt.push_back(t);
-      }
-      h.end = (int32_t)jt.size();
-      jc.push_back(h);
-    }
-    jc_ptr.push_back((int32_t)jc.size());
-  }
+    t.scratch = JAC_PER_RXN * chunk + std::max(typed_most, 0);
+    return t;
+  };
+  // the wide form's scratch takes the matrix's place in shared memory: all
+  // reactions at once where they fit it (or 24 KB)
+  const int room = std::max(NN, 3072);
+  const JacHost jw = jac_table(JAC_PER_RXN * R + (R - first_typed) <= room ? std::max(R, 1)
+                                                                            : shares(room / (JAC_PER_RXN + 1)));
+  const JacHost jn = jac_table(shares(n1 <= 64 ? 64 : 60));
   // species ordered by the length of their CSR rows (longest first), so
   // that the lanes of one warp gather similar counts in the RHS
   std::vector<int16_t> rsp(S);
@@ -432,9 +450,17 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   }
   const size_t off_csr = place(sizeof(CsrTerm) * csr.size());
   const size_t off_csr_cptr = place(sizeof(int32_t) * csr_cptr.size());
-  const size_t off_jc_ptr = place(sizeof(int32_t) * jc_ptr.size());
-  const size_t off_jc = place(sizeof(JcEntry) * jc.size());
-  const size_t off_jt = place(sizeof(JcTerm) * jt.size());
+  struct JacOff {
+    size_t ptr, jc, jt;
+  };
+  auto place_jac = [&](const JacHost& t) {
+    JacOff o;
+    o.ptr = place(sizeof(int32_t) * t.jc_ptr.size());
+    o.jc = place(sizeof(JcEntry) * t.jc.size());
+    o.jt = place(sizeof(JcTerm) * t.jt.size());
+    return o;
+  };
+  const JacOff ow = place_jac(jw), on = place_jac(jn);
   const size_t off_rsp = place(sizeof(int16_t) * rsp.size());
   const size_t off_err = place(sizeof(int32_t) * 4);
   const size_t total = off;
@@ -454,9 +480,13 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   put(off_csr_ptr, csr_ptr.data(), sizeof(int32_t) * (S + 1));
   put(off_csr, csr.data(), sizeof(CsrTerm) * csr.size());
   put(off_csr_cptr, csr_cptr.data(), sizeof(int32_t) * csr_cptr.size());
-  put(off_jc_ptr, jc_ptr.data(), sizeof(int32_t) * jc_ptr.size());
-  put(off_jc, jc.data(), sizeof(JcEntry) * jc.size());
-  put(off_jt, jt.data(), sizeof(JcTerm) * jt.size());
+  auto put_jac = [&](const JacOff& o, const JacHost& t) {
+    put(o.ptr, t.jc_ptr.data(), sizeof(int32_t) * t.jc_ptr.size());
+    put(o.jc, t.jc.data(), sizeof(JcEntry) * t.jc.size());
+    put(o.jt, t.jt.data(), sizeof(JcTerm) * t.jt.size());
+  };
+  put_jac(ow, jw);
+  put_jac(on, jn);
   put(off_rsp, rsp.data(), sizeof(int16_t) * rsp.size());
 
   ck_mech* m = new ck_mech;
@@ -501,14 +531,16 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   dm.tab = reinterpret_cast<const double*>(b + L.tab);
   dm.csr_ptr = reinterpret_cast<const int32_t*>(b + off_csr_ptr);
   dm.csr = reinterpret_cast<const CsrTerm*>(b + off_csr);
-  dm.chunk = chunk;
-  dm.n_chunks = n_chunks;
   dm.rhs_chunk = rhs_chunk;
   dm.n_rhs_chunks = n_rhs_chunks;
+  dm.first_typed = first_typed;
   dm.csr_cptr = reinterpret_cast<const int32_t*>(b + off_csr_cptr);
-  dm.jc_ptr = reinterpret_cast<const int32_t*>(b + off_jc_ptr);
-  dm.jc = reinterpret_cast<const JcEntry*>(b + off_jc);
-  dm.jt = reinterpret_cast<const JcTerm*>(b + off_jt);
+  auto view_jac = [&](const JacOff& o, const JacHost& t) {
+    return JacTab{t.chunk, t.n_chunks, t.scratch, reinterpret_cast<const int32_t*>(b + o.ptr),
+                  reinterpret_cast<const JcEntry*>(b + o.jc), reinterpret_cast<const JcTerm*>(b + o.jt)};
+  };
+  dm.wide = view_jac(ow, jw);
+  dm.narrow = view_jac(on, jn);
   dm.rsp = reinterpret_cast<const int16_t*>(b + off_rsp);
   hm.n_contrib = n_jterms;
   hm.csr_nnz = (int)csr_rx.size();

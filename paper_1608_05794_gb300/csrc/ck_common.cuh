@@ -49,9 +49,11 @@ struct __align__(16) RxnRec {
 };
 static_assert(sizeof(RxnRec) == 112, "RxnRec layout");
 
-// Jacobian partials stored per reaction: reactant slots 0..2, product slots
-// 3..5, and slot 6 = dc/d[M] * (k_f prod' - k_r prod'').
-constexpr int JP = 7;
+// Per-reaction values of a chunk of c reactions that the Jacobian is
+// assembled from: q, dq/dT and D (c each), six partials a reaction (reactant
+// slots 0..2, product slots 3..5), and dc/d[M] (k_f prod' - k_r prod'') of
+// the chunk's third-body and fall-off reactions (its last ones).
+constexpr int JAC_PER_RXN = 9;
 
 // Per species and temperature range: 18 doubles
 //   cp/R  : c0 + c1 T + c2 T^2 + c3 T^3 + c4 T^4               [0..4]
@@ -76,6 +78,20 @@ struct __align__(16) JcTerm {   // coef * P[pidx]
 };
 static_assert(sizeof(CsrTerm) == 16 && sizeof(JcEntry) == 16 && sizeof(JcTerm) == 16, "packed records");
 
+// One way of assembling the Jacobian: the reactions in chunks of `chunk`
+// (scratch doubles of per-reaction values), and per chunk c the targets
+// jc[e], e in [jc_ptr[c], jc_ptr[c+1]) (flat index idx: the species-block
+// entry J[idx] below n^2, else the per-species sums wd, aT, E, u at idx -
+// n^2), which add the sum over t in [jc[e].beg, jc[e].end) of jt[t].coef *
+// src[jt[t].pidx] (src: the chunk's per-reaction values).  Chunk 0 lists
+// every target, those without a term too.
+struct JacTab {
+  int chunk, n_chunks, scratch;
+  const int32_t* jc_ptr;
+  const JcEntry* jc;
+  const JcTerm* jt;
+};
+
 // Device view of a loaded mechanism.  All pointers are device memory (one
 // allocation, 16-byte aligned sections).
 struct DevMech {
@@ -96,21 +112,16 @@ struct DevMech {
   const CsrTerm* csr;     // [csr_nnz]
   const double* tab;      // [256] 2^(j/256)
   const double* revp;     // [n_rev][3] explicit reverse: log2 A_r, beta_r, Ea_r / (R ln 2)
-  // Team kernels walk the reactions in chunks: of `chunk` for the Jacobian,
-  // of `rhs_chunk` for a right-hand side whose team has no room for all R
-  // rates.  csr_cptr[k (n_rhs_chunks + 1) + c] = first CSR entry of species k
-  // whose reaction lies in right-hand-side chunk c or later.  Jacobian
-  // assembly, chunk c: the
-  // targets jc[e], e in [jc_ptr[c], jc_ptr[c+1]) (flat index idx: the
-  // species-block entry J[idx] below n^2, else the per-species sums wd, aT,
-  // E, u at idx - n^2), each add the sum over t in [jc[e].beg, jc[e].end)
-  // of jt[t].coef * src[jt[t].pidx] (src: the chunk's q, dq/dT, D and
-  // partials P, JP per reaction, contiguous).
-  int chunk, n_chunks, rhs_chunk, n_rhs_chunks;
+  // A right-hand side whose team has no room for all R rates takes the
+  // reactions in chunks of rhs_chunk.  csr_cptr[k (n_rhs_chunks + 1) + c] =
+  // first CSR entry of species k whose reaction lies in chunk c or later.
+  int rhs_chunk, n_rhs_chunks;
+  int first_typed;        // reactions from here on are third-body or fall-off
   const int32_t* csr_cptr;
-  const int32_t* jc_ptr;
-  const JcEntry* jc;
-  const JcTerm* jt;
+  // Jacobian tables: for teams that may assemble in device memory (the
+  // per-reaction values then take the place of the matrix in shared memory,
+  // usually of all reactions at once), and for those that may not.
+  JacTab wide, narrow;
   const int16_t* rsp;     // [S] species order of the RHS gather, longest row first
 };
 

@@ -18,20 +18,20 @@ namespace ck {
 static int team_size(int n) { return n <= 24 ? 32 : (n <= 64 ? 96 : 256); }
 
 // ------------------------------------------------------------------ Jacobian
+// The matrix is assembled in place in the output (its lines stay in L2), so
+// that a CTA's shared memory holds the per-reaction values instead.
 __global__ void __launch_bounds__(256) k_jacobian(const __grid_constant__ DevMech d, int64_t N,
                                                   const double* __restrict__ p, const double* __restrict__ y,
                                                   double* __restrict__ jac) {
   extern __shared__ __align__(16) double sm[];
   const int n = d.n;
-  double* J = sm;
-  double* ys = J + (size_t)n * n;
+  double* ys = sm + d.wide.scratch;
   double* fs = ys + n;
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
     team_sync();
-    team_jacobian(d, d.tab, p[r], ys, fs, J, carve_bufs(fs + n, d.S, d.chunk, 256));
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = J[e];
-    team_sync();
+    team_jacobian(d, d.wide, d.tab, p[r], ys, fs, jac + r * (int64_t)n * n, nullptr,
+                  carve_bufs(fs + n, d.S, sm, d.wide.chunk, 256));
   }
 }
 
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ D
   double* red = sm + bufs;
   const RhsQ qq{bufs + species_doubles(d.S), d.rhs_chunk};
   const bool fixed = sp.fixed_h > 0.0;
-  const int tid = threadIdx.x, P = blockDim.x;
+  const int tid = (int)threadIdx.x, P = blockDim.x;
   double* k0 = kk;
   double* k1 = kk + n;
   double* k2 = kk + 2 * n;
@@ -261,7 +261,7 @@ cudaError_t launch_jacobian(const HostMech& hm, int64_t n, const double* p, cons
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
   const size_t smem =
-      sizeof(double) * ((size_t)nn * nn + 2 * nn + species_doubles(hm.S) + jac_doubles(hm.S, hm.d.chunk));
+      sizeof(double) * ((size_t)hm.d.wide.scratch + 2 * nn + species_doubles(hm.S) + 3 * hm.S);
   const int threads = team_size(nn);
   const int grid = team_grid(k_jacobian, threads, smem, n, cfg);
   k_jacobian<<<grid, threads, smem, st>>>(hm.d, n, p, y, jac);

@@ -10,17 +10,20 @@
 namespace ck {
 
 // Stage solve of the precision form: the iteration matrix is factored in
-// FP32 (M32, rof, invd32) and each solve is refined against the FP64 matrix
-// M64 (the CTA's copy in global memory, L2-resident): x = LU32^-1 b, then
-// REFINE times r = b - M64 x (FP64), x += LU32^-1 r.
-// b (in u) is overwritten with x; xf (n floats) and x (n doubles) are scratch
-// that must not hold anything the caller still needs.
-static __device__ void refined_solve(const double* M64, const float* M32, int n, const int* rof,
-                              const float* invd32, double* u, float* xf, double* x, int refine) {
-  const int tid = threadIdx.x, P = blockDim.x;
+// FP32 (at the start of shared memory) and each solve is refined against the
+// FP64 matrix M64 (the CTA's copy in global memory, L2-resident): x = LU32^-1
+// b, then refine times r = b - M64 x (FP64), x += LU32^-1 r.  Arrays by offset
+// in shared memory: b (in u) is overwritten with x; the second half of invd (n
+// floats) and x (n doubles) are scratch.
+static __device__ __noinline__ void refined_solve(const double* M64, int n, int rof_o, int invd_o, int u_o, int x_o,
+                                                  int refine) {
+  extern __shared__ __align__(16) double sm[];
+  const int tid = threadIdx.x, P = blockDim.x, xf_o = 2 * invd_o + n;
+  float* xf = reinterpret_cast<float*>(sm) + xf_o;
+  double *u = sm + u_o, *x = sm + x_o;
   for (int i = tid; i < n; i += P) xf[i] = (float)u[i];
   team_sync();
-  if (tid < 32) warp_lu_solve<true>(M32, n, rof, invd32, xf);
+  if (tid < 32) warp_solve<float>(0, n, rof_o, invd_o, xf_o);
   team_sync();
   for (int i = tid; i < n; i += P) x[i] = (double)xf[i];
   team_sync();
@@ -39,7 +42,7 @@ static __device__ void refined_solve(const double* M64, const float* M32, int n,
       xf[i] = (float)((s0 + s1) + (s2 + s3));
     }
     team_sync();
-    if (tid < 32) warp_lu_solve<true>(M32, n, rof, invd32, xf);
+    if (tid < 32) warp_solve<float>(0, n, rof_o, invd_o, xf_o);
     team_sync();
     for (int i = tid; i < n; i += P) x[i] += (double)xf[i];
     team_sync();
@@ -92,28 +95,23 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
                                                  double* h_io, SolverParams sp, int32_t* steps,
                                                  int32_t* status, int32_t* queue, double* __restrict__ m64g) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ int slot, flag;
+  __shared__ int slot;
   __shared__ Ros4Ctl ctl;
   using F = typename std::conditional<PREC == 0, double, float>::type;  // type of the factors
   const int n = d.n, nn = n * n;
   const double* tab = d.tab;  // 2 KB, stays in L1
-  const Ros4Layout L(n, d.S, d.chunk, d.rhs_chunk);
+  const Ros4Layout L(d, m64g != nullptr, nn);
   double* M = sm;
   double* yv = sm + L.yv;
   double* F0 = sm + L.f0;
   double* Yt = sm + L.yt;
   double* ub = sm + L.ub;
-  double* invd = sm + L.invd;
-  int* rof = reinterpret_cast<int*>(sm + L.rof);
   double* red = sm + L.bufs;
-  LuRow<F>* lr = reinterpret_cast<LuRow<F>*>(sm + L.lr);
   F* MF = reinterpret_cast<F*>(M);         // PREC >= 1: FP32 factors over the FP64 matrix
-  F* invF = reinterpret_cast<F*>(invd);
-  float* xf = reinterpret_cast<float*>(invd) + n;  // PREC >= 1: the other half of invd
   double* Mg = m64g ? m64g + (size_t)blockIdx.x * ros4_scratch_doubles(n) : nullptr;
   const bool keep_j = Mg != nullptr && sp.jac == 0;
   const bool fixed = sp.fixed_h > 0.0;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = (int)threadIdx.x, warp = tid >> 5;
   const bool own = tid < n;
   for (;;) {
     const int r = team_next(queue, &slot);
@@ -172,11 +170,17 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
         // J and f at y (or the copy kept since a rejected attempt at the
         // same y); A = J - I/(hh gamma) = -M; LU of A
         if (!have_j) {
-          if (sp.jac == 1) team_jacobian_fd(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, M, L.yt, L.ub, L.bufs, L.vp, L.rhs_q, have_f);
-          else team_jacobian(d, tab, pr, yv, F0, M, carve_bufs(sm + L.bufs, d.S, d.chunk, L.vp));
-          if (Mg && (keep_j || PREC)) {
-            for (int e = tid; e < nn; e += P) Mg[e] = M[e];
-            if (PREC && own) Mg[nn + tid] = M[(size_t)tid * n + tid];
+          if (sp.jac == 1) {
+            team_jacobian_fd(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, L.yt, L.ub, L.bufs, L.vp,
+                             L.rhs_q, have_f);
+          } else {
+            // assembled in the copy Mg where there is one
+            const JacTab& jt = Mg ? d.wide : d.narrow;
+            team_jacobian(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr,
+                          carve_bufs(sm + L.bufs, d.S, sm + L.jscr, jt.chunk, L.vp));
+          }
+          if (PREC) {
+            if (own) Mg[nn + tid] = Mg[(size_t)tid * n + tid];
             team_sync();
           }
           have_j = keep_j;
@@ -193,7 +197,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           for (int e = tid; e < nn; e += P) MF[e] = (F)Mg[e];
         }
         team_sync();
-        const int info = lu_flat<true>(MF, n, rof, nullptr, invF, lr, &flag);
+        const int info = team_lu<F>(0, n, L.rof, L.invd, L.lr, L.bufs + TEAM_RED_DOUBLES - 1);
         if (info) {
           if (warp == 0) {
             ++rej;
@@ -212,10 +216,10 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
         auto solve = [&]() {  // ub <- A^-1 ub
           team_sync();
           if constexpr (PREC == 0) {
-            if (warp == 0) warp_lu_solve<true>(M, n, rof, invd, ub);
+            if (warp == 0) warp_solve<double>(0, n, L.rof, L.invd, L.ub);
             team_sync();
           } else {
-            refined_solve(Mg, MF, n, rof, invF, ub, xf, Yt, PREC);
+            refined_solve(Mg, n, L.rof, L.invd, L.ub, L.yt, PREC);
           }
         };
         double u1 = 0.0, u2 = 0.0, u3 = 0.0, u4 = 0.0, f3 = 0.0;
@@ -333,10 +337,10 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
                              int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, double* scratch,
                              size_t scratch_bytes, bool may_alloc) {
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * Ros4Layout(nn, hm.S, hm.d.chunk, hm.d.rhs_chunk).doubles;
   auto kern = cfg.precision == 2 ? k_ros4<P, MINB, 2>
                                  : (cfg.precision == 1 ? k_ros4<P, MINB, 1> : k_ros4<P, MINB, 0>);
-  const int grid = team_grid(kern, P, smem, n, cfg);
+  size_t smem = sizeof(double) * Ros4Layout(hm.d, true, nn * nn).doubles;
+  int grid = team_grid(kern, P, smem, n, cfg);
   // per-CTA copies of J (every form) and the FP64 iteration matrices of
   // the precision form: the caller's scratch when it is large enough, else
   // a stream-ordered allocation around the launch, else (allocation-free
@@ -352,6 +356,9 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
     owned = true;
   } else if (cfg.precision) {
     return cudaErrorNotSupported;
+  } else {
+    smem = sizeof(double) * Ros4Layout(hm.d, false, nn * nn).doubles;
+    grid = team_grid(kern, P, smem, n, cfg);
   }
   kern<<<grid, P, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);
   cudaError_t k = cudaGetLastError();

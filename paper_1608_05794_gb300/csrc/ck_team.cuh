@@ -85,10 +85,9 @@ __device__ __forceinline__ void team_sync() {
 }
 
 // Shared-memory work arrays of one team.
-// The Jacobian processes reactions in chunks of m.chunk, so the per-reaction
-// arrays hold one chunk; the right-hand side, which keeps one value per
-// reaction, takes all reactions at once when the caller's q holds them, else
-// chunks of m.rhs_chunk.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
+// The Jacobian processes reactions in the chunks of its table (JacTab); the
+// right-hand side, which keeps one value per reaction, takes all reactions at
+// once or chunks of m.rhs_chunk.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
 // (S/R - H/RT)_k / ln 2, so that 1/K_c of Eq. kc is a product of species
 // factors.  Entry S of X, Gp, Gm (1) and hRT (0) stands for an empty reaction
 // slot.  After the reaction passes of the Jacobian, X, Gp and Gm are reused
@@ -96,19 +95,17 @@ __device__ __forceinline__ void team_sync() {
 struct TeamBufs {
   double *X, *Gp, *Gm, *hRT;              // [S + 1]
   double *cpR, *wd, *aT, *E, *u;          // [S]; wd, aT, E, u contiguous
-  double *q, *dqT, *D;                    // [chunk]
-  double* P;                              // [chunk * JP] Jacobian partials
+  double *q, *dqT, *D, *P, *w;            // per-reaction values of a chunk (JAC_PER_RXN)
   double* red;                            // [TEAM_RED_DOUBLES] reductions and scalars (SC_*)
   int vp;                                 // lanes that the species sums are grouped by (64 or 256)
 };
 
-// [red | X Gp Gm hRT | cpR | wd ... : a right-hand side needs species_doubles(S)
-// doubles up to and with wd; a Jacobian continues with aT E u and the chunk.
+// [red | X Gp Gm hRT | cpR | wd], species_doubles(S) doubles; a Jacobian
+// continues with aT E u (3 S).
 constexpr int TEAM_RED_DOUBLES = 64;
 __host__ __device__ __forceinline__ constexpr int species_doubles(int S) { return TEAM_RED_DOUBLES + 4 * (S + 1) + 2 * S; }
-__host__ __device__ __forceinline__ constexpr int jac_doubles(int S, int chunk) { return 3 * S + (3 + JP) * chunk; }
 
-__device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH, int vp) {
+__device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, double* scratch, int chunk, int vp) {
   TeamBufs b;
   b.red = base;
   b.X = b.red + TEAM_RED_DOUBLES;
@@ -120,10 +117,11 @@ __device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, int CH, int 
   b.aT = b.wd + S;
   b.E = b.aT + S;
   b.u = b.E + S;
-  b.q = b.u + S;
-  b.dqT = b.q + CH;
-  b.D = b.dqT + CH;
-  b.P = b.D + CH;
+  b.q = scratch;
+  b.dqT = b.q + chunk;
+  b.D = b.dqT + chunk;
+  b.P = b.D + chunk;
+  b.w = b.P + 6 * chunk;
   b.vp = vp;
   return b;
 }
@@ -144,7 +142,7 @@ struct Mix {
 };
 
 // Where a right-hand side keeps its rates of progress: offset in shared
-// memory and how many (all m.R, or m.rhs_chunk).
+// memory and how many at a time (all m.R, or m.rhs_chunk).
 struct RhsQ {
   int off, chunk;
 };
@@ -157,10 +155,9 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // through log T) are formed side by side by two warps, everything else of
 // the species by all of them: a polynomial pass of 32 species is one work
 // item, dealt to the warps in turn.
-template <bool JAC>
 __device__ __forceinline__ void team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
-  const int S = m.S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int S = m.S, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int SG = species_groups(S);
   double* red = b.red;
   const double T = y[0];
@@ -223,8 +220,6 @@ __device__ __forceinline__ void team_species(const DevMech& m, double p, const d
       b.hRT[S] = 0.0;
     }
   }
-  if (JAC)
-    for (int k = threadIdx.x; k < 4 * S; k += blockDim.x) b.wd[k] = 0.0;  // wd, aT, E, u
   team_sync();
   x.invT = red[SC_INVT];
   x.log2T = red[SC_LOG2T];
@@ -267,12 +262,12 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 
 // Rates of one reaction at the mixture state.  JAC: also the partial-
 // derivative pieces used by the Jacobian (see team_jacobian).  i: index of
-// the reaction inside the current chunk.  Empty slots read the neutral
+// the reaction inside the current chunk, iw: among its typed reactions.  Empty slots read the neutral
 // entries of the species arrays (a product with 1, a sum with 0, exact), so
 // that reactions of every molecularity take the same instructions.
 template <bool JAC>
 __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
-                                              const TeamBufs& b, const double* tab, int i) {
+                                              const TeamBufs& b, const double* tab, int i, int iw) {
   const RxnRec r = load_rxn(src);
   const double* X = b.X;
   const double l2kf = fma(-r.EoR2, x.invT, fma(r.beta, x.log2T, r.lA2));
@@ -342,14 +337,14 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
       ckf = c * kf;
       ckr = c * kr;
       w = dcdM * net;
-      b.P[(size_t)i * JP + 6] = w;
+      b.w[iw] = w;
     }
   }
   b.q[i] = q;
   if (JAC) {
     // d q / d[X] slot by slot: c k_f prod of the other reactant slots, and
     // -c k_r prod of the other product slots
-    double* P = b.P + (size_t)i * JP;
+    double* P = b.P + 6 * i;
     P[0] = ckf * (x1 * x2);
     P[1] = ckf * (x0 * x2);
     P[2] = ckf * (x0 * x1);
@@ -377,19 +372,17 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
 // f(y) for one reactor.  Arrays by their offsets (doubles) in the CTA's
 // dynamic shared memory, so that this out-of-line function still addresses
 // shared memory directly: y_o, f_o the vectors (n = S + 1; f may not be y),
-// bufs_o the work arrays (species_doubles), q_o the rates of progress (m.R
-// doubles if they fit the caller's layout, else m.rhs_chunk; q_all tells).
+// bufs_o the work arrays (species_doubles), qq the rates of progress.
 static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
   extern __shared__ __align__(16) double sm[];
   const double* y = sm + y_o;
   double* f = sm + f_o;
-  TeamBufs b = carve_bufs(sm + bufs_o, m.S, 0, vp);
-  b.q = sm + qq.off;
+  TeamBufs b = carve_bufs(sm + bufs_o, m.S, sm + qq.off, 0, vp);
   Mix x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int S = m.S, SG = species_groups(S);
-  team_species<false>(m, p, y, b, x, tab);
+  team_species(m, p, y, b, x, tab);
   team_sync();
   const double invrho = x.invrho;
   // every chunk: its rates of progress, then one fixed-order gather per
@@ -398,10 +391,13 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   const int CH = qq.chunk;
   for (int base = 0;;) {
     const int cnt = m.R - base < CH ? m.R - base : CH;
-    for (int li = threadIdx.x; li < cnt; li += blockDim.x) team_reaction<false>(m, m.rxn + base + li, x, b, tab, li);
+    // last reactions first: the expensive ones (fall-off) then fill whole
+    // warps, and the warp that is left partly empty has the cheapest
+    for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+      team_reaction<false>(m, m.rxn + base + li, x, b, tab, li, 0);
     team_sync();
     const bool last = base + cnt >= m.R;
-    for (int kk = threadIdx.x; kk < S; kk += blockDim.x) {
+    for (int kk = tid; kk < S; kk += blockDim.x) {
       const int k = m.rsp[kk];
       int e = m.csr_ptr[k], e1 = m.csr_ptr[k + 1];
       double w = 0.0;
@@ -465,9 +461,10 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   team_sync();
 }
 
-// Analytic Jacobian J = df/d(T, Y) at constant p, written row-major into J
-// (shared memory, n x n), and f(y) into f.  Derivation (chain rule through
-// rho(T, Y) and [X](rho, Y); dlnK_c/dT = (sum nu H/RT - dnu)/T):
+// Analytic Jacobian J = df/d(T, Y) at constant p, written row-major (n x n)
+// into A, and into M too unless that is NULL, and f(y) into f.  Derivation
+// (chain rule through rho(T, Y) and [X](rho, Y); dlnK_c/dT = (sum nu H/RT -
+// dnu)/T):
 //   A_kj   = sum_i nu_ki dq_i/d[X_j] (sparse mass-action part and the
 //            (eff - 1) corrections) + u_k (dense third-body part, u_k = sum nu_ki w_i),
 //   E_k    = sum_i nu_ki D_i,  a_k = sum_i nu_ki dq_i/dT,
@@ -482,52 +479,51 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 //   J[1+k][1+j] = W_k (A_kj + u_k) / W_j,   J[1+k][0] = W_k a_k / rho,
 //   J[0][1+j]   = -(T cs_j / cvm + Tdot cv_j / cvm) / W_j,
 //   J[0][0]     = -(sum cv_k wdot_k + T sum U_k/RT a_k)/(rho cvm) - Tdot dcpm/cvm.
+// The species block is accumulated in A.  With A in device memory (where it
+// stays in L2) the per-reaction values (b.q and on) may lie where M is: they
+// are read for the last time before M is written, so that a team needs shared
+// memory for the larger of the two only, and takes all reactions in one pass.
 // Needs b.vp >= S (one species a lane in the sums).
-static __device__ void team_jacobian(const DevMech& m, const double* tab, double p, const double* y,
-                              double* f, double* J, TeamBufs b) {
+static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const double* tab, double p, const double* y,
+                                     double* f, double* A, double* M, TeamBufs b) {
   Mix x;
   const int S = m.S, n = m.n, SG = species_groups(S);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  team_species<true>(m, p, y, b, x, tab);
-  // species block A starts at zero (the whole matrix is cleared: the
-  // temperature row and column are written whole further down); chunk by
-  // chunk, every entry touched by the chunk and every species sum (wdot,
-  // d wdot/dT, E = sum nu D and the dense third-body part u) adds its
-  // fixed-order sum of contributions, one thread per target, the targets in
-  // one list sorted by length so that a warp's lanes do similar work
-  for (int e = threadIdx.x; e < n * n; e += blockDim.x) J[e] = 0.0;
+  const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  team_species(m, p, y, b, x, tab);
   team_sync();
-  const int NC = m.n_chunks, CH = m.chunk;
-  for (int c = 0; c < NC; ++c) {
-    const int base = c * CH;
-    for (int li = threadIdx.x; li < CH; li += blockDim.x)
-      if (base + li < m.R) team_reaction<true>(m, m.rxn + base + li, x, b, tab, li);
+  // chunk by chunk, every target (species-block entries and the per-species
+  // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
+  // fixed-order sum of terms; one thread per target, no conflicts, the
+  // targets sorted by length so that a warp's lanes do similar work
+  for (int c = 0; c < jt.n_chunks; ++c) {
+    const int base = c * jt.chunk, cnt = m.R - base < jt.chunk ? m.R - base : jt.chunk;
+    const int ft = m.first_typed > base ? m.first_typed - base : 0;
+    for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+      team_reaction<true>(m, m.rxn + base + li, x, b, tab, li, li - ft);
     team_sync();
-    // every target of the chunk (species-block entries and the per-species
-    // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
-    // fixed-order sum of terms; one thread per target, no conflicts
-    for (int e = m.jc_ptr[c] + threadIdx.x; e < m.jc_ptr[c + 1]; e += blockDim.x) {
-      const JcEntry h = m.jc[e];
-      double* tgt = h.idx < n * n ? J + h.idx : b.wd + (h.idx - n * n);
-      double a = *tgt;
+    for (int e = jt.jc_ptr[c] + tid; e < jt.jc_ptr[c + 1]; e += blockDim.x) {
+      const JcEntry h = jt.jc[e];
+      double a = 0.0;
+      if (c > 0) a = h.idx < n * n ? A[h.idx] : b.wd[h.idx - n * n];
       for (int t = h.beg; t < h.end; ++t) {
-        const JcTerm ct = m.jt[t];
+        const JcTerm ct = jt.jt[t];
         a = fma(ct.coef, b.q[ct.pidx], a);
       }
-      *tgt = a;
+      if (h.idx < n * n) A[h.idx] = a;
+      else b.wd[h.idx - n * n] = a;
     }
     team_sync();
   }
   // Constant volume: rho is fixed, so every term that comes from d rho/dT or
   // d rho/dY (cpf) drops out, and U/RT = H/RT - 1, cv/R = cp/R - 1 take the
   // places of H/RT and cp/R (cvf).  The contributions were pre-scaled by
-  // W_k/W_j, so J holds A'_kj = W_k A_kj / W_j here.
+  // W_k/W_j, so A holds A'_kj = W_k A_kj / W_j here.
   const double invrho = x.invrho;
   const double cvf = m.cv ? 1.0 : 0.0, cpf = 1.0 - cvf;
   double* eW = b.Gm;     // e_k / W_k, for the column sums
   double* dense = b.X;   // dense part of the species block, W_k u_k + W_k Wbar (wdot_k - E_k) / rho
   double* cs = b.Gp;
-  for (int k = threadIdx.x; k < S; k += blockDim.x) {
+  for (int k = tid; k < S; k += blockDim.x) {
     f[1 + k] = b.wd[k] * (m.W[k] * invrho);
     eW[k] = (b.hRT[k] - cvf) * m.invW[k];
     dense[k] = m.W[k] * fma(cpf * x.Wbar * invrho, b.wd[k] - b.E[k], b.u[k]);
@@ -573,23 +569,25 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
     const int j = 32 * g + lane;
     if (j < S) {
       double s = 0.0;
-      for (int k = 0; k < S; ++k) s = fma(eW[k], J[(size_t)(1 + k) * n + 1 + j], s);
+      const double* a = A + n + 1 + j;
+#pragma unroll 8
+      for (int k = 0; k < S; ++k) s = fma(eW[k], a[k * n], s);
       cs[j] = s;
     }
   }
   team_sync();
   const double dcpm = sums[1], he = sums[3], cw = sums[4], ha = sums[5], eu = sums[6];
   const double Tdot = b.red[SC_TDOT], inv_cpm = b.red[SC_ICPM];
-  // species block (J_kj = A'_kj + dense_k / W_j) and temperature column and
-  // row, each product rounded as written
-  // entries e = k S + j of the species block, (k, j) advanced without
-  // dividing by the runtime S
+  // species block (J_kj = A'_kj + dense_k / W_j), entries e = k S + j, (k, j)
+  // advanced without dividing by the runtime S
   {
     const int P = blockDim.x, dk = P / S, dj = P - (P / S) * S;
-    int k = threadIdx.x / S, j = threadIdx.x - k * S;
+    int k = tid / S, j = tid - k * S;
     for (; k < S;) {
-      double* a = J + (size_t)(1 + k) * n + 1 + j;
-      *a = fma(dense[k], m.invW[j], *a);
+      const int o = (1 + k) * n + 1 + j;
+      const double v = fma(dense[k], m.invW[j], A[o]);
+      A[o] = v;
+      if (M) M[o] = v;
       k += dk;
       j += dj;
       if (j >= S) {
@@ -598,19 +596,27 @@ static __device__ void team_jacobian(const DevMech& m, const double* tab, double
       }
     }
   }
-  for (int k = threadIdx.x; k < S; k += blockDim.x)
-    J[(size_t)(1 + k) * n] = m.W[k] * invrho * fma(cpf * b.wd[k], x.invT, b.aT[k]);
+  // temperature column and row (each product rounded where it is written)
+  for (int k = tid; k < S; k += blockDim.x) {
+    const double v = m.W[k] * invrho * fma(cpf * b.wd[k], x.invT, b.aT[k]);
+    A[(1 + k) * n] = v;
+    if (M) M[(1 + k) * n] = v;
+  }
   const double inv_rc = invrho * inv_cpm;
-  for (int j = threadIdx.x; j < S; j += blockDim.x) {
+  for (int j = tid; j < S; j += blockDim.x) {
     // cs_j = sum_k e_k (A_kj + u_k) = W_j sum_k (e_k / W_k) A'_kj + sum_k e_k u_k
     const double csj = fma(m.W[j], cs[j], eu);
     const double cW = __dmul_rn(cpf, x.Wbar);
     const double in = fma(x.rho, csj, -__dmul_rn(cW, he));
     const double tt = fma(__dmul_rn(x.T, in), inv_rc, __dmul_rn(Tdot, fma(b.cpR[j] - cvf, inv_cpm, -cW)));
-    J[1 + j] = -tt * m.invW[j];
+    const double v = -tt * m.invW[j];
+    A[1 + j] = v;
+    if (M) M[1 + j] = v;
   }
-  if (threadIdx.x == 0) {
-    J[0] = fma(-fma(x.T, ha, cw), inv_rc, -__dmul_rn(Tdot, fma(dcpm, inv_cpm, -cpf * x.invT)));
+  if (tid == 0) {
+    const double v = fma(-fma(x.T, ha, cw), inv_rc, -__dmul_rn(Tdot, fma(dcpm, inv_cpm, -cpf * x.invT)));
+    A[0] = v;
+    if (M) M[0] = v;
     f[0] = Tdot;
   }
   team_sync();
@@ -748,8 +754,39 @@ __device__ __forceinline__ void lu_panel(F* A, int n, int k, int* rof, int* lpiv
 // integer, far more than its rounding error of 2^-22 e / c).
 __device__ __forceinline__ int flat_row(int e, float rc) { return (int)(((float)e + 0.5f) * rc); }
 
+// Rows i0, i0 + step, .. of the m x c trailing matrix at A2, updated with the
+// pivot row U and the multipliers in R.
+template <class F>
+__device__ __forceinline__ void lu_rows(F* A2, const F* U, const LuRow<F>* R, int m, int c, int i0, int step) {
+  constexpr int Q = (LU_MAX_N + 31) / 32;
+  const int lane = threadIdx.x & 31;
+  F u[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) u[q] = lane + 32 * q < c ? U[lane + 32 * q] : F(0);
+  for (int i = i0; i < m; i += 2 * step) {
+    const bool two = i + step < m;
+    const LuRow<F> r0 = R[i], r1 = R[two ? i + step : i];
+    F* a0 = A2 + (r0.pk >> 8) + lane;
+    F* a1 = A2 + (r1.pk >> 8) + lane;
+    F v0[Q], v1[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const bool in = lane + 32 * q < c;
+      v0[q] = in ? a0[32 * q] : F(0);
+      v1[q] = in ? a1[32 * q] : F(0);
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      if (lane + 32 * q < c) {
+        a0[32 * q] = fma(-r0.l, u[q], v0[q]);
+        if (two) a1[32 * q] = fma(-r1.l, u[q], v1[q]);
+      }
+    }
+  }
+}
+
 template <bool PRE, class F>
-__device__ __noinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd, LuRow<F>* lr, int* flag) {
+__device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd, LuRow<F>* lr, int* flag) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   for (int i = tid; i < n; i += blockDim.x) {
     lr[n + i].pk = (i * n) << 8 | i;
@@ -764,6 +801,19 @@ __device__ __noinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd, L
   int pw = 1 % nw;        // the warp of the next panel
   for (int k = 0; k + 1 < n; ++k) {
     const int m = n - 1 - k, mc = m - 1, E = m * mc, NG = (E + 31) >> 5;
+    if constexpr (sizeof(F) == 4) {
+      // FP32 (the precision form): the arithmetic is cheap and the index work
+      // of the flat list would set the pace, so a lane keeps its columns and
+      // the other warps take rows in turn
+      if (warp == pw) lu_panel(A, n, k + 1, rof, lpiv, invd, lr, flag);
+      if (warp != pw || nw == 1)
+        lu_rows(A + k + 2, A + (rof[k] >> 8) + k + 2, lr + (k & 1) * n + k + 1, m, mc,
+                nw == 1 ? 0 : (warp > pw ? warp - pw - 1 : warp - pw - 1 + nw), nw == 1 ? 1 : nw - 1);
+      if (++pw == nw) pw = 0;
+      team_sync();
+      if (*flag) return *flag;
+      continue;
+    }
     // groups of 32 elements: the panel's warp takes the last gp, the others
     // share the rest
     int gp = NG, g0 = 0, gs = 1, g1 = NG;
@@ -921,6 +971,23 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     if (act) b[i] = s;
     __syncwarp();
   }
+}
+
+// lu_flat<true> and its solve out of line (one copy of each in a kernel that
+// calls them often), with their arrays by offset (doubles; b_o in elements) in
+// the CTA's dynamic shared memory so that they still address it directly.
+template <class F>
+static __device__ __noinline__ int team_lu(int a_o, int n, int rof_o, int invd_o, int lr_o, int flag_o) {
+  extern __shared__ __align__(16) double sm[];
+  return lu_flat<true>(reinterpret_cast<F*>(sm + a_o), n, reinterpret_cast<int*>(sm + rof_o), nullptr,
+                       reinterpret_cast<F*>(sm + invd_o), reinterpret_cast<LuRow<F>*>(sm + lr_o),
+                       reinterpret_cast<int*>(sm + flag_o));
+}
+template <class F>
+static __device__ __noinline__ void warp_solve(int a_o, int n, int rof_o, int invd_o, int b_o) {
+  extern __shared__ __align__(16) double sm[];
+  warp_lu_solve<true>(reinterpret_cast<const F*>(sm + a_o), n, reinterpret_cast<const int*>(sm + rof_o),
+                      reinterpret_cast<const F*>(sm + invd_o), reinterpret_cast<F*>(sm) + b_o);
 }
 
 }  // namespace ck

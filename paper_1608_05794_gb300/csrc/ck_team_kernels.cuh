@@ -36,11 +36,11 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
   const double* f0 = sm + f0_o;
   const double* F = sm + f_o;
   double* Yt = sm + yt_o;
-  const int n = d.n;
+  const int n = d.n, tid = (int)threadIdx.x;
   if (!have_f0) team_rhs(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
   double s = 0.0;
-  if ((int)threadIdx.x < vp)
-    for (int i = threadIdx.x; i < n; i += vp) {
+  if (tid < vp)
+    for (int i = tid; i < n; i += vp) {
       const double v = f0[i] / (atol + rtol * fabs(y[i]));
       s = fma(v, v, s);
       Yt[i] = y[i];
@@ -51,11 +51,11 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
   const double s0 = (fn != 0.0) ? 1000.0 * fabs(h) * U * n * fn : 1.0;
   for (int j = 0; j < n; ++j) {
     const double sj = fmax(srur * fabs(y[j]), s0 * (atol + rtol * fabs(y[j])));
-    if (threadIdx.x == 0) Yt[j] = y[j] + sj;
+    if (tid == 0) Yt[j] = y[j] + sj;
     team_sync();
     team_rhs(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) J[(size_t)i * n + j] = (F[i] - f0[i]) / sj;
-    if (threadIdx.x == 0) Yt[j] = y[j];
+    for (int i = tid; i < n; i += blockDim.x) J[(size_t)i * n + j] = (F[i] - f0[i]) / sj;
+    if (tid == 0) Yt[j] = y[j];
     team_sync();
   }
 }
@@ -76,9 +76,10 @@ static __device__ __forceinline__ double team_pow(double x, double q, double* re
 // that the components are dealt to (as the species sums).
 static __device__ __forceinline__ double team_wrms(int n, const double* e, const double* y0, const double* y1,
                                                    double rtol, double atol, double* red, int vp) {
+  const int tid = threadIdx.x;
   double s = 0.0;
-  if ((int)threadIdx.x < vp)
-    for (int i = threadIdx.x; i < n; i += vp) {
+  if (tid < vp)
+    for (int i = tid; i < n; i += vp) {
       const double sc = atol + rtol * fmax(fabs(y0[i]), fabs(y1[i]));
       const double v = e[i] / sc;
       s = fma(v, v, s);
@@ -95,12 +96,12 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   extern __shared__ __align__(16) double sm[];
   const double *y0 = sm + y0_o, *f0 = sm + f0_o, *f1 = sm + f1_o;
   double *y1 = sm + y1_o, *red = sm + bufs_o;
-  const int n = d.n;
-  const bool lane_in = (int)threadIdx.x < vp;
+  const int n = d.n, tid = (int)threadIdx.x;
+  const bool lane_in = tid < vp;
   team_rhs(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
   double s0 = 0.0, s1 = 0.0;
   if (lane_in)
-    for (int i = threadIdx.x; i < n; i += vp) {
+    for (int i = tid; i < n; i += vp) {
       const double sc = atol + rtol * fabs(y0[i]);
       s0 = fma(y0[i] / sc, y0[i] / sc, s0);
       s1 = fma(f0[i] / sc, f0[i] / sc, s1);
@@ -108,12 +109,12 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   const double d0 = sqrt(team_sum(s0, red) / n);
   const double d1 = sqrt(team_sum(s1, red) / n);
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) y1[i] = fma(ha, f0[i], y0[i]);
+  for (int i = tid; i < n; i += blockDim.x) y1[i] = fma(ha, f0[i], y0[i]);
   team_sync();
   team_rhs(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
   double s2 = 0.0;
   if (lane_in)
-    for (int i = threadIdx.x; i < n; i += vp) {
+    for (int i = tid; i < n; i += vp) {
       const double sc = atol + rtol * fabs(y0[i]);
       const double v = (f1[i] - f0[i]) / sc;
       s2 = fma(v, v, s2);
@@ -124,20 +125,23 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
 
-// Shared memory of one k_ros4 CTA, in doubles: the matrix, y and f(y), the
-// team's work arrays, and behind them the Jacobian's chunk or, at other times,
-// the stage vectors, the factors' row table and the rates of progress (or the
-// LU's scratch).
+// Shared memory of one k_ros4 CTA, in doubles: the matrix (mat: n^2 FP64, or
+// FP32 factors), y and f(y), the team's work arrays, and the stage vectors,
+// the factors' row table and the rates of progress (or the LU's scratch).  The
+// Jacobian's per-reaction values lie over the matrix (wide: it is assembled in
+// device memory) or behind the work arrays, over the stage vectors.
 struct Ros4Layout {
-  int vp, yv, f0, bufs, yt, ub, invd, rof, lr;
+  int vp, yv, f0, bufs, jscr, yt, ub, invd, rof, lr;
   RhsQ rhs_q;
   size_t doubles;
-  __host__ __device__ Ros4Layout(int n, int S, int chunk, int rhs_chunk) {
+  __host__ __device__ Ros4Layout(const DevMech& d, bool wide, int mat) {
+    const int n = d.n;
     vp = n > 64 ? 256 : 64;
-    yv = n * n;
+    yv = wide && d.wide.scratch > mat ? d.wide.scratch : mat;
     f0 = yv + n;
     bufs = f0 + n;
-    const int t = bufs + species_doubles(S);
+    const int t = bufs + species_doubles(d.S), tj = t + 3 * d.S;
+    jscr = wide ? 0 : tj;
     yt = t;
     ub = yt + n;
     invd = ub + n;
@@ -145,10 +149,10 @@ struct Ros4Layout {
     const int after = (rof + (n + 1) / 2 + 1) & ~1;  // 16-byte aligned
     lr = after;
     rhs_q.off = after;
-    rhs_q.chunk = rhs_chunk;
-    int most = t + jac_doubles(S, chunk);
+    rhs_q.chunk = d.rhs_chunk;
+    int most = wide ? tj : tj + d.narrow.scratch;
     if (after + 4 * n > most) most = after + 4 * n;
-    if (after + rhs_chunk > most) most = after + rhs_chunk;
+    if (after + d.rhs_chunk > most) most = after + d.rhs_chunk;
     doubles = (size_t)most;
   }
 };
