@@ -199,6 +199,66 @@ __device__ __forceinline__ double rt_over_p0_pow(int dnu, double T, double invT)
   return a == 0 ? 1.0 : (a == 1 ? q : q * q);
 }
 
+// ---------------------------------------------------------------- products off the FP64 pipe
+// a * b rounded to nearest even, in integer arithmetic: the 53-bit
+// significands are multiplied in full (b's shifted up by 11, so that the upper
+// 64 bits of the product hold the result and the lower 64 its rounding), the
+// leading bit normalised and the rest rounded.  About 42 issue cycles of one
+// scheduler; the FP64 unit, which the SM's four schedulers share, takes 64 of
+// them for a warp instruction, and the integer units are idle beside it.  The
+// same bits as the FP64 instruction while both operands and the product are
+// normal numbers (nothing else is handled: callers check the ranges).
+__device__ __forceinline__ double mul_int(double a, double b) {
+  const uint32_t ah = (uint32_t)__double2hiint(a), al = (uint32_t)__double2loint(a);
+  const uint32_t bh = (uint32_t)__double2hiint(b), bl = (uint32_t)__double2loint(b);
+  const uint32_t mh = (ah & 0xfffffu) | 0x100000u, nh = (bh & 0xfffffu) | 0x100000u;
+  const uint32_t Bh = __funnelshift_l(bl, nh, 11), Bl = bl << 11;
+  const uint64_t t0 = (uint64_t)al * Bl;
+  const uint64_t t1 = (uint64_t)al * Bh + (uint32_t)(t0 >> 32);
+  const uint64_t t2 = (uint64_t)mh * Bl + (uint32_t)t1;
+  const uint64_t t3 = (uint64_t)mh * Bh + (uint32_t)(t1 >> 32) + (uint32_t)(t2 >> 32);
+  uint32_t H1 = (uint32_t)(t3 >> 32), H0 = (uint32_t)t3, L1 = (uint32_t)t2;
+  const uint32_t L0 = (uint32_t)t0;
+  const int s = (int)(H1 >> 20) ^ 1;  // 1: the product of the significands is below 2
+  H1 = __funnelshift_l(H0, H1, s);
+  H0 = __funnelshift_l(L1, H0, s);
+  L1 = __funnelshift_l(L0, L1, s);
+  const uint32_t sticky = (L1 << 1) | L0;
+  const uint32_t up = (L1 >> 31) & (H0 | (sticky != 0 ? 1u : 0u));
+  const uint64_t m = (((uint64_t)H1 << 32) | H0) + (up & 1u);
+  // biased exponents add up; the leading bit of m adds the last one
+  const int e = (int)((ah >> 20) & 0x7ff) + (int)((bh >> 20) & 0x7ff) - 1023 - s;
+  const uint32_t rh = ((uint32_t)e << 20) + (uint32_t)(m >> 32);
+  return __hiloint2double((int)(rh | ((ah ^ bh) & 0x80000000u)), (int)(uint32_t)m);
+}
+template <bool INT>
+__device__ __forceinline__ double mul_sel(double a, double b) {
+  if constexpr (INT) return mul_int(a, b);
+  else return __dmul_rn(a, b);
+}
+
+// Ranges in which the products of a reaction's concentrations and Gibbs
+// factors stay normal: up to three concentrations within 2^+-300 (not zero),
+// and (R T/p0)^dnu, within 2^+-46 for T in [2^-9, 2^21), times up to six
+// factors 2^(+-g), |g| < 160.
+__device__ __forceinline__ bool conc_in_range(double x) {
+  const uint32_t e = ((uint32_t)__double2hiint(x) >> 20) & 0x7ff;
+  return e - (1023u - 300u) < 600u;
+}
+__device__ __forceinline__ bool gibbs_in_range(double g) {
+  return ((uint32_t)__double2hiint(g) & 0x7fffffffu) < 0x40640000u;  // |g| < 160
+}
+__device__ __forceinline__ bool temp_in_range(double T) {
+  const uint32_t h = (uint32_t)__double2hiint(T);
+  return h - 0x3f600000u < 0x41400000u - 0x3f600000u;
+}
+// c k_f and c k_r within 2^+-400: their products with two concentrations are
+// normal too.
+__device__ __forceinline__ bool rate_in_range(double k) {
+  const uint32_t e = ((uint32_t)__double2hiint(k) >> 20) & 0x7ff;
+  return e - (1023u - 400u) < 800u;
+}
+
 // ---------------------------------------------------------------- statuses
 enum : int32_t { ST_OK = 0, ST_MAXSTEPS = 1, ST_HMIN = 2, ST_NONFINITE = 3, ST_SINGULAR = 4,
                  ST_BADINPUT = 5 };

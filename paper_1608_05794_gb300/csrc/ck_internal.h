@@ -42,6 +42,8 @@ struct LaunchCfg {
 
 cudaError_t launch_rhs(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                        cudaStream_t st);
+cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
+                            cudaStream_t st);
 cudaError_t launch_jacobian(const HostMech& hm, int64_t n, const double* p, const double* y,
                             double* jac, cudaStream_t st, const LaunchCfg& cfg);
 cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, const double* y, const double* h,

@@ -11,16 +11,27 @@
 
 namespace ck {
 
-// Threads of a team for a mechanism or matrix of dimension n: one warp for
-// the smallest (no barriers), otherwise three warps (an odd number spreads
-// the single-warp phases of neighbouring CTAs over the SM's four schedulers)
-// or eight.
-static int team_size(int n) { return n <= 24 ? 32 : (n <= 64 ? 96 : 256); }
+// ------------------------------------------------------------------ RHS (team)
+template <bool INT>
+__global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N,
+                                                  const double* __restrict__ p, const double* __restrict__ y,
+                                                  double* __restrict__ f) {
+  extern __shared__ __align__(16) double sm[];
+  const int n = d.n;
+  const RhsQ qq{2 * n + species_doubles(d.S), d.rhs_chunk};
+  for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = y[r * n + i];
+    team_sync();
+    team_rhs<INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) f[r * n + i] = sm[n + i];
+  }
+}
 
 // ------------------------------------------------------------------ Jacobian
 // The matrix is assembled in place in the output (its lines stay in L2), so
 // that a CTA's shared memory holds the per-reaction values instead.
-__global__ void __launch_bounds__(256) k_jacobian(const __grid_constant__ DevMech d, int64_t N,
+template <int P, int MINB>
+__global__ void __launch_bounds__(P, MINB) k_jacobian(const __grid_constant__ DevMech d, int64_t N,
                                                   const double* __restrict__ p, const double* __restrict__ y,
                                                   double* __restrict__ jac) {
   extern __shared__ __align__(16) double sm[];
@@ -30,7 +41,7 @@ __global__ void __launch_bounds__(256) k_jacobian(const __grid_constant__ DevMec
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
     team_sync();
-    team_jacobian(d, d.wide, d.tab, p[r], ys, fs, jac + r * (int64_t)n * n, nullptr,
+    team_jacobian<(P > 64)>(d, d.wide, d.tab, p[r], ys, fs, jac + r * (int64_t)n * n, nullptr,
                   carve_bufs(fs + n, d.S, sm, d.wide.chunk, 256));
   }
 }
@@ -47,7 +58,7 @@ __global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ Dev
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[ys + i] = y[r * n + i];
     team_sync();
-    team_jacobian_fd(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, ys + 2 * n, ys + 3 * n, ys + 4 * n,
+    team_jacobian_fd<false>(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, ys + 2 * n, ys + 3 * n, ys + 4 * n,
                      n > 64 ? 256 : 64, qq);
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = sm[e];
     team_sync();
@@ -114,7 +125,8 @@ __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu
 // right-hand sides are evaluated by the team, so a reactor's working set
 // (8 n-vectors and one chunk of reaction scratch) stays in shared memory and
 // the number of steps of one reactor never holds back another.
-__global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
+template <bool INT>
+__global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
                                                    double* __restrict__ y, const double* __restrict__ dt,
                                                    double* h_io, SolverParams sp, int32_t* steps,
                                                    int32_t* status, int32_t* queue) {
@@ -155,7 +167,7 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ D
       if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
+      else h = team_h0<INT>(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
       const double hmin = 1e-15 * tf;
       double t = 0.0;
       bool last_rej = false, last_nf = false;
@@ -165,38 +177,38 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ D
         const double hh = clamped ? tf - t : h;
         if (hh < hmin) { st = last_nf ? ST_NONFINITE : ST_HMIN; break; }
         // k_s = hh f(y + sum_j a_sj k_j)
-        team_rhs(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k0[i] *= hh;
           yt[i] = fma(RK_A21, k0[i], yv[i]);
         }
         team_sync();
-        team_rhs(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k1[i] *= hh;
           yt[i] = fma(RK_A32, k1[i], fma(RK_A31, k0[i], yv[i]));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k2[i] *= hh;
           yt[i] = fma(RK_A43, k2[i], fma(RK_A42, k1[i], fma(RK_A41, k0[i], yv[i])));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k3[i] *= hh;
           yt[i] = fma(RK_A54, k3[i], fma(RK_A53, k2[i], fma(RK_A52, k1[i], fma(RK_A51, k0[i], yv[i]))));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k4[i] *= hh;
           yt[i] = fma(RK_A65, k4[i],
                       fma(RK_A64, k3[i], fma(RK_A63, k2[i], fma(RK_A62, k1[i], fma(RK_A61, k0[i], yv[i])))));
         }
         team_sync();
-        team_rhs(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
+        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k1, whose weights are 0)
         int nf = 0;
         for (int i = tid; i < n; i += P) {
@@ -256,15 +268,29 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_team(const __grid_constant__ D
 }
 
 // ------------------------------------------------------------------ launchers
+cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
+                            cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  const int nn = hm.d.n;
+  const size_t smem = sizeof(double) * (2 * (size_t)nn + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 128);
+  LaunchCfg cfg;
+  auto kern = hm.S > 32 ? k_rhs_team<true> : k_rhs_team<false>;
+  const int grid = team_grid(kern, threads, smem, n, cfg);
+  kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, f);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_jacobian(const HostMech& hm, int64_t n, const double* p, const double* y,
                             double* jac, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
   const size_t smem =
       sizeof(double) * ((size_t)hm.d.wide.scratch + 2 * nn + species_doubles(hm.S) + 3 * hm.S);
-  const int threads = team_size(nn);
-  const int grid = team_grid(k_jacobian, threads, smem, n, cfg);
-  k_jacobian<<<grid, threads, smem, st>>>(hm.d, n, p, y, jac);
+  auto kern = nn <= 24 ? k_jacobian<64, 12> : (nn <= 64 ? k_jacobian<128, 6> : k_jacobian<256, 2>);
+  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 128 : 256);
+  const int grid = team_grid(kern, threads, smem, n, cfg);
+  kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, jac);
   return cudaGetLastError();
 }
 
@@ -273,7 +299,7 @@ cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, c
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
   const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + species_doubles(hm.S) + hm.d.rhs_chunk);
-  const int threads = team_size(nn);
+  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 256);
   const int grid = team_grid(k_jacobian_fd, threads, smem, n, cfg);
   k_jacobian_fd<<<grid, threads, smem, st>>>(hm.d, n, p, y, h, rtol, atol, jac);
   return cudaGetLastError();
@@ -284,7 +310,9 @@ cudaError_t launch_lu_factor(int64_t batch, int dim, double* a, int32_t* piv, in
   if (batch <= 0) return cudaSuccess;
   LaunchCfg cfg;
   const size_t smem = sizeof(double) * lu_doubles(dim);
-  const int threads = team_size(dim);
+  // a warp alone needs no barriers and is enough for the smallest matrices;
+  // measured for 4096 matrices of 54: 96 threads 712 us, 128 680
+  const int threads = dim <= 24 ? 32 : (dim <= 64 ? 128 : 256);
   const int grid = team_grid(k_lu_factor, threads, smem, batch, cfg);
   k_lu_factor<<<grid, threads, smem, st>>>(batch, dim, a, piv, info);
   return cudaGetLastError();
@@ -333,11 +361,15 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
   const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + hm.d.rhs_chunk);
-  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 128);
-  const int grid = team_grid(k_rkf45_team, threads, smem, n, cfg);
+  // four warps shorten a step while the batch leaves the SMs room; two keep
+  // their lanes busier in one that does not (53 species, four / two warps: 300
+  // reactors 13.0 / 19.0 ms, 1000 23.4 / 26.5, 2000 41.5 / 39.1, 16384 278 / 268)
+  const int threads = nn <= 24 ? 64 : (nn > 64 || n < (int64_t)12 * sm_count() ? 128 : 64);
+  auto kern = hm.S > 32 ? k_rkf45_team<true> : k_rkf45_team<false>;
+  const int grid = team_grid(kern, threads, smem, n, cfg);
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  k_rkf45_team<<<grid, threads, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
+  kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
   return cudaGetLastError();
 }
 

@@ -87,10 +87,7 @@ __device__ __forceinline__ MechView view_of(const DevMech& d, const StageLayout&
 constexpr uint32_t STAGE_HDR = 16;
 
 // ------------------------------------------------------------------ RHS
-// R reactors a thread (rhs_thread_r); the last group of a batch repeats
-// reactor N - 1 in its missing places (the same thread writes the same
-// values there).
-template <int MAXS, int R>
+template <int MAXS, bool INT>
 __global__ void __launch_bounds__(128) k_rhs(DevMech d, StageLayout L, int staged, int64_t N,
                                              const double* __restrict__ p,
                                              const double* __restrict__ y, double* __restrict__ f,
@@ -102,26 +99,10 @@ __global__ void __launch_bounds__(128) k_rhs(DevMech d, StageLayout L, int stage
     base = smem + STAGE_HDR;
   }
   const MechView m = view_of(d, L, base);
-  double X[R * MAXS], G[2 * R * MAXS], wd[R * MAXS];
+  double X[MAXS], G[2 * MAXS], wd[MAXS];
   const int n = d.n;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * R; r < N;
-       r += (int64_t)gridDim.x * blockDim.x * R) {
-    if constexpr (R == 1) {
-      rhs_thread(m, p[r], y + r * n, 1, f + r * n, 1, X, G, wd);
-    } else {
-      double pr[R];
-      const double* yr[R];
-      double* fr[R];
-#pragma unroll
-      for (int j = 0; j < R; ++j) {
-        const int64_t rj = r + j < N ? r + j : N - 1;
-        pr[j] = p[rj];
-        yr[j] = y + rj * n;
-        fr[j] = f + rj * n;
-      }
-      rhs_thread_r<R>(m, pr, yr, fr, X, G, wd);
-    }
-  }
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < N; r += (int64_t)gridDim.x * blockDim.x)
+    rhs_thread<INT>(m, p[r], y + r * n, 1, f + r * n, 1, X, G, wd);
 }
 
 // ------------------------------------------------------------------ RKF45
@@ -141,7 +122,7 @@ __device__ __forceinline__ double wrms_thread(int n, const double* e, const doub
 __device__ double h0_thread(const MechView& m, int n, double p, const double* y0, double tspan,
                             double rtol, double atol, double* f0, double* y1, double* f1, double* X,
                             double* G, double* wd) {
-  rhs_thread(m, p, y0, 1, f0, 1, X, G, wd);
+  rhs_thread<false>(m, p, y0, 1, f0, 1, X, G, wd);
   double d0 = 0.0, d1 = 0.0;
   for (int i = 0; i < n; ++i) {
     const double sc = atol + rtol * fabs(y0[i]);
@@ -152,7 +133,7 @@ __device__ double h0_thread(const MechView& m, int n, double p, const double* y0
   d1 = sqrt(d1 / n);
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   for (int i = 0; i < n; ++i) y1[i] = fma(ha, f0[i], y0[i]);
-  rhs_thread(m, p, y1, 1, f1, 1, X, G, wd);
+  rhs_thread<false>(m, p, y1, 1, f1, 1, X, G, wd);
   double d2 = 0.0;
   for (int i = 0; i < n; ++i) {
     const double sc = atol + rtol * fabs(y0[i]);
@@ -231,28 +212,28 @@ __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int sta
         finish = true;
       } else {
         // stages k_s = hh f(y + sum_j a_sj k_j)
-        rhs_thread(m, pr, yv, 1, k[0], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yv, 1, k[0], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[0][i] *= hh;
         for (int i = 0; i < n; ++i) yt[i] = fma(RK_A21, k[0][i], yv[i]);
-        rhs_thread(m, pr, yt, 1, k[1], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yt, 1, k[1], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[1][i] *= hh;
         for (int i = 0; i < n; ++i) yt[i] = fma(RK_A32, k[1][i], fma(RK_A31, k[0][i], yv[i]));
-        rhs_thread(m, pr, yt, 1, k[2], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yt, 1, k[2], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[2][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A43, k[2][i], fma(RK_A42, k[1][i], fma(RK_A41, k[0][i], yv[i])));
-        rhs_thread(m, pr, yt, 1, k[3], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yt, 1, k[3], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[3][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A54, k[3][i],
                       fma(RK_A53, k[2][i], fma(RK_A52, k[1][i], fma(RK_A51, k[0][i], yv[i]))));
-        rhs_thread(m, pr, yt, 1, k[4], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yt, 1, k[4], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[4][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A65, k[4][i],
                       fma(RK_A64, k[3][i],
                           fma(RK_A63, k[2][i], fma(RK_A62, k[1][i], fma(RK_A61, k[0][i], yv[i])))));
-        rhs_thread(m, pr, yt, 1, k[5], 1, X, G, wd);
+        rhs_thread<false>(m, pr, yt, 1, k[5], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[5][i] *= hh;
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k[1], whose b is 0)
         bool nf = false;
@@ -357,23 +338,14 @@ static int blocks_for(K kernel, int threads, size_t smem) {
   return per_sm * sm_count();
 }
 
-// Reactors a thread of k_rhs, for mechanisms above and up to 32 species.
-// Two and four (rhs_thread_r, each table record read once for all of them)
-// measured slower on GB300: 33.2 and 22.7 M evaluations/s against 38.1 M on
-// the 53-species mechanism, 9.4 and 5.2 M against 13.4 M on the 111-species
-// one, 392 and 383 M against 440 M on the 10-species one (twice and four
-// times the per-lane scratch in local memory, and fewer resident threads).
-constexpr int RHS_REACTORS = 1;
-constexpr int RHS_REACTORS_SMALL = 1;
-
-template <int MAXS, int R>
+template <int MAXS, bool INT>
 static cudaError_t rhs_impl(const HostMech& hm, int64_t n, const double* p, const double* y,
                             double* f, cudaStream_t st) {
-  auto kern = k_rhs<MAXS, R>;
+  auto kern = k_rhs<MAXS, INT>;
   const int threads = 128;
   size_t smem = 0;
   const int staged = stage_pays(hm, kern, threads, &smem);
-  int64_t want = (n + (int64_t)threads * R - 1) / ((int64_t)threads * R);
+  int64_t want = (n + threads - 1) / threads;
   int64_t cap = blocks_for(kern, threads, smem);
   int blocks = (int)(want < cap ? want : cap);
   if (blocks < 1) blocks = 1;
@@ -381,11 +353,22 @@ static cudaError_t rhs_impl(const HostMech& hm, int64_t n, const double* p, cons
   return cudaGetLastError();
 }
 
+// One reactor a thread only for batches that fill the SMs with threads: below
+// that a thread's serial chain through all reactions sets the time whatever
+// the batch, and one team a reactor is faster.  Measured on GB300 (thread /
+// team, us): 10 species 55 / 17 at 512 reactors, 55 / 58 at 4000, 55 / 198 at
+// 16000; 53 species 880 / 231 at 8000, 1992 / 1792 at 65536, 2983 / 3637 at
+// 131072; 111 species 3421 / 1247 at 20011, 6634 / 4933 at 80000.  Products in
+// integer arithmetic (mul_int) pay once the FP64 unit is the bound: 10 species
+// 55 -> 65 us at 16000, 711 -> 571 us at 300000; 53 species 3440 -> 2983 us.
 cudaError_t launch_rhs(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                        cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (hm.S <= 32) return rhs_impl<32, RHS_REACTORS_SMALL>(hm, n, p, y, f, st);
-  return rhs_impl<128, RHS_REACTORS>(hm, n, p, y, f, st);
+  const int64_t per_sm = n / sm_count();
+  if (hm.S > 64 || per_sm < (hm.S > 32 ? 512 : 26)) return launch_rhs_team(hm, n, p, y, f, st);
+  if (hm.S > 32) return rhs_impl<128, true>(hm, n, p, y, f, st);
+  if (per_sm < 256) return rhs_impl<32, false>(hm, n, p, y, f, st);
+  return rhs_impl<32, true>(hm, n, p, y, f, st);
 }
 
 template <int MAXS>

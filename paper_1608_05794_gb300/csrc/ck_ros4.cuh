@@ -28,18 +28,23 @@ static __device__ __noinline__ void refined_solve(const double* M64, int n, int 
   for (int i = tid; i < n; i += P) x[i] = (double)xf[i];
   team_sync();
   for (int it = 0; it < refine; ++it) {
-    for (int i = tid; i < n; i += P) {
-      const double* row = M64 + (size_t)i * n;
-      double s0 = u[i], s1 = 0.0, s2 = 0.0, s3 = 0.0;
-      int j = 0;
-      for (; j + 4 <= n; j += 4) {
-        s0 = fma(-row[j], x[j], s0);
-        s1 = fma(-row[j + 1], x[j + 1], s1);
-        s2 = fma(-row[j + 2], x[j + 2], s2);
-        s3 = fma(-row[j + 3], x[j + 3], s3);
+    // four lanes a row, one of four partial sums each (every fourth column;
+    // the last n % 4 join the first), added as (s0 + s1) + (s2 + s3)
+    const int n4 = n & ~3, q = tid & 3;
+    for (int w = tid; w < ((4 * n + 31) & ~31); w += P) {
+      const int i = w >> 2;
+      double s = 0.0;
+      if (i < n) {
+        const double* row = M64 + (size_t)i * n;
+        if (q == 0) s = u[i];
+#pragma unroll 4
+        for (int j = q; j < n4; j += 4) s = fma(-row[j], x[j], s);
+        if (q == 0)
+          for (int j = n4; j < n; ++j) s = fma(-row[j], x[j], s);
       }
-      for (; j < n; ++j) s0 = fma(-row[j], x[j], s0);
-      xf[i] = (float)((s0 + s1) + (s2 + s3));
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (q == 0 && i < n) xf[i] = (float)s;
     }
     team_sync();
     if (tid < 32) warp_solve<float>(0, n, rof_o, invd_o, xf_o);
@@ -97,6 +102,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
   extern __shared__ __align__(16) double sm[];
   __shared__ int slot;
   __shared__ Ros4Ctl ctl;
+  constexpr bool INT = P == 256;  // products in integer arithmetic (see team_rhs)
   using F = typename std::conditional<PREC == 0, double, float>::type;  // type of the factors
   const int n = d.n, nn = n * n;
   const double* tab = d.tab;  // 2 KB, stays in L1
@@ -133,7 +139,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
       if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0(d, tab, pr, L.yv, tf, sp.rtol, sp.atol, L.f0, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+      else h = team_h0<INT>(d, tab, pr, L.yv, tf, sp.rtol, sp.atol, L.f0, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
       const double hmin = 1e-15 * tf;
       // the next attempt: its step size, or the end of the integration
       auto next = [&](int accept) {
@@ -171,12 +177,12 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
         // same y); A = J - I/(hh gamma) = -M; LU of A
         if (!have_j) {
           if (sp.jac == 1) {
-            team_jacobian_fd(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, L.yt, L.ub, L.bufs, L.vp,
+            team_jacobian_fd<INT>(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, L.yt, L.ub, L.bufs, L.vp,
                              L.rhs_q, have_f);
           } else {
             // assembled in the copy Mg where there is one
             const JacTab& jt = Mg ? d.wide : d.narrow;
-            team_jacobian(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr,
+            team_jacobian<INT>(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr,
                           carve_bufs(sm + L.bufs, d.S, sm + L.jscr, jt.chunk, L.vp));
           }
           if (PREC) {
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           Yt[tid] = fma(-ROS_A21, u1, yi);
         }
         team_sync();
-        team_rhs(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        team_rhs<INT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
         if (own) ub[tid] = fma(ctl.c21, u1, ub[tid]);
         solve();
         // stage 3: M u3 = f(y + a31 u1 + a32 u2) + (c31 u1 + c32 u2)/h
@@ -242,7 +248,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           Yt[tid] = fma(-ROS_A32, u2, fma(-ROS_A31, u1, yi));
         }
         team_sync();
-        team_rhs(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        team_rhs<INT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
         if (own) {
           f3 = ub[tid];
           ub[tid] = fma(ctl.c32, u2, fma(ctl.c31, u1, f3));

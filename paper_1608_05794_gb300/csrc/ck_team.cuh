@@ -155,13 +155,17 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // through log T) are formed side by side by two warps, everything else of
 // the species by all of them: a polynomial pass of 32 species is one work
 // item, dealt to the warps in turn.
-__device__ __forceinline__ void team_species(const DevMech& m, double p, const double* y,
+// Ends with a barrier and returns (the same in every thread) whether the
+// ranges allow the reactions' products to be taken in integer arithmetic
+// (mul_int).
+__device__ __forceinline__ bool team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
   const int S = m.S, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int SG = species_groups(S);
   double* red = b.red;
   const double T = y[0];
   x.T = T;
+  bool ok = temp_in_range(T);
   if (warp == nw - 1) {
     const double invT = rcp_rn(T), lnT = log(T);
     const double T2 = T * T, T3 = T2 * T;
@@ -206,7 +210,10 @@ __device__ __forceinline__ void team_species(const DevMech& m, double p, const d
       if (q < SG) {
         const int k = 32 * q + lane;
         const double xk = k < S ? rho * yw[q] : 0.0;
-        if (k < S) b.X[k] = xk;
+        if (k < S) {
+          b.X[k] = xk;
+          ok &= conc_in_range(xk);
+        }
         if (q >= 2 && fold) part[q - 2] += xk;
         else part[q] = xk;
       }
@@ -240,6 +247,7 @@ __device__ __forceinline__ void team_species(const DevMech& m, double p, const d
         g = fma(a[15], T3, g);
         g = fma(a[16], T4, g);
         g = fma(a[17], x.invT, g);
+        ok &= gibbs_in_range(g);
         ck_exp2_pm(g, tab, b.Gp[k], b.Gm[k]);
       } else {
         b.cpR[k] = fma(a[4], T4, fma(a[3], T3, fma(a[2], T2, fma(a[1], T, a[0]))));
@@ -247,6 +255,7 @@ __device__ __forceinline__ void team_species(const DevMech& m, double p, const d
       }
     }
   }
+  return __syncthreads_and(ok);
 }
 
 // A reaction record without its fall-off limit (the last two vectors) in
@@ -262,10 +271,13 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 
 // Rates of one reaction at the mixture state.  JAC: also the partial-
 // derivative pieces used by the Jacobian (see team_jacobian).  i: index of
-// the reaction inside the current chunk, iw: among its typed reactions.  Empty slots read the neutral
-// entries of the species arrays (a product with 1, a sum with 0, exact), so
-// that reactions of every molecularity take the same instructions.
-template <bool JAC>
+// the reaction inside the current chunk, iw: among its typed reactions.
+// Empty slots read the neutral entries of the species arrays (a product with
+// 1, a sum with 0, exact), so that reactions of every molecularity take the
+// same instructions.  INT: the products of concentrations and of Gibbs factors
+// in integer arithmetic, beside the FP64 unit, which bounds the team kernels
+// (10 of the 23 FP64 instructions of a rate, 20 of 49 with its derivatives).
+template <bool JAC, bool INT>
 __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
                                               const TeamBufs& b, const double* tab, int i, int iw) {
   const RxnRec r = load_rxn(src);
@@ -274,28 +286,28 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
   const double kf = ck_exp2(l2kf, tab);
   const int s0 = r.sp[0], s1 = r.sp[1], s2 = r.sp[2], s3 = r.sp[3], s4 = r.sp[4], s5 = r.sp[5];
   const double x0 = X[s0], x1 = X[s1], x2 = X[s2], y0 = X[s3], y1 = X[s4], y2 = X[s5];
-  const double fwd = x0 * x1 * x2;
+  const double fwd = mul_sel<INT>(mul_sel<INT>(x0, x1), x2);
   double kr = 0.0, rv = 0.0, dlnkc = 0.0;
   if (r.rev == 2) {
     // explicit reverse Arrhenius; for the Jacobian, d ln k_r/dT enters as
     // d ln k_f/dT - d ln K_c/dT, so dlnkc carries their difference
     const double* ra = m.revp + 3 * r.rev_ix;
     kr = ck_exp2(fma(-ra[2], x.invT, fma(ra[1], x.log2T, ra[0])), tab);
-    rv = y0 * y1 * y2;
+    rv = mul_sel<INT>(mul_sel<INT>(y0, y1), y2);
     if (JAC) {
       const double dlnkf = fma(r.EoR, x.invT, r.beta) * x.invT;
       dlnkc = dlnkf - fma(ra[2] * LN2, x.invT, ra[1]) * x.invT;
     }
   } else if (r.rev) {
     // 1/K_c = (R T/p0)^dnu prod_reactants Gp prod_products Gm (Eq. kc)
-    double kci = b.red[SC_PW + 2 + r.dnu] * b.Gp[s0];
-    kci *= b.Gm[s3];
-    kci *= b.Gp[s1];
-    kci *= b.Gm[s4];
-    kci *= b.Gp[s2];
-    kci *= b.Gm[s5];
+    double kci = mul_sel<INT>(b.red[SC_PW + 2 + r.dnu], b.Gp[s0]);
+    kci = mul_sel<INT>(kci, b.Gm[s3]);
+    kci = mul_sel<INT>(kci, b.Gp[s1]);
+    kci = mul_sel<INT>(kci, b.Gm[s4]);
+    kci = mul_sel<INT>(kci, b.Gp[s2]);
+    kci = mul_sel<INT>(kci, b.Gm[s5]);
     kr = kf * kci;
-    rv = y0 * y1 * y2;
+    rv = mul_sel<INT>(mul_sel<INT>(y0, y1), y2);
     if (JAC) {
       // d ln K_c / dT = (sum_j nu_j H_j/(R T) - dnu) / T
       double hs = b.hRT[s3];
@@ -345,13 +357,27 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
     // d q / d[X] slot by slot: c k_f prod of the other reactant slots, and
     // -c k_r prod of the other product slots
     double* P = b.P + 6 * i;
-    P[0] = ckf * (x1 * x2);
-    P[1] = ckf * (x0 * x2);
-    P[2] = ckf * (x0 * x1);
-    if (r.rev) {
-      P[3] = -ckr * (y1 * y2);
-      P[4] = -ckr * (y0 * y2);
-      P[5] = -ckr * (y0 * y1);
+    const double x12 = mul_sel<INT>(x1, x2), x02 = mul_sel<INT>(x0, x2), x01 = mul_sel<INT>(x0, x1);
+    const double y12 = mul_sel<INT>(y1, y2), y02 = mul_sel<INT>(y0, y2), y01 = mul_sel<INT>(y0, y1);
+    const bool in = INT && rate_in_range(ckf) && (!r.rev || rate_in_range(ckr));
+    if (INT && __all_sync(__activemask(), in)) {
+      P[0] = mul_sel<INT>(ckf, x12);
+      P[1] = mul_sel<INT>(ckf, x02);
+      P[2] = mul_sel<INT>(ckf, x01);
+      if (r.rev) {
+        P[3] = mul_sel<INT>(-ckr, y12);
+        P[4] = mul_sel<INT>(-ckr, y02);
+        P[5] = mul_sel<INT>(-ckr, y01);
+      }
+    } else {
+      P[0] = ckf * x12;
+      P[1] = ckf * x02;
+      P[2] = ckf * x01;
+      if (r.rev) {
+        P[3] = -ckr * y12;
+        P[4] = -ckr * y02;
+        P[5] = -ckr * y01;
+      }
     }
     // D = sum_j dq/d[X_j] [X_j]: Euler's theorem for the mass-action
     // products (homogeneous of degree nreac / nprod) plus the [M] part.
@@ -373,6 +399,13 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
 // dynamic shared memory, so that this out-of-line function still addresses
 // shared memory directly: y_o, f_o the vectors (n = S + 1; f may not be y),
 // bufs_o the work arrays (species_doubles), qq the rates of progress.
+// INT: products in integer arithmetic where the ranges allow it.  That pays
+// where the FP64 unit is the bound (RKF45 on 16384 reactors of the 53-species
+// mechanism: 278 against 321 ms), not where a team waits for its chain of
+// operations (a product is 106 cycles of it in integers, 72 in FP64: ROS4 on
+// 512 reactors of the 10-species mechanism, 245 against 230 ms) or is short of
+// registers (ROS4 on 4096 of the 53-species one, 617 against 600 ms).
+template <bool INT>
 static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
   extern __shared__ __align__(16) double sm[];
@@ -382,8 +415,7 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   Mix x;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int S = m.S, SG = species_groups(S);
-  team_species(m, p, y, b, x, tab);
-  team_sync();
+  const bool in = team_species(m, p, y, b, x, tab);
   const double invrho = x.invrho;
   // every chunk: its rates of progress, then one fixed-order gather per
   // species, longest rows first so that the lanes of a warp do similar work
@@ -393,8 +425,13 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
     const int cnt = m.R - base < CH ? m.R - base : CH;
     // last reactions first: the expensive ones (fall-off) then fill whole
     // warps, and the warp that is left partly empty has the cheapest
-    for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
-      team_reaction<false>(m, m.rxn + base + li, x, b, tab, li, 0);
+    if (INT && in) {
+      for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+        team_reaction<false, INT>(m, m.rxn + base + li, x, b, tab, li, 0);
+    } else {
+      for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+        team_reaction<false, false>(m, m.rxn + base + li, x, b, tab, li, 0);
+    }
     team_sync();
     const bool last = base + cnt >= m.R;
     for (int kk = tid; kk < S; kk += blockDim.x) {
@@ -484,13 +521,13 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 // are read for the last time before M is written, so that a team needs shared
 // memory for the larger of the two only, and takes all reactions in one pass.
 // Needs b.vp >= S (one species a lane in the sums).
+template <bool INT>
 static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const double* tab, double p, const double* y,
                                      double* f, double* A, double* M, TeamBufs b) {
   Mix x;
   const int S = m.S, n = m.n, SG = species_groups(S);
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  team_species(m, p, y, b, x, tab);
-  team_sync();
+  const bool in = team_species(m, p, y, b, x, tab);
   // chunk by chunk, every target (species-block entries and the per-species
   // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
   // fixed-order sum of terms; one thread per target, no conflicts, the
@@ -498,8 +535,13 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
   for (int c = 0; c < jt.n_chunks; ++c) {
     const int base = c * jt.chunk, cnt = m.R - base < jt.chunk ? m.R - base : jt.chunk;
     const int ft = m.first_typed > base ? m.first_typed - base : 0;
-    for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
-      team_reaction<true>(m, m.rxn + base + li, x, b, tab, li, li - ft);
+    if (INT && in) {
+      for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+        team_reaction<true, INT>(m, m.rxn + base + li, x, b, tab, li, li - ft);
+    } else {
+      for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
+        team_reaction<true, false>(m, m.rxn + base + li, x, b, tab, li, li - ft);
+    }
     team_sync();
     for (int e = jt.jc_ptr[c] + tid; e < jt.jc_ptr[c + 1]; e += blockDim.x) {
       const JcEntry h = jt.jc[e];
@@ -607,8 +649,8 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
     // cs_j = sum_k e_k (A_kj + u_k) = W_j sum_k (e_k / W_k) A'_kj + sum_k e_k u_k
     const double csj = fma(m.W[j], cs[j], eu);
     const double cW = __dmul_rn(cpf, x.Wbar);
-    const double in = fma(x.rho, csj, -__dmul_rn(cW, he));
-    const double tt = fma(__dmul_rn(x.T, in), inv_rc, __dmul_rn(Tdot, fma(b.cpR[j] - cvf, inv_cpm, -cW)));
+    const double d0 = fma(x.rho, csj, -__dmul_rn(cW, he));
+    const double tt = fma(__dmul_rn(x.T, d0), inv_rc, __dmul_rn(Tdot, fma(b.cpR[j] - cvf, inv_cpm, -cW)));
     const double v = -tt * m.invW[j];
     A[1 + j] = v;
     if (M) M[1 + j] = v;

@@ -28,6 +28,7 @@ static __device__ __forceinline__ int team_next(int32_t* queue, int* slot) {
 // for this y) and reused as the first stage's f; the n columns cost n team
 // RHS evaluations.  y_o, f0_o, yt_o, f_o: offsets of n-vectors in shared
 // memory (the last two scratch); bufs_o, vp, qq as in team_rhs.
+template <bool INT>
 static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const double* tab, double p, int y_o, double h,
                                                      double rtol, double atol, int f0_o, double* J, int yt_o,
                                                      int f_o, int bufs_o, int vp, RhsQ qq, bool have_f0 = false) {
@@ -37,7 +38,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
   const double* F = sm + f_o;
   double* Yt = sm + yt_o;
   const int n = d.n, tid = (int)threadIdx.x;
-  if (!have_f0) team_rhs(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
+  if (!have_f0) team_rhs<INT>(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
   double s = 0.0;
   if (tid < vp)
     for (int i = tid; i < n; i += vp) {
@@ -53,7 +54,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
     const double sj = fmax(srur * fabs(y[j]), s0 * (atol + rtol * fabs(y[j])));
     if (tid == 0) Yt[j] = y[j] + sj;
     team_sync();
-    team_rhs(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
+    team_rhs<INT>(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
     for (int i = tid; i < n; i += blockDim.x) J[(size_t)i * n + j] = (F[i] - f0[i]) / sj;
     if (tid == 0) Yt[j] = y[j];
     team_sync();
@@ -90,6 +91,7 @@ static __device__ __forceinline__ double team_wrms(int n, const double* e, const
 
 // Initial step, Hairer-Norsett-Wanner starting-step algorithm (order 4).
 // Offsets, vp and qq as in team_rhs; f0, y1, f1 are scratch vectors.
+template <bool INT>
 static __device__ __noinline__ double team_h0(const DevMech& d, const double* tab, double p, int y0_o, double tspan,
                                               double rtol, double atol, int f0_o, int y1_o, int f1_o, int bufs_o,
                                               int vp, RhsQ qq) {
@@ -98,7 +100,7 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   double *y1 = sm + y1_o, *red = sm + bufs_o;
   const int n = d.n, tid = (int)threadIdx.x;
   const bool lane_in = tid < vp;
-  team_rhs(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
+  team_rhs<INT>(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
   double s0 = 0.0, s1 = 0.0;
   if (lane_in)
     for (int i = tid; i < n; i += vp) {
@@ -111,7 +113,7 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   for (int i = tid; i < n; i += blockDim.x) y1[i] = fma(ha, f0[i], y0[i]);
   team_sync();
-  team_rhs(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
+  team_rhs<INT>(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
   double s2 = 0.0;
   if (lane_in)
     for (int i = tid; i < n; i += vp) {

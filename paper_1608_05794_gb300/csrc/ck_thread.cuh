@@ -22,72 +22,41 @@ struct MechView {
   int cv;             // 1: constant volume (p is the density)
 };
 
-// f = (dT/dt, dY_k/dt) at state y (Eqs. ydot, tdot, wdot, kfor, krev, kc,
-// tfits).  y and f are strided (element k at y[k*ys]); X and wd are per-lane
-// scratch of S doubles, G of 2S (the species factors 2^(g_k), 2^(-g_k)).
-//   rho = p Wbar / (R T), [X_k] = rho Y_k / W_k,
-//   k_f = 2^(log2 A + beta log2 T - Ea/(R T ln 2)),
-//   1/K_c = (R T/p0)^dnu prod_reactants 2^(g_j) prod_products 2^(-g_j), g_j = (S/R - H/RT)_j / ln 2,
-//   k_r = k_f / K_c,
-//   c = 1, [M], or P_r/(1+P_r) with P_r = 2^(log2 k0 - log2 k_inf) [M],
-//   q = c (k_f prod [X]^nu' - k_r prod [X]^nu''),  wdot_k = sum (nu'' - nu') q,
-//   dY_k/dt = wdot_k W_k / rho, dT/dt = -T sum_k (H_k/RT) wdot_k / (rho sum_k Y_k (cp_k/R)/W_k).
-// Explicit reverse rows: k_r = 2^(log2 A_r + beta_r log2 T - Ea_r/(R T ln 2)).
-// Constant volume (Sec. 3): rho = p (the parameter is the density) and
-// H/RT -> U/RT = H/RT - 1, cp/R -> cv/R = cp/R - 1 in dT/dt.
-__device__ __forceinline__ void rhs_thread(const MechView& m, double p, const double* y, int ys,
-                                           double* f, int fs, double* X, double* G, double* wd) {
-  const int S = m.S;
-  const double T = y[0];
-  const double invT = __drcp_rn(T);
-  const double lnT = log(T);
-  const double log2T = lnT * INV_LN2;
-  const double T2 = T * T, T3 = T2 * T, T4 = T3 * T;
-  double sumYW = 0.0;
-  for (int k = 0; k < S; ++k) sumYW = fma(y[(1 + k) * ys], m.invW[k], sumYW);
-  const double rho = m.cv ? p : p / (R_GAS * T * sumYW);
-  double Ctot = 0.0;
-  for (int k = 0; k < S; ++k) {
-    const double xk = rho * (y[(1 + k) * ys] * m.invW[k]);
-    X[k] = xk;
-    Ctot += xk;
-    const double* a = m.th + k * TH_PER_SPECIES + (T < m.tmid[k] ? 0 : TH_STRIDE);
-    double g = fma(a[11], lnT, a[12]);
-    g = fma(a[13], T, g);
-    g = fma(a[14], T2, g);
-    g = fma(a[15], T3, g);
-    g = fma(a[16], T4, g);
-    g = fma(a[17], invT, g);
-    ck_exp2_pm(g, m.tab, G[k], G[S + k]);
-    wd[k] = 0.0;
-  }
-  const double* Gm = G + S;
+// The reaction loop of rhs_thread: wd_k += nu q of every reaction, in order.
+// INT: the products of concentrations and of Gibbs factors in integer
+// arithmetic, beside the FP64 unit (see mul_int).
+template <bool INT>
+__device__ __forceinline__ void rates_thread(const MechView& m, double T, double invT, double log2T, double Ctot,
+                                             const double* X, const double* G, const double* Gm, double* wd) {
+  const double up = T * R_OVER_P0, up2 = up * up, dw = invT * P0_OVER_R, dw2 = dw * dw;
   for (int i = 0; i < m.R; ++i) {
     const RxnRec& r = m.rx[i];
     const double l2kf = fma(-r.EoR2, invT, fma(r.beta, log2T, r.lA2));
     const double kf = ck_exp2(l2kf, m.tab);
     double fwd = X[r.sp[0]];
-    if (r.nreac > 1) fwd *= X[r.sp[1]];
-    if (r.nreac > 2) fwd *= X[r.sp[2]];
+    if (r.nreac > 1) fwd = mul_sel<INT>(fwd, X[r.sp[1]]);
+    if (r.nreac > 2) fwd = mul_sel<INT>(fwd, X[r.sp[2]]);
     double net = kf * fwd;
     if (r.rev == 2) {
       const double* ra = m.revp + 3 * r.rev_ix;
       const double kr = ck_exp2(fma(-ra[2], invT, fma(ra[1], log2T, ra[0])), m.tab);
       double rv = X[r.sp[3]];
-      if (r.nprod > 1) rv *= X[r.sp[4]];
-      if (r.nprod > 2) rv *= X[r.sp[5]];
+      if (r.nprod > 1) rv = mul_sel<INT>(rv, X[r.sp[4]]);
+      if (r.nprod > 2) rv = mul_sel<INT>(rv, X[r.sp[5]]);
       net = fma(-kr, rv, net);
     } else if (r.rev) {
-      double kci = rt_over_p0_pow(r.dnu, T, invT) * G[r.sp[0]];
-      kci *= Gm[r.sp[3]];
-      if (r.nreac > 1) kci *= G[r.sp[1]];
-      if (r.nprod > 1) kci *= Gm[r.sp[4]];
-      if (r.nreac > 2) kci *= G[r.sp[2]];
-      if (r.nprod > 2) kci *= Gm[r.sp[5]];
+      const int dn = r.dnu;
+      const double q = dn >= 0 ? (dn == 0 ? 1.0 : (dn == 1 ? up : up2)) : (dn == -1 ? dw : dw2);
+      double kci = mul_sel<INT>(q, G[r.sp[0]]);
+      kci = mul_sel<INT>(kci, Gm[r.sp[3]]);
+      if (r.nreac > 1) kci = mul_sel<INT>(kci, G[r.sp[1]]);
+      if (r.nprod > 1) kci = mul_sel<INT>(kci, Gm[r.sp[4]]);
+      if (r.nreac > 2) kci = mul_sel<INT>(kci, G[r.sp[2]]);
+      if (r.nprod > 2) kci = mul_sel<INT>(kci, Gm[r.sp[5]]);
       const double kr = kf * kci;
       double rv = X[r.sp[3]];
-      if (r.nprod > 1) rv *= X[r.sp[4]];
-      if (r.nprod > 2) rv *= X[r.sp[5]];
+      if (r.nprod > 1) rv = mul_sel<INT>(rv, X[r.sp[4]]);
+      if (r.nprod > 2) rv = mul_sel<INT>(rv, X[r.sp[5]]);
       net = fma(-kr, rv, net);
     }
     double q = net;
@@ -109,6 +78,54 @@ __device__ __forceinline__ void rhs_thread(const MechView& m, double p, const do
     if (r.nprod > 1) wd[r.sp[4]] += q;
     if (r.nprod > 2) wd[r.sp[5]] += q;
   }
+}
+
+// f = (dT/dt, dY_k/dt) at state y (Eqs. ydot, tdot, wdot, kfor, krev, kc,
+// tfits).  y and f are strided (element k at y[k*ys]); X and wd are per-lane
+// scratch of S doubles, G of 2S (the species factors 2^(g_k), 2^(-g_k)).
+//   rho = p Wbar / (R T), [X_k] = rho Y_k / W_k,
+//   k_f = 2^(log2 A + beta log2 T - Ea/(R T ln 2)),
+//   1/K_c = (R T/p0)^dnu prod_reactants 2^(g_j) prod_products 2^(-g_j), g_j = (S/R - H/RT)_j / ln 2,
+//   k_r = k_f / K_c,
+//   c = 1, [M], or P_r/(1+P_r) with P_r = 2^(log2 k0 - log2 k_inf) [M],
+//   q = c (k_f prod [X]^nu' - k_r prod [X]^nu''),  wdot_k = sum (nu'' - nu') q,
+//   dY_k/dt = wdot_k W_k / rho, dT/dt = -T sum_k (H_k/RT) wdot_k / (rho sum_k Y_k (cp_k/R)/W_k).
+// Explicit reverse rows: k_r = 2^(log2 A_r + beta_r log2 T - Ea_r/(R T ln 2)).
+// Constant volume (Sec. 3): rho = p (the parameter is the density) and
+// H/RT -> U/RT = H/RT - 1, cp/R -> cv/R = cp/R - 1 in dT/dt.
+template <bool INT>
+__device__ __forceinline__ void rhs_thread(const MechView& m, double p, const double* y, int ys,
+                                           double* f, int fs, double* X, double* G, double* wd) {
+  const int S = m.S;
+  const double T = y[0];
+  const double invT = __drcp_rn(T);
+  const double lnT = log(T);
+  const double log2T = lnT * INV_LN2;
+  const double T2 = T * T, T3 = T2 * T, T4 = T3 * T;
+  double sumYW = 0.0;
+  for (int k = 0; k < S; ++k) sumYW = fma(y[(1 + k) * ys], m.invW[k], sumYW);
+  const double rho = m.cv ? p : p / (R_GAS * T * sumYW);
+  double Ctot = 0.0;
+  bool in = temp_in_range(T);
+  for (int k = 0; k < S; ++k) {
+    const double xk = rho * (y[(1 + k) * ys] * m.invW[k]);
+    X[k] = xk;
+    Ctot += xk;
+    in &= conc_in_range(xk);
+    const double* a = m.th + k * TH_PER_SPECIES + (T < m.tmid[k] ? 0 : TH_STRIDE);
+    double g = fma(a[11], lnT, a[12]);
+    g = fma(a[13], T, g);
+    g = fma(a[14], T2, g);
+    g = fma(a[15], T3, g);
+    g = fma(a[16], T4, g);
+    g = fma(a[17], invT, g);
+    in &= gibbs_in_range(g);
+    ck_exp2_pm(g, m.tab, G[k], G[S + k]);
+    wd[k] = 0.0;
+  }
+  const double* Gm = G + S;
+  if (INT && __all_sync(__activemask(), in)) rates_thread<INT>(m, T, invT, log2T, Ctot, X, G, Gm, wd);
+  else rates_thread<false>(m, T, invT, log2T, Ctot, X, G, Gm, wd);
   const double invrho = __drcp_rn(rho);
   const double cvf = m.cv ? 1.0 : 0.0;
   double cpm = 0.0, hw = 0.0;
