@@ -305,6 +305,22 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     }
   }
   csr_ptr[S] = (int32_t)csr_rx.size();
+  // the same one slot at a time (mechanisms of at most 32 species, which a
+  // thread may integrate alone)
+  std::vector<int32_t> slot_ptr(S + 1, 0);
+  std::vector<CsrTerm> slot;
+  if (S <= 32)
+    for (int k = 0; k < S; ++k) {
+      for (int i = 0; i < R; ++i)
+        for (int s = 0; s < 6; ++s)
+          if (rx[i].sp[s] == k) {
+            CsrTerm t{};
+            t.nu = s < 3 ? -1.0 : 1.0;
+            t.rx = i;
+            slot.push_back(t);
+          }
+      slot_ptr[k + 1] = (int32_t)slot.size();
+    }
   // team kernels walk the reactions in chunks: equal shares of at most what
   // the team's shared memory has room for
   const int n1 = S + 1, NN = n1 * n1;
@@ -327,23 +343,24 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   // memory):
   // - species-block entries A[k][j] += nu_ki * P[i][slot] for every slot of
   //   reaction i holding species j (and nu_ki (eff_ij - 1) * w[i] for the
-  //   third-body corrections), target index (1 + k) n + 1 + j;
+  //   third-body corrections), target index (1 + k) ld + 1 + j;
   // - per species k the four sums over its reactions in the chunk, wdot_k
   //   (nu q), a_k (nu dq/dT), E_k (nu D) and u_k (nu w), target index
-  //   n^2 + a S + k for a = 0..3, terms in the CSR order.
+  //   n ld + a S + k for a = 0..3, terms in the CSR order.
   // Longest lists first, so that lanes running the same iteration do similar
   // amounts of work.  The terms of a target come in reaction order whatever
   // the chunks, so its sum does not depend on them.
   struct JacHost {
-    int chunk = 1, n_chunks = 1, scratch = 0;
+    int chunk = 1, n_chunks = 1, scratch = 0, ld = 0;
     std::vector<int32_t> jc_ptr;
     std::vector<JcEntry> jc;
     std::vector<JcTerm> jt;
   };
   int n_jterms = 0;
-  auto jac_table = [&](int chunk) {
+  auto jac_table = [&](int chunk, int ld) {
     JacHost t;
     t.chunk = chunk;
+    t.ld = ld;
     t.n_chunks = R ? (R + chunk - 1) / chunk : 1;
     t.jc_ptr.push_back(0);
     n_jterms = 0;
@@ -386,10 +403,10 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
         JcEntry h{};
         if (e < S * S) {
           const int k = e / S, j = e % S;
-          h.idx = (1 + k) * n1 + 1 + j;
+          h.idx = (1 + k) * ld + 1 + j;
           n_jterms += (int)ent[e].size();
         } else {
-          h.idx = NN + (e - S * S);
+          h.idx = n1 * ld + (e - S * S);
         }
         h.beg = (int32_t)t.jt.size();
         for (auto& cc : ent[e]) {
@@ -410,8 +427,10 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   // reactions at once where they fit it (or 24 KB)
   const int room = std::max(NN, 3072);
   const JacHost jw = jac_table(JAC_PER_RXN * R + (R - first_typed) <= room ? std::max(R, 1)
-                                                                            : shares(room / (JAC_PER_RXN + 1)));
-  const JacHost jn = jac_table(shares(n1 <= 64 ? 64 : 60));
+                                                                            : shares(room / (JAC_PER_RXN + 1)),
+                               n1);
+  const JacHost jn = jac_table(shares(n1 <= 64 ? 64 : 60), n1 | 1);  // in the LU's matrix
+
   // species ordered by the length of their CSR rows (longest first), so
   // that the lanes of one warp gather similar counts in the RHS
   std::vector<int16_t> rsp(S);
@@ -449,6 +468,8 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     csr[e].pad = 0;
   }
   const size_t off_csr = place(sizeof(CsrTerm) * csr.size());
+  const size_t off_slot_ptr = place(sizeof(int32_t) * slot_ptr.size());
+  const size_t off_slot = place(sizeof(CsrTerm) * slot.size());
   const size_t off_csr_cptr = place(sizeof(int32_t) * csr_cptr.size());
   struct JacOff {
     size_t ptr, jc, jt;
@@ -479,6 +500,8 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   put(L.tab, tab.data(), sizeof(double) * 256);
   put(off_csr_ptr, csr_ptr.data(), sizeof(int32_t) * (S + 1));
   put(off_csr, csr.data(), sizeof(CsrTerm) * csr.size());
+  put(off_slot_ptr, slot_ptr.data(), sizeof(int32_t) * slot_ptr.size());
+  put(off_slot, slot.data(), sizeof(CsrTerm) * slot.size());
   put(off_csr_cptr, csr_cptr.data(), sizeof(int32_t) * csr_cptr.size());
   auto put_jac = [&](const JacOff& o, const JacHost& t) {
     put(o.ptr, t.jc_ptr.data(), sizeof(int32_t) * t.jc_ptr.size());
@@ -531,12 +554,14 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   dm.tab = reinterpret_cast<const double*>(b + L.tab);
   dm.csr_ptr = reinterpret_cast<const int32_t*>(b + off_csr_ptr);
   dm.csr = reinterpret_cast<const CsrTerm*>(b + off_csr);
+  dm.slot_ptr = reinterpret_cast<const int32_t*>(b + off_slot_ptr);
+  dm.slot = reinterpret_cast<const CsrTerm*>(b + off_slot);
   dm.rhs_chunk = rhs_chunk;
   dm.n_rhs_chunks = n_rhs_chunks;
   dm.first_typed = first_typed;
   dm.csr_cptr = reinterpret_cast<const int32_t*>(b + off_csr_cptr);
   auto view_jac = [&](const JacOff& o, const JacHost& t) {
-    return JacTab{t.chunk, t.n_chunks, t.scratch, reinterpret_cast<const int32_t*>(b + o.ptr),
+    return JacTab{t.chunk, t.n_chunks, t.scratch, t.ld, reinterpret_cast<const int32_t*>(b + o.ptr),
                   reinterpret_cast<const JcEntry*>(b + o.jc), reinterpret_cast<const JcTerm*>(b + o.jt)};
   };
   dm.wide = view_jac(ow, jw);
@@ -766,7 +791,7 @@ int integrate(int method, const ck_mech* m, int64_t n, const double* p, double* 
     else if (rkf45_team(m->hm, o.form, n))
       e = ck::launch_rkf45_team(m->hm, n, dp, dy, ddt, dh, sp, ds, dst, queue, st, cfg);
     else
-      e = ck::launch_rkf45(m->hm, n, dp, dy, ddt, dh, sp, ds, dst, queue, st, cfg);
+      e = ck::launch_rkf45(m->hm, n, dp, dy, ddt, dh, sp, ds, dst, queue, st, cfg, true);
     cudaFreeAsync(queue, st);
   }
   if (host) {

@@ -81,12 +81,12 @@ static_assert(sizeof(CsrTerm) == 16 && sizeof(JcEntry) == 16 && sizeof(JcTerm) =
 // One way of assembling the Jacobian: the reactions in chunks of `chunk`
 // (scratch doubles of per-reaction values), and per chunk c the targets
 // jc[e], e in [jc_ptr[c], jc_ptr[c+1]) (flat index idx: the species-block
-// entry J[idx] below n^2, else the per-species sums wd, aT, E, u at idx -
-// n^2), which add the sum over t in [jc[e].beg, jc[e].end) of jt[t].coef *
+// entry J[idx], rows ld apart, below n ld, else the per-species sums wd, aT,
+// E, u at idx - n ld), which add the sum over t in [jc[e].beg, jc[e].end) of jt[t].coef *
 // src[jt[t].pidx] (src: the chunk's per-reaction values).  Chunk 0 lists
 // every target, those without a term too.
 struct JacTab {
-  int chunk, n_chunks, scratch;
+  int chunk, n_chunks, scratch, ld;
   const int32_t* jc_ptr;
   const JcEntry* jc;
   const JcTerm* jt;
@@ -110,6 +110,8 @@ struct DevMech {
   const double* eff_m1;   // [n_eff] efficiency - 1
   const int32_t* csr_ptr; // [S+1] species -> (reaction, net nu) lists
   const CsrTerm* csr;     // [csr_nnz]
+  const int32_t* slot_ptr;  // [S+1] species -> its reaction slots one by one, -1 a reactant, +1 a product,
+  const CsrTerm* slot;      // in the order in which rhs_thread adds them
   const double* tab;      // [256] 2^(j/256)
   const double* revp;     // [n_rev][3] explicit reverse: log2 A_r, beta_r, Ea_r / (R ln 2)
   // A right-hand side whose team has no room for all R rates takes the
@@ -301,6 +303,14 @@ constexpr double RK_D1 = 16.0 / 135.0 - 25.0 / 216.0, RK_D3 = 6656.0 / 12825.0 -
 // Per-CTA global scratch of the ROS4 kernel, in doubles: -J of the current
 // state (n x n) and its diagonal (n).
 __host__ __device__ constexpr size_t ros4_scratch_doubles(int n) { return (size_t)n * n + (size_t)n; }
+
+// A reactor that the thread-per-reactor RKF45 hands to a team after
+// RK_THREAD_STEPS attempts (its state is in the caller's y).
+struct RkCont {
+  double t, h;
+  int32_t r, acc, rej;
+  int16_t last_rej, last_nf;
+};
 
 struct SolverParams {
   double rtol, atol, h0, fixed_h;

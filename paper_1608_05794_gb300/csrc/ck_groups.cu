@@ -72,7 +72,7 @@ cudaError_t launch_group(int method, const ck_group& g, int32_t* queue, cudaStre
                            true);
   const bool team = o.form == 2 || (o.form == 0 && (hm.S > 32 || g.n < (int64_t)4 * 128 * ck::sm_count()));
   if (team) return ck::launch_rkf45_team(hm, g.n, g.p, g.y, g.dt, g.h_inout, sp, g.steps, g.status, queue, st, cfg);
-  return ck::launch_rkf45(hm, g.n, g.p, g.y, g.dt, g.h_inout, sp, g.steps, g.status, queue, st, cfg);
+  return ck::launch_rkf45(hm, g.n, g.p, g.y, g.dt, g.h_inout, sp, g.steps, g.status, queue, st, cfg, true);
 }
 
 // Record the fork / kernels / join sequence on `st` (captured or not), in

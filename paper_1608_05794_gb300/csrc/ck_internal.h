@@ -73,9 +73,15 @@ CK_ROS4_TILE_LAUNCHER(launch_ros4_w2)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w4)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w8)
 #undef CK_ROS4_TILE_LAUNCHER
+// may_alloc: hand reactors of many steps from their threads to teams through
+// a stream-ordered list (mechanisms of at most 32 species); same results.
 cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                          double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,
-                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg);
+                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, bool may_alloc);
+// The teams' part: reactors list[0 .. min(*count, cap)); queue: a zeroed counter.
+cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
+                              const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
+                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st);
 
 cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, double* y,
                               const double* dt, double* h_io, const SolverParams& sp, int32_t* steps,

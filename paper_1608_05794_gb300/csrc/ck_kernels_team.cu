@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(P, MINB) k_jacobian(const __grid_constant__ De
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) ys[i] = y[r * n + i];
     team_sync();
-    team_jacobian<(P > 64)>(d, d.wide, d.tab, p[r], ys, fs, jac + r * (int64_t)n * n, nullptr,
+    team_jacobian<(P > 64)>(d, d.wide, d.tab, p[r], ys, fs, jac + r * (int64_t)n * n, nullptr, 0,
                   carve_bufs(fs + n, d.S, sm, d.wide.chunk, 256));
   }
 }
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ Dev
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[ys + i] = y[r * n + i];
     team_sync();
-    team_jacobian_fd<false>(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, ys + 2 * n, ys + 3 * n, ys + 4 * n,
+    team_jacobian_fd<false>(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, n, ys + 2 * n, ys + 3 * n, ys + 4 * n,
                      n > 64 ? 256 : 64, qq);
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = sm[e];
     team_sync();
@@ -66,29 +66,45 @@ __global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ Dev
 }
 
 // ------------------------------------------------------------------ batched LU
+// A dim x dim matrix into shared memory, rows ld apart, eight loads a thread
+// in flight.
+static __device__ __forceinline__ void load_matrix(double* A, int ld, const double* __restrict__ src, int dim, float rc) {
+  const int nn = dim * dim, P = blockDim.x;
+  for (int e0 = threadIdx.x; e0 < nn; e0 += 8 * P) {
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = e0 + u * P < nn ? src[e0 + u * P] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = e0 + u * P;
+      if (e < nn) A[e + flat_row(e, rc) * (ld - dim)] = v[u];
+    }
+  }
+}
+
 // Shared memory, in doubles: the matrix, 1 / U_kk, the row tables and pivots.
 static __host__ __device__ __forceinline__ size_t lu_doubles(int dim) {
-  return (((size_t)dim * dim + 1) & ~(size_t)1) + 4 * (size_t)dim + 2 * (size_t)dim;
+  return (((size_t)dim * lu_ld(dim) + 1) & ~(size_t)1) + 4 * (size_t)dim + 2 * (size_t)dim;
 }
 __global__ void __launch_bounds__(256) k_lu_factor(int64_t batch, int dim, double* __restrict__ a,
                                                    int32_t* __restrict__ piv, int32_t* __restrict__ info) {
   extern __shared__ __align__(16) double sm[];
   __shared__ int flag;
-  const int nn = dim * dim;
+  const int nn = dim * dim, ld = lu_ld(dim), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   double* A = sm;
-  LuRow<double>* lr = reinterpret_cast<LuRow<double>*>(A + ((nn + 1) & ~1));
+  LuRow<double>* lr = reinterpret_cast<LuRow<double>*>(A + ((dim * lu_ld(dim) + 1) & ~1));
   double* invd = reinterpret_cast<double*>(lr + 2 * dim);
   int* rof = reinterpret_cast<int*>(invd + dim);
   int* pv = rof + dim;
   const float rc = 1.0f / (float)dim;
   for (int64_t m = blockIdx.x; m < batch; m += gridDim.x) {
     double* am = a + m * nn;
-    for (int e = threadIdx.x; e < nn; e += blockDim.x) A[e] = am[e];
+    load_matrix(A, ld, am, dim, rc);
     team_sync();
     const int inf = lu_flat<false>(A, dim, rof, pv, invd, lr, &flag);
-    for (int e = threadIdx.x; e < nn; e += blockDim.x) {
-      const int i = flat_row(e, rc);
-      am[e] = A[(rof[i] >> 8) + (e - i * dim)];
+    for (int i = warp; i < dim; i += nw) {
+      const double* row = A + (rof[i] >> 8);
+      for (int j = lane; j < dim; j += 32) am[i * dim + j] = row[j];
     }
     for (int i = threadIdx.x; i < dim; i += blockDim.x) piv[m * dim + i] = pv[i];
     if (threadIdx.x == 0) info[m] = inf;
@@ -99,24 +115,25 @@ __global__ void __launch_bounds__(256) k_lu_factor(int64_t batch, int dim, doubl
 __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu,
                            const int32_t* __restrict__ piv, double* __restrict__ bvec) {
   extern __shared__ __align__(16) double sm[];
+  const int nn = dim * dim, ld = lu_ld(dim);
   double* A = sm;
-  double* invd = A + (size_t)dim * dim;
+  double* invd = A + dim * ld;
   int* pv = reinterpret_cast<int*>(invd + dim);
   double* x = invd + 2 * dim;
-  const int64_t nn = (int64_t)dim * dim;
+  const float rc = 1.0f / (float)dim;
   for (int64_t m = blockIdx.x; m < batch; m += gridDim.x) {
-    for (int64_t e = threadIdx.x; e < nn; e += blockDim.x) A[e] = lu[m * nn + e];
+    load_matrix(A, ld, lu + m * nn, dim, rc);
     for (int i = threadIdx.x; i < dim; i += blockDim.x) {
       pv[i] = piv[m * dim + i];
       x[i] = bvec[m * dim + i];
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < dim; i += blockDim.x) invd[i] = rcp_rn(A[(size_t)i * dim + i]);
-    __syncthreads();
+    team_sync();
+    for (int i = threadIdx.x; i < dim; i += blockDim.x) invd[i] = rcp_rn(A[i * ld + i]);
+    team_sync();
     if (threadIdx.x < 32) warp_lu_solve(A, dim, pv, invd, x);
-    __syncthreads();
+    team_sync();
     for (int i = threadIdx.x; i < dim; i += blockDim.x) bvec[m * dim + i] = x[i];
-    __syncthreads();
+    team_sync();
   }
 }
 
@@ -125,11 +142,16 @@ __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu
 // right-hand sides are evaluated by the team, so a reactor's working set
 // (8 n-vectors and one chunk of reaction scratch) stays in shared memory and
 // the number of steps of one reactor never holds back another.
-template <bool INT>
-__global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N, const double* __restrict__ p,
-                                                   double* __restrict__ y, const double* __restrict__ dt,
-                                                   double* h_io, SolverParams sp, int32_t* steps,
-                                                   int32_t* status, int32_t* queue) {
+//
+// TAIL: reactors that the thread-per-reactor kernel handed on (the entries of
+// list, *count of them but cap at most), taken up where it left them; every sum
+// is then in that kernel's order, so that its results do not depend on where
+// a reactor is finished.
+template <bool INT, bool TAIL>
+static __device__ __forceinline__ void rkf45_team(const DevMech& d, int64_t N, const double* __restrict__ p,
+                                                  double* __restrict__ y, const double* __restrict__ dt,
+                                                  double* h_io, const SolverParams& sp, int32_t* steps,
+                                                  int32_t* status, int32_t* queue, const RkCont* list) {
   extern __shared__ __align__(16) double sm[];
   __shared__ int slot;
   const int n = d.n;
@@ -149,66 +171,72 @@ __global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ D
   double* k4 = kk + 4 * n;
   double* k5 = kk + 5 * n;
   for (;;) {
-    const int r = team_next(queue, &slot);
+    int r = team_next(queue, &slot);
     if (r >= N) break;
+    RkCont from{};
+    if (TAIL) {
+      from = list[r];
+      r = from.r;
+    }
     for (int i = tid; i < n; i += P) yv[i] = y[(int64_t)r * n + i];
     const double pr = p[r];
     const double tf = dt[r];
-    __syncthreads();
+    team_sync();
     int bad = 0;
     for (int i = tid; i < n; i += P) bad |= !isfinite(yv[i]);
     bad = __syncthreads_or(bad);
     bad |= !(pr > 0.0) || !isfinite(pr) || !(yv[0] > 0.0) || !isfinite(tf) || !(tf >= 0.0);
-    int st = ST_OK, acc = 0, rej = 0;
+    int st = ST_OK, acc = from.acc, rej = from.rej;
     double h = 0.0;
-    if (bad) {
+    if (!TAIL && bad) {
       st = ST_BADINPUT;
     } else if (tf > 0.0) {
-      if (fixed) h = sp.fixed_h;
+      if (TAIL) h = from.h;
+      else if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
       else h = team_h0<INT>(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
       const double hmin = 1e-15 * tf;
-      double t = 0.0;
-      bool last_rej = false, last_nf = false;
+      double t = from.t;
+      bool last_rej = from.last_rej != 0, last_nf = from.last_nf != 0;
       while (t < tf) {
         if (acc + rej >= sp.max_steps) { st = ST_MAXSTEPS; break; }
         const bool clamped = h >= tf - t;
         const double hh = clamped ? tf - t : h;
         if (hh < hmin) { st = last_nf ? ST_NONFINITE : ST_HMIN; break; }
         // k_s = hh f(y + sum_j a_sj k_j)
-        team_rhs<INT>(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k0[i] *= hh;
           yt[i] = fma(RK_A21, k0[i], yv[i]);
         }
         team_sync();
-        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k1[i] *= hh;
           yt[i] = fma(RK_A32, k1[i], fma(RK_A31, k0[i], yv[i]));
         }
         team_sync();
-        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k2[i] *= hh;
           yt[i] = fma(RK_A43, k2[i], fma(RK_A42, k1[i], fma(RK_A41, k0[i], yv[i])));
         }
         team_sync();
-        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k3[i] *= hh;
           yt[i] = fma(RK_A54, k3[i], fma(RK_A53, k2[i], fma(RK_A52, k1[i], fma(RK_A51, k0[i], yv[i]))));
         }
         team_sync();
-        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k4[i] *= hh;
           yt[i] = fma(RK_A65, k4[i],
                       fma(RK_A64, k3[i], fma(RK_A63, k2[i], fma(RK_A62, k1[i], fma(RK_A61, k0[i], yv[i])))));
         }
         team_sync();
-        team_rhs<INT>(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
+        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k1, whose weights are 0)
         int nf = 0;
         for (int i = tid; i < n; i += P) {
@@ -227,7 +255,7 @@ __global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ D
           ++acc;
           continue;
         }
-        const double e = team_wrms(n, k1, yv, yt, sp.rtol, sp.atol, red, vp);
+        const double e = team_wrms<TAIL>(n, k1, yv, yt, sp.rtol, sp.atol, red, vp);
         if (nf || !isfinite(e)) {
           ++rej;
           h = FAC_MIN * hh;
@@ -265,6 +293,24 @@ __global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ D
     }
     __syncthreads();
   }
+}
+
+template <bool INT>
+__global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N,
+                                                       const double* __restrict__ p, double* __restrict__ y,
+                                                       const double* __restrict__ dt, double* h_io, SolverParams sp,
+                                                       int32_t* steps, int32_t* status, int32_t* queue) {
+  rkf45_team<INT, false>(d, N, p, y, dt, h_io, sp, steps, status, queue, nullptr);
+}
+
+__global__ void __launch_bounds__(128, 8) k_rkf45_tail(const __grid_constant__ DevMech d,
+                                                       const double* __restrict__ p, double* __restrict__ y,
+                                                       const double* __restrict__ dt, double* h_io, SolverParams sp,
+                                                       int32_t* steps, int32_t* status, int32_t* queue,
+                                                       const RkCont* __restrict__ list,
+                                                       const int32_t* __restrict__ count, int cap) {
+  const int n = *count < cap ? *count : cap;
+  rkf45_team<false, true>(d, n, p, y, dt, h_io, sp, steps, status, queue, list);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -321,9 +367,9 @@ cudaError_t launch_lu_factor(int64_t batch, int dim, double* a, int32_t* piv, in
 cudaError_t launch_lu_solve(int64_t batch, int dim, const double* lu, const int32_t* piv,
                             double* b, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  const size_t smem = sizeof(double) * ((size_t)dim * dim + 3 * dim);
+  const size_t smem = sizeof(double) * ((size_t)dim * lu_ld(dim) + 3 * dim);
   LaunchCfg cfg;
-  const int threads = dim <= 24 ? 32 : (dim <= 64 ? 64 : 128);
+  const int threads = dim <= 24 ? 32 : 128;  // one warp solves, all load
   const int grid = team_grid(k_lu_solve, threads, smem, batch, cfg);
   k_lu_solve<<<grid, threads, smem, st>>>(batch, dim, lu, piv, b);
   return cudaGetLastError();
@@ -370,6 +416,17 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
   kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
+                              const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
+                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st) {
+  const size_t smem = sizeof(double) * (8 * (size_t)hm.d.n + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const int threads = 64;
+  LaunchCfg cfg;
+  const int grid = team_grid(k_rkf45_tail, threads, smem, cap, cfg);
+  k_rkf45_tail<<<grid, threads, smem, st>>>(hm.d, p, y, dt, h_io, sp, steps, status, queue, list, count, cap);
   return cudaGetLastError();
 }
 

@@ -146,16 +146,27 @@ __device__ double h0_thread(const MechView& m, int n, double p, const double* y0
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
 
+// Attempts after which a thread hands its reactor on, and how many reactors
+// may be.  Longer keeps more of the work where the lanes are full, but a warp
+// then runs on for its slowest lanes.  10 species over 1e-5 s (70 attempts a
+// reactor on average, 1900 at most), 100003 / 300000 reactors: 96 attempts 389
+// / 1051 ms, 128 372 / 906, 192 411 / 808, 320 536 / 889, never 670 / -.
+constexpr int RK_THREAD_STEPS = 160;
+constexpr int64_t RK_LIST_MAX = 1 << 18;
+
 // One lane integrates one reactor at a time and fetches the next reactor
 // from a global atomic counter as soon as it finishes (dynamic scheduling
 // with granularity one, per lane), so lanes of a warp never wait for a
-// slower neighbour beyond one step.
+// slower neighbour beyond one step.  With a list, a reactor that is not done
+// after RK_THREAD_STEPS attempts is handed on (k_rkf45_tail): a step takes a
+// thread 410 us however few are left, a team 50.
 template <int MAXS>
 __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int staged, int64_t N,
                                                const double* __restrict__ p, double* __restrict__ y,
                                                const double* __restrict__ dt, double* h_io,
                                                SolverParams sp, int32_t* steps, int32_t* status,
-                                               int32_t* queue, int32_t* err) {
+                                               int32_t* queue, RkCont* list, int32_t* count, int cap,
+                                               int32_t* err) {
   extern __shared__ __align__(16) unsigned char smem[];
   const unsigned char* base = reinterpret_cast<const unsigned char*>(d.rxn);
   if (staged) {
@@ -274,6 +285,14 @@ __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int sta
           }
         }
         if (t >= tf) finish = true;
+        if (!finish && list && acc + rej >= RK_THREAD_STEPS) {
+          const int at = *count < cap ? atomicAdd(count, 1) : cap;
+          if (at < cap) {
+            for (int i = 0; i < n; ++i) y[r * n + i] = yv[i];
+            list[at] = RkCont{t, h, (int32_t)r, acc, rej, (int16_t)last_rej, (int16_t)last_nf};
+            r = -1;
+          }
+        }
       }
     }
     if (finish) {
@@ -375,7 +394,7 @@ template <int MAXS>
 static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, double* y,
                               const double* dt, double* h_io, const SolverParams& sp,
                               int32_t* steps, int32_t* status, int32_t* queue, cudaStream_t st,
-                              const LaunchCfg& cfg) {
+                              const LaunchCfg& cfg, bool may_alloc) {
   auto kern = k_rkf45<MAXS>;
   const int threads = 128;
   size_t smem = 0;
@@ -387,17 +406,36 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   if (blocks < 1) blocks = 1;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, threads, smem, st>>>(hm.d, hm.L, staged, n, p, y, dt, h_io, sp, steps, status,
-                                      queue, hm.dev_err);
-  return cudaGetLastError();
+  // the list of reactors handed on, behind its two counters (8 MB at most)
+  RkCont* list = nullptr;
+  int32_t* count = nullptr;
+  const int list_cap = (int)(n < RK_LIST_MAX ? n : RK_LIST_MAX);
+  if (MAXS <= 32 && may_alloc && hm.R <= hm.d.rhs_chunk && n <= INT32_MAX) {
+    e = cudaMallocAsync(reinterpret_cast<void**>(&count), 16 + sizeof(RkCont) * (size_t)list_cap, st);
+    if (e != cudaSuccess) return e;
+    list = reinterpret_cast<RkCont*>(count + 4);
+    e = cudaMemsetAsync(count, 0, 16, st);
+  }
+  if (e == cudaSuccess) {
+    kern<<<blocks, threads, smem, st>>>(hm.d, hm.L, staged, n, p, y, dt, h_io, sp, steps, status,
+                                        queue, list, count, list_cap, hm.dev_err);
+    e = cudaGetLastError();
+  }
+  if (list) {
+    if (e == cudaSuccess)
+      e = launch_rkf45_tail(hm, p, y, dt, h_io, sp, steps, status, count + 1, list, count, list_cap, st);
+    const cudaError_t f = cudaFreeAsync(count, st);
+    if (e == cudaSuccess) e = f;
+  }
+  return e;
 }
 
 cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                          double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,
-                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg) {
+                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, bool may_alloc) {
   if (n <= 0) return cudaSuccess;
-  if (hm.S <= 32) return rkf45_impl<32>(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg);
-  return rkf45_impl<128>(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg);
+  if (hm.S <= 32) return rkf45_impl<32>(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg, may_alloc);
+  return rkf45_impl<128>(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg, false);
 }
 
 }  // namespace ck

@@ -106,7 +106,9 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
   using F = typename std::conditional<PREC == 0, double, float>::type;  // type of the factors
   const int n = d.n, nn = n * n;
   const double* tab = d.tab;  // 2 KB, stays in L1
-  const Ros4Layout L(d, m64g != nullptr, nn);
+  const int ld = lu_ld(n);
+  const float rc = 1.0f / (float)n;
+  const Ros4Layout L(d, m64g != nullptr);
   double* M = sm;
   double* yv = sm + L.yv;
   double* F0 = sm + L.f0;
@@ -177,12 +179,12 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
         // same y); A = J - I/(hh gamma) = -M; LU of A
         if (!have_j) {
           if (sp.jac == 1) {
-            team_jacobian_fd<INT>(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, L.yt, L.ub, L.bufs, L.vp,
+            team_jacobian_fd<INT>(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, PREC ? n : ld, L.yt, L.ub, L.bufs, L.vp,
                              L.rhs_q, have_f);
           } else {
             // assembled in the copy Mg where there is one
             const JacTab& jt = Mg ? d.wide : d.narrow;
-            team_jacobian<INT>(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr,
+            team_jacobian<INT>(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr, ld,
                           carve_bufs(sm + L.bufs, d.S, sm + L.jscr, jt.chunk, L.vp));
           }
           if (PREC) {
@@ -192,15 +194,15 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           have_j = keep_j;
           have_f = true;
         } else if (PREC == 0) {
-          for (int e = tid; e < nn; e += P) M[e] = Mg[e];
+          for (int e = tid; e < nn; e += P) M[e + flat_row(e, rc) * (ld - n)] = Mg[e];
           team_sync();
         }
         if (PREC == 0) {
-          if (own) M[(size_t)tid * n + tid] -= ctl.dg;
+          if (own) M[tid * ld + tid] -= ctl.dg;
         } else {
           if (own) Mg[(size_t)tid * n + tid] = Mg[nn + tid] - ctl.dg;
           __syncthreads();
-          for (int e = tid; e < nn; e += P) MF[e] = (F)Mg[e];
+          for (int e = tid; e < nn; e += P) MF[e + flat_row(e, rc) * (ld - n)] = (F)Mg[e];
         }
         team_sync();
         const int info = team_lu<F>(0, n, L.rof, L.invd, L.lr, L.bufs + TEAM_RED_DOUBLES - 1);
@@ -345,7 +347,7 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
   const int nn = hm.d.n;
   auto kern = cfg.precision == 2 ? k_ros4<P, MINB, 2>
                                  : (cfg.precision == 1 ? k_ros4<P, MINB, 1> : k_ros4<P, MINB, 0>);
-  size_t smem = sizeof(double) * Ros4Layout(hm.d, true, nn * nn).doubles;
+  size_t smem = sizeof(double) * Ros4Layout(hm.d, true).doubles;
   int grid = team_grid(kern, P, smem, n, cfg);
   // per-CTA copies of J (every form) and the FP64 iteration matrices of
   // the precision form: the caller's scratch when it is large enough, else
@@ -363,7 +365,7 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
   } else if (cfg.precision) {
     return cudaErrorNotSupported;
   } else {
-    smem = sizeof(double) * Ros4Layout(hm.d, false, nn * nn).doubles;
+    smem = sizeof(double) * Ros4Layout(hm.d, false).doubles;
     grid = team_grid(kern, P, smem, n, cfg);
   }
   kern<<<grid, P, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);

@@ -198,7 +198,7 @@ void launch_chunk(ck_server* s, Slot& sl, Request* r) {
       e = ck::launch_ros4(hm, cnt, pp, yy, tt, nullptr, sp, ss, st, sl.queue, sl.stream, cfg, sl.scratch,
                           sl.scratch_bytes, false);
     else if (r->opts.form == 1)
-      e = ck::launch_rkf45(hm, cnt, pp, yy, tt, nullptr, sp, ss, st, sl.queue, sl.stream, cfg);
+      e = ck::launch_rkf45(hm, cnt, pp, yy, tt, nullptr, sp, ss, st, sl.queue, sl.stream, cfg, false);
     else
       e = ck::launch_rkf45_team(hm, cnt, pp, yy, tt, nullptr, sp, ss, st, sl.queue, sl.stream, cfg);
   }

@@ -158,6 +158,9 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // Ends with a barrier and returns (the same in every thread) whether the
 // ranges allow the reactions' products to be taken in integer arithmetic
 // (mul_int).
+// ORD: the species sums one species after another, as a thread that evaluates
+// a reactor alone takes them (rhs_thread), instead of by trees.
+template <bool ORD>
 __device__ __forceinline__ bool team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
   const int S = m.S, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -199,7 +202,12 @@ __device__ __forceinline__ bool team_species(const DevMech& m, double p, const d
         else part[q] = yw[q];
       }
     }
-    const double sumYW = warp_sum_groups(part, ng);
+    double sumYW = 0.0;
+    if (ORD) {
+      for (int k = 0; k < S; ++k) sumYW = fma(y[1 + k], m.invW[k], sumYW);
+    } else {
+      sumYW = warp_sum_groups(part, ng);
+    }
     const double Wbar = rcp_rn(sumYW);
     const double rho = m.cv ? p : p / (R_GAS * T * sumYW);  // constant volume: p is the density
     const double invrho = rcp_rn(rho);
@@ -217,7 +225,13 @@ __device__ __forceinline__ bool team_species(const DevMech& m, double p, const d
         if (q >= 2 && fold) part[q - 2] += xk;
         else part[q] = xk;
       }
-    const double Ctot = warp_sum_groups(part, ng);
+    double Ctot = 0.0;
+    if (ORD) {
+      __syncwarp();
+      for (int k = 0; k < S; ++k) Ctot += b.X[k];
+    } else {
+      Ctot = warp_sum_groups(part, ng);
+    }
     if (lane == 0) {
       red[SC_WBAR] = Wbar;
       red[SC_RHO] = rho;
@@ -277,7 +291,8 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 // same instructions.  INT: the products of concentrations and of Gibbs factors
 // in integer arithmetic, beside the FP64 unit, which bounds the team kernels
 // (10 of the 23 FP64 instructions of a rate, 20 of 49 with its derivatives).
-template <bool JAC, bool INT>
+// ORD: the fall-off factor by a division, as rhs_thread forms it.
+template <bool JAC, bool INT, bool ORD = false>
 __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
                                               const TeamBufs& b, const double* tab, int i, int iw) {
   const RxnRec r = load_rxn(src);
@@ -335,6 +350,10 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
       const double l2k0 = fma(-f1.x, x.invT, fma(f0.y, x.log2T, f0.x));
       const double k0_kf = ck_exp2(l2k0 - l2kf, tab);
       const double Pr = k0_kf * M;
+      if (ORD) {
+        b.q[i] = net * (Pr / (1.0 + Pr));
+        return;
+      }
       const double inv1p = rcp_rn(1.0 + Pr);
       c = Pr * inv1p;
       dcdM = k0_kf * inv1p * inv1p;
@@ -405,7 +424,9 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
 // operations (a product is 106 cycles of it in integers, 72 in FP64: ROS4 on
 // 512 reactors of the 10-species mechanism, 245 against 230 ms) or is short of
 // registers (ROS4 on 4096 of the 53-species one, 617 against 600 ms).
-template <bool INT>
+// ORD: every sum in the order of rhs_thread, whose values it then returns bit
+// for bit (one pass over all reactions: qq.chunk >= m.R).
+template <bool INT, bool ORD = false>
 static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
   extern __shared__ __align__(16) double sm[];
@@ -415,7 +436,7 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   Mix x;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int S = m.S, SG = species_groups(S);
-  const bool in = team_species(m, p, y, b, x, tab);
+  const bool in = team_species<ORD>(m, p, y, b, x, tab);
   const double invrho = x.invrho;
   // every chunk: its rates of progress, then one fixed-order gather per
   // species, longest rows first so that the lanes of a warp do similar work
@@ -430,15 +451,17 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
         team_reaction<false, INT>(m, m.rxn + base + li, x, b, tab, li, 0);
     } else {
       for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
-        team_reaction<false, false>(m, m.rxn + base + li, x, b, tab, li, 0);
+        team_reaction<false, false, ORD>(m, m.rxn + base + li, x, b, tab, li, 0);
     }
     team_sync();
     const bool last = base + cnt >= m.R;
     for (int kk = tid; kk < S; kk += blockDim.x) {
       const int k = m.rsp[kk];
-      int e = m.csr_ptr[k], e1 = m.csr_ptr[k + 1];
+      const int32_t* ptr = ORD ? m.slot_ptr : m.csr_ptr;
+      const CsrTerm* terms = ORD ? m.slot : m.csr;
+      int e = ptr[k], e1 = ptr[k + 1];
       double w = 0.0;
-      if (CH < m.R) {
+      if (!ORD && CH < m.R) {
         const int c = base / CH;
         const int* cp = m.csr_cptr + k * (m.n_rhs_chunks + 1) + c;
         e = cp[0];
@@ -446,7 +469,7 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
         if (c) w = b.wd[k];
       }
       for (; e < e1; ++e) {
-        const CsrTerm t = m.csr[e];
+        const CsrTerm t = terms[e];
         w = fma(t.nu, b.q[t.rx - base], w);
       }
       b.wd[k] = w;
@@ -483,7 +506,22 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
         }
       }
     double sc, sh;
-    if (ng <= 2) {
+    if (ORD) {
+      // lane 0 the heat capacity, lane 1 the enthalpy, both from one chain
+      // (the factors side by side in the Gibbs arrays, free by now)
+      for (int k = lane; k < S; k += 32) {
+        b.Gp[k] = y[1 + k] * m.invW[k];
+        b.Gm[k] = m.cv ? b.cpR[k] - 1.0 : b.cpR[k];
+        if (m.cv) b.hRT[k] -= 1.0;
+      }
+      __syncwarp();
+      const double* a0 = lane & 1 ? b.hRT : b.Gp;
+      const double* a1 = lane & 1 ? b.wd : b.Gm;
+      double s = 0.0;
+      for (int k = 0; k < S; ++k) s = fma(a0[k], a1[k], s);
+      sc = __shfl_sync(0xffffffffu, s, 0);
+      sh = __shfl_sync(0xffffffffu, s, 1);
+    } else if (ng <= 2) {
       const double v = warp_sum_pack4(cpm[0], cpm[1], hw[0], hw[1]);
       // lanes 0-15: cpm, 16-31: hw, both from one add
       const double s = v + __shfl_xor_sync(0xffffffffu, v, 8);
@@ -498,8 +536,9 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   team_sync();
 }
 
-// Analytic Jacobian J = df/d(T, Y) at constant p, written row-major (n x n)
-// into A, and into M too unless that is NULL, and f(y) into f.  Derivation
+// Analytic Jacobian J = df/d(T, Y) at constant p, written row-major into A
+// (rows jt.ld apart), and into M too (rows ldm apart) unless that is NULL, and
+// f(y) into f.  Derivation
 // (chain rule through rho(T, Y) and [X](rho, Y); dlnK_c/dT = (sum nu H/RT -
 // dnu)/T):
 //   A_kj   = sum_i nu_ki dq_i/d[X_j] (sparse mass-action part and the
@@ -523,11 +562,11 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 // Needs b.vp >= S (one species a lane in the sums).
 template <bool INT>
 static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const double* tab, double p, const double* y,
-                                     double* f, double* A, double* M, TeamBufs b) {
+                                     double* f, double* A, double* M, int ldm, TeamBufs b) {
   Mix x;
-  const int S = m.S, n = m.n, SG = species_groups(S);
+  const int S = m.S, lda = jt.ld, na = m.n * lda, SG = species_groups(S);
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const bool in = team_species(m, p, y, b, x, tab);
+  const bool in = team_species<false>(m, p, y, b, x, tab);
   // chunk by chunk, every target (species-block entries and the per-species
   // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
   // fixed-order sum of terms; one thread per target, no conflicts, the
@@ -546,13 +585,13 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
     for (int e = jt.jc_ptr[c] + tid; e < jt.jc_ptr[c + 1]; e += blockDim.x) {
       const JcEntry h = jt.jc[e];
       double a = 0.0;
-      if (c > 0) a = h.idx < n * n ? A[h.idx] : b.wd[h.idx - n * n];
+      if (c > 0) a = h.idx < na ? A[h.idx] : b.wd[h.idx - na];
       for (int t = h.beg; t < h.end; ++t) {
         const JcTerm ct = jt.jt[t];
         a = fma(ct.coef, b.q[ct.pidx], a);
       }
-      if (h.idx < n * n) A[h.idx] = a;
-      else b.wd[h.idx - n * n] = a;
+      if (h.idx < na) A[h.idx] = a;
+      else b.wd[h.idx - na] = a;
     }
     team_sync();
   }
@@ -611,9 +650,9 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
     const int j = 32 * g + lane;
     if (j < S) {
       double s = 0.0;
-      const double* a = A + n + 1 + j;
+      const double* a = A + lda + 1 + j;
 #pragma unroll 8
-      for (int k = 0; k < S; ++k) s = fma(eW[k], a[k * n], s);
+      for (int k = 0; k < S; ++k) s = fma(eW[k], a[k * lda], s);
       cs[j] = s;
     }
   }
@@ -626,10 +665,10 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
     const int P = blockDim.x, dk = P / S, dj = P - (P / S) * S;
     int k = tid / S, j = tid - k * S;
     for (; k < S;) {
-      const int o = (1 + k) * n + 1 + j;
-      const double v = fma(dense[k], m.invW[j], A[o]);
-      A[o] = v;
-      if (M) M[o] = v;
+      double* a = A + (1 + k) * lda + 1 + j;
+      const double v = fma(dense[k], m.invW[j], *a);
+      *a = v;
+      if (M) M[(1 + k) * ldm + 1 + j] = v;
       k += dk;
       j += dj;
       if (j >= S) {
@@ -641,8 +680,8 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
   // temperature column and row (each product rounded where it is written)
   for (int k = tid; k < S; k += blockDim.x) {
     const double v = m.W[k] * invrho * fma(cpf * b.wd[k], x.invT, b.aT[k]);
-    A[(1 + k) * n] = v;
-    if (M) M[(1 + k) * n] = v;
+    A[(1 + k) * lda] = v;
+    if (M) M[(1 + k) * ldm] = v;
   }
   const double inv_rc = invrho * inv_cpm;
   for (int j = tid; j < S; j += blockDim.x) {
@@ -665,7 +704,7 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
 }
 
 // LU with partial pivoting of the n x n row-major matrix A (shared memory,
-// n <= 144) by the whole team, in place.  An FP64 instruction costs a full
+// n <= 144, rows ld = lu_ld(n) apart) by the whole team, in place.  An FP64 instruction costs a full
 // warp slot of a pipe that takes 64 cycles a slot, while shared memory has
 // bandwidth to spare beside it (an update moves 3 loads and a store per
 // slot), so the trailing matrix stays in shared memory and its elements are
@@ -708,6 +747,12 @@ __device__ __forceinline__ unsigned long long inf_key(double) { return 0x7ff0000
 __device__ __forceinline__ unsigned long long inf_key(float) { return 0x7f80000000000000ULL; }
 
 constexpr int LU_MAX_N = 144;
+
+// Distance of the rows of a factored matrix in shared memory: odd, so that
+// the lanes of a warp reading one column (a row each: the pivot search, the
+// substitutions) touch different banks.  At n = 112 every such load took 32
+// turns.
+__host__ __device__ __forceinline__ constexpr int lu_ld(int n) { return n | 1; }
 
 // Pivot k, by one warp: column k updated with pivot k - 1, the pivot of rows
 // k.., and the multipliers and row order of the rows below it.
@@ -791,7 +836,7 @@ __device__ __forceinline__ void lu_panel(F* A, int n, int k, int* rof, int* lpiv
   }
 }
 
-// Element e of a list of rows of c elements: its row, for e < 2^14, c <= 144
+// Element e of a list of rows of c elements: its row, for e < 2^15, c <= 144
 // (rc = 1 / c in FP32: (e + 1/2) / c is at least 1 / (2 c) away from an
 // integer, far more than its rounding error of 2^-22 e / c).
 __device__ __forceinline__ int flat_row(int e, float rc) { return (int)(((float)e + 0.5f) * rc); }
@@ -831,7 +876,7 @@ template <bool PRE, class F>
 __device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd, LuRow<F>* lr, int* flag) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   for (int i = tid; i < n; i += blockDim.x) {
-    lr[n + i].pk = (i * n) << 8 | i;
+    lr[n + i].pk = (i * lu_ld(n)) << 8 | i;
     if (lpiv) lpiv[i] = i;
   }
   if (tid == 0) *flag = 0;
@@ -933,7 +978,7 @@ __device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd
 // value is broadcast by a shuffle.
 // PRE: the factors come from lu_flat<true> (rows listed in its row table rof,
 // passed as piv: gather by it, U pre-divided by its diagonal); else rows in
-// order and piv[k] the row swapped with row k.
+// order, lu_ld(n) apart, and piv[k] the row swapped with row k.
 template <bool PRE = false, class F>
 __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv, const F* invd, F* b) {
   const int lane = threadIdx.x & 31;
@@ -967,7 +1012,7 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     const int i = B0 + lane;
     const bool act = i < n;
     F s0 = act ? b[i] : F(0), s1 = F(0), s2 = F(0), s3 = F(0);
-    const F* Li = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * n);
+    const F* Li = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * lu_ld(n));
     if (act) {
       int j = 0;
       for (; j + 4 <= B0; j += 4) {
@@ -993,7 +1038,7 @@ __device__ __forceinline__ void warp_lu_solve(const F* A, int n, const int* piv,
     const bool act = i < n;
     const int m = min(32, n - B1);
     F s0 = act ? (PRE ? b[i] * invd[i] : b[i]) : F(0), s1 = F(0), s2 = F(0), s3 = F(0);
-    const F* Ui = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * n);
+    const F* Ui = A + (PRE ? (act ? piv[i] >> 8 : 0) : (act ? i : 0) * lu_ld(n));
     if (act) {
       int j = B1 + 32;
       for (; j + 4 <= n; j += 4) {

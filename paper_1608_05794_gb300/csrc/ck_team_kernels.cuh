@@ -30,7 +30,7 @@ static __device__ __forceinline__ int team_next(int32_t* queue, int* slot) {
 // memory (the last two scratch); bufs_o, vp, qq as in team_rhs.
 template <bool INT>
 static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const double* tab, double p, int y_o, double h,
-                                                     double rtol, double atol, int f0_o, double* J, int yt_o,
+                                                     double rtol, double atol, int f0_o, double* J, int ldj, int yt_o,
                                                      int f_o, int bufs_o, int vp, RhsQ qq, bool have_f0 = false) {
   extern __shared__ __align__(16) double sm[];
   const double* y = sm + y_o;
@@ -55,7 +55,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
     if (tid == 0) Yt[j] = y[j] + sj;
     team_sync();
     team_rhs<INT>(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
-    for (int i = tid; i < n; i += blockDim.x) J[(size_t)i * n + j] = (F[i] - f0[i]) / sj;
+    for (int i = tid; i < n; i += blockDim.x) J[(size_t)i * ldj + j] = (F[i] - f0[i]) / sj;
     if (tid == 0) Yt[j] = y[j];
     team_sync();
   }
@@ -74,8 +74,10 @@ static __device__ __forceinline__ double team_pow(double x, double q, double* re
 
 // Weighted RMS norm over the team (reading shared with the oracle:
 // sqrt(mean (e_i / (atol + rtol max(|y_i|, |ynew_i|)))^2)).  vp: the lanes
-// that the components are dealt to (as the species sums).
-static __device__ __forceinline__ double team_wrms(int n, const double* e, const double* y0, const double* y1,
+// that the components are dealt to (as the species sums).  ORD: the components
+// one after another (the sum by every thread).
+template <bool ORD = false>
+static __device__ __forceinline__ double team_wrms(int n, double* e, const double* y0, const double* y1,
                                                    double rtol, double atol, double* red, int vp) {
   const int tid = threadIdx.x;
   double s = 0.0;
@@ -83,9 +85,16 @@ static __device__ __forceinline__ double team_wrms(int n, const double* e, const
     for (int i = tid; i < n; i += vp) {
       const double sc = atol + rtol * fmax(fabs(y0[i]), fabs(y1[i]));
       const double v = e[i] / sc;
-      s = fma(v, v, s);
+      if (ORD) e[i] = v;
+      else s = fma(v, v, s);
     }
-  s = team_sum(s, red);
+  if (ORD) {
+    team_sync();
+    for (int i = 0; i < n; ++i) s = fma(e[i], e[i], s);
+    team_sync();
+  } else {
+    s = team_sum(s, red);
+  }
   return sqrt(s / n);
 }
 
@@ -127,8 +136,7 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
 
-// Shared memory of one k_ros4 CTA, in doubles: the matrix (mat: n^2 FP64, or
-// FP32 factors), y and f(y), the team's work arrays, and the stage vectors,
+// Shared memory of one k_ros4 CTA, in doubles: the matrix, y and f(y), the team's work arrays, and the stage vectors,
 // the factors' row table and the rates of progress (or the LU's scratch).  The
 // Jacobian's per-reaction values lie over the matrix (wide: it is assembled in
 // device memory) or behind the work arrays, over the stage vectors.
@@ -136,8 +144,8 @@ struct Ros4Layout {
   int vp, yv, f0, bufs, jscr, yt, ub, invd, rof, lr;
   RhsQ rhs_q;
   size_t doubles;
-  __host__ __device__ Ros4Layout(const DevMech& d, bool wide, int mat) {
-    const int n = d.n;
+  __host__ __device__ Ros4Layout(const DevMech& d, bool wide) {
+    const int n = d.n, mat = n * lu_ld(n);
     vp = n > 64 ? 256 : 64;
     yv = wide && d.wide.scratch > mat ? d.wide.scratch : mat;
     f0 = yv + n;

@@ -105,3 +105,39 @@ def test_more_reactions_than_the_scratch(ck, name, times):
     yo = om.integrate(ORA_ROS4, p, y, dt)[0]
     assert np.max(np.abs(ends[0][:, 0] - yo[:, 0]) / yo[:, 0]) <= 1e-6
     assert np.max(np.abs(ends[0][:, 1:] - yo[:, 1:])) <= 1e-8
+
+
+@pytest.mark.parametrize("cv", [0, 1])
+def test_rkf45_threads_hand_reactors_to_teams(ck, cv):
+    # reactors of more than 160 attempts move from their threads to teams,
+    # which take every sum in the threads' order; the server's launches keep
+    # them in threads: the same bits
+    m = load_mechanism(CONFIGS["small"]["mech"])
+    gm = ck.load_mechanism(m, reactor=cv)
+    n = 200
+    y, p = reactor_states("small", n=n, seed_offset=47)
+    if cv:
+        p = np.linspace(0.2, 2.5, n)
+    dt = np.linspace(1e-6, 6e-5, n)
+    opts = ck.SolverOpts.make(form=1)
+    yd, st = _dev(y), torch.empty(n, dtype=torch.int32, device="cuda")
+    steps, h = torch.empty((n, 2), dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.float64, device="cuda")
+    ck.integrate_rkf45(gm, _dev(p), yd, _dev(dt), st, steps=steps, h_inout=h, opts=opts)
+    torch.cuda.synchronize()
+    total = steps.sum(1).cpu().numpy()
+    assert (total > 160).sum() >= 20 and (total < 160).sum() >= 20
+    srv = ck.Server(hbm_budget_bytes=1 << 30, streams=1)
+    ys, ss = y.copy(), np.zeros((n, 2), np.int32)
+    sts = np.zeros(n, np.int32)
+    t = srv.submit(gm, ck.Server.RKF45, np.ascontiguousarray(p), ys, dt, sts, ss, opts)
+    srv.wait(t)
+    srv.release(t)
+    srv.close()
+    assert np.array_equal(yd.cpu().numpy(), ys)
+    assert np.array_equal(steps.cpu().numpy(), ss) and np.array_equal(st.cpu().numpy(), sts)
+    # a step limit inside and beyond the threads' share
+    for limit in (100, 160, 161, 300):
+        o = ck.SolverOpts.make(form=1, max_steps=limit)
+        yl = _dev(y)
+        ck.integrate_rkf45(gm, _dev(p), yl, _dev(dt), st, steps=steps, opts=o)
+        assert np.array_equal(steps.sum(1).cpu().numpy(), np.minimum(total, limit))
