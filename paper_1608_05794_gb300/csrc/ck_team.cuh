@@ -160,7 +160,7 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // (mul_int).
 // ORD: the species sums one species after another, as a thread that evaluates
 // a reactor alone takes them (rhs_thread), instead of by trees.
-template <bool ORD>
+template <bool ORD, bool INT>
 __device__ __forceinline__ bool team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
   const int S = m.S, tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -170,7 +170,7 @@ __device__ __forceinline__ bool team_species(const DevMech& m, double p, const d
   x.T = T;
   bool ok = temp_in_range(T);
   if (warp == nw - 1) {
-    const double invT = rcp_rn(T), lnT = log(T);
+    const double invT = rcp_sel<INT>(T), lnT = log(T);
     const double T2 = T * T, T3 = T2 * T;
     const double up = T * R_OVER_P0, dn = invT * P0_OVER_R;
     if (lane == 0) {
@@ -197,7 +197,7 @@ __device__ __forceinline__ bool team_species(const DevMech& m, double p, const d
       if (q < SG) {
         const int k = 32 * q + lane;
         const double yk = k < S ? y[1 + k] : 0.0, iw = k < S ? m.invW[k] : 0.0;
-        yw[q] = yk * iw;
+        yw[q] = __dmul_rn(yk, iw);  // (rounded: a sum over lanes must not take the product in)
         if (q >= 2 && fold) part[q - 2] = fma(yk, iw, part[q - 2]);
         else part[q] = yw[q];
       }
@@ -208,16 +208,16 @@ __device__ __forceinline__ bool team_species(const DevMech& m, double p, const d
     } else {
       sumYW = warp_sum_groups(part, ng);
     }
-    const double Wbar = rcp_rn(sumYW);
+    const double Wbar = rcp_sel<INT>(sumYW);
     const double rho = m.cv ? p : p / (R_GAS * T * sumYW);  // constant volume: p is the density
-    const double invrho = rcp_rn(rho);
+    const double invrho = rcp_sel<INT>(rho);
 #pragma unroll
     for (int q = 0; q < 4; ++q) part[q] = 0.0;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
       if (q < SG) {
         const int k = 32 * q + lane;
-        const double xk = k < S ? rho * yw[q] : 0.0;
+        const double xk = k < S ? __dmul_rn(rho, yw[q]) : 0.0;
         if (k < S) {
           b.X[k] = xk;
           ok &= conc_in_range(xk);
@@ -349,12 +349,12 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
       const double2 f1 = __ldg(reinterpret_cast<const double2*>(src) + 6);  // E0oR2, E0oR
       const double l2k0 = fma(-f1.x, x.invT, fma(f0.y, x.log2T, f0.x));
       const double k0_kf = ck_exp2(l2k0 - l2kf, tab);
-      const double Pr = k0_kf * M;
+      const double Pr = __dmul_rn(k0_kf, M);
       if (ORD) {
         b.q[i] = net * (Pr / (1.0 + Pr));
         return;
       }
-      const double inv1p = rcp_rn(1.0 + Pr);
+      const double inv1p = rcp_rn(__dadd_rn(1.0, Pr));
       c = Pr * inv1p;
       dcdM = k0_kf * inv1p * inv1p;
       if (JAC) {
@@ -436,7 +436,7 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   Mix x;
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   const int S = m.S, SG = species_groups(S);
-  const bool in = team_species<ORD>(m, p, y, b, x, tab);
+  const bool in = team_species<ORD, INT>(m, p, y, b, x, tab);
   const double invrho = x.invrho;
   // every chunk: its rates of progress, then one fixed-order gather per
   // species, longest rows first so that the lanes of a warp do similar work
@@ -566,7 +566,7 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
   Mix x;
   const int S = m.S, lda = jt.ld, na = m.n * lda, SG = species_groups(S);
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const bool in = team_species<false>(m, p, y, b, x, tab);
+  const bool in = team_species<false, INT>(m, p, y, b, x, tab);
   // chunk by chunk, every target (species-block entries and the per-species
   // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
   // fixed-order sum of terms; one thread per target, no conflicts, the
@@ -813,7 +813,7 @@ __device__ __forceinline__ void lu_panel(F* A, int n, int k, int* rof, int* lpiv
   bpk = __shfl_sync(0xffffffffu, bpk, from);
   const F vk = __shfl_sync(0xffffffffu, v[0], 0);
   const int pkk = __shfl_sync(0xffffffffu, pk[0], 0);
-  const F ip = rcp_rn(bv);
+  const F ip = rcp_int(bv);
   if (lane == 0) {
     rof[k] = bpk;
     A[(bpk >> 8) + k] = bv;
