@@ -71,6 +71,7 @@ size_t ros4_scratch_bytes_max();
                    const LaunchCfg& cfg, double* scratch, size_t scratch_bytes, bool may_alloc);
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w2)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w4)
+CK_ROS4_TILE_LAUNCHER(launch_ros4_w4_lat)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w8)
 #undef CK_ROS4_TILE_LAUNCHER
 // may_alloc: hand reactors of many steps from their threads to teams through

@@ -22,7 +22,7 @@ __global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMec
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = y[r * n + i];
     team_sync();
-    team_rhs<INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
+    team_rhs_any<INT, false, !INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
     for (int i = threadIdx.x; i < n; i += blockDim.x) f[r * n + i] = sm[n + i];
   }
 }
@@ -195,7 +195,7 @@ static __device__ __forceinline__ void rkf45_team(const DevMech& d, int64_t N, c
       else if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0<INT>(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
+      else h = team_h0<INT, !INT>(d, d.tab, pr, o_y, tf, sp.rtol, sp.atol, o_k, o_t, o_k + n, bufs, vp, qq);
       const double hmin = 1e-15 * tf;
       double t = from.t;
       bool last_rej = from.last_rej != 0, last_nf = from.last_nf != 0;
@@ -205,38 +205,38 @@ static __device__ __forceinline__ void rkf45_team(const DevMech& d, int64_t N, c
         const double hh = clamped ? tf - t : h;
         if (hh < hmin) { st = last_nf ? ST_NONFINITE : ST_HMIN; break; }
         // k_s = hh f(y + sum_j a_sj k_j)
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_y, o_k, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k0[i] *= hh;
           yt[i] = fma(RK_A21, k0[i], yv[i]);
         }
         team_sync();
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_t, o_k + 1 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k1[i] *= hh;
           yt[i] = fma(RK_A32, k1[i], fma(RK_A31, k0[i], yv[i]));
         }
         team_sync();
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_t, o_k + 2 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k2[i] *= hh;
           yt[i] = fma(RK_A43, k2[i], fma(RK_A42, k1[i], fma(RK_A41, k0[i], yv[i])));
         }
         team_sync();
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_t, o_k + 3 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k3[i] *= hh;
           yt[i] = fma(RK_A54, k3[i], fma(RK_A53, k2[i], fma(RK_A52, k1[i], fma(RK_A51, k0[i], yv[i]))));
         }
         team_sync();
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_t, o_k + 4 * n, bufs, vp, qq);
         for (int i = tid; i < n; i += P) {
           k4[i] *= hh;
           yt[i] = fma(RK_A65, k4[i],
                       fma(RK_A64, k3[i], fma(RK_A63, k2[i], fma(RK_A62, k1[i], fma(RK_A61, k0[i], yv[i])))));
         }
         team_sync();
-        team_rhs<INT, TAIL>(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
+        team_rhs_any<INT, TAIL, !INT>(d, d.tab, pr, o_t, o_k + 5 * n, bufs, vp, qq);
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k1, whose weights are 0)
         int nf = 0;
         for (int i = tid; i < n; i += P) {
@@ -318,8 +318,8 @@ cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, cons
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * (2 * (size_t)nn + species_doubles(hm.S) + hm.d.rhs_chunk);
-  const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 128);
+  const size_t smem = sizeof(double) * (2 * (size_t)nn + species_doubles(hm.S) + rhs_doubles(hm.d));
+  const int threads = hm.S > 32 && nn <= 64 ? 96 : 128;
   LaunchCfg cfg;
   auto kern = hm.S > 32 ? k_rhs_team<true> : k_rhs_team<false>;
   const int grid = team_grid(kern, threads, smem, n, cfg);
@@ -344,7 +344,7 @@ cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, c
                                double rtol, double atol, double* jac, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + species_doubles(hm.S) + rhs_doubles(hm.d));
   const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 256);
   const int grid = team_grid(k_jacobian_fd, threads, smem, n, cfg);
   k_jacobian_fd<<<grid, threads, smem, st>>>(hm.d, n, p, y, h, rtol, atol, jac);
@@ -389,6 +389,7 @@ size_t ros4_scratch_bytes_max() {
 }
 
 
+constexpr int64_t ROS4_LAT_PER_SM = 4;
 cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                         double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,
                         int32_t* queue, cudaStream_t st, const LaunchCfg& cfg, double* scratch,
@@ -397,7 +398,12 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
   const int nn = hm.d.n;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  auto* fn = cfg.grid_side == 16 ? launch_ros4_w8 : (nn <= 24 ? launch_ros4_w2 : (nn <= 64 ? launch_ros4_w4 : launch_ros4_w8));
+  // the smallest mechanisms: the latency form while its teams (four an SM) are
+  // enough for the batch
+  const bool lat = hm.S <= 32 && n <= ROS4_LAT_PER_SM * sm_count();
+  auto* fn = cfg.grid_side == 16 ? launch_ros4_w8
+             : nn <= 24          ? (lat ? launch_ros4_w4_lat : launch_ros4_w2)
+                                 : (nn <= 64 ? launch_ros4_w4 : launch_ros4_w8);
   return fn(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg, scratch, scratch_bytes, may_alloc);
 }
 
@@ -406,11 +412,11 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
                               int32_t* status, int32_t* queue, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + hm.d.rhs_chunk);
+  const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + rhs_doubles(hm.d));
   // four warps shorten a step while the batch leaves the SMs room; two keep
   // their lanes busier in one that does not (53 species, four / two warps: 300
   // reactors 13.0 / 19.0 ms, 1000 23.4 / 26.5, 2000 41.5 / 39.1, 16384 278 / 268)
-  const int threads = nn <= 24 ? 64 : (nn > 64 || n < (int64_t)12 * sm_count() ? 128 : 64);
+  const int threads = nn > 64 || hm.S <= 32 || n < (int64_t)12 * sm_count() ? 128 : 64;
   auto kern = hm.S > 32 ? k_rkf45_team<true> : k_rkf45_team<false>;
   const int grid = team_grid(kern, threads, smem, n, cfg);
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
@@ -422,8 +428,8 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
 cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
                               const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
                               const RkCont* list, const int32_t* count, int cap, cudaStream_t st) {
-  const size_t smem = sizeof(double) * (8 * (size_t)hm.d.n + species_doubles(hm.S) + hm.d.rhs_chunk);
-  const int threads = 64;
+  const size_t smem = sizeof(double) * (8 * (size_t)hm.d.n + species_doubles(hm.S) + rhs_doubles(hm.d));
+  const int threads = 128;
   LaunchCfg cfg;
   const int grid = team_grid(k_rkf45_tail, threads, smem, cap, cfg);
   k_rkf45_tail<<<grid, threads, smem, st>>>(hm.d, p, y, dt, h_io, sp, steps, status, queue, list, count, cap);

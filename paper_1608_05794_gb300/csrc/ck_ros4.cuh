@@ -102,7 +102,8 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
   extern __shared__ __align__(16) double sm[];
   __shared__ int slot;
   __shared__ Ros4Ctl ctl;
-  constexpr bool INT = P == 256;  // products in integer arithmetic (see team_rhs)
+  constexpr bool INT = P == 256;               // products in integer arithmetic (see team_rhs)
+  constexpr bool LAT = P == 128 && MINB == 4;  // right-hand sides in the latency form (team_rhs_lat)
   using F = typename std::conditional<PREC == 0, double, float>::type;  // type of the factors
   const int n = d.n, nn = n * n;
   const double* tab = d.tab;  // 2 KB, stays in L1
@@ -141,7 +142,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
       if (fixed) h = sp.fixed_h;
       else if (h_io && h_io[r] > 0.0) h = h_io[r];
       else if (sp.h0 > 0.0) h = sp.h0;
-      else h = team_h0<INT>(d, tab, pr, L.yv, tf, sp.rtol, sp.atol, L.f0, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+      else h = team_h0<INT, LAT>(d, tab, pr, L.yv, tf, sp.rtol, sp.atol, L.f0, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
       const double hmin = 1e-15 * tf;
       // the next attempt: its step size, or the end of the integration
       auto next = [&](int accept) {
@@ -179,12 +180,12 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
         // same y); A = J - I/(hh gamma) = -M; LU of A
         if (!have_j) {
           if (sp.jac == 1) {
-            team_jacobian_fd<INT>(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, PREC ? n : ld, L.yt, L.ub, L.bufs, L.vp,
+            team_jacobian_fd<INT, LAT>(d, tab, pr, L.yv, ctl.hh, sp.rtol, sp.atol, L.f0, PREC ? Mg : M, PREC ? n : ld, L.yt, L.ub, L.bufs, L.vp,
                              L.rhs_q, have_f);
           } else {
             // assembled in the copy Mg where there is one
             const JacTab& jt = Mg ? d.wide : d.narrow;
-            team_jacobian<INT>(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr, ld,
+            team_jacobian<INT, LAT>(d, jt, tab, pr, yv, F0, Mg ? Mg : M, Mg && !PREC ? M : nullptr, ld,
                           carve_bufs(sm + L.bufs, d.S, sm + L.jscr, jt.chunk, L.vp));
           }
           if (PREC) {
@@ -241,7 +242,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           Yt[tid] = fma(-ROS_A21, u1, yi);
         }
         team_sync();
-        team_rhs<INT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        team_rhs_any<INT, false, LAT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
         if (own) ub[tid] = fma(ctl.c21, u1, ub[tid]);
         solve();
         // stage 3: M u3 = f(y + a31 u1 + a32 u2) + (c31 u1 + c32 u2)/h
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(P, MINB) k_ros4(const __grid_constant__ DevMec
           Yt[tid] = fma(-ROS_A32, u2, fma(-ROS_A31, u1, yi));
         }
         team_sync();
-        team_rhs<INT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
+        team_rhs_any<INT, false, LAT>(d, tab, pr, L.yt, L.ub, L.bufs, L.vp, L.rhs_q);
         if (own) {
           f3 = ub[tid];
           ub[tid] = fma(ctl.c32, u2, fma(ctl.c31, u1, f3));

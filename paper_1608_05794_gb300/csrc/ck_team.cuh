@@ -291,14 +291,15 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 // same instructions.  INT: the products of concentrations and of Gibbs factors
 // in integer arithmetic, beside the FP64 unit, which bounds the team kernels
 // (10 of the 23 FP64 instructions of a rate, 20 of 49 with its derivatives).
-// ORD: the fall-off factor by a division, as rhs_thread forms it.
-template <bool JAC, bool INT, bool ORD = false>
+// ORD: the fall-off factor by a division, as rhs_thread forms it.  PRE: k_f
+// and k_0/k_inf are at hand in b.q[i] and b.w[iw] (team_species_lat).
+template <bool JAC, bool INT, bool ORD = false, bool PRE = false>
 __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
                                               const TeamBufs& b, const double* tab, int i, int iw) {
   const RxnRec r = load_rxn(src);
   const double* X = b.X;
   const double l2kf = fma(-r.EoR2, x.invT, fma(r.beta, x.log2T, r.lA2));
-  const double kf = ck_exp2(l2kf, tab);
+  const double kf = PRE ? b.q[i] : ck_exp2(l2kf, tab);
   const int s0 = r.sp[0], s1 = r.sp[1], s2 = r.sp[2], s3 = r.sp[3], s4 = r.sp[4], s5 = r.sp[5];
   const double x0 = X[s0], x1 = X[s1], x2 = X[s2], y0 = X[s3], y1 = X[s4], y2 = X[s5];
   const double fwd = mul_sel<INT>(mul_sel<INT>(x0, x1), x2);
@@ -348,7 +349,7 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
       const double2 f0 = __ldg(reinterpret_cast<const double2*>(src) + 5);  // lA02, beta0
       const double2 f1 = __ldg(reinterpret_cast<const double2*>(src) + 6);  // E0oR2, E0oR
       const double l2k0 = fma(-f1.x, x.invT, fma(f0.y, x.log2T, f0.x));
-      const double k0_kf = ck_exp2(l2k0 - l2kf, tab);
+      const double k0_kf = PRE ? b.w[iw] : ck_exp2(l2k0 - l2kf, tab);
       const double Pr = __dmul_rn(k0_kf, M);
       if (ORD) {
         b.q[i] = net * (Pr / (1.0 + Pr));
@@ -412,6 +413,185 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
     b.D[i] = D;
     b.dqT[i] = m.cv ? dqTX : fma(-D, x.invT, dqTX);
   }
+}
+
+// team_species for a team of four warps on a mechanism of at most 32 species,
+// arranged for the shortest chain: one warp issues an FP64 instruction every
+// 68 cycles however independent they are, so the mixture, log T, 1/T and the
+// powers go to one warp each, then the two Gibbs factors, the heat-capacity
+// and enthalpy polynomials, and the rate constants k_f (kf[R]) and k_0/k_inf
+// (k0, of the fall-off reactions among the typed ones), which need T alone.
+// JAC: the mean molar mass too.  The same values as team_species.
+template <bool ORD, bool JAC>
+__device__ __forceinline__ void team_species_lat(const DevMech& m, double p, const double* y, TeamBufs& b, Mix& x,
+                                                 const double* tab, double* kf, double* k0) {
+  const int S = m.S, R = m.R, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* red = b.red;
+  const double T = y[0];
+  const bool in = lane < S;
+  const double yw = in ? __dmul_rn(y[1 + lane], m.invW[lane]) : 0.0;  // (every warp: the sums below)
+  x.T = T;
+  if (warp == 0) {
+    double sumYW = 0.0;
+    if (ORD) {
+      for (int k = 0; k < S; ++k) sumYW = fma(y[1 + k], m.invW[k], sumYW);
+    } else {
+      sumYW = warp_allsum(yw);
+    }
+    const double rho = m.cv ? p : p / (R_GAS * T * sumYW);
+    if (in) b.X[lane] = __dmul_rn(rho, yw);
+    if (lane == 0) {
+      red[SC_RHO] = rho;
+      red[SC_SUM] = sumYW;
+      b.X[S] = b.Gp[S] = b.Gm[S] = 1.0;
+      b.hRT[S] = 0.0;
+    }
+  } else if (warp == 1) {
+    const double lnT = log(T);
+    if (lane == 0) {
+      red[SC_LNT] = lnT;
+      red[SC_LOG2T] = lnT * INV_LN2;
+    }
+  } else if (warp == 2) {
+    const double invT = rcp_rn(T), T2 = T * T, T3 = T2 * T;
+    const double up = T * R_OVER_P0, dn = invT * P0_OVER_R;
+    if (lane == 0) {
+      red[SC_INVT] = invT;
+      red[SC_T2] = T2;
+      red[SC_T3] = T3;
+      red[SC_T4] = T3 * T;
+      red[SC_PW] = dn * dn;
+      red[SC_PW + 1] = dn;
+      red[SC_PW + 2] = 1.0;
+      red[SC_PW + 3] = up;
+      red[SC_PW + 4] = up * up;
+    }
+  }
+  __syncthreads();
+  x.invT = red[SC_INVT];
+  x.log2T = red[SC_LOG2T];
+  x.rho = red[SC_RHO];
+  const double T2 = red[SC_T2], T3 = red[SC_T3], T4 = red[SC_T4];
+  if (warp == 0) {
+    if (in) {
+      const double* a = m.thermo + lane * TH_PER_SPECIES + (T < m.tmid[lane] ? 0 : TH_STRIDE);
+      double g = fma(a[11], red[SC_LNT], a[12]);
+      g = fma(a[13], T, g);
+      g = fma(a[14], T2, g);
+      g = fma(a[15], T3, g);
+      g = fma(a[16], T4, g);
+      g = fma(a[17], x.invT, g);
+      ck_exp2_pm(g, tab, b.Gp[lane], b.Gm[lane]);
+    }
+  } else if (warp == 1) {
+    if (in) {
+      const double* a = m.thermo + lane * TH_PER_SPECIES + (T < m.tmid[lane] ? 0 : TH_STRIDE);
+      b.cpR[lane] = fma(a[4], T4, fma(a[3], T3, fma(a[2], T2, fma(a[1], T, a[0]))));
+      b.hRT[lane] = fma(a[10], x.invT, fma(a[9], T4, fma(a[8], T3, fma(a[7], T2, fma(a[6], T, a[5])))));
+    }
+    const double invrho = rcp_rn(x.rho);
+    if (lane == 0) red[SC_INVRHO] = invrho;
+  } else {
+    if (warp == 3) {
+      double c = 0.0;
+      if (ORD) {
+        for (int k = 0; k < S; ++k) c += b.X[k];
+      } else {
+        c = warp_allsum(in ? b.X[lane] : 0.0);
+      }
+      if (lane == 0) red[SC_CTOT] = c;
+      if (JAC) {
+        const double Wbar = rcp_rn(red[SC_SUM]);
+        if (lane == 0) red[SC_WBAR] = Wbar;
+      }
+    }
+    for (int i = threadIdx.x - 64; i < R; i += 64) {
+      const RxnRec* src = m.rxn + i;
+      kf[i] = ck_exp2(fma(-src->EoR2, x.invT, fma(src->beta, x.log2T, src->lA2)), tab);
+    }
+    for (int i = m.first_typed + (threadIdx.x ^ 32) - 64; i < R; i += 64) {
+      const RxnRec* src = m.rxn + i;
+      if (src->type == 2) {
+        const double l2kf = fma(-src->EoR2, x.invT, fma(src->beta, x.log2T, src->lA2));
+        const double l2k0 = fma(-src->E0oR2, x.invT, fma(src->beta0, x.log2T, src->lA02));
+        k0[i - m.first_typed] = ck_exp2(l2k0 - l2kf, tab);
+      }
+    }
+  }
+  __syncthreads();
+  x.invrho = red[SC_INVRHO];
+  x.Ctot = red[SC_CTOT];
+  x.Wbar = JAC ? red[SC_WBAR] : 0.0;
+}
+
+// The reaction that place s of a team's walk over R reactions takes, or -1:
+// elementary reactions first, the others from a warp of their own on, so that
+// the two kinds run side by side.
+__device__ __forceinline__ int lat_slots(int R, int ft) { return ((ft + 31) & ~31) + R - ft; }
+__device__ __forceinline__ int lat_reaction(int s, int ft) {
+  const int es = (ft + 31) & ~31;
+  return s < ft ? s : (s >= es ? ft + s - es : -1);
+}
+
+// team_rhs arranged like team_species_lat (four warps, at most 32 species, q of
+// m.R doubles and one more for each third-body or fall-off reaction).  ORD: see
+// team_rhs.  The same values.  One evaluation alone on an SM, 10 species: see
+// k_rkf45_team.
+template <bool ORD>
+static __device__ __noinline__ void team_rhs_lat(const DevMech& m, const double* tab, double p, int y_o, int f_o,
+                                                 int bufs_o, int q_o) {
+  extern __shared__ __align__(16) double sm[];
+  const double* y = sm + y_o;
+  double* f = sm + f_o;
+  TeamBufs b = carve_bufs(sm + bufs_o, m.S, sm + q_o, 0, 64);
+  b.w = b.q + m.R;
+  Mix x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, S = m.S;
+  team_species_lat<ORD, false>(m, p, y, b, x, tab, b.q, b.w);
+  for (int s = threadIdx.x; s < lat_slots(m.R, m.first_typed); s += blockDim.x) {
+    const int i = lat_reaction(s, m.first_typed);
+    if (i >= 0) team_reaction<false, false, ORD, true>(m, m.rxn + i, x, b, tab, i, i - m.first_typed);
+  }
+  if (warp == 3) {  // rho c_p meanwhile
+    double c = 0.0, yk = 0.0;
+    if (lane < S) {
+      c = m.cv ? b.cpR[lane] - 1.0 : b.cpR[lane];
+      yk = __dmul_rn(y[1 + lane], m.invW[lane]);
+    }
+    double cpm = 0.0;
+    if (ORD) {
+      for (int k = 0; k < S; ++k) cpm = fma(__shfl_sync(0xffffffffu, yk, k), __shfl_sync(0xffffffffu, c, k), cpm);
+    } else {
+      cpm = warp_allsum(fma(yk, c, 0.0));
+    }
+    if (lane == 0) b.red[SC_ICPM] = x.rho * cpm;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    double w = 0.0, h = 0.0;
+    if (lane < S) {
+      const int32_t* ptr = ORD ? m.slot_ptr : m.csr_ptr;
+      const CsrTerm* terms = ORD ? m.slot : m.csr;
+      int e = ptr[lane];
+      const int e1 = ptr[lane + 1];
+      for (; e + 4 <= e1; e += 4) {
+        const CsrTerm t0 = terms[e], t1 = terms[e + 1], t2 = terms[e + 2], t3 = terms[e + 3];
+        const double q0 = b.q[t0.rx], q1 = b.q[t1.rx], q2 = b.q[t2.rx], q3 = b.q[t3.rx];
+        w = fma(t3.nu, q3, fma(t2.nu, q2, fma(t1.nu, q1, fma(t0.nu, q0, w))));
+      }
+      for (; e < e1; ++e) w = fma(terms[e].nu, b.q[terms[e].rx], w);
+      f[1 + lane] = w * (m.W[lane] * x.invrho);
+      h = m.cv ? b.hRT[lane] - 1.0 : b.hRT[lane];
+    }
+    double hw = 0.0;
+    if (ORD) {
+      for (int k = 0; k < S; ++k) hw = fma(__shfl_sync(0xffffffffu, h, k), __shfl_sync(0xffffffffu, w, k), hw);
+    } else {
+      hw = warp_allsum(fma(h, w, 0.0));
+    }
+    if (lane == 0) f[0] = -x.T * hw / b.red[SC_ICPM];
+  }
+  __syncthreads();
 }
 
 // f(y) for one reactor.  Arrays by their offsets (doubles) in the CTA's
@@ -536,6 +716,15 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
   team_sync();
 }
 
+// The right-hand side of a kernel: LAT kernels (four warps, at most 32 species)
+// take the latency form where q holds all reactions.
+template <bool INT, bool ORD, bool LAT>
+__device__ __forceinline__ void team_rhs_any(const DevMech& m, const double* tab, double p, int y_o, int f_o,
+                                             int bufs_o, int vp, RhsQ qq) {
+  if (LAT && m.R <= qq.chunk) team_rhs_lat<ORD>(m, tab, p, y_o, f_o, bufs_o, qq.off);
+  else team_rhs<INT, ORD>(m, tab, p, y_o, f_o, bufs_o, vp, qq);
+}
+
 // Analytic Jacobian J = df/d(T, Y) at constant p, written row-major into A
 // (rows jt.ld apart), and into M too (rows ldm apart) unless that is NULL, and
 // f(y) into f.  Derivation
@@ -560,13 +749,16 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 // are read for the last time before M is written, so that a team needs shared
 // memory for the larger of the two only, and takes all reactions in one pass.
 // Needs b.vp >= S (one species a lane in the sums).
-template <bool INT>
+template <bool INT, bool LAT = false>
 static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const double* tab, double p, const double* y,
                                      double* f, double* A, double* M, int ldm, TeamBufs b) {
   Mix x;
   const int S = m.S, lda = jt.ld, na = m.n * lda, SG = species_groups(S);
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const bool in = team_species<false, INT>(m, p, y, b, x, tab);
+  const bool lat = LAT && jt.n_chunks == 1;
+  bool in = false;
+  if (lat) team_species_lat<false, true>(m, p, y, b, x, tab, b.q, b.w);
+  else in = team_species<false, INT>(m, p, y, b, x, tab);
   // chunk by chunk, every target (species-block entries and the per-species
   // sums wdot, a, E, u, whose arrays wd, aT, E, u are contiguous) adds its
   // fixed-order sum of terms; one thread per target, no conflicts, the
@@ -574,7 +766,12 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
   for (int c = 0; c < jt.n_chunks; ++c) {
     const int base = c * jt.chunk, cnt = m.R - base < jt.chunk ? m.R - base : jt.chunk;
     const int ft = m.first_typed > base ? m.first_typed - base : 0;
-    if (INT && in) {
+    if (lat) {
+      for (int s = tid; s < lat_slots(cnt, m.first_typed); s += blockDim.x) {
+        const int li = lat_reaction(s, m.first_typed);
+        if (li >= 0) team_reaction<true, false, false, true>(m, m.rxn + li, x, b, tab, li, li - ft);
+      }
+    } else if (INT && in) {
       for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
         team_reaction<true, INT>(m, m.rxn + base + li, x, b, tab, li, li - ft);
     } else {

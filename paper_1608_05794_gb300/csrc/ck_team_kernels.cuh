@@ -28,7 +28,7 @@ static __device__ __forceinline__ int team_next(int32_t* queue, int* slot) {
 // for this y) and reused as the first stage's f; the n columns cost n team
 // RHS evaluations.  y_o, f0_o, yt_o, f_o: offsets of n-vectors in shared
 // memory (the last two scratch); bufs_o, vp, qq as in team_rhs.
-template <bool INT>
+template <bool INT, bool LAT = false>
 static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const double* tab, double p, int y_o, double h,
                                                      double rtol, double atol, int f0_o, double* J, int ldj, int yt_o,
                                                      int f_o, int bufs_o, int vp, RhsQ qq, bool have_f0 = false) {
@@ -38,7 +38,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
   const double* F = sm + f_o;
   double* Yt = sm + yt_o;
   const int n = d.n, tid = (int)threadIdx.x;
-  if (!have_f0) team_rhs<INT>(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
+  if (!have_f0) team_rhs_any<INT, false, LAT>(d, tab, p, y_o, f0_o, bufs_o, vp, qq);
   double s = 0.0;
   if (tid < vp)
     for (int i = tid; i < n; i += vp) {
@@ -54,7 +54,7 @@ static __device__ __noinline__ void team_jacobian_fd(const DevMech& d, const dou
     const double sj = fmax(srur * fabs(y[j]), s0 * (atol + rtol * fabs(y[j])));
     if (tid == 0) Yt[j] = y[j] + sj;
     team_sync();
-    team_rhs<INT>(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
+    team_rhs_any<INT, false, LAT>(d, tab, p, yt_o, f_o, bufs_o, vp, qq);
     for (int i = tid; i < n; i += blockDim.x) J[(size_t)i * ldj + j] = (F[i] - f0[i]) / sj;
     if (tid == 0) Yt[j] = y[j];
     team_sync();
@@ -100,7 +100,7 @@ static __device__ __forceinline__ double team_wrms(int n, double* e, const doubl
 
 // Initial step, Hairer-Norsett-Wanner starting-step algorithm (order 4).
 // Offsets, vp and qq as in team_rhs; f0, y1, f1 are scratch vectors.
-template <bool INT>
+template <bool INT, bool LAT = false>
 static __device__ __noinline__ double team_h0(const DevMech& d, const double* tab, double p, int y0_o, double tspan,
                                               double rtol, double atol, int f0_o, int y1_o, int f1_o, int bufs_o,
                                               int vp, RhsQ qq) {
@@ -109,7 +109,7 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   double *y1 = sm + y1_o, *red = sm + bufs_o;
   const int n = d.n, tid = (int)threadIdx.x;
   const bool lane_in = tid < vp;
-  team_rhs<INT>(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
+  team_rhs_any<INT, false, LAT>(d, tab, p, y0_o, f0_o, bufs_o, vp, qq);
   double s0 = 0.0, s1 = 0.0;
   if (lane_in)
     for (int i = tid; i < n; i += vp) {
@@ -122,7 +122,7 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   for (int i = tid; i < n; i += blockDim.x) y1[i] = fma(ha, f0[i], y0[i]);
   team_sync();
-  team_rhs<INT>(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
+  team_rhs_any<INT, false, LAT>(d, tab, p, y1_o, f1_o, bufs_o, vp, qq);
   double s2 = 0.0;
   if (lane_in)
     for (int i = tid; i < n; i += vp) {
@@ -134,6 +134,11 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   const double dm = fmax(d1, d2);
   const double hb = (dm <= 1e-15) ? fmax(1e-6, ha * 1e-3) : pow(0.01 / dm, 0.2);
   return fmin(fmin(100.0 * ha, hb), tspan);
+}
+
+// Room for a right-hand side's rates of progress (team_rhs, team_rhs_lat).
+__host__ __device__ __forceinline__ int rhs_doubles(const DevMech& d) {
+  return d.rhs_chunk + (d.S <= 32 ? d.R - d.first_typed : 0);
 }
 
 // Shared memory of one k_ros4 CTA, in doubles: the matrix, y and f(y), the team's work arrays, and the stage vectors,
@@ -162,7 +167,7 @@ struct Ros4Layout {
     rhs_q.chunk = d.rhs_chunk;
     int most = wide ? tj : tj + d.narrow.scratch;
     if (after + 4 * n > most) most = after + 4 * n;
-    if (after + d.rhs_chunk > most) most = after + d.rhs_chunk;
+    if (after + rhs_doubles(d) > most) most = after + rhs_doubles(d);
     doubles = (size_t)most;
   }
 };
