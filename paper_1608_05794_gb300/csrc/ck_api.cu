@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -512,8 +513,10 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   put_jac(on, jn);
   put(off_rsp, rsp.data(), sizeof(int16_t) * rsp.size());
 
+  static std::atomic<uint64_t> loads{0};
   ck_mech* m = new ck_mech;
   HostMech& hm = m->hm;
+  hm.id = ++loads;
   cudaError_t e = cudaGetDevice(&hm.device);
   if (e != cudaSuccess) {
     delete m;

@@ -43,11 +43,18 @@ void destroy(GraphEntry& e) {
   if (e.queues) cudaFree(e.queues);
 }
 
+// The arguments, and the load that each mechanism handle comes from: a graph
+// holds the addresses of its mechanisms' tables, and a handle loaded after
+// another was freed may have that one's address.
 std::vector<unsigned char> make_key(int method, int ng, const ck_group* g, int device, int flags) {
-  std::vector<unsigned char> k(sizeof(int) * 4 + sizeof(ck_group) * ng);
+  std::vector<unsigned char> k(sizeof(int) * 4 + (sizeof(ck_group) + sizeof(uint64_t)) * ng);
   int head[4] = {method, ng, device, flags};
-  std::memcpy(k.data(), head, sizeof(head));
-  std::memcpy(k.data() + sizeof(head), g, sizeof(ck_group) * ng);
+  unsigned char* o = k.data();
+  std::memcpy(o, head, sizeof(head));
+  o += sizeof(head);
+  std::memcpy(o, g, sizeof(ck_group) * ng);
+  o += sizeof(ck_group) * ng;
+  for (int i = 0; i < ng; ++i) std::memcpy(o + sizeof(uint64_t) * i, &g[i].mech->hm.id, sizeof(uint64_t));
   return k;
 }
 

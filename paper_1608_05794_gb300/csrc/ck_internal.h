@@ -19,6 +19,7 @@ struct StageLayout {
 
 struct HostMech {
   int device = -1;
+  uint64_t id = 0;          // of this load, never used again (a freed handle's address may be)
   DevMech d{};
   StageLayout L{};
   void* blob = nullptr;     // device allocation holding every table

@@ -141,3 +141,27 @@ def test_rkf45_threads_hand_reactors_to_teams(ck, cv):
         yl = _dev(y)
         ck.integrate_rkf45(gm, _dev(p), yl, _dev(dt), st, steps=steps, opts=o)
         assert np.array_equal(steps.sum(1).cpu().numpy(), np.minimum(total, limit))
+
+
+def test_graph_of_a_freed_mechanism_is_not_replayed(ck):
+    # a mechanism loaded after another was freed may get its handle's address;
+    # a cached graph of the old one, whose tables are gone, must not match
+    m = load_mechanism(CONFIGS["medium"]["mech"])
+    y, p = reactor_states("medium", n=12, seed_offset=51)
+    pd, rho, dt = _dev(p), _dev(np.linspace(0.3, 2.0, 12)), _dev(np.full(12, 1e-7))
+    yd, st = _dev(y), torch.empty(12, dtype=torch.int32, device="cuda")
+    par = torch.empty_like(pd)  # the same buffers in every call
+    ends = []
+    for cv in (0, 1, 0, 1):
+        gm = ck.load_mechanism(m, reactor=cv)
+        par.copy_(rho if cv else pd)
+        yd.copy_(_dev(y))
+        ck.integrate_groups(1, [dict(mech=gm, p=par, y=yd, dt=dt, status=st)], use_graph=True)
+        torch.cuda.synchronize()
+        yr = _dev(y)
+        ck.integrate_rkf45(gm, par, yr, dt, st)
+        assert torch.equal(yd, yr)
+        ends.append(yr)
+        gm.close()
+    assert torch.equal(ends[0], ends[2]) and not torch.equal(ends[0], ends[1])
+    ck.graph_cache_clear()
