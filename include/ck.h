@@ -139,8 +139,8 @@ typedef struct {
   int32_t variant;  /* 0: as many resident CTAs / blocks per SM as fit; > 0: cap per SM */
   int32_t form;     /* RKF45 mapping: 0 automatic, 1 one thread per reactor (shallow),
                        2 one CTA per reactor (deep); ROS4 always uses one CTA per reactor */
-  int32_t team;     /* ROS4 thread grid of a reactor team: 0 automatic, 8 (8x8 threads, n <= 56)
-                       or 16 (16x16 threads, n <= 112) */
+  int32_t team;     /* ROS4 team of a reactor: 0 or 8 automatic (64 to 256 threads by mechanism
+                       and batch size), 16 always 256 threads */
   int32_t jac;      /* ROS4 Jacobian: 0 analytic (Sec. 6), 1 forward differences as the paper
                        ran it (Sec. 5; see ck_jacobian_fd), n further RHS evaluations a step */
 } ck_solver_opts;

@@ -296,14 +296,14 @@ static __device__ __forceinline__ void rkf45_team(const DevMech& d, int64_t N, c
 }
 
 template <bool INT>
-__global__ void __launch_bounds__(128, 8) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N,
+__global__ void __launch_bounds__(128, INT ? 8 : 5) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N,
                                                        const double* __restrict__ p, double* __restrict__ y,
                                                        const double* __restrict__ dt, double* h_io, SolverParams sp,
                                                        int32_t* steps, int32_t* status, int32_t* queue) {
   rkf45_team<INT, false>(d, N, p, y, dt, h_io, sp, steps, status, queue, nullptr);
 }
 
-__global__ void __launch_bounds__(128, 8) k_rkf45_tail(const __grid_constant__ DevMech d,
+__global__ void __launch_bounds__(128, 5) k_rkf45_tail(const __grid_constant__ DevMech d,
                                                        const double* __restrict__ p, double* __restrict__ y,
                                                        const double* __restrict__ dt, double* h_io, SolverParams sp,
                                                        int32_t* steps, int32_t* status, int32_t* queue,

@@ -150,7 +150,8 @@ __device__ double h0_thread(const MechView& m, int n, double p, const double* y0
 // may be.  Longer keeps more of the work where the lanes are full, but a warp
 // then runs on for its slowest lanes.  10 species over 1e-5 s (70 attempts a
 // reactor on average, 1900 at most), 100003 / 300000 reactors: 96 attempts 389
-// / 1051 ms, 128 372 / 906, 192 411 / 808, 320 536 / 889, never 670 / -.
+// / 1051 ms, 128 372 / 906, 192 411 / 808, 320 536 / 889, never 670 / -; 160
+// (and the teams' latency form) 365 / 944.
 constexpr int RK_THREAD_STEPS = 160;
 constexpr int64_t RK_LIST_MAX = 1 << 18;
 
@@ -412,9 +413,14 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   const int list_cap = (int)(n < RK_LIST_MAX ? n : RK_LIST_MAX);
   if (MAXS <= 32 && may_alloc && hm.R <= hm.d.rhs_chunk && n <= INT32_MAX) {
     e = cudaMallocAsync(reinterpret_cast<void**>(&count), 16 + sizeof(RkCont) * (size_t)list_cap, st);
-    if (e != cudaSuccess) return e;
-    list = reinterpret_cast<RkCont*>(count + 4);
-    e = cudaMemsetAsync(count, 0, 16, st);
+    if (e == cudaSuccess) {
+      list = reinterpret_cast<RkCont*>(count + 4);
+      e = cudaMemsetAsync(count, 0, 16, st);
+    } else {  // no room for it: the threads finish every reactor themselves
+      cudaGetLastError();
+      count = nullptr;
+      e = cudaSuccess;
+    }
   }
   if (e == cudaSuccess) {
     kern<<<blocks, threads, smem, st>>>(hm.d, hm.L, staged, n, p, y, dt, h_io, sp, steps, status,

@@ -292,7 +292,8 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 // in integer arithmetic, beside the FP64 unit, which bounds the team kernels
 // (10 of the 23 FP64 instructions of a rate, 20 of 49 with its derivatives).
 // ORD: the fall-off factor by a division, as rhs_thread forms it.  PRE: k_f
-// and k_0/k_inf are at hand in b.q[i] and b.w[iw] (team_species_lat).
+// is at hand in b.q[i], and in b.w[iw] k_0/k_inf (JAC) or the whole factor of the
+// net rate (team_species_lat).
 template <bool JAC, bool INT, bool ORD = false, bool PRE = false>
 __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* src, const Mix& x,
                                               const TeamBufs& b, const double* tab, int i, int iw) {
@@ -338,6 +339,10 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
   const double net = fma(-kr, rv, kf * fwd);
   double q = net, ckf = kf, ckr = kr, w = 0.0, M = 0.0, dcdT = 0.0;
   const double dlnkf = fma(r.EoR, x.invT, r.beta) * x.invT;
+  if (PRE && !JAC) {
+    b.q[i] = r.type ? b.w[iw] * net : net;
+    return;
+  }
   if (r.type) {
     double c, dcdM;
     M = x.Ctot;
@@ -415,13 +420,22 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
   }
 }
 
+// Named barriers of the first 128 threads' teams: `sync` waits until n threads
+// have come, `arrive` counts the caller's warp without waiting.
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+
 // team_species for a team of four warps on a mechanism of at most 32 species,
 // arranged for the shortest chain: one warp issues an FP64 instruction every
-// 68 cycles however independent they are, so the mixture, log T, 1/T and the
-// powers go to one warp each, then the two Gibbs factors, the heat-capacity
-// and enthalpy polynomials, and the rate constants k_f (kf[R]) and k_0/k_inf
-// (k0, of the fall-off reactions among the typed ones), which need T alone.
-// JAC: the mean molar mass too.  The same values as team_species.
+// 68 cycles however independent they are, so that every warp takes its own
+// share: warp 1 log T, warp 2 1/T and the powers; then, without waiting for
+// the mixture, warp 3 the Gibbs factors, warp 1 the heat capacities and
+// enthalpies, warp 2 the rate constants k_f (kf[R]), which need T alone; warp 0
+// the mixture and, of the third-body and fall-off reactions, k_0/k_inf (k0,
+// JAC) or the whole factor that multiplies their net rate (k0, else).  JAC: the
+// mean molar mass too.  The same values as team_species and team_reaction.
 template <bool ORD, bool JAC>
 __device__ __forceinline__ void team_species_lat(const DevMech& m, double p, const double* y, TeamBufs& b, Mix& x,
                                                  const double* tab, double* kf, double* k0) {
@@ -429,9 +443,9 @@ __device__ __forceinline__ void team_species_lat(const DevMech& m, double p, con
   double* red = b.red;
   const double T = y[0];
   const bool in = lane < S;
-  const double yw = in ? __dmul_rn(y[1 + lane], m.invW[lane]) : 0.0;  // (every warp: the sums below)
   x.T = T;
   if (warp == 0) {
+    const double yw = in ? __dmul_rn(y[1 + lane], m.invW[lane]) : 0.0;
     double sumYW = 0.0;
     if (ORD) {
       for (int k = 0; k < S; ++k) sumYW = fma(y[1 + k], m.invW[k], sumYW);
@@ -439,89 +453,103 @@ __device__ __forceinline__ void team_species_lat(const DevMech& m, double p, con
       sumYW = warp_allsum(yw);
     }
     const double rho = m.cv ? p : p / (R_GAS * T * sumYW);
-    if (in) b.X[lane] = __dmul_rn(rho, yw);
+    const double xk = in ? __dmul_rn(rho, yw) : 0.0;
+    if (in) b.X[lane] = xk;
     if (lane == 0) {
       red[SC_RHO] = rho;
-      red[SC_SUM] = sumYW;
       b.X[S] = b.Gp[S] = b.Gm[S] = 1.0;
       b.hRT[S] = 0.0;
     }
-  } else if (warp == 1) {
-    const double lnT = log(T);
-    if (lane == 0) {
-      red[SC_LNT] = lnT;
-      red[SC_LOG2T] = lnT * INV_LN2;
+    __syncwarp();
+    double c = 0.0;
+    if (ORD) {
+      for (int k = 0; k < S; ++k) c += b.X[k];
+    } else {
+      c = warp_allsum(xk);
     }
-  } else if (warp == 2) {
-    const double invT = rcp_rn(T), T2 = T * T, T3 = T2 * T;
-    const double up = T * R_OVER_P0, dn = invT * P0_OVER_R;
-    if (lane == 0) {
-      red[SC_INVT] = invT;
-      red[SC_T2] = T2;
-      red[SC_T3] = T3;
-      red[SC_T4] = T3 * T;
-      red[SC_PW] = dn * dn;
-      red[SC_PW + 1] = dn;
-      red[SC_PW + 2] = 1.0;
-      red[SC_PW + 3] = up;
-      red[SC_PW + 4] = up * up;
+    if (lane == 0) red[SC_CTOT] = c;
+    if (JAC) {
+      const double Wbar = rcp_rn(sumYW), invrho = rcp_rn(rho);
+      if (lane == 0) {
+        red[SC_WBAR] = Wbar;
+        red[SC_INVRHO] = invrho;
+      }
+    }
+    bar_sync(2, 96);  // the functions of T, from warps 1 and 2
+    for (int i = m.first_typed + lane; i < R; i += 32) {
+      const RxnRec* src = m.rxn + i;
+      const bool fall = src->type == 2;
+      double k0kf = 0.0;
+      if (fall) {
+        const double l2kf = fma(-src->EoR2, red[SC_INVT], fma(src->beta, red[SC_LOG2T], src->lA2));
+        const double l2k0 = fma(-src->E0oR2, red[SC_INVT], fma(src->beta0, red[SC_LOG2T], src->lA02));
+        k0kf = ck_exp2(l2k0 - l2kf, tab);
+      }
+      if (!JAC) {
+        double M = c;
+        for (int e = src->eff_beg; e < src->eff_beg + src->eff_cnt; ++e) M = fma(m.eff_m1[e], b.X[m.eff_sp[e]], M);
+        if (fall) {
+          const double Pr = __dmul_rn(k0kf, M);
+          k0kf = ORD ? Pr / __dadd_rn(1.0, Pr) : __dmul_rn(Pr, rcp_rn(__dadd_rn(1.0, Pr)));
+        } else {
+          k0kf = M;
+        }
+      }
+      k0[i - m.first_typed] = k0kf;
+    }
+  } else {
+    if (warp == 1) {
+      const double lnT = log(T);
+      if (lane == 0) {
+        red[SC_LNT] = lnT;
+        red[SC_LOG2T] = lnT * INV_LN2;
+      }
+      bar_arrive(2, 96);
+    } else if (warp == 2) {
+      const double invT = rcp_rn(T), T2 = T * T, T3 = T2 * T;
+      const double up = T * R_OVER_P0, dn = invT * P0_OVER_R;
+      if (lane == 0) {
+        red[SC_INVT] = invT;
+        red[SC_T2] = T2;
+        red[SC_T3] = T3;
+        red[SC_T4] = T3 * T;
+        red[SC_PW] = dn * dn;
+        red[SC_PW + 1] = dn;
+        red[SC_PW + 2] = 1.0;
+        red[SC_PW + 3] = up;
+        red[SC_PW + 4] = up * up;
+      }
+      bar_arrive(2, 96);
+    }
+    bar_sync(1, 96);  // warps 1 to 3
+    const double invT = red[SC_INVT], log2T = red[SC_LOG2T];
+    const double T2 = red[SC_T2], T3 = red[SC_T3], T4 = red[SC_T4];
+    const double* a = m.thermo + lane * TH_PER_SPECIES + (in && T < m.tmid[lane] ? 0 : TH_STRIDE);
+    if (warp == 3 && in) {
+      double g = fma(a[11], red[SC_LNT], a[12]);
+      g = fma(a[13], T, g);
+      g = fma(a[14], T2, g);
+      g = fma(a[15], T3, g);
+      g = fma(a[16], T4, g);
+      g = fma(a[17], invT, g);
+      ck_exp2_pm(g, tab, b.Gp[lane], b.Gm[lane]);
+    } else if (warp == 1 && in) {
+      b.cpR[lane] = fma(a[4], T4, fma(a[3], T3, fma(a[2], T2, fma(a[1], T, a[0]))));
+      b.hRT[lane] = fma(a[10], invT, fma(a[9], T4, fma(a[8], T3, fma(a[7], T2, fma(a[6], T, a[5])))));
+    } else if (warp == 2) {
+      for (int i = lane; i < R; i += 32) {
+        const RxnRec* src = m.rxn + i;
+        kf[i] = ck_exp2(fma(-src->EoR2, invT, fma(src->beta, log2T, src->lA2)), tab);
+      }
     }
   }
   __syncthreads();
   x.invT = red[SC_INVT];
   x.log2T = red[SC_LOG2T];
   x.rho = red[SC_RHO];
-  const double T2 = red[SC_T2], T3 = red[SC_T3], T4 = red[SC_T4];
-  if (warp == 0) {
-    if (in) {
-      const double* a = m.thermo + lane * TH_PER_SPECIES + (T < m.tmid[lane] ? 0 : TH_STRIDE);
-      double g = fma(a[11], red[SC_LNT], a[12]);
-      g = fma(a[13], T, g);
-      g = fma(a[14], T2, g);
-      g = fma(a[15], T3, g);
-      g = fma(a[16], T4, g);
-      g = fma(a[17], x.invT, g);
-      ck_exp2_pm(g, tab, b.Gp[lane], b.Gm[lane]);
-    }
-  } else if (warp == 1) {
-    if (in) {
-      const double* a = m.thermo + lane * TH_PER_SPECIES + (T < m.tmid[lane] ? 0 : TH_STRIDE);
-      b.cpR[lane] = fma(a[4], T4, fma(a[3], T3, fma(a[2], T2, fma(a[1], T, a[0]))));
-      b.hRT[lane] = fma(a[10], x.invT, fma(a[9], T4, fma(a[8], T3, fma(a[7], T2, fma(a[6], T, a[5])))));
-    }
-    const double invrho = rcp_rn(x.rho);
-    if (lane == 0) red[SC_INVRHO] = invrho;
-  } else {
-    if (warp == 3) {
-      double c = 0.0;
-      if (ORD) {
-        for (int k = 0; k < S; ++k) c += b.X[k];
-      } else {
-        c = warp_allsum(in ? b.X[lane] : 0.0);
-      }
-      if (lane == 0) red[SC_CTOT] = c;
-      if (JAC) {
-        const double Wbar = rcp_rn(red[SC_SUM]);
-        if (lane == 0) red[SC_WBAR] = Wbar;
-      }
-    }
-    for (int i = threadIdx.x - 64; i < R; i += 64) {
-      const RxnRec* src = m.rxn + i;
-      kf[i] = ck_exp2(fma(-src->EoR2, x.invT, fma(src->beta, x.log2T, src->lA2)), tab);
-    }
-    for (int i = m.first_typed + (threadIdx.x ^ 32) - 64; i < R; i += 64) {
-      const RxnRec* src = m.rxn + i;
-      if (src->type == 2) {
-        const double l2kf = fma(-src->EoR2, x.invT, fma(src->beta, x.log2T, src->lA2));
-        const double l2k0 = fma(-src->E0oR2, x.invT, fma(src->beta0, x.log2T, src->lA02));
-        k0[i - m.first_typed] = ck_exp2(l2k0 - l2kf, tab);
-      }
-    }
-  }
-  __syncthreads();
-  x.invrho = red[SC_INVRHO];
   x.Ctot = red[SC_CTOT];
   x.Wbar = JAC ? red[SC_WBAR] : 0.0;
+  x.invrho = JAC ? red[SC_INVRHO] : 0.0;
 }
 
 // The reaction that place s of a team's walk over R reactions takes, or -1:
@@ -565,22 +593,40 @@ static __device__ __noinline__ void team_rhs_lat(const DevMech& m, const double*
       cpm = warp_allsum(fma(yk, c, 0.0));
     }
     if (lane == 0) b.red[SC_ICPM] = x.rho * cpm;
+  } else if (warp == 2) {  // and 1 / rho
+    const double invrho = rcp_rn(x.rho);
+    if (lane == 0) b.red[SC_INVRHO] = invrho;
+  }
+  // the gather's terms are read ahead of the rates
+  constexpr int PF = 8;
+  const int32_t* ptr = ORD ? m.slot_ptr : m.csr_ptr;
+  const CsrTerm* terms = ORD ? m.slot : m.csr;
+  int e = 0, e1 = 0;
+  CsrTerm t[PF];
+  if (warp == 0 && lane < S) {
+    e = ptr[lane];
+    e1 = ptr[lane + 1];
+#pragma unroll
+    for (int u = 0; u < PF; ++u)
+      if (e + u < e1) t[u] = terms[e + u];
   }
   __syncthreads();
   if (warp == 0) {
     double w = 0.0, h = 0.0;
     if (lane < S) {
-      const int32_t* ptr = ORD ? m.slot_ptr : m.csr_ptr;
-      const CsrTerm* terms = ORD ? m.slot : m.csr;
-      int e = ptr[lane];
-      const int e1 = ptr[lane + 1];
-      for (; e + 4 <= e1; e += 4) {
-        const CsrTerm t0 = terms[e], t1 = terms[e + 1], t2 = terms[e + 2], t3 = terms[e + 3];
-        const double q0 = b.q[t0.rx], q1 = b.q[t1.rx], q2 = b.q[t2.rx], q3 = b.q[t3.rx];
-        w = fma(t3.nu, q3, fma(t2.nu, q2, fma(t1.nu, q1, fma(t0.nu, q0, w))));
+      while (e < e1) {
+        double q[PF];
+#pragma unroll
+        for (int u = 0; u < PF; ++u) q[u] = e + u < e1 ? b.q[t[u].rx] : 0.0;
+#pragma unroll
+        for (int u = 0; u < PF; ++u)
+          if (e + u < e1) w = fma(t[u].nu, q[u], w);
+        e += PF;
+#pragma unroll
+        for (int u = 0; u < PF; ++u)
+          if (e + u < e1) t[u] = terms[e + u];
       }
-      for (; e < e1; ++e) w = fma(terms[e].nu, b.q[terms[e].rx], w);
-      f[1 + lane] = w * (m.W[lane] * x.invrho);
+      f[1 + lane] = w * (m.W[lane] * b.red[SC_INVRHO]);
       h = m.cv ? b.hRT[lane] - 1.0 : b.hRT[lane];
     }
     double hw = 0.0;
