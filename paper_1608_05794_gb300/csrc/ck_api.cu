@@ -294,15 +294,20 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
   // species -> (reaction, net nu), in the sorted reaction order
   std::vector<int32_t> csr_ptr(S + 1, 0), csr_rx;
   std::vector<double> csr_nu;
+  std::vector<std::vector<std::pair<int32_t, double>>> rows(S);
+  for (int i = 0; i < R; ++i)
+    for (int s = 0; s < 6; ++s) {
+      const int k = rx[i].sp[s];
+      if (k == S || (!rows[k].empty() && rows[k].back().first == i)) continue;
+      int nu = 0;
+      for (int q = 0; q < 3; ++q) nu += (rx[i].sp[3 + q] == k) - (rx[i].sp[q] == k);
+      if (nu != 0) rows[k].push_back({i, (double)nu});
+    }
   for (int k = 0; k < S; ++k) {
     csr_ptr[k] = (int32_t)csr_rx.size();
-    for (int i = 0; i < R; ++i) {
-      int nu = 0;
-      for (int s = 0; s < 3; ++s) nu += (rx[i].sp[3 + s] == k) - (rx[i].sp[s] == k);
-      if (nu != 0) {
-        csr_rx.push_back(i);
-        csr_nu.push_back((double)nu);
-      }
+    for (auto& t : rows[k]) {
+      csr_rx.push_back(t.first);
+      csr_nu.push_back(t.second);
     }
   }
   csr_ptr[S] = (int32_t)csr_rx.size();
@@ -358,6 +363,9 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     std::vector<JcTerm> jt;
   };
   int n_jterms = 0;
+  std::vector<double> w_ratio((size_t)S * S);
+  for (int k = 0; k < S; ++k)
+    for (int j = 0; j < S; ++j) w_ratio[(size_t)k * S + j] = (double)((long double)W[k] / (long double)W[j]);
   auto jac_table = [&](int chunk, int ld) {
     JacHost t;
     t.chunk = chunk;
@@ -366,59 +374,73 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     t.jc_ptr.push_back(0);
     n_jterms = 0;
     int typed_most = 0;
+    const int NE = S * S + 4 * S;
+    std::vector<int32_t> at(csr_ptr.begin(), csr_ptr.end() - 1);  // the next CSR entry of every species
+    std::vector<int32_t> first(NE + 1), put_at(NE), by_len;
     for (int c = 0; c < t.n_chunks; ++c) {
       const int base = c * chunk, end = std::min(R, base + chunk), ft = std::max(first_typed - base, 0);
       typed_most = std::max(typed_most, end - std::max(base, first_typed));
-      std::vector<std::vector<std::pair<double, int32_t>>> ent((size_t)S * S + 4 * (size_t)S);
-      for (int k = 0; k < S; ++k) {
-        for (int e = csr_ptr[k]; e < csr_ptr[k + 1]; ++e) {
-          const int i = csr_rx[e];
-          if (i < base || i >= end) continue;
-          const int li = i - base;
-          const double nu = csr_nu[e];
-          const RxnRec& r = rx[i];
-          const int32_t pbase = 3 * chunk + li * 6, pw = JAC_PER_RXN * chunk + li - ft;
-          // coefficients carry W_k / W_j, the factor of the species block
-          // dY_k/dY_j (so the assembly needs no per-entry rescaling)
-          auto wr = [&](int j) { return (double)((long double)W[k] / (long double)W[j]); };
-          for (int s2 = 0; s2 < r.nreac; ++s2)
-            ent[(size_t)k * S + r.sp[s2]].push_back({nu * wr(r.sp[s2]), pbase + s2});
-          if (r.rev)
-            for (int s2 = 0; s2 < r.nprod; ++s2)
-              ent[(size_t)k * S + r.sp[3 + s2]].push_back({nu * wr(r.sp[3 + s2]), pbase + 3 + s2});
-          for (int q = r.eff_beg; q < r.eff_beg + r.eff_cnt; ++q)
-            ent[(size_t)k * S + eff_sp[q]].push_back({nu * eff_m1[q] * wr(eff_sp[q]), pw});
-          const size_t sb = (size_t)S * S;
-          ent[sb + 0 * S + k].push_back({nu, li});
-          ent[sb + 1 * S + k].push_back({nu, chunk + li});
-          ent[sb + 2 * S + k].push_back({nu, 2 * chunk + li});
-          if (r.type) ent[sb + 3 * S + k].push_back({nu, pw});
+      // every term of the chunk, target by target, in the order of the CSR
+      auto walk = [&](auto&& term) {
+        for (int k = 0; k < S; ++k)
+          for (int e = at[k]; e < csr_ptr[k + 1] && csr_rx[e] < end; ++e) {
+            const int li = csr_rx[e] - base;
+            const double nu = csr_nu[e];
+            const RxnRec& r = rx[csr_rx[e]];
+            const int32_t pbase = 3 * chunk + li * 6, pw = JAC_PER_RXN * chunk + li - ft;
+            // coefficients carry W_k / W_j, the factor of the species block
+            // dY_k/dY_j (so the assembly needs no per-entry rescaling)
+            const double* wr = &w_ratio[(size_t)k * S];
+            for (int s2 = 0; s2 < r.nreac; ++s2) term(k * S + r.sp[s2], nu * wr[r.sp[s2]], pbase + s2);
+            if (r.rev)
+              for (int s2 = 0; s2 < r.nprod; ++s2) term(k * S + r.sp[3 + s2], nu * wr[r.sp[3 + s2]], pbase + 3 + s2);
+            for (int q = r.eff_beg; q < r.eff_beg + r.eff_cnt; ++q)
+              term(k * S + eff_sp[q], nu * eff_m1[q] * wr[eff_sp[q]], pw);
+            const int sb = S * S + k;
+            term(sb, nu, li);
+            term(sb + S, nu, chunk + li);
+            term(sb + 2 * S, nu, 2 * chunk + li);
+            if (r.type) term(sb + 3 * S, nu, pw);
+          }
+      };
+      std::fill(first.begin(), first.end(), 0);
+      walk([&](int e, double, int32_t) { ++first[e + 1]; });
+      int longest = 0;
+      for (int e = 0; e < NE; ++e) longest = std::max(longest, (int)first[e + 1]);
+      // targets, longest first (equal lengths in order), and their terms
+      by_len.assign(longest + 2, 0);
+      for (int e = 0; e < NE; ++e) ++by_len[longest - first[e + 1] + 1];
+      for (int l = 0; l <= longest; ++l) by_len[l + 1] += by_len[l];
+      const size_t jc0 = t.jc.size();
+      const int kept = c == 0 ? NE : by_len[longest];  // those of no term in chunk 0 only
+      t.jc.resize(jc0 + kept);
+      for (int e = 0; e < NE; ++e) {
+        const int len = first[e + 1], i = by_len[longest - len]++;
+        if (i < kept) {
+          JcEntry& h = t.jc[jc0 + i];
+          h.idx = e < S * S ? (1 + e / S) * ld + 1 + e % S : n1 * ld + (e - S * S);
+          h.beg = e;  // the target, until its terms have a place
+          h.end = len;
         }
+        if (e < S * S) n_jterms += len;
       }
-      std::vector<int> order_e;
-      for (size_t e = 0; e < ent.size(); ++e)
-        if (c == 0 || !ent[e].empty()) order_e.push_back((int)e);
-      std::stable_sort(order_e.begin(), order_e.end(),
-                       [&](int a, int b) { return ent[a].size() > ent[b].size(); });
-      for (int e : order_e) {
-        JcEntry h{};
-        if (e < S * S) {
-          const int k = e / S, j = e % S;
-          h.idx = (1 + k) * ld + 1 + j;
-          n_jterms += (int)ent[e].size();
-        } else {
-          h.idx = n1 * ld + (e - S * S);
-        }
-        h.beg = (int32_t)t.jt.size();
-        for (auto& cc : ent[e]) {
-          JcTerm u{};
-          u.coef = cc.first;
-          u.pidx = cc.second;
-          t.jt.push_back(u);
-        }
-        h.end = (int32_t)t.jt.size();
-        t.jc.push_back(h);
+      int32_t at_term = (int32_t)t.jt.size();
+      for (size_t i = jc0; i < t.jc.size(); ++i) {
+        JcEntry& h = t.jc[i];
+        const int len = h.end;
+        put_at[h.beg] = at_term;
+        h.beg = at_term;
+        at_term += len;
+        h.end = at_term;
       }
+      t.jt.resize(at_term);
+      walk([&](int e, double coef, int32_t pidx) {
+        JcTerm& u = t.jt[put_at[e]++];
+        u.coef = coef;
+        u.pidx = pidx;
+      });
+      for (int k = 0; k < S; ++k)
+        while (at[k] < csr_ptr[k + 1] && csr_rx[at[k]] < end) ++at[k];
       t.jc_ptr.push_back((int32_t)t.jc.size());
     }
     t.scratch = JAC_PER_RXN * chunk + std::max(typed_most, 0);
