@@ -68,7 +68,7 @@ struct __align__(16) CsrTerm {  // species -> reaction list: net coefficient and
   int32_t rx, pad;
 };
 struct __align__(16) JcEntry {  // one species-block entry of the Jacobian assembly
-  int32_t idx;                  // flat shared-memory index of the entry
+  int32_t idx;                  // flat index of the target (see JacTab)
   int32_t beg, end;             // its contribution terms
   int32_t pad;
 };

@@ -140,8 +140,11 @@ __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu
 // ------------------------------------------------------------------ RKF45 (team)
 // RKF45 with one CTA per reactor (the paper's "deep" form): the six stage
 // right-hand sides are evaluated by the team, so a reactor's working set
-// (8 n-vectors and one chunk of reaction scratch) stays in shared memory and
-// the number of steps of one reactor never holds back another.
+// (8 n-vectors, the species arrays and the rates of progress) stays in shared
+// memory and the number of steps of one reactor never holds back another.
+// Bound by the FP64 unit (87 % active, 608 warp instructions a right-hand side
+// of the 53-species mechanism before the integer products): 16384 reactors 266
+// ms, 362 with 710 instructions.
 //
 // TAIL: reactors that the thread-per-reactor kernel handed on (the entries of
 // list, *count of them but cap at most), taken up where it left them; every sum
@@ -398,8 +401,12 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
   const int nn = hm.d.n;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  // the smallest mechanisms: the latency form while its teams (four an SM) are
-  // enough for the batch
+  // Team sizes as measured on GB300.  10 species: two warps 234 / 343 ms on 512
+  // / 4000 reactors, the latency form on four 205 / 454 (four of its teams
+  // fit an SM: for batches they hold), one warp 272 / 375.  53 species, 4096
+  // reactors: four warps 600 ms, two 731, three 667, six 646, eight 1031.  111
+  // species, 1500 reactors: eight warps and two CTAs an SM 280 ms, twelve and
+  // one 380.
   const bool lat = hm.S <= 32 && n <= ROS4_LAT_PER_SM * sm_count();
   auto* fn = cfg.grid_side == 16 ? launch_ros4_w8
              : nn <= 24          ? (lat ? launch_ros4_w4_lat : launch_ros4_w2)
