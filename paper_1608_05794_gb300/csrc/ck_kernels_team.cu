@@ -89,7 +89,7 @@ static __host__ __device__ __forceinline__ size_t lu_doubles(int dim) {
 __global__ void __launch_bounds__(256) k_lu_factor(int64_t batch, int dim, double* __restrict__ a,
                                                    int32_t* __restrict__ piv, int32_t* __restrict__ info) {
   extern __shared__ __align__(16) double sm[];
-  __shared__ int flag;
+  __shared__ int flag[2];
   const int nn = dim * dim, ld = lu_ld(dim), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   double* A = sm;
   LuRow<double>* lr = reinterpret_cast<LuRow<double>*>(A + ((dim * lu_ld(dim) + 1) & ~1));
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) k_lu_factor(int64_t batch, int dim, doubl
     double* am = a + m * nn;
     load_matrix(A, ld, am, dim, rc);
     team_sync();
-    const int inf = lu_flat<false>(A, dim, rof, pv, invd, lr, &flag);
+    const int inf = lu_flat<false>(A, dim, rof, pv, invd, lr, flag);
     for (int i = warp; i < dim; i += nw) {
       const double* row = A + (rof[i] >> 8);
       for (int j = lane; j < dim; j += 32) am[i * dim + j] = row[j];

@@ -980,7 +980,11 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
 // pivot k was swapped with (LAPACK order).  Returns 0, or k + 1 when pivot k
 // is zero or not finite (the same in every thread; A then holds the matrix as
 // updated by the pivots before k).
-// lr: 2 n entries of scratch, flag: one int of shared memory.
+// lr: 2 n entries of scratch, flag: two ints of shared memory.  Pivot k raises
+// flag[k & 1]: the panel of pivot k + 1 may run while a slower warp has yet to
+// read pivot k's, behind the barrier that both have passed, and a flag that it
+// saw too early would take that warp out of the loop one barrier before its
+// team.
 template <class F>
 struct __align__(2 * sizeof(F)) LuRow {
   F l;      // multiplier
@@ -1056,7 +1060,7 @@ __device__ __forceinline__ void lu_panel(F* A, int n, int k, int* rof, int* lpiv
         rof[i] = pk[q];  // the row order as it stands
       }
     }
-    if (lane == 0) *flag = k + 1;
+    if (lane == 0) flag[k & 1] = k + 1;
     return;
   }
   const int from = (p - k) & 31;
@@ -1130,11 +1134,11 @@ __device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd
     lr[n + i].pk = (i * lu_ld(n)) << 8 | i;
     if (lpiv) lpiv[i] = i;
   }
-  if (tid == 0) *flag = 0;
+  if (tid < 2) flag[tid] = 0;
   team_sync();
   if (warp == 0) lu_panel(A, n, 0, rof, lpiv, invd, lr, flag);
   team_sync();
-  if (*flag) return *flag;
+  if (flag[0]) return flag[0];
   constexpr int C0 = 10;  // a panel costs its warp about as much as this many updates of 32 elements
   int pw = 1 % nw;        // the warp of the next panel
   for (int k = 0; k + 1 < n; ++k) {
@@ -1149,7 +1153,7 @@ __device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd
                 nw == 1 ? 0 : (warp > pw ? warp - pw - 1 : warp - pw - 1 + nw), nw == 1 ? 1 : nw - 1);
       if (++pw == nw) pw = 0;
       team_sync();
-      if (*flag) return *flag;
+      if (flag[(k + 1) & 1]) return flag[(k + 1) & 1];
       continue;
     }
     // groups of 32 elements: the panel's warp takes the last gp, the others
@@ -1204,7 +1208,7 @@ __device__ __forceinline__ int lu_flat(F* A, int n, int* rof, int* lpiv, F* invd
     }
     if (++pw == nw) pw = 0;
     team_sync();
-    if (*flag) return *flag;
+    if (flag[(k + 1) & 1]) return flag[(k + 1) & 1];
   }
   if (PRE) {
     // rows r and n - 2 - r of the strict upper triangle have n elements together
