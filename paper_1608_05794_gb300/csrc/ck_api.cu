@@ -14,6 +14,7 @@
 
 #include "../../include/ck.h"
 #include "ck_internal.h"
+#include "ck_layout.cuh"
 
 namespace {
 
@@ -329,11 +330,11 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     }
   // team kernels walk the reactions in chunks: equal shares of at most what
   // the team's shared memory has room for
-  const int n1 = S + 1, NN = n1 * n1;
-  auto shares = [&](int most) { return R ? (R + (R + most - 1) / most - 1) / ((R + most - 1) / most) : 1; };
+  const int n1 = S + 1;
   int first_typed = 0;
   while (first_typed < R && rx[first_typed].type == 0) ++first_typed;
-  const int rhs_chunk = shares(n1 <= 64 ? 512 : 392);
+  const TeamChunks chunks = team_chunks(S, R, R - first_typed);
+  const int rhs_chunk = chunks.rhs;
   const int n_rhs_chunks = (R + rhs_chunk - 1) / rhs_chunk;
   std::vector<int32_t> csr_cptr((size_t)S * (n_rhs_chunks + 1));  // first CSR entry of every species and chunk
   for (int k = 0; k < S; ++k) {
@@ -446,13 +447,8 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     t.scratch = JAC_PER_RXN * chunk + std::max(typed_most, 0);
     return t;
   };
-  // the wide form's scratch takes the matrix's place in shared memory: all
-  // reactions at once where they fit it (or 24 KB)
-  const int room = std::max(NN, 3072);
-  const JacHost jw = jac_table(JAC_PER_RXN * R + (R - first_typed) <= room ? std::max(R, 1)
-                                                                            : shares(room / (JAC_PER_RXN + 1)),
-                               n1);
-  const JacHost jn = jac_table(shares(n1 <= 64 ? 64 : 60), n1 | 1);  // in the LU's matrix
+  const JacHost jw = jac_table(chunks.wide, n1);
+  const JacHost jn = jac_table(chunks.narrow, lu_ld(n1));  // in the LU's matrix
 
   // species ordered by the length of their CSR rows (longest first), so
   // that the lanes of one warp gather similar counts in the RHS

@@ -7,6 +7,7 @@
 // takes the same branch and results are bitwise reproducible.
 #pragma once
 #include "ck_common.cuh"
+#include "ck_layout.cuh"
 
 namespace ck {
 
@@ -84,7 +85,8 @@ __device__ __forceinline__ void team_sync() {
   else __syncthreads();
 }
 
-// Shared-memory work arrays of one team.
+// Shared-memory work arrays of one team (species_doubles: [red | X Gp Gm hRT |
+// cpR | wd]; a Jacobian continues with aT E u).
 // The Jacobian processes reactions in the chunks of its table (JacTab); the
 // right-hand side, which keeps one value per reaction, takes all reactions at
 // once or chunks of m.rhs_chunk.  Gp_k = 2^(g_k) and Gm_k = 2^(-g_k) with g_k =
@@ -99,11 +101,6 @@ struct TeamBufs {
   double* red;                            // [TEAM_RED_DOUBLES] reductions and scalars (SC_*)
   int vp;                                 // lanes that the species sums are grouped by (64 or 256)
 };
-
-// [red | X Gp Gm hRT | cpR | wd], species_doubles(S) doubles; a Jacobian
-// continues with aT E u (3 S).
-constexpr int TEAM_RED_DOUBLES = 64;
-__host__ __device__ __forceinline__ constexpr int species_doubles(int S) { return TEAM_RED_DOUBLES + 4 * (S + 1) + 2 * S; }
 
 __device__ __forceinline__ TeamBufs carve_bufs(double* base, int S, double* scratch, int chunk, int vp) {
   TeamBufs b;
@@ -139,12 +136,6 @@ enum : int {
 // Mixture quantities shared by the RHS and the Jacobian.
 struct Mix {
   double T, invT, log2T, rho, invrho, Wbar, Ctot;
-};
-
-// Where a right-hand side keeps its rates of progress: offset in shared
-// memory and how many at a time (all m.R, or m.rhs_chunk).
-struct RhsQ {
-  int off, chunk;
 };
 
 // Groups of 32 species (at most 4).
@@ -1002,12 +993,6 @@ __device__ __forceinline__ unsigned long long inf_key(double) { return 0x7ff0000
 __device__ __forceinline__ unsigned long long inf_key(float) { return 0x7f80000000000000ULL; }
 
 constexpr int LU_MAX_N = 144;
-
-// Distance of the rows of a factored matrix in shared memory: odd, so that
-// the lanes of a warp reading one column (a row each: the pivot search, the
-// substitutions) touch different banks.  At n = 112 every such load took 32
-// turns.
-__host__ __device__ __forceinline__ constexpr int lu_ld(int n) { return n | 1; }
 
 // Pivot k, by one warp: column k updated with pivot k - 1, the pivot of rows
 // k.., and the multipliers and row order of the rows below it.

@@ -136,42 +136,6 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
 
-// Room for a right-hand side's rates of progress (team_rhs, team_rhs_lat).
-__host__ __device__ __forceinline__ int rhs_doubles(const DevMech& d) {
-  return d.rhs_chunk + (d.S <= 32 ? d.R - d.first_typed : 0);
-}
-
-// Shared memory of one k_ros4 CTA, in doubles: the matrix, y and f(y), the team's work arrays, and the stage vectors,
-// the factors' row table and the rates of progress (or the LU's scratch).  The
-// Jacobian's per-reaction values lie over the matrix (wide: it is assembled in
-// device memory) or behind the work arrays, over the stage vectors.
-struct Ros4Layout {
-  int vp, yv, f0, bufs, jscr, yt, ub, invd, rof, lr;
-  RhsQ rhs_q;
-  size_t doubles;
-  __host__ __device__ Ros4Layout(const DevMech& d, bool wide) {
-    const int n = d.n, mat = n * lu_ld(n);
-    vp = n > 64 ? 256 : 64;
-    yv = wide && d.wide.scratch > mat ? d.wide.scratch : mat;
-    f0 = yv + n;
-    bufs = f0 + n;
-    const int t = bufs + species_doubles(d.S), tj = t + 3 * d.S;
-    jscr = wide ? 0 : tj;
-    yt = t;
-    ub = yt + n;
-    invd = ub + n;
-    rof = invd + n;
-    const int after = (rof + (n + 1) / 2 + 1) & ~1;  // 16-byte aligned
-    lr = after;
-    rhs_q.off = after;
-    rhs_q.chunk = d.rhs_chunk;
-    int most = wide ? tj : tj + d.narrow.scratch;
-    if (after + 4 * n > most) most = after + 4 * n;
-    if (after + rhs_doubles(d) > most) most = after + rhs_doubles(d);
-    doubles = (size_t)most;
-  }
-};
-
 // ------------------------------------------------------------------ launch helpers
 // Persistent grid: as many CTAs of `kernel` as fit on every SM (or the
 // caller's cap), at most one per work item.
