@@ -348,8 +348,8 @@ constexpr double RK_D1 = 16.0 / 135.0 - 25.0 / 216.0, RK_D3 = 6656.0 / 12825.0 -
 // state (n x n) and its diagonal (n).
 __host__ __device__ constexpr size_t ros4_scratch_doubles(int n) { return (size_t)n * n + (size_t)n; }
 
-// A reactor that the thread-per-reactor RKF45 hands to a team after
-// RK_THREAD_STEPS attempts (its state is in the caller's y).
+// A reactor that the thread-per-reactor RKF45 hands to a team part-way (its
+// state is in the caller's y).
 struct RkCont {
   double t, h;
   int32_t r, acc, rej;

@@ -75,7 +75,7 @@ CK_ROS4_TILE_LAUNCHER(launch_ros4_w4)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w4_lat)
 CK_ROS4_TILE_LAUNCHER(launch_ros4_w8)
 #undef CK_ROS4_TILE_LAUNCHER
-// may_alloc: hand reactors of many steps from their threads to teams through
+// may_alloc: hand a warp's last reactors from their threads to teams through
 // a stream-ordered list (mechanisms of at most 32 species); same results.
 cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,
                          double* h_io, const SolverParams& sp, int32_t* steps, int32_t* status,

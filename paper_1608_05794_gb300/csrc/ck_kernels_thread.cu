@@ -146,21 +146,26 @@ __device__ double h0_thread(const MechView& m, int n, double p, const double* y0
   return fmin(fmin(100.0 * ha, hb), tspan);
 }
 
-// Attempts after which a thread hands its reactor on, and how many reactors
-// may be.  Longer keeps more of the work where the lanes are full, but a warp
-// then runs on for its slowest lanes.  10 species over 1e-5 s (70 attempts a
-// reactor on average, 1900 at most), 100003 / 300000 reactors: 96 attempts 389
-// / 1051 ms, 128 372 / 906, 192 411 / 808, 320 536 / 889, never 670 / -; 160
-// (and the teams' latency form) 365 / 944.
-constexpr int RK_THREAD_STEPS = 160;
-constexpr int64_t RK_LIST_MAX = 1 << 18;
+// Once the queue is empty, a warp with this many reactors left or fewer hands
+// them on to teams.  A warp's step takes the same time however few of its lanes
+// are live; with all of them a full GPU of threads takes about five times the
+// steps of a full GPU of teams (100000 reactors of the 10-species mechanism,
+// 1000 fixed steps each: 1.61 s, teams alone 7.8), so that a team beats a lane
+// in a warp with less than a quarter of them.  10 species, never handed on / at
+// 4, 8, 12, 16, 24 lanes, ms: 100003 reactors over 1e-5 s 689 / 417, 415, 478,
+// 549, 655; 300000 1316 / 1161, 1080, 1143, 1241, 1428; 100000 over 1e-4 s 9154
+// / 2652, 2240, 2210, 2249, 2341; 30 species and 300 reactions, 80000 over 1e-6
+// s 904 / 309, 244, 205, 195, 176.  A count of attempts (160) instead: 397, 864,
+// 2358, 866, but reactors that all take more go to teams while the warps are
+// full (the fixed steps above: 7.8 s).
+constexpr int RK_HAND_ON_LANES = 8;
 
 // One lane integrates one reactor at a time and fetches the next reactor
 // from a global atomic counter as soon as it finishes (dynamic scheduling
 // with granularity one, per lane), so lanes of a warp never wait for a
-// slower neighbour beyond one step.  With a list, a reactor that is not done
-// after RK_THREAD_STEPS attempts is handed on (k_rkf45_tail): a step takes a
-// thread 410 us however few are left, a team 50.
+// slower neighbour beyond one step.  With a list, the last reactors of a warp
+// are handed on (k_rkf45_tail): a step takes a thread 410 us however few are
+// left, a team 50.
 template <int MAXS>
 __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int staged, int64_t N,
                                                const double* __restrict__ p, double* __restrict__ y,
@@ -286,8 +291,9 @@ __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int sta
           }
         }
         if (t >= tf) finish = true;
-        if (!finish && list && acc + rej >= RK_THREAD_STEPS) {
-          const int at = *count < cap ? atomicAdd(count, 1) : cap;
+        if (!finish && list && __popc(__activemask()) <= RK_HAND_ON_LANES &&
+            *static_cast<volatile int32_t*>(queue) >= N) {
+          const int at = atomicAdd(count, 1);
           if (at < cap) {
             for (int i = 0; i < n; ++i) y[r * n + i] = yv[i];
             list[at] = RkCont{t, h, (int32_t)r, acc, rej, (int16_t)last_rej, (int16_t)last_nf};
@@ -407,11 +413,12 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   if (blocks < 1) blocks = 1;
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  // the list of reactors handed on, behind its two counters (8 MB at most)
+  // the list of reactors handed on, behind its two counters: what all warps may
+  // hand on at once (32 bytes each)
   RkCont* list = nullptr;
   int32_t* count = nullptr;
-  const int list_cap = (int)(n < RK_LIST_MAX ? n : RK_LIST_MAX);
-  if (MAXS <= 32 && may_alloc && hm.R <= hm.d.rhs_chunk && n <= INT32_MAX) {
+  const int list_cap = blocks * (threads / 32) * RK_HAND_ON_LANES;
+  if (MAXS <= 32 && may_alloc && hm.R <= hm.d.rhs_chunk) {
     e = cudaMallocAsync(reinterpret_cast<void**>(&count), 16 + sizeof(RkCont) * (size_t)list_cap, st);
     if (e == cudaSuccess) {
       list = reinterpret_cast<RkCont*>(count + 4);
