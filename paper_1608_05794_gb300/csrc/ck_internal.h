@@ -83,7 +83,8 @@ cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double*
 // The teams' part: reactors list[0 .. min(*count, cap)); queue: a zeroed counter.
 cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
                               const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
-                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st);
+                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st,
+                              const LaunchCfg& cfg);
 
 cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, double* y,
                               const double* dt, double* h_io, const SolverParams& sp, int32_t* steps,

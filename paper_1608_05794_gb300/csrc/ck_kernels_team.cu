@@ -434,10 +434,10 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
 
 cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
                               const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
-                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st) {
+                              const RkCont* list, const int32_t* count, int cap, cudaStream_t st,
+                              const LaunchCfg& cfg) {
   const size_t smem = sizeof(double) * (8 * (size_t)hm.d.n + species_doubles(hm.S) + rhs_doubles(hm.d));
   const int threads = 128;
-  LaunchCfg cfg;
   const int grid = team_grid(k_rkf45_tail, threads, smem, cap, cfg);
   k_rkf45_tail<<<grid, threads, smem, st>>>(hm.d, p, y, dt, h_io, sp, steps, status, queue, list, count, cap);
   return cudaGetLastError();

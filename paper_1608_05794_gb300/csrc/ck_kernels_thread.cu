@@ -436,7 +436,7 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   }
   if (list) {
     if (e == cudaSuccess)
-      e = launch_rkf45_tail(hm, p, y, dt, h_io, sp, steps, status, count + 1, list, count, list_cap, st);
+      e = launch_rkf45_tail(hm, p, y, dt, h_io, sp, steps, status, count + 1, list, count, list_cap, st, cfg);
     const cudaError_t f = cudaFreeAsync(count, st);
     if (e == cudaSuccess) e = f;
   }
