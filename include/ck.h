@@ -164,7 +164,9 @@ int ck_free_mechanism(ck_mech* mech);
 int ck_mech_info(const ck_mech* mech, int32_t* n_species, int32_t* n_reactions);
 
 /* Right-hand side of Eqs. ydot/tdot for n reactors: dydt[i*(S+1)+0] = dT/dt,
- * dydt[i*(S+1)+1+k] = dY_k/dt.  p[n] Pa, y[n][S+1].  One thread per reactor. */
+ * dydt[i*(S+1)+1+k] = dY_k/dt.  p[n] Pa, y[n][S+1].  One CTA per reactor for
+ * small batches and for more than 64 species, else one thread; a reactor's
+ * result is bitwise the same in a batch of any size. */
 int ck_rhs(const ck_mech* mech, int64_t n, const double* p, const double* y, double* dydt,
            void* stream);
 

@@ -312,22 +312,20 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
     }
   }
   csr_ptr[S] = (int32_t)csr_rx.size();
-  // the same one slot at a time (mechanisms of at most 32 species, which a
-  // thread may integrate alone)
+  // the same one slot at a time (mechanisms of at most 64 species, which a
+  // thread may evaluate alone)
   std::vector<int32_t> slot_ptr(S + 1, 0);
   std::vector<CsrTerm> slot;
-  if (S <= 32)
+  if (S <= 64) {
+    std::vector<std::vector<CsrTerm>> of(S);
+    for (int i = 0; i < R; ++i)
+      for (int s = 0; s < 6; ++s)
+        if (rx[i].sp[s] != S) of[rx[i].sp[s]].push_back(CsrTerm{s < 3 ? -1.0 : 1.0, i, 0});
     for (int k = 0; k < S; ++k) {
-      for (int i = 0; i < R; ++i)
-        for (int s = 0; s < 6; ++s)
-          if (rx[i].sp[s] == k) {
-            CsrTerm t{};
-            t.nu = s < 3 ? -1.0 : 1.0;
-            t.rx = i;
-            slot.push_back(t);
-          }
+      slot.insert(slot.end(), of[k].begin(), of[k].end());
       slot_ptr[k + 1] = (int32_t)slot.size();
     }
+  }
   // team kernels walk the reactions in chunks: equal shares of at most what
   // the team's shared memory has room for
   const int n1 = S + 1;

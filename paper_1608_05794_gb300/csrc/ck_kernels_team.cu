@@ -12,17 +12,18 @@
 namespace ck {
 
 // ------------------------------------------------------------------ RHS (team)
-template <bool INT>
-__global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N,
+// ORD: the sums in the order of k_rhs (all reactions at once), with its bits.
+template <bool INT, bool ORD>
+__global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N, int chunk,
                                                   const double* __restrict__ p, const double* __restrict__ y,
                                                   double* __restrict__ f) {
   extern __shared__ __align__(16) double sm[];
   const int n = d.n;
-  const RhsQ qq{2 * n + species_doubles(d.S), d.rhs_chunk};
+  const RhsQ qq{2 * n + species_doubles(d.S), chunk};
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = y[r * n + i];
     team_sync();
-    team_rhs_any<INT, false, !INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
+    team_rhs_any<INT, ORD, !INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
     for (int i = threadIdx.x; i < n; i += blockDim.x) f[r * n + i] = sm[n + i];
   }
 }
@@ -317,16 +318,26 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_tail(const __grid_constant__ D
 }
 
 // ------------------------------------------------------------------ launchers
+// Room for all R rates (and, up to 32 species, the latency form's factors) of
+// a right-hand side by team.
+static size_t rhs_team_doubles(const HostMech& hm, int rates) {
+  return 2 * (size_t)hm.d.n + species_doubles(hm.S) + rates + (hm.S <= 32 ? hm.R - hm.d.first_typed : 0);
+}
+bool rhs_team_takes_all(const HostMech& hm) {
+  return rhs_team_doubles(hm, hm.R) <= (size_t)smem_doubles(4);
+}
+
 cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * (2 * (size_t)nn + species_doubles(hm.S) + rhs_doubles(hm.d));
-  const int threads = hm.S > 32 && nn <= 64 ? 96 : 128;
+  const int chunk = rhs_team_takes_all(hm) ? hm.R : hm.d.rhs_chunk;
+  const size_t smem = sizeof(double) * rhs_team_doubles(hm, chunk);
+  const int threads = hm.S > 32 && nn <= 65 ? 96 : 128;
   LaunchCfg cfg;
-  auto kern = hm.S > 32 ? k_rhs_team<true> : k_rhs_team<false>;
+  auto kern = hm.S > 64 ? k_rhs_team<true, false> : (hm.S > 32 ? k_rhs_team<true, true> : k_rhs_team<false, true>);
   const int grid = team_grid(kern, threads, smem, n, cfg);
-  kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, f);
+  kern<<<grid, threads, smem, st>>>(hm.d, n, chunk, p, y, f);
   return cudaGetLastError();
 }
 

@@ -6,6 +6,8 @@
 // TMA copy (cp.async.bulk + mbarrier); otherwise they are read through L1.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "ck_internal.h"
 #include "ck_thread.cuh"
 
@@ -370,8 +372,8 @@ static cudaError_t rhs_impl(const HostMech& hm, int64_t n, const double* p, cons
   auto kern = k_rhs<MAXS, INT>;
   const int threads = 128;
   size_t smem = 0;
+  const int64_t want = (n + threads - 1) / threads;
   const int staged = stage_pays(hm, kern, threads, &smem);
-  int64_t want = (n + threads - 1) / threads;
   int64_t cap = blocks_for(kern, threads, smem);
   int blocks = (int)(want < cap ? want : cap);
   if (blocks < 1) blocks = 1;
@@ -380,21 +382,37 @@ static cudaError_t rhs_impl(const HostMech& hm, int64_t n, const double* p, cons
 }
 
 // One reactor a thread only for batches that fill the SMs with threads: below
-// that a thread's serial chain through all reactions sets the time whatever
-// the batch, and one team a reactor is faster.  Measured on GB300 (thread /
-// team, us): 10 species 55 / 17 at 512 reactors, 55 / 58 at 4000, 55 / 198 at
-// 16000; 53 species 880 / 231 at 8000, 1992 / 1792 at 65536, 2983 / 3637 at
-// 131072; 111 species 3421 / 1247 at 20011, 6634 / 4933 at 80000.  Products in
-// integer arithmetic (mul_int) pay once the FP64 unit is the bound: 10 species
-// 55 -> 65 us at 16000, 711 -> 571 us at 300000; 53 species 3440 -> 2983 us.
+// that a thread's serial chain through all species and reactions sets the time
+// whatever the batch, and one team a reactor is faster.  Up to 64 species both
+// add in the same order, so that a reactor's bits do not depend on the batch;
+// above, teams take every batch (111 species, 20011 reactors: 1.10 ms against
+// 2.77).  Measured on GB300 (thread / team, us): 10 species 54 / 16 at 512
+// reactors, 54 / 52 at 3000, 54 / 96 at 6000; 53 species 708 / 284 at 8000, 1069
+// / 692 at 20000, 1389 / 1364 at 40000.  The line: reactors an SM at which both
+// took the same time were 21 (10 species, 20 reactions), 41 (100), 77 (280), 88
+// (600); 33 (20, 40), 85 (200); 54 (30, 60), 147 (300); 74 (40, 80), 166 (320);
+// 70 (50, 100); 82 (60, 120), 195 (480); 179 (53, 325), 214 (650), each with
+// half of the mass fractions zero, which costs teams more.  They grow with the
+// reactions, the faster the fewer, and up to 32 species with these; the two
+// formulas lie at or below them (91 against the 88).
+static bool rhs_by_team(const HostMech& hm, int64_t n) {
+  if (hm.S > 64) return true;
+  const double line =
+      hm.S > 32 ? std::fmin(35.0 + 0.35 * hm.R, 190.0) : (2.4 + 0.13 * hm.S) * std::sqrt((double)hm.R);
+  return (double)n < line * sm_count() && rhs_team_takes_all(hm);
+}
+
+// Products in integer arithmetic (mul_int) pay once the FP64 unit is the bound:
+// up to 32 species from 256 reactors an SM (10 species 55 -> 65 us at 16000
+// reactors, 711 -> 571 at 300000), above from 512 (53 species 3458 -> 3030 us at
+// 131072; 708 -> 884 at 8000, 40 species 339 -> 409 at 20000).
 cudaError_t launch_rhs(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                        cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const int64_t per_sm = n / sm_count();
-  if (hm.S > 64 || per_sm < (hm.S > 32 ? 512 : 26)) return launch_rhs_team(hm, n, p, y, f, st);
-  if (hm.S > 32) return rhs_impl<128, true>(hm, n, p, y, f, st);
-  if (per_sm < 256) return rhs_impl<32, false>(hm, n, p, y, f, st);
-  return rhs_impl<32, true>(hm, n, p, y, f, st);
+  if (rhs_by_team(hm, n)) return launch_rhs_team(hm, n, p, y, f, st);
+  const bool many = n / sm_count() >= (hm.S > 32 ? 512 : 256);
+  if (hm.S > 32) return many ? rhs_impl<128, true>(hm, n, p, y, f, st) : rhs_impl<128, false>(hm, n, p, y, f, st);
+  return many ? rhs_impl<32, true>(hm, n, p, y, f, st) : rhs_impl<32, false>(hm, n, p, y, f, st);
 }
 
 template <int MAXS>
@@ -405,8 +423,8 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   auto kern = k_rkf45<MAXS>;
   const int threads = 128;
   size_t smem = 0;
+  const int64_t want = (n + threads - 1) / threads;
   const int staged = stage_pays(hm, kern, threads, &smem);
-  int64_t want = (n + threads - 1) / threads;
   int64_t cap = blocks_for(kern, threads, smem);
   if (cfg.ctas_per_sm > 0) cap = (int64_t)cfg.ctas_per_sm * sm_count();
   int blocks = (int)(want < cap ? want : cap);

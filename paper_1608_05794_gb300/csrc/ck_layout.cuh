@@ -16,6 +16,13 @@ __host__ __device__ __forceinline__ constexpr int species_doubles(int S) { retur
 // turns.
 __host__ __device__ __forceinline__ constexpr int lu_ld(int n) { return n | 1; }
 
+// Dynamic shared memory, in doubles, with which `ctas` of them fit an SM: 228 KB
+// an SM and 227 KB a CTA, less the 1 KB that every CTA reserves and 80 bytes of
+// static shared memory (k_ros4's step control).
+__host__ __device__ __forceinline__ constexpr int smem_doubles(int ctas) {
+  return ((ctas > 1 ? 228 * 1024 / ctas - 1024 : 227 * 1024) - 80) / 8;
+}
+
 // Where a right-hand side keeps its rates of progress: offset in shared
 // memory and how many at a time (all m.R, or m.rhs_chunk).
 struct RhsQ {

@@ -666,7 +666,7 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
     // warps, and the warp that is left partly empty has the cheapest
     if (INT && in) {
       for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
-        team_reaction<false, INT>(m, m.rxn + base + li, x, b, tab, li, 0);
+        team_reaction<false, INT, ORD>(m, m.rxn + base + li, x, b, tab, li, 0);
     } else {
       for (int li = cnt - 1 - tid; li >= 0; li -= blockDim.x)
         team_reaction<false, false, ORD>(m, m.rxn + base + li, x, b, tab, li, 0);
