@@ -755,11 +755,13 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 }
 
 // The right-hand side of a kernel: LAT kernels (four warps, at most 32 species)
-// take the latency form where q holds all reactions.
+// take the latency form where q holds all reactions, and with ORD are launched
+// only then.
 template <bool INT, bool ORD, bool LAT>
 __device__ __forceinline__ void team_rhs_any(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
-  if (LAT && m.R <= qq.chunk) team_rhs_lat<ORD>(m, tab, p, y_o, f_o, bufs_o, qq.off);
+  if constexpr (LAT && ORD) team_rhs_lat<true>(m, tab, p, y_o, f_o, bufs_o, qq.off);
+  else if (LAT && m.R <= qq.chunk) team_rhs_lat<ORD>(m, tab, p, y_o, f_o, bufs_o, qq.off);
   else team_rhs<INT, ORD>(m, tab, p, y_o, f_o, bufs_o, vp, qq);
 }
 
