@@ -431,10 +431,12 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
   const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + rhs_doubles(hm.d));
-  // four warps shorten a step while the batch leaves the SMs room; two keep
-  // their lanes busier in one that does not (53 species, four / two warps: 300
-  // reactors 13.0 / 19.0 ms, 1000 23.4 / 26.5, 2000 41.5 / 39.1, 16384 278 / 268)
-  const int threads = nn > 64 || hm.S <= 32 || n < (int64_t)12 * sm_count() ? 128 : 64;
+  // four warps shorten a step while the batch, or the caller's cap, leaves the
+  // SMs room; two keep their lanes busier where neither does (53 species, four /
+  // two warps: 300 reactors 13.0 / 19.0 ms, 1000 23.4 / 26.5, 2000 41.5 / 39.1,
+  // 16384 278 / 268; 2000 capped at three CTAs an SM 18.3 / 23.1)
+  const bool room = n < (int64_t)12 * sm_count() || (cfg.ctas_per_sm > 0 && cfg.ctas_per_sm < 12);
+  const int threads = nn > 64 || hm.S <= 32 || room ? 128 : 64;
   auto kern = hm.S > 32 ? k_rkf45_team<true> : k_rkf45_team<false>;
   const int grid = team_grid(kern, threads, smem, n, cfg);
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
