@@ -14,12 +14,12 @@ namespace ck {
 // ------------------------------------------------------------------ RHS (team)
 // ORD: the sums in the order of k_rhs (all reactions at once), with its bits.
 template <bool INT, bool ORD>
-__global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N, int chunk,
+__global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N,
                                                   const double* __restrict__ p, const double* __restrict__ y,
                                                   double* __restrict__ f) {
   extern __shared__ __align__(16) double sm[];
   const int n = d.n;
-  const RhsQ qq{2 * n + species_doubles(d.S), chunk};
+  const RhsQ qq{2 * n + species_doubles(d.S), d.rhs_chunk};
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = y[r * n + i];
     team_sync();
@@ -299,15 +299,16 @@ static __device__ __forceinline__ void rkf45_team(const DevMech& d, int64_t N, c
   }
 }
 
+constexpr int RKF45_LAT_CTAS = 5;  // CTAs an SM of the latency form, by registers
 template <bool INT>
-__global__ void __launch_bounds__(128, INT ? 8 : 5) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N,
+__global__ void __launch_bounds__(128, INT ? 8 : RKF45_LAT_CTAS) k_rkf45_team(const __grid_constant__ DevMech d, int64_t N,
                                                        const double* __restrict__ p, double* __restrict__ y,
                                                        const double* __restrict__ dt, double* h_io, SolverParams sp,
                                                        int32_t* steps, int32_t* status, int32_t* queue) {
   rkf45_team<INT, false>(d, N, p, y, dt, h_io, sp, steps, status, queue, nullptr);
 }
 
-__global__ void __launch_bounds__(128, 5) k_rkf45_tail(const __grid_constant__ DevMech d,
+__global__ void __launch_bounds__(128, RKF45_LAT_CTAS) k_rkf45_tail(const __grid_constant__ DevMech d,
                                                        const double* __restrict__ p, double* __restrict__ y,
                                                        const double* __restrict__ dt, double* h_io, SolverParams sp,
                                                        int32_t* steps, int32_t* status, int32_t* queue,
@@ -318,26 +319,28 @@ __global__ void __launch_bounds__(128, 5) k_rkf45_tail(const __grid_constant__ D
 }
 
 // ------------------------------------------------------------------ launchers
-// Room for all R rates (and, up to 32 species, the latency form's factors) of
-// a right-hand side by team.
-static size_t rhs_team_doubles(const HostMech& hm, int rates) {
-  return 2 * (size_t)hm.d.n + species_doubles(hm.S) + rates + (hm.S <= 32 ? hm.R - hm.d.first_typed : 0);
+// Shared memory beside the rates, in doubles, and the CTAs an SM to leave room
+// for.
+static DevMech rhs_mech(const HostMech& hm, size_t* fixed) {
+  *fixed = 2 * (size_t)hm.d.n + species_doubles(hm.S);
+  return with_rates(hm, *fixed, 4);
 }
 bool rhs_team_takes_all(const HostMech& hm) {
-  return rhs_team_doubles(hm, hm.R) <= (size_t)smem_doubles(4);
+  size_t fixed;
+  return rhs_mech(hm, &fixed).rhs_chunk >= hm.R;
 }
 
 cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  const int nn = hm.d.n;
-  const int chunk = rhs_team_takes_all(hm) ? hm.R : hm.d.rhs_chunk;
-  const size_t smem = sizeof(double) * rhs_team_doubles(hm, chunk);
-  const int threads = hm.S > 32 && nn <= 65 ? 96 : 128;
+  size_t fixed;
+  const DevMech d = rhs_mech(hm, &fixed);
+  const size_t smem = sizeof(double) * (fixed + rhs_doubles(d));
+  const int threads = hm.S > 32 && hm.S <= 64 ? 96 : 128;
   LaunchCfg cfg;
   auto kern = hm.S > 64 ? k_rhs_team<true, false> : (hm.S > 32 ? k_rhs_team<true, true> : k_rhs_team<false, true>);
   const int grid = team_grid(kern, threads, smem, n, cfg);
-  kern<<<grid, threads, smem, st>>>(hm.d, n, chunk, p, y, f);
+  kern<<<grid, threads, smem, st>>>(d, n, p, y, f);
   return cudaGetLastError();
 }
 
@@ -425,12 +428,18 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
   return fn(hm, n, p, y, dt, h_io, sp, steps, status, queue, st, cfg, scratch, scratch_bytes, may_alloc);
 }
 
+// Shared memory of a team RKF45 beside its rates, in doubles: eight vectors and
+// the species arrays.
+static size_t rkf45_fixed(const HostMech& hm) { return 8 * (size_t)hm.d.n + species_doubles(hm.S); }
+
 cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, double* y,
                               const double* dt, double* h_io, const SolverParams& sp, int32_t* steps,
                               int32_t* status, int32_t* queue, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * (8 * (size_t)nn + species_doubles(hm.S) + rhs_doubles(hm.d));
+  const size_t fixed = rkf45_fixed(hm);
+  const DevMech d = with_rates(hm, fixed, hm.S > 32 ? 8 : RKF45_LAT_CTAS);
+  const size_t smem = sizeof(double) * (fixed + rhs_doubles(d));
   // four warps shorten a step while the batch, or the caller's cap, leaves the
   // SMs room; two keep their lanes busier where neither does (53 species, four /
   // two warps: 300 reactors 13.0 / 19.0 ms, 1000 23.4 / 26.5, 2000 41.5 / 39.1,
@@ -441,18 +450,24 @@ cudaError_t launch_rkf45_team(const HostMech& hm, int64_t n, const double* p, do
   const int grid = team_grid(kern, threads, smem, n, cfg);
   cudaError_t e = cudaMemsetAsync(queue, 0, sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  kern<<<grid, threads, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue);
+  kern<<<grid, threads, smem, st>>>(d, n, p, y, dt, h_io, sp, steps, status, queue);
   return cudaGetLastError();
+}
+
+bool rkf45_tail_takes(const HostMech& hm) {
+  return with_rates(hm, rkf45_fixed(hm), RKF45_LAT_CTAS).rhs_chunk >= hm.R;
 }
 
 cudaError_t launch_rkf45_tail(const HostMech& hm, const double* p, double* y, const double* dt, double* h_io,
                               const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue,
                               const RkCont* list, const int32_t* count, int cap, cudaStream_t st,
                               const LaunchCfg& cfg) {
-  const size_t smem = sizeof(double) * (8 * (size_t)hm.d.n + species_doubles(hm.S) + rhs_doubles(hm.d));
+  const size_t fixed = rkf45_fixed(hm);
+  const DevMech d = with_rates(hm, fixed, RKF45_LAT_CTAS);
+  const size_t smem = sizeof(double) * (fixed + rhs_doubles(d));
   const int threads = 128;
   const int grid = team_grid(k_rkf45_tail, threads, smem, cap, cfg);
-  k_rkf45_tail<<<grid, threads, smem, st>>>(hm.d, p, y, dt, h_io, sp, steps, status, queue, list, count, cap);
+  k_rkf45_tail<<<grid, threads, smem, st>>>(d, p, y, dt, h_io, sp, steps, status, queue, list, count, cap);
   return cudaGetLastError();
 }
 

@@ -436,7 +436,7 @@ static cudaError_t rkf45_impl(const HostMech& hm, int64_t n, const double* p, do
   RkCont* list = nullptr;
   int32_t* count = nullptr;
   const int list_cap = blocks * (threads / 32) * RK_HAND_ON_LANES;
-  if (MAXS <= 32 && may_alloc && hm.R <= hm.d.rhs_chunk) {
+  if (MAXS <= 32 && may_alloc && rkf45_tail_takes(hm)) {
     e = cudaMallocAsync(reinterpret_cast<void**>(&count), 16 + sizeof(RkCont) * (size_t)list_cap, st);
     if (e == cudaSuccess) {
       list = reinterpret_cast<RkCont*>(count + 4);

@@ -755,13 +755,11 @@ static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab
 }
 
 // The right-hand side of a kernel: LAT kernels (four warps, at most 32 species)
-// take the latency form where q holds all reactions, and with ORD are launched
-// only then.
+// take the latency form for mechanisms of few reactions, whose rates q holds all.
 template <bool INT, bool ORD, bool LAT>
 __device__ __forceinline__ void team_rhs_any(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
-  if constexpr (LAT && ORD) team_rhs_lat<true>(m, tab, p, y_o, f_o, bufs_o, qq.off);
-  else if (LAT && m.R <= qq.chunk) team_rhs_lat<ORD>(m, tab, p, y_o, f_o, bufs_o, qq.off);
+  if (LAT && latency_form(m)) team_rhs_lat<ORD>(m, tab, p, y_o, f_o, bufs_o, qq.off);
   else team_rhs<INT, ORD>(m, tab, p, y_o, f_o, bufs_o, vp, qq);
 }
 
@@ -799,7 +797,7 @@ static __device__ void team_jacobian(const DevMech& m, const JacTab& jt, const d
   Mix x;
   const int S = m.S, lda = jt.ld, na = m.n * lda, SG = species_groups(S);
   const int tid = (int)threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const bool lat = LAT && jt.n_chunks == 1;
+  const bool lat = LAT && latency_form(m);
   bool in = false;
   if (lat) team_species_lat<false, true>(m, p, y, b, x, tab, b.q, b.w);
   else in = team_species<false, INT>(m, p, y, b, x, tab);

@@ -137,6 +137,16 @@ static __device__ __noinline__ double team_h0(const DevMech& d, const double* ta
 }
 
 // ------------------------------------------------------------------ launch helpers
+// The mechanism for a kernel that keeps `fixed` doubles beside its rates of
+// progress: with all of them at once where that leaves room for `ctas` CTAs an
+// SM, else in the loader's chunks (the same sums in the same order).
+static inline DevMech with_rates(const HostMech& hm, size_t fixed, int ctas) {
+  DevMech d = hm.d;
+  if (hm.R > 0) d.rhs_chunk = hm.R;
+  if (fixed + rhs_doubles(d) > (size_t)smem_doubles(ctas)) d.rhs_chunk = hm.d.rhs_chunk;
+  return d;
+}
+
 // Persistent grid: as many CTAs of `kernel` as fit on every SM (or the
 // caller's cap), at most one per work item.
 template <class K>

@@ -24,9 +24,17 @@ def _dev(a):
     return torch.as_tensor(np.array(a, dtype=np.float64), device="cuda")
 
 
-def _both(ck, n, dt, opts, repeats=1):
-    """States, step counts and the best time of the call and of threads alone."""
-    gm = ck.load_mechanism(load_mechanism(CONFIGS["small"]["mech"]))
+def _both(ck, n, dt, opts, repeats=1, times=1):
+    """States, step counts and the best time of the call and of threads alone;
+    times: the mechanism's reactions several times over, at lower rates."""
+    m = load_mechanism(CONFIGS["small"]["mech"])
+    n_eff = len(m["eff_sp"])
+    m["eff_ptr"] = np.concatenate([m["eff_ptr"][:-1] + i * n_eff for i in range(times)] + [[times * n_eff]])
+    for k in ("reac", "prod", "rtype", "rev", "arrh", "arrh0", "eff_sp", "eff_val"):
+        m[k] = np.concatenate([m[k]] * times)
+    for k in ("arrh", "arrh0"):
+        m[k] = m[k] / np.array([times, 1.0, 1.0])
+    gm = ck.load_mechanism(m)
     y, p = reactor_states("small", n=n, seed_offset=61)
     y0, pd, dtd = _dev(y), _dev(p), _dev(dt)
     st = torch.empty(n, dtype=torch.int32, device="cuda")
@@ -61,7 +69,9 @@ def test_full_warps_keep_reactors_of_many_steps(ck):
     assert t < 1.5 * ts
 
 
+# 20 reactions: teams in the latency form; 80 in the general one
+@pytest.mark.parametrize("times", [1, 4])
 @pytest.mark.parametrize("n", [1, 8, 9, 33, 129, 5000])
-def test_same_bits_wherever_a_reactor_is_finished(ck, n):
-    (y, steps, _), (ys, ss, _) = _both(ck, n, np.geomspace(1e-7, 3e-5, n), ck.SolverOpts.make(form=1))
+def test_same_bits_wherever_a_reactor_is_finished(ck, n, times):
+    (y, steps, _), (ys, ss, _) = _both(ck, n, np.geomspace(1e-7, 1e-5, n), ck.SolverOpts.make(form=1), times=times)
     assert np.array_equal(y, ys) and np.array_equal(steps, ss)

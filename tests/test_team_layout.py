@@ -70,3 +70,41 @@ def test_every_accepted_size_fits_a_cta(layout):
         # the kernels without a matrix: eight vectors, the species arrays and the rates
         assert rates + 8 * (8 * (S + 1) + 64 + 4 * (S + 1) + 2 * S) <= MAX_SMEM - 256, (S, R, typed)
         assert 1 <= rhs <= max(R, 1) and 1 <= wide <= max(R, 1) and 1 <= narrow <= max(R, 1)
+
+
+def _ctas(size):
+    return 228 * 1024 // (size + 1024 + 80)
+
+
+def test_chunks_follow_the_shared_memory(layout):
+    # no step in the number of passes just above the sizes of any one mechanism:
+    # as many reactions at a time as the residency of the kernel leaves room for
+    sizes = [(S, R, R // 7) for S in (10, 23, 24, 40, 53, 58, 64, 80, 106, 111, 112, 128)
+             for R in (20, 200, 325, 340, 400, 650, 784, 785, 800, 852, 1568, 5000)]
+    for (S, R, typed), (rhs, wide, narrow, ros4, ros4_narrow, _) in zip(sizes, layout(sizes)):
+        n = S + 1
+        species = 64 + 4 * (S + 1) + 2 * S
+        before = (n * (n | 1) + 5 * n + (n + 1) // 2 + 1 + species) & ~1  # matrix, vectors, species arrays, row table
+        want = 8 if n <= 24 else (6 if n <= 64 else 2)
+        while want > 1 and _ctas(8 * (before + 4 * n)) < want:
+            want -= 1
+        assert _ctas(ros4) >= want and _ctas(ros4_narrow) >= want, (S, R)
+        # the separate Jacobian kernel's values
+        assert _ctas(8 * (9 * wide + 2 * n + species + 3 * S)) >= (8 if n <= 24 else (6 if n <= 64 else 2)), (S, R)
+        # one pass fewer would not have fitted
+        room = ((228 * 1024 // want - 1024 if want > 1 else 227 * 1024) - 80) // 8
+        fewer = lambda chunk: -(-R // (-(-R // chunk) - 1))  # noqa: E731
+        if rhs < R:
+            assert before + fewer(rhs) > room, (S, R)
+        if narrow < R:
+            assert n * (n | 1) + 2 * n + species + 3 * S + (9 * R + typed if fewer(narrow) >= R else 10 * fewer(narrow)) > room
+    assert [c[:2] for c in layout([(53, 325, 50), (53, 340, 52), (53, 380, 58)])] == [(325, 325), (340, 340), (380, 380)]
+    assert [c[:2] for c in layout([(111, 784, 120), (111, 785, 120), (111, 852, 130)])] == [(392, 784), (393, 785),
+                                                                                          (426, 852)]
+
+
+def test_latency_form_holds_all_reactions(layout):
+    # up to 32 species and 64 reactions the kernels take them in one pass
+    cases = [(S, R, typed) for S in (1, 2, 10, 23, 24, 25, 31, 32) for R in (1, 20, 63, 64) for typed in sorted({0, R // 7, R})]
+    for (S, R, typed), (rhs, wide, narrow, *_) in zip(cases, layout(cases)):
+        assert rhs == wide == narrow == R, (S, R, typed)
