@@ -48,7 +48,9 @@ __global__ void __launch_bounds__(P, MINB) k_jacobian(const __grid_constant__ De
 }
 
 // Forward-difference Jacobians (one CTA per reactor), as ROS4 builds them
-// with the forward-difference option at step size h[r].
+// with the forward-difference option at step size h[r].  INT: products in integer
+// arithmetic (111 species: 150 reactors 2.40 ms against 3.05).
+template <bool INT>
 __global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ DevMech d, int64_t N,
                                                      const double* __restrict__ p, const double* __restrict__ y,
                                                      const double* __restrict__ h, double rtol, double atol,
@@ -59,8 +61,8 @@ __global__ void __launch_bounds__(256) k_jacobian_fd(const __grid_constant__ Dev
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[ys + i] = y[r * n + i];
     team_sync();
-    team_jacobian_fd<false>(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, n, ys + 2 * n, ys + 3 * n, ys + 4 * n,
-                     n > 64 ? 256 : 64, qq);
+    team_jacobian_fd<INT>(d, d.tab, p[r], ys, h[r], rtol, atol, ys + n, sm, n, ys + 2 * n, ys + 3 * n, ys + 4 * n,
+                          n > 64 ? 256 : 64, qq);
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) jac[r * (int64_t)n * n + e] = sm[e];
     team_sync();
   }
@@ -361,10 +363,13 @@ cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, c
                                double rtol, double atol, double* jac, cudaStream_t st, const LaunchCfg& cfg) {
   if (n <= 0) return cudaSuccess;
   const int nn = hm.d.n;
-  const size_t smem = sizeof(double) * ((size_t)nn * nn + 4 * nn + species_doubles(hm.S) + rhs_doubles(hm.d));
+  const size_t fixed = (size_t)nn * nn + 4 * nn + species_doubles(hm.S);
+  const DevMech d = with_rates(hm, fixed, n <= sm_count() ? 1 : team_ctas(nn));
+  const size_t smem = sizeof(double) * (fixed + rhs_doubles(d));
   const int threads = nn <= 24 ? 64 : (nn <= 64 ? 96 : 256);
-  const int grid = team_grid(k_jacobian_fd, threads, smem, n, cfg);
-  k_jacobian_fd<<<grid, threads, smem, st>>>(hm.d, n, p, y, h, rtol, atol, jac);
+  auto kern = nn > 64 ? k_jacobian_fd<true> : k_jacobian_fd<false>;
+  const int grid = team_grid(kern, threads, smem, n, cfg);
+  kern<<<grid, threads, smem, st>>>(d, n, p, y, h, rtol, atol, jac);
   return cudaGetLastError();
 }
 

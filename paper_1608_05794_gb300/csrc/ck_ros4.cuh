@@ -348,7 +348,13 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
   const int nn = hm.d.n;
   auto kern = cfg.precision == 2 ? k_ros4<P, MINB, 2>
                                  : (cfg.precision == 1 ? k_ros4<P, MINB, 1> : k_ros4<P, MINB, 0>);
-  size_t smem = sizeof(double) * Ros4Layout(hm.d, true).doubles;
+  // with at most one reactor an SM, all rates of progress at once
+  DevMech d = hm.d;
+  if (n <= sm_count() && hm.R > 0) {
+    d.rhs_chunk = hm.R;
+    if (Ros4Layout(d, true).doubles > (size_t)smem_doubles(1)) d.rhs_chunk = hm.d.rhs_chunk;
+  }
+  size_t smem = sizeof(double) * Ros4Layout(d, true).doubles;
   int grid = team_grid(kern, P, smem, n, cfg);
   // per-CTA copies of J (every form) and the FP64 iteration matrices of
   // the precision form: the caller's scratch when it is large enough, else
@@ -366,10 +372,10 @@ cudaError_t launch_ros4_team(const HostMech& hm, int64_t n, const double* p, dou
   } else if (cfg.precision) {
     return cudaErrorNotSupported;
   } else {
-    smem = sizeof(double) * Ros4Layout(hm.d, false).doubles;
+    smem = sizeof(double) * Ros4Layout(d, false).doubles;
     grid = team_grid(kern, P, smem, n, cfg);
   }
-  kern<<<grid, P, smem, st>>>(hm.d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);
+  kern<<<grid, P, smem, st>>>(d, n, p, y, dt, h_io, sp, steps, status, queue, m64g);
   cudaError_t k = cudaGetLastError();
   if (owned) {
     cudaError_t f = cudaFreeAsync(m64g, st);
