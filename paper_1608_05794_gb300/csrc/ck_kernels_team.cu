@@ -120,9 +120,9 @@ __global__ void k_lu_solve(int64_t batch, int dim, const double* __restrict__ lu
   extern __shared__ __align__(16) double sm[];
   const int nn = dim * dim, ld = lu_ld(dim);
   double* A = sm;
-  double* invd = A + dim * ld;
+  double* invd = A + (dim - 1) * ld + dim;
   int* pv = reinterpret_cast<int*>(invd + dim);
-  double* x = invd + 2 * dim;
+  double* x = invd + dim + (dim + 1) / 2;
   const float rc = 1.0f / (float)dim;
   for (int64_t m = blockIdx.x; m < batch; m += gridDim.x) {
     load_matrix(A, ld, lu + m * nn, dim, rc);
@@ -378,9 +378,11 @@ cudaError_t launch_lu_factor(int64_t batch, int dim, double* a, int32_t* piv, in
   if (batch <= 0) return cudaSuccess;
   LaunchCfg cfg;
   const size_t smem = sizeof(double) * lu_doubles(dim);
-  // a warp alone needs no barriers and is enough for the smallest matrices;
-  // measured for 4096 matrices of 54: 96 threads 712 us, 128 680
-  const int threads = dim <= 24 ? 32 : (dim <= 64 ? 128 : 256);
+  // a warp alone needs no barriers and is enough for the smallest matrices,
+  // except in a batch that leaves the SMs room (24: 300 matrices 40 us with one
+  // warp, 32 with two; 1200 42 / 36; 2400 52 / 54); measured for 4096 matrices of
+  // 54: 96 threads 712 us, 128 680
+  const int threads = dim <= 24 ? (batch <= 8 * (int64_t)sm_count() ? 64 : 32) : (dim <= 64 ? 128 : 256);
   const int grid = team_grid(k_lu_factor, threads, smem, batch, cfg);
   k_lu_factor<<<grid, threads, smem, st>>>(batch, dim, a, piv, info);
   return cudaGetLastError();
@@ -389,9 +391,11 @@ cudaError_t launch_lu_factor(int64_t batch, int dim, double* a, int32_t* piv, in
 cudaError_t launch_lu_solve(int64_t batch, int dim, const double* lu, const int32_t* piv,
                             double* b, cudaStream_t st) {
   if (batch <= 0) return cudaSuccess;
-  const size_t smem = sizeof(double) * ((size_t)dim * lu_ld(dim) + 3 * dim);
+  const size_t smem = sizeof(double) * ((size_t)(dim - 1) * lu_ld(dim) + 3 * dim + (dim + 1) / 2);
   LaunchCfg cfg;
-  const int threads = dim <= 24 ? 32 : 128;  // one warp solves, all load
+  // one warp solves, all load: as many as leave the residency to shared memory
+  // (32: 4096 systems 35 us with 64 threads, 39 with 128; 54: 81 / 76)
+  const int threads = dim <= 24 ? 32 : (dim <= 40 ? 64 : 128);
   const int grid = team_grid(k_lu_solve, threads, smem, batch, cfg);
   k_lu_solve<<<grid, threads, smem, st>>>(batch, dim, lu, piv, b);
   return cudaGetLastError();

@@ -79,3 +79,26 @@ def test_rkf45_teams(ck, name, n):
         assert torch.equal(y, y[:8][torch.as_tensor(rows, device="cuda")])
         outs.append(y[:8].clone())
     assert all(torch.equal(outs[0], o) for o in outs[1:])
+
+
+# one, two and more warps a matrix, at the sizes where they change
+@pytest.mark.parametrize("dim", [1, 2, 24, 25, 40, 41, 54, 128])
+def test_lu_and_solve(ck, dim):
+    rng = np.random.default_rng(dim)
+    a0 = rng.standard_normal((8, dim, dim)) + 2.0 * np.eye(dim)
+    b0 = rng.standard_normal((8, dim))
+    outs = []
+    for n in (8, 8 * _sms(), 8 * _sms() + 1):
+        rows = np.arange(n) % 8
+        a, b = (torch.as_tensor(v[rows], device="cuda") for v in (a0, b0))
+        piv, info = (torch.empty(s, dtype=torch.int32, device="cuda") for s in ((n, dim), (n,)))
+        ck.lu_factor(a, piv, info)
+        ck.lu_solve(a, piv, b)
+        for v in (a, b, piv, info):
+            assert torch.equal(v, v[:8][torch.as_tensor(rows, device="cuda")])
+        outs.append([v[:8].clone() for v in (a, b, piv, info)])
+    for other in outs[1:]:
+        assert all(torch.equal(u, v) for u, v in zip(outs[0], other))
+    assert int(outs[0][3].abs().sum()) == 0
+    x = np.linalg.solve(a0, b0[:, :, None])[:, :, 0]
+    assert np.abs(outs[0][1].cpu().numpy() - x).max() <= 1e-12 * np.linalg.cond(a0).max() * np.abs(x).max()
