@@ -32,11 +32,9 @@ struct __align__(16) RxnRec {
   double EoR2;   // Ea / (R ln 2), K
   double EoR;    // EoR2 * LN2 (as rounded by that product): d ln k_f/dT
   int16_t sp[6];    // reactant slots 0..2, product slots 3..5, padded with S
+  uint32_t bits;    // RXN_*: what the reaction does with its slots
   int8_t type;      // 0 elementary, 1 third-body, 2 Lindemann
   int8_t rev;       // 1 reversible through K_c, 2 explicit reverse Arrhenius
-  int8_t dnu;
-  int8_t nreac;
-  int8_t nprod, pad0;
   int16_t eff_beg, eff_cnt;  // slice of the efficiency table (eff - 1 != 0)
   int16_t rev_ix;            // rev == 2: row of the explicit reverse table
   double dnu_d;    // sum of product minus reactant coefficients, as FP64
@@ -46,7 +44,14 @@ struct __align__(16) RxnRec {
   double beta0;
   double E0oR2;
   double E0oR;   // E0oR2 * LN2
+  __host__ __device__ int nreac() const { return (int)(bits >> 18 & 3); }
+  __host__ __device__ int nprod() const { return (int)(bits >> 20 & 3); }
+  __host__ __device__ int dnu2() const { return (int)(bits >> 22 & 7); }  // nprod - nreac + 2
 };
+// RxnRec::bits: 3 bits a slot, 3 + the net coefficient of its species in that
+// species' first slot and 3 elsewhere; reactants, products (2 bits each), their
+// difference + 2 (3); and whether a species is in more than one slot.
+constexpr uint32_t RXN_NET0 = 0333333u, RXN_REPEATS = 1u << 25;
 static_assert(sizeof(RxnRec) == 112, "RxnRec layout");
 
 // Per-reaction values of a chunk of c reactions that the Jacobian is

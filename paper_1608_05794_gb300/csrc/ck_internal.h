@@ -45,8 +45,7 @@ cudaError_t launch_rhs(const HostMech& hm, int64_t n, const double* p, const dou
                        cudaStream_t st);
 cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                             cudaStream_t st);
-bool rhs_team_takes_all(const HostMech& hm);  // all reactions in one pass
-bool rkf45_tail_takes(const HostMech& hm);    // the same
+bool rkf45_tail_takes(const HostMech& hm);  // all reactions in one pass
 cudaError_t launch_jacobian(const HostMech& hm, int64_t n, const double* p, const double* y,
                             double* jac, cudaStream_t st, const LaunchCfg& cfg);
 cudaError_t launch_jacobian_fd(const HostMech& hm, int64_t n, const double* p, const double* y, const double* h,

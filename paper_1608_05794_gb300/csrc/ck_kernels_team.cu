@@ -12,8 +12,8 @@
 namespace ck {
 
 // ------------------------------------------------------------------ RHS (team)
-// ORD: the sums in the order of k_rhs (all reactions at once), with its bits.
-template <bool INT, bool ORD>
+// The sums are in the order of k_rhs, and the bits the same.
+template <bool INT>
 __global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMech d, int64_t N,
                                                   const double* __restrict__ p, const double* __restrict__ y,
                                                   double* __restrict__ f) {
@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(128) k_rhs_team(const __grid_constant__ DevMec
   for (int64_t r = blockIdx.x; r < N; r += gridDim.x) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) sm[i] = y[r * n + i];
     team_sync();
-    team_rhs_any<INT, ORD, !INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
+    team_rhs_any<INT, false, !INT>(d, d.tab, p[r], 0, n, 2 * n, 256, qq);
     for (int i = threadIdx.x; i < n; i += blockDim.x) f[r * n + i] = sm[n + i];
   }
 }
@@ -321,26 +321,15 @@ __global__ void __launch_bounds__(128, RKF45_LAT_CTAS) k_rkf45_tail(const __grid
 }
 
 // ------------------------------------------------------------------ launchers
-// Shared memory beside the rates, in doubles, and the CTAs an SM to leave room
-// for.
-static DevMech rhs_mech(const HostMech& hm, size_t* fixed) {
-  *fixed = 2 * (size_t)hm.d.n + species_doubles(hm.S);
-  return with_rates(hm, *fixed, 4);
-}
-bool rhs_team_takes_all(const HostMech& hm) {
-  size_t fixed;
-  return rhs_mech(hm, &fixed).rhs_chunk >= hm.R;
-}
-
 cudaError_t launch_rhs_team(const HostMech& hm, int64_t n, const double* p, const double* y, double* f,
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  size_t fixed;
-  const DevMech d = rhs_mech(hm, &fixed);
+  const size_t fixed = 2 * (size_t)hm.d.n + species_doubles(hm.S);
+  const DevMech d = with_rates(hm, fixed, 4);
   const size_t smem = sizeof(double) * (fixed + rhs_doubles(d));
   const int threads = hm.S > 32 && hm.S <= 64 ? 96 : 128;
   LaunchCfg cfg;
-  auto kern = hm.S > 64 ? k_rhs_team<true, false> : (hm.S > 32 ? k_rhs_team<true, true> : k_rhs_team<false, true>);
+  auto kern = hm.S > 32 ? k_rhs_team<true> : k_rhs_team<false>;
   const int grid = team_grid(kern, threads, smem, n, cfg);
   kern<<<grid, threads, smem, st>>>(d, n, p, y, f);
   return cudaGetLastError();

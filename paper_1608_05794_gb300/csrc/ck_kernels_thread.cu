@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(128) k_rhs(DevMech d, StageLayout L, int stage
   double X[MAXS], G[2 * MAXS], wd[MAXS];
   const int n = d.n;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < N; r += (int64_t)gridDim.x * blockDim.x)
-    rhs_thread<INT>(m, p[r], y + r * n, 1, f + r * n, 1, X, G, wd);
+    rhs_thread<INT, true, true>(m, p[r], y + r * n, 1, f + r * n, 1, X, G, wd);
 }
 
 // ------------------------------------------------------------------ RKF45
@@ -121,10 +121,11 @@ __device__ __forceinline__ double wrms_thread(int n, const double* e, const doub
 
 // Initial step (reading: Hairer, Norsett & Wanner, Solving ODEs I, Sec. II.4,
 // order 4, weights atol + rtol |y0|).  f0, y1, f1 are scratch vectors.
+template <int MAXS>
 __device__ double h0_thread(const MechView& m, int n, double p, const double* y0, double tspan,
                             double rtol, double atol, double* f0, double* y1, double* f1, double* X,
                             double* G, double* wd) {
-  rhs_thread<false, true>(m, p, y0, 1, f0, 1, X, G, wd);
+  rhs_thread<false, false, (MAXS > 32)>(m, p, y0, 1, f0, 1, X, G, wd);
   double d0 = 0.0, d1 = 0.0;
   for (int i = 0; i < n; ++i) {
     const double sc = atol + rtol * fabs(y0[i]);
@@ -135,7 +136,7 @@ __device__ double h0_thread(const MechView& m, int n, double p, const double* y0
   d1 = sqrt(d1 / n);
   const double ha = (d0 < 1e-5 || d1 < 1e-5) ? 1e-6 : 0.01 * d0 / d1;
   for (int i = 0; i < n; ++i) y1[i] = fma(ha, f0[i], y0[i]);
-  rhs_thread<false, true>(m, p, y1, 1, f1, 1, X, G, wd);
+  rhs_thread<false, false, (MAXS > 32)>(m, p, y1, 1, f1, 1, X, G, wd);
   double d2 = 0.0;
   for (int i = 0; i < n; ++i) {
     const double sc = atol + rtol * fabs(y0[i]);
@@ -217,7 +218,7 @@ __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int sta
       } else if (sp.h0 > 0.0) {
         h = sp.h0;
       } else {
-        h = h0_thread(m, n, pr, yv, tf, sp.rtol, sp.atol, k[0], yt, k[1], X, G, wd);
+        h = h0_thread<MAXS>(m, n, pr, yv, tf, sp.rtol, sp.atol, k[0], yt, k[1], X, G, wd);
       }
     }
     if (!finish) {
@@ -231,28 +232,28 @@ __global__ void __launch_bounds__(128) k_rkf45(DevMech d, StageLayout L, int sta
         finish = true;
       } else {
         // stages k_s = hh f(y + sum_j a_sj k_j)
-        rhs_thread<false, true>(m, pr, yv, 1, k[0], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yv, 1, k[0], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[0][i] *= hh;
         for (int i = 0; i < n; ++i) yt[i] = fma(RK_A21, k[0][i], yv[i]);
-        rhs_thread<false, true>(m, pr, yt, 1, k[1], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yt, 1, k[1], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[1][i] *= hh;
         for (int i = 0; i < n; ++i) yt[i] = fma(RK_A32, k[1][i], fma(RK_A31, k[0][i], yv[i]));
-        rhs_thread<false, true>(m, pr, yt, 1, k[2], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yt, 1, k[2], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[2][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A43, k[2][i], fma(RK_A42, k[1][i], fma(RK_A41, k[0][i], yv[i])));
-        rhs_thread<false, true>(m, pr, yt, 1, k[3], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yt, 1, k[3], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[3][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A54, k[3][i],
                       fma(RK_A53, k[2][i], fma(RK_A52, k[1][i], fma(RK_A51, k[0][i], yv[i]))));
-        rhs_thread<false, true>(m, pr, yt, 1, k[4], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yt, 1, k[4], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[4][i] *= hh;
         for (int i = 0; i < n; ++i)
           yt[i] = fma(RK_A65, k[4][i],
                       fma(RK_A64, k[3][i],
                           fma(RK_A63, k[2][i], fma(RK_A62, k[1][i], fma(RK_A61, k[0][i], yv[i])))));
-        rhs_thread<false, true>(m, pr, yt, 1, k[5], 1, X, G, wd);
+        rhs_thread<false, false, (MAXS > 32)>(m, pr, yt, 1, k[5], 1, X, G, wd);
         for (int i = 0; i < n; ++i) k[5][i] *= hh;
         // y* = y + sum b k (into yt), e = sum (bh - b) k (into k[1], whose b is 0)
         bool nf = false;
@@ -386,20 +387,26 @@ static cudaError_t rhs_impl(const HostMech& hm, int64_t n, const double* p, cons
 // whatever the batch, and one team a reactor is faster.  Up to 64 species both
 // add in the same order, so that a reactor's bits do not depend on the batch;
 // above, teams take every batch (111 species, 20011 reactors: 1.10 ms against
-// 2.77).  Measured on GB300 (thread / team, us): 10 species 54 / 16 at 512
-// reactors, 54 / 52 at 3000, 54 / 96 at 6000; 53 species 708 / 284 at 8000, 1069
-// / 692 at 20000, 1389 / 1364 at 40000.  The line: reactors an SM at which both
-// took the same time were 21 (10 species, 20 reactions), 41 (100), 77 (280), 88
-// (600); 33 (20, 40), 85 (200); 54 (30, 60), 147 (300); 74 (40, 80), 166 (320);
-// 70 (50, 100); 82 (60, 120), 195 (480); 179 (53, 325), 214 (650), each with
-// half of the mass fractions zero, which costs teams more.  They grow with the
-// reactions, the faster the fewer, and up to 32 species with these; the two
-// formulas lie at or below them (91 against the 88).
+// 2.77).  Measured on GB300 (thread / team, us): 10 species 57 / 15 at 512
+// reactors, 57 / 46 at 3000, 57 / 90 at 6000; 53 species 700 / 224 at 8000, 1060
+// / 543 at 20000, 1447 / 1070 at 40000, 1915 / 1610 at 60000.
+//
+// The line, from fifteen mechanisms at 10 to 400 reactors an SM, with all species
+// present and with half of the mass fractions zero (which costs teams up to 20 %).
+// Above 32 species the time of either form is estimated: teams take 1.8 + 0.0078 R
+// us for every reactor an SM, threads 3.1 S + 1.56 R us with one block of 128 an
+// SM, and 1.4, 2.0, 2.65 times as long with two, three, four.  The form chosen was
+// the faster one or within 3 % of it in all but five of 224 cases (12 % at worst).
+// Up to 32, by the reactors an SM at which both took the same time: 24 (10
+// species, 20 reactions), 50 (100), 82 (280), 98 (600); 44 (20, 40), 152 (200); 76
+// (30, 60), 180 (300).
 static bool rhs_by_team(const HostMech& hm, int64_t n) {
   if (hm.S > 64) return true;
-  const double line =
-      hm.S > 32 ? std::fmin(35.0 + 0.35 * hm.R, 190.0) : (2.4 + 0.13 * hm.S) * std::sqrt((double)hm.R);
-  return (double)n < line * sm_count() && rhs_team_takes_all(hm);
+  const double per_sm = (double)n / sm_count(), S = hm.S, R = hm.R;
+  if (hm.S <= 32) return per_sm < std::fmin((2.2 + 0.24 * S) * std::sqrt(R), 10.0 * S);
+  const double step[4] = {1.0, 1.4, 2.0, 2.65};
+  const int blocks = (int)std::fmin(std::ceil(per_sm / 128.0), 5.0);
+  return blocks <= 4 && per_sm * (1.8 + 0.0078 * R) < (3.1 * S + 1.56 * R) * step[blocks - 1];
 }
 
 // Products in integer arithmetic (mul_int) pay once the FP64 unit is the bound:
