@@ -330,9 +330,10 @@ int sm_count() {
   return cached;
 }
 
+constexpr int STAGE_MAX = 200 * 1024;
 static bool stage_fits(const HostMech& hm, size_t* smem) {
   *smem = STAGE_HDR + hm.L.bytes;
-  return *smem <= 200 * 1024;
+  return *smem <= STAGE_MAX;
 }
 
 // Stage the tables in shared memory (one bulk copy a CTA) only when the
@@ -348,7 +349,8 @@ static int stage_pays(const HostMech& hm, K kernel, int threads, size_t* smem) {
     *smem = 0;
     return 0;
   }
-  if (*smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  // (the same limit in every call, whatever other threads launch)
+  if (*smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGE_MAX);
   int with = 0, without = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&with, kernel, threads, *smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&without, kernel, threads, 0);

@@ -151,7 +151,10 @@ static inline DevMech with_rates(const HostMech& hm, size_t fixed, int ctas) {
 // caller's cap), at most one per work item.
 template <class K>
 static inline int team_grid(K kernel, int threads, size_t smem, int64_t work, const LaunchCfg& cfg) {
-  if (smem > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the same limit in every call: another thread may be about to launch this
+  // kernel with more
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(double) * smem_doubles(1));
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
   if (per_sm < 1) per_sm = 1;
