@@ -252,13 +252,16 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
       nr += d->reac[i * 3 + s] >= 0;
       np += d->prod[i * 3 + s] >= 0;
     }
-    r.bits = RXN_NET0 + ((uint32_t)nr << 18) + ((uint32_t)np << 20) + ((uint32_t)(np - nr + 2) << 22);
-    for (int s = 0; s < 6; ++s) {
-      if (r.sp[s] == S) continue;
-      const int at = (int)(std::find(r.sp, r.sp + s, r.sp[s]) - r.sp);  // the species' first slot
-      r.bits += (s < 3 ? -1u : 1u) << 3 * at;
-      if (at != s) r.bits |= RXN_REPEATS;
-    }
+    auto same = [&](const int16_t* a, int n) {
+      const bool s01 = n > 1 && a[0] == a[1], s02 = n > 2 && a[0] == a[2], s12 = n > 2 && a[1] == a[2];
+      return s01 && s12 ? REP_ALL : s01 ? REP_01 : s02 ? REP_02 : s12 ? REP_12 : REP_NONE;
+    };
+    r.repeats = (uint8_t)(same(r.sp, nr) | same(r.sp + 3, np) << 3);
+    for (int s = 0; s < nr; ++s)
+      if (std::find(r.sp + 3, r.sp + 3 + np, r.sp[s]) != r.sp + 3 + np) r.repeats |= REP_BOTH_SIDES;
+    r.nreac = (int8_t)nr;
+    r.nprod = (int8_t)np;
+    r.dnu = (int8_t)(np - nr);
     r.dnu_d = (double)(np - nr);
     r.nreac_d = (double)nr;
     r.nprod_d = (double)np;
@@ -394,9 +397,9 @@ int ck_load_mechanism(const ck_mech_desc* d, ck_mech** out) {
             // coefficients carry W_k / W_j, the factor of the species block
             // dY_k/dY_j (so the assembly needs no per-entry rescaling)
             const double* wr = &w_ratio[(size_t)k * S];
-            for (int s2 = 0; s2 < r.nreac(); ++s2) term(k * S + r.sp[s2], nu * wr[r.sp[s2]], pbase + s2);
+            for (int s2 = 0; s2 < r.nreac; ++s2) term(k * S + r.sp[s2], nu * wr[r.sp[s2]], pbase + s2);
             if (r.rev)
-              for (int s2 = 0; s2 < r.nprod(); ++s2) term(k * S + r.sp[3 + s2], nu * wr[r.sp[3 + s2]], pbase + 3 + s2);
+              for (int s2 = 0; s2 < r.nprod; ++s2) term(k * S + r.sp[3 + s2], nu * wr[r.sp[3 + s2]], pbase + 3 + s2);
             for (int q = r.eff_beg; q < r.eff_beg + r.eff_cnt; ++q)
               term(k * S + eff_sp[q], nu * eff_m1[q] * wr[eff_sp[q]], pw);
             const int sb = S * S + k;
@@ -830,10 +833,10 @@ double rhs_count(const ck::HostMech& hm) {
   // 2^(+-g_k) (8 each) per species
   double c = 20.0 + 40.0 * hm.S;
   for (const auto& r : hm.rx) {
-    c += 2 + 8 + (r.nreac() - 1) + 1 + (r.nreac() + r.nprod());
+    c += 2 + 8 + (r.nreac - 1) + 1 + (r.nreac + r.nprod);
     // 1/K_c as a product of species factors, then k_r and the reverse product
-    if (r.rev == 1) c += 1 + (r.nreac() + r.nprod()) + 1 + (r.nprod() - 1) + 1;
-    if (r.rev == 2) c += 2 + 8 + (r.nprod() - 1) + 1;
+    if (r.rev == 1) c += 1 + (r.nreac + r.nprod) + 1 + (r.nprod - 1) + 1;
+    if (r.rev == 2) c += 2 + 8 + (r.nprod - 1) + 1;
     if (r.type) c += r.eff_cnt + 1;
     if (r.type == 2) c += 2 + 1 + 8 + 1 + 1 + 1 + 1;
   }
@@ -851,11 +854,11 @@ double jac_count(const ck::HostMech& hm) {
   double c = 4.0 * S + S * S + S * S + 14.0 * S + 30.0;
   for (const auto& r : hm.rx) {
     double per = 3 + 3 + 4 + 1 + 6 + 1;  // dlnkf, c k, w, D, dq/dT
-    if (r.rev == 1) per += (r.nreac() + r.nprod()) + 2;
+    if (r.rev == 1) per += (r.nreac + r.nprod) + 2;
     if (r.rev == 2) per += 2;
     if (r.type == 2) per += 7;
-    per += (r.nreac() == 2 ? 2 : (r.nreac() == 3 ? 6 : 0));
-    if (r.rev) per += (r.nprod() == 2 ? 2 : (r.nprod() == 3 ? 6 : 1));
+    per += (r.nreac == 2 ? 2 : (r.nreac == 3 ? 6 : 0));
+    if (r.rev) per += (r.nprod == 2 ? 2 : (r.nprod == 3 ? 6 : 1));
     c += per;
   }
   c += hm.n_contrib;          // one FMA per contribution
@@ -886,15 +889,15 @@ Ops rhs_ops(const ck::HostMech& hm) {
   for (const auto& r : hm.rx) {
     o.fma += 2;           // log2 k_f
     o.transc += 1;        // k_f
-    o.other += r.nreac() - 1;  // forward product
+    o.other += r.nreac - 1;  // forward product
     if (r.rev == 1) {
-      o.other += (r.nreac() + r.nprod()) - (r.dnu2() == 2 ? 1 : 0) + (r.dnu2() % 4 == 0 ? 1 : 0) + 1 + (r.nprod() - 1);
+      o.other += (r.nreac + r.nprod) - (r.dnu == 0 ? 1 : 0) + (std::abs((int)r.dnu) == 2 ? 1 : 0) + 1 + (r.nprod - 1);
       o.other += 1;
       o.fma += 1;         // q = k_f prod' - k_r prod''
     } else if (r.rev == 2) {
       o.fma += 2;
       o.transc += 1;
-      o.other += (r.nprod() - 1) + 1;
+      o.other += (r.nprod - 1) + 1;
       o.fma += 1;
     } else {
       o.other += 1;
@@ -921,7 +924,7 @@ Ops jac_ops(const ck::HostMech& hm) {
   for (const auto& r : hm.rx) {
     o.fma += 1;           // d ln k_f / dT
     o.other += 2;
-    if (r.rev == 1) o.other += r.nreac() + r.nprod() + 1;      // d ln K_c / dT
+    if (r.rev == 1) o.other += r.nreac + r.nprod + 1;      // d ln K_c / dT
     if (r.rev == 2) {
       o.fma += 1;
       o.other += 3;
@@ -931,8 +934,8 @@ Ops jac_ops(const ck::HostMech& hm) {
       o.other += 8;       // d ln k0/dT, dc/dT, dc/d[M]
     }
     o.other += 2 + (r.type ? 1 : 0);  // c k_f, c k_r, dc/d[M] net
-    o.other += (r.nreac() == 2 ? 2 : (r.nreac() == 3 ? 6 : 0));
-    if (r.rev) o.other += (r.nprod() == 2 ? 2 : (r.nprod() == 3 ? 6 : 0));
+    o.other += (r.nreac == 2 ? 2 : (r.nreac == 3 ? 6 : 0));
+    if (r.rev) o.other += (r.nprod == 2 ? 2 : (r.nprod == 3 ? 6 : 0));
     o.fma += r.type ? 2 : 1;  // D (Euler sum)
     o.other += 3;
     o.other += 4;             // dq/dT at fixed [X]

@@ -32,9 +32,12 @@ struct __align__(16) RxnRec {
   double EoR2;   // Ea / (R ln 2), K
   double EoR;    // EoR2 * LN2 (as rounded by that product): d ln k_f/dT
   int16_t sp[6];    // reactant slots 0..2, product slots 3..5, padded with S
-  uint32_t bits;    // RXN_*: what the reaction does with its slots
   int8_t type;      // 0 elementary, 1 third-body, 2 Lindemann
   int8_t rev;       // 1 reversible through K_c, 2 explicit reverse Arrhenius
+  int8_t dnu;
+  int8_t nreac;
+  int8_t nprod;
+  uint8_t repeats;  // species in more than one slot: REP_*
   int16_t eff_beg, eff_cnt;  // slice of the efficiency table (eff - 1 != 0)
   int16_t rev_ix;            // rev == 2: row of the explicit reverse table
   double dnu_d;    // sum of product minus reactant coefficients, as FP64
@@ -44,15 +47,15 @@ struct __align__(16) RxnRec {
   double beta0;
   double E0oR2;
   double E0oR;   // E0oR2 * LN2
-  __host__ __device__ int nreac() const { return (int)(bits >> 18 & 3); }
-  __host__ __device__ int nprod() const { return (int)(bits >> 20 & 3); }
-  __host__ __device__ int dnu2() const { return (int)(bits >> 22 & 7); }  // nprod - nreac + 2
 };
-// RxnRec::bits: 3 bits a slot, 3 + the net coefficient of its species in that
-// species' first slot and 3 elsewhere; reactants, products (2 bits each), their
-// difference + 2 (3); and whether a species is in more than one slot.
-constexpr uint32_t RXN_NET0 = 0333333u, RXN_REPEATS = 1u << 25;
 static_assert(sizeof(RxnRec) == 112, "RxnRec layout");
+// RxnRec::repeats: which slots of a side hold the same species (reactants in the
+// low three bits, products in the next three), and whether a species is on both
+// sides.  REP_NET has 2 bits a slot, 6 a pattern: how often the species of a slot
+// is in the pattern's side, in its first slot, else 0.
+enum : uint8_t { REP_NONE = 0, REP_01 = 1, REP_02 = 2, REP_12 = 3, REP_ALL = 4, REP_BOTH_SIDES = 64 };
+constexpr uint32_t REP_NET = (1u | 1u << 2 | 1u << 4) | (2u | 1u << 4) << 6 | (2u | 1u << 2) << 12 |
+                             (1u | 2u << 2) << 18 | 3u << 24;
 
 // Per-reaction values of a chunk of c reactions that the Jacobian is
 // assembled from: q, dq/dT and D (c each), six partials a reaction (reactant

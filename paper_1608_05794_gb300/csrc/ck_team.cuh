@@ -308,7 +308,7 @@ __device__ __forceinline__ void team_reaction(const DevMech& m, const RxnRec* sr
     }
   } else if (r.rev) {
     // 1/K_c = (R T/p0)^dnu prod_reactants Gp prod_products Gm (Eq. kc)
-    double kci = mul_sel<INT>(b.red[SC_PW + r.dnu2()], b.Gp[s0]);
+    double kci = mul_sel<INT>(b.red[SC_PW + 2 + r.dnu], b.Gp[s0]);
     kci = mul_sel<INT>(kci, b.Gm[s3]);
     kci = mul_sel<INT>(kci, b.Gp[s1]);
     kci = mul_sel<INT>(kci, b.Gm[s4]);

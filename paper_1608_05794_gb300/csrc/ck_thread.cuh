@@ -70,9 +70,9 @@ __device__ __forceinline__ V tree_sum(int S, F value) {
 // INT: the products of concentrations and of Gibbs factors in integer
 // arithmetic, beside the FP64 unit (see mul_int).  TEAM: see rhs_thread; without
 // it, also, the powers of R T/p0 formed where they are used, for a kernel short
-// of registers.  WHOLE: a record's slots and bits in one 16-byte load, taken apart in
+// of registers.  WHOLE: a record's slots and kinds in two vector loads, taken apart in
 // registers, instead of loads that wait for each other: the right-hand side of 53
-// species 3050 -> 2925 us on 131072 reactors, RKF45 on 2000 325 -> 272 ms; the small
+// species 3050 -> 2960 us on 131072 reactors, RKF45 on 2000 325 -> 274 ms; the small
 // mechanisms' RKF45 lacks the registers (1000 fixed steps of 100000 reactors 1.60 ->
 // 1.71 s).
 template <bool INT, bool TEAM, bool WHOLE>
@@ -81,17 +81,19 @@ __device__ __forceinline__ void rates_thread(const MechView& m, double T, double
   const double up = T * R_OVER_P0, up2 = up * up, dw = invT * P0_OVER_R, dw2 = dw * dw;
   for (int i = 0; i < m.R; ++i) {
     const RxnRec& r = m.rx[i];
-    uint4 h{};  // slots and bits
     int sp[6];
+    int type, rev, dnu, nreac, nprod, repeats;
     if (WHOLE) {
-      h = *reinterpret_cast<const uint4*>(&r.sp);
+      const uint4 h = *reinterpret_cast<const uint4*>(r.sp);
+      const uint32_t g = *reinterpret_cast<const uint32_t*>(&r.nprod);
       sp[0] = h.x & 0xffff, sp[1] = h.x >> 16, sp[2] = h.y & 0xffff;
       sp[3] = h.y >> 16, sp[4] = h.z & 0xffff, sp[5] = h.z >> 16;
+      type = h.w & 255, rev = h.w >> 8 & 255, dnu = (int8_t)(h.w >> 16), nreac = h.w >> 24;
+      nprod = g & 255, repeats = g >> 8 & 255;
+    } else {
+      type = r.type, rev = r.rev, dnu = r.dnu, nreac = r.nreac, nprod = r.nprod, repeats = r.repeats;
     }
-    const uint32_t bits = WHOLE ? h.w : r.bits;
     auto slot = [&](int q) { return WHOLE ? sp[q] : (int)r.sp[q]; };
-    const int nreac = bits >> 18 & 3, nprod = bits >> 20 & 3, dnu = (int)(bits >> 22 & 7) - 2;
-    const int type = r.type, rev = r.rev;
     const double l2kf = fma(-r.EoR2, invT, fma(r.beta, log2T, r.lA2));
     const double kf = ck_exp2(l2kf, m.tab);
     double fwd = X[slot(0)];
@@ -132,20 +134,36 @@ __device__ __forceinline__ void rates_thread(const MechView& m, double T, double
         q = net * (TEAM ? Pr * __drcp_rn(__dadd_rn(1.0, Pr)) : Pr / __dadd_rn(1.0, Pr));
       }
     }
-    if (TEAM && (bits & RXN_REPEATS)) {  // a species in several slots: its net coefficient at once
-      auto add = [&](int k, int s) {
-        const int nu = (int)(bits >> 3 * s & 7) - 3;
+    if (TEAM && repeats) {  // a species in several slots: its net coefficient at once
+      auto add = [&](int k, int nu) {
         if (nu == 0) return;
         const int a = nu < 0 ? -nu : nu;  // 1.0, 2.0 or 3.0 and the sign
         const int hi = (a == 1 ? 0x3ff00000 : (a == 2 ? 0x40000000 : 0x40080000)) | (nu & (int)0x80000000);
         wd[k] = fma(__hiloint2double(hi, 0), q, wd[k]);
       };
-      add(slot(0), 0);
-      add(slot(1), 1);
-      add(slot(2), 2);
-      add(slot(3), 3);
-      add(slot(4), 4);
-      add(slot(5), 5);
+      const uint32_t rn = REP_NET >> 6 * (repeats & 7), pn = REP_NET >> 6 * (repeats >> 3 & 7);
+      if (repeats & REP_BOTH_SIDES) {
+        // (rare: how often the species of slot k is on the other side, less)
+        auto on = [&](int k, int from, int n) {
+          int c = slot(from) == k;
+          if (n > 1) c += slot(from + 1) == k;
+          if (n > 2) c += slot(from + 2) == k;
+          return c;
+        };
+        if (rn & 3) add(slot(0), on(slot(0), 3, nprod) - (int)(rn & 3));
+        if (nreac > 1 && (rn >> 2 & 3)) add(slot(1), on(slot(1), 3, nprod) - (int)(rn >> 2 & 3));
+        if (nreac > 2 && (rn >> 4 & 3)) add(slot(2), on(slot(2), 3, nprod) - (int)(rn >> 4 & 3));
+        if ((pn & 3) && !on(slot(3), 0, nreac)) add(slot(3), (int)(pn & 3));
+        if (nprod > 1 && (pn >> 2 & 3) && !on(slot(4), 0, nreac)) add(slot(4), (int)(pn >> 2 & 3));
+        if (nprod > 2 && (pn >> 4 & 3) && !on(slot(5), 0, nreac)) add(slot(5), (int)(pn >> 4 & 3));
+      } else {
+        add(slot(0), -(int)(rn & 3));
+        if (nreac > 1) add(slot(1), -(int)(rn >> 2 & 3));
+        if (nreac > 2) add(slot(2), -(int)(rn >> 4 & 3));
+        add(slot(3), (int)(pn & 3));
+        if (nprod > 1) add(slot(4), (int)(pn >> 2 & 3));
+        if (nprod > 2) add(slot(5), (int)(pn >> 4 & 3));
+      }
     } else {
       wd[slot(0)] -= q;
       if (nreac > 1) wd[slot(1)] -= q;
