@@ -209,8 +209,10 @@ int ck_integrate_ros4(const ck_mech* mech, int64_t n, const double* p, double* y
                       double* h_inout, const ck_solver_opts* opts, int32_t* steps, int32_t* status,
                       void* stream);
 /* Same with RKF45 (Sec. 2, App. B: six stages, fourth-order solution
- * propagated, error = sum (bh - b) k).  One thread per reactor; each thread
- * takes the next reactor from the work queue when its reactor finishes. */
+ * propagated, error = sum (bh - b) k).  One CTA or one thread per reactor
+ * (opts.form); each takes the next reactor from the work queue when its reactor
+ * finishes, and the last reactors of a warp of threads are finished by CTAs (at
+ * most 32 species; the same results). */
 int ck_integrate_rkf45(const ck_mech* mech, int64_t n, const double* p, double* y, const double* dt,
                        double* h_inout, const ck_solver_opts* opts, int32_t* steps, int32_t* status,
                        void* stream);

@@ -119,7 +119,7 @@ struct DevMech {
   const int32_t* csr_ptr; // [S+1] species -> (reaction, net nu) lists
   const CsrTerm* csr;     // [csr_nnz]
   const int32_t* slot_ptr;  // [S+1] species -> its reaction slots one by one, -1 a reactant, +1 a product,
-  const CsrTerm* slot;      // in the order in which rhs_thread adds them
+  const CsrTerm* slot;      // in the order in which RKF45's threads add them (at most 32 species)
   const double* tab;      // [256] 2^(j/256)
   const double* revp;     // [n_rev][3] explicit reverse: log2 A_r, beta_r, Ea_r / (R ln 2)
   // A right-hand side whose team has no room for all R rates takes the

@@ -67,15 +67,15 @@ cudaError_t launch_ros4(const HostMech& hm, int64_t n, const double* p, double* 
 size_t ros4_scratch_bytes_max();
 // launch_ros4 for one team size (warps), each in its own translation unit
 // (ck_ros4_wN.cu).
-#define CK_ROS4_TILE_LAUNCHER(NAME)                                                                          \
+#define CK_ROS4_TEAM_LAUNCHER(NAME)                                                                          \
   cudaError_t NAME(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt, double* h_io, \
                    const SolverParams& sp, int32_t* steps, int32_t* status, int32_t* queue, cudaStream_t st,   \
                    const LaunchCfg& cfg, double* scratch, size_t scratch_bytes, bool may_alloc);
-CK_ROS4_TILE_LAUNCHER(launch_ros4_w2)
-CK_ROS4_TILE_LAUNCHER(launch_ros4_w4)
-CK_ROS4_TILE_LAUNCHER(launch_ros4_w4_lat)
-CK_ROS4_TILE_LAUNCHER(launch_ros4_w8)
-#undef CK_ROS4_TILE_LAUNCHER
+CK_ROS4_TEAM_LAUNCHER(launch_ros4_w2)
+CK_ROS4_TEAM_LAUNCHER(launch_ros4_w4)
+CK_ROS4_TEAM_LAUNCHER(launch_ros4_w4_lat)
+CK_ROS4_TEAM_LAUNCHER(launch_ros4_w8)
+#undef CK_ROS4_TEAM_LAUNCHER
 // may_alloc: hand a warp's last reactors from their threads to teams through
 // a stream-ordered list (mechanisms of at most 32 species); same results.
 cudaError_t launch_rkf45(const HostMech& hm, int64_t n, const double* p, double* y, const double* dt,

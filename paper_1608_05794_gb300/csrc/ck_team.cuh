@@ -149,8 +149,8 @@ __device__ __forceinline__ int species_groups(int S) { return (S + 31) >> 5; }
 // Ends with a barrier and returns (the same in every thread) whether the
 // ranges allow the reactions' products to be taken in integer arithmetic
 // (mul_int).
-// ORD: the species sums one species after another, as a thread that evaluates
-// a reactor alone takes them (rhs_thread), instead of by trees.
+// ORD: the species sums one species after another, as the threads of RKF45 take
+// them (rhs_thread without TEAM), instead of by trees.
 template <bool ORD, bool INT>
 __device__ __forceinline__ bool team_species(const DevMech& m, double p, const double* y,
                                              TeamBufs& b, Mix& x, const double* tab) {
@@ -282,7 +282,7 @@ __device__ __forceinline__ RxnRec load_rxn(const RxnRec* src) {
 // same instructions.  INT: the products of concentrations and of Gibbs factors
 // in integer arithmetic, beside the FP64 unit, which bounds the team kernels
 // (10 of the 23 FP64 instructions of a rate, 20 of 49 with its derivatives).
-// ORD: the fall-off factor by a division, as rhs_thread forms it.  PRE: k_f
+// ORD: the fall-off factor by a division, as RKF45's threads form it.  PRE: k_f
 // is at hand in b.q[i], and in b.w[iw] k_0/k_inf (JAC) or the whole factor of the
 // net rate (team_species_lat).
 template <bool JAC, bool INT, bool ORD = false, bool PRE = false>
@@ -642,8 +642,9 @@ static __device__ __noinline__ void team_rhs_lat(const DevMech& m, const double*
 // operations (a product is 106 cycles of it in integers, 72 in FP64: ROS4 on
 // 512 reactors of the 10-species mechanism, 245 against 230 ms) or is short of
 // registers (ROS4 on 4096 of the 53-species one, 617 against 600 ms).
-// ORD: every sum in the order of rhs_thread, whose values it then returns bit
-// for bit (one pass over all reactions: qq.chunk >= m.R).
+// ORD: every sum in the order of RKF45's threads (rhs_thread without TEAM), whose
+// values it then returns bit for bit (one pass over all reactions: qq.chunk >=
+// m.R).
 template <bool INT, bool ORD = false>
 static __device__ __noinline__ void team_rhs(const DevMech& m, const double* tab, double p, int y_o, int f_o,
                                              int bufs_o, int vp, RhsQ qq) {
